@@ -16,7 +16,10 @@ struct pcf_ctx {
   int mode_thr = 128;    // threads per CTA of the single per-mode kernel
   int thr_ya = 256, thr_yy = 128;  // threads per CTA of the split analysis and synthesis
   bool mixed = false;    // mixed-precision form (FP32 planes, split-BF16 Chebyshev, FP64 solves)
-  int plane_kind = 0;    // arithmetic of the x-z plane kernels: 0 FP64, 1 FP32, 2 float-float
+  int plane_kind = 0;    // 0 FP64 form, 1 mixed form, 2 float-float form
+  // fixed-point plane kernels: threads per CTA; some side above 64
+  int thr_synth = 64, thr_prod = 64;
+  bool plane_big = false;
   bool plane_warp = false;  // FP32 plane kernels with the transforms in warp registers
   bool tc05 = false;        // Chebyshev contractions of the mixed form on tcgen05 (else mma.sync)
   // descent steps in the symmetric subspace run the per-mode kernels on the modes m >= 0 only

@@ -364,30 +364,27 @@ std::vector<double2> make_twiddles(int L) {
   return w;
 }
 
-// Tangent form of the twiddles w^q = c + i s (w = e^{-2 pi i/L}) for the FMA butterflies:
-// w^q = m (1 + i t) with t = s/c, m = c where |c| >= |s|; else w^q = m i (1 + i t) with
-// m = s, t = -c/s (rot = 1).  |t| <= 1 either way.  rot[q] = 1 exactly where the angle's
-// distance to the nearest multiple of pi exceeds pi/4: 2q mod L in (L/4, 3L/4), decided in
-// integers.  tan[0, L): w^q; tan[L, 2L): its conjugate c - i s (t -> -t, and m -> -m where
-// rot = 1).
-void make_tangent_twiddles(int L, std::vector<double2>* tan, std::vector<unsigned char>* rot) {
-  tan->assign(2 * (size_t)L, make_double2(0.0, 0.0));
-  rot->assign(L, 0);
+// Fixed-point twiddles: e^{-2 pi i q/L}, then their conjugates, in units of 2^-62 split into a
+// high word and a signed low word.
+std::vector<fxtw> make_fx_twiddles(int L) {
+  auto split = [](long double v, int* h, int* l) {
+    const long long z = std::llrint(std::ldexp(v, 62));
+    int lo = (int)(uint32_t)(uint64_t)z;
+    *h = (int)((z - lo) >> 32);
+    *l = lo == INT32_MIN ? lo + 1 : lo;  // its negative is a word too
+  };
+  std::vector<fxtw> w(2 * (size_t)L);
   for (int q = 0; q < L; ++q) {
-    const double a = -2.0 * kPi * (double)q / (double)L;
-    const double c = std::cos(a), s = std::sin(a);
-    const int r2 = (2 * q) % L;
-    const bool r = 4 * r2 > L && 4 * r2 < 3 * L;
-    (*rot)[q] = r ? 1 : 0;
-    if (!r) {
-      (*tan)[q] = make_double2(s / c, c);
-      (*tan)[L + q] = make_double2(-s / c, c);
-    } else {
-      (*tan)[q] = make_double2(-c / s, s);
-      (*tan)[L + q] = make_double2(c / s, -s);
-    }
+    const long double a = -2.0L * 3.14159265358979323846264338327950288L * q / L;
+    split(std::cos(a), &w[q].ch, &w[q].cl);
+    split(std::sin(a), &w[q].sh, &w[q].sl);
+    w[L + q] = w[q];
+    split(-std::sin(a), &w[L + q].sh, &w[L + q].sl);
   }
+  return w;
 }
+// floor(2^32/d) + 1: __umulhi(t, .) = t / d for t d < 2^32
+unsigned div_mul(int d) { return (unsigned)((1ULL << 32) / (unsigned)d) + 1u; }
 
 template <class T>
 cudaError_t upload(const std::vector<T>& h, T** d) {
@@ -414,7 +411,9 @@ pcf_status push_descriptors(pcf_ctx* c) {
   return PCF_OK;
 }
 
-LaunchInfo li_of(pcf_ctx* c, const int* pre) { return LaunchInfo{c->dinst, pre, c->B}; }
+LaunchInfo li_of(pcf_ctx* c, const int* pre, int ctas = 0) {
+  return LaunchInfo{c->dinst, pre, c->B, c->uniform ? ctas / c->B : 0};
+}
 
 // kernel launch with optional per-class event timing
 template <class F>
@@ -439,9 +438,9 @@ pcf_status timed(pcf_ctx* c, int cls, F&& launch) {
   return PCF_OK;
 }
 
-pcf_status launch_mode(pcf_ctx* c, int op, int sig, int step_index) {
+pcf_status launch_mode(pcf_ctx* c, int op, int sig) {
   return timed(c, op == MODE_PHI ? 3 : (op == MODE_SYNTH_ONLY ? 0 : 6), [&] {
-    k_mode<<<c->cta_mode, c->mode_thr, c->sm_mode, c->cs>>>(li_of(c, c->pre_mode), op, sig, c->mpc, step_index);
+    k_mode<<<c->cta_mode, c->mode_thr, c->sm_mode, c->cs>>>(li_of(c, c->pre_mode), op, sig, c->mpc);
   });
 }
 pcf_status launch_synth(pcf_ctx* c, int slot, int nf) {
@@ -449,22 +448,34 @@ pcf_status launch_synth(pcf_ctx* c, int slot, int nf) {
   const int ctas = nf == kFieldsSynth ? c->cta_synth11 : c->cta_synth3;
   return timed(c, slot == 0 ? 1 : 4, [&] {
     if (c->plane_warp) launch_xzsynth_warp(ctas, c->sm_synth, c->cs, li_of(c, pre), slot, nf);
-    else launch_xzsynth(c->plane_kind, ctas, c->sm_synth, c->cs, li_of(c, pre), slot, nf);
+    else if (c->mixed) launch_xzsynth(ctas, c->sm_synth, c->cs, li_of(c, pre), slot, nf);
+    else launch_xzsynth_fx(c->plane_big, ctas, c->thr_synth, c->sm_synth, c->cs, li_of(c, pre, ctas), slot, nf);
   });
 }
 pcf_status launch_prodM(pcf_ctx* c) {
   return timed(c, 2, [&] {
     if (c->plane_warp) launch_prod_warp(false, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod), -1);
-    else launch_prod(c->plane_kind, false, c->suction, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod));
+    else if (c->mixed) launch_prod(false, c->suction, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod));
+    else
+      launch_prod_fx(c->plane_big, false, c->cta_prod, c->thr_prod, c->sm_prod, c->cs,
+                     li_of(c, c->pre_prod, c->cta_prod), -1);
   });
 }
 pcf_status launch_prodN(pcf_ctx* c, int step_index = -1) {
   return timed(c, 5, [&] {
     if (c->plane_warp) launch_prod_warp(true, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod), step_index);
+    else if (c->mixed)
+      launch_prod(true, c->suction, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod), step_index);
     else
-      launch_prod(c->plane_kind, true, c->suction, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod),
-                  step_index);
+      launch_prod_fx(c->plane_big, true, c->cta_prod, c->thr_prod, c->sm_prod, c->cs,
+                     li_of(c, c->pre_prod, c->cta_prod), step_index);
   });
+}
+
+// plane sums of the squared velocity of a slot
+void launch_plane_sums(pcf_ctx* c, int slot) {
+  if (c->mixed) launch_norm_planes(c->cta_synth3, c->cs, li_of(c, c->pre_synth3), slot);
+  else launch_norm_planes_fx(c->cta_synth3, c->cs, li_of(c, c->pre_synth3, c->cta_synth3), slot);
 }
 
 pcf_status launch_tc_synth(pcf_ctx* c, int slot) {
@@ -522,7 +533,7 @@ pcf_status launch_split_synth(pcf_ctx* c, int slot, int in_step, bool red = fals
 pcf_status launch_ysynth(pcf_ctx* c, int slot) {
   if (c->mixed) return launch_tc_synth(c, slot);
   if (c->split) return launch_split_synth(c, slot, 0);
-  return launch_mode(c, MODE_SYNTH_ONLY, slot, 0);
+  return launch_mode(c, MODE_SYNTH_ONLY, slot);
 }
 
 // projection onto the symmetric subspace: each instance's own mask (mask_override < 0) or mask
@@ -570,12 +581,12 @@ pcf_status step_body(pcf_ctx* c, int s) {
     PCF_TRY(launch_synth(c, 0, kFieldsSynth));
     PCF_TRY(launch_prodM(c));
     PCF_TRY(launch_tc_analysis(c));
-    PCF_TRY(launch_mode(c, MODE_PHI, 0, s));
+    PCF_TRY(launch_mode(c, MODE_PHI, 0));
     PCF_TRY(launch_tc_synth(c, 1));
     PCF_TRY(launch_synth(c, 1, kFieldsSynth));
     PCF_TRY(launch_prodN(c, s));  // with J, its history entry and the convergence mask
     PCF_TRY(launch_tc_analysis(c));
-    PCF_TRY(launch_mode(c, MODE_PSI_UPDATE, 1, -1));
+    PCF_TRY(launch_mode(c, MODE_PSI_UPDATE, 1));
     if (c->any_sym) PCF_TRY(launch_sym(c, -1));  // the next step's synthesis reads the projected state
     return PCF_OK;
   }
@@ -615,10 +626,10 @@ pcf_status step_body(pcf_ctx* c, int s) {
   }
   PCF_TRY(launch_synth(c, 0, kFieldsSynth));
   PCF_TRY(launch_prodM(c));
-  PCF_TRY(launch_mode(c, MODE_PHI, 0, s));
+  PCF_TRY(launch_mode(c, MODE_PHI, 0));
   PCF_TRY(launch_synth(c, 1, kFieldsSynth));
   PCF_TRY(launch_prodN(c, s));  // with J, its history entry and the convergence mask
-  PCF_TRY(launch_mode(c, MODE_PSI_UPDATE, 1, -1));
+  PCF_TRY(launch_mode(c, MODE_PSI_UPDATE, 1));
   if (c->any_sym) {
     PCF_TRY(launch_sym(c, -1));
     PCF_TRY(launch_ysynth(c, 0));
@@ -632,21 +643,21 @@ pcf_status step_body(pcf_ctx* c, int s) {
 pcf_status dns_body(pcf_ctx* c) {
   PCF_TRY(launch_synth(c, 0, kFieldsSynth));
   PCF_TRY(timed(c, 11, [&] {
-    launch_norm_planes(c->plane_kind, c->cta_synth3, c->cs, li_of(c, c->pre_synth3), 0);
+    launch_plane_sums(c, 0);
     launch_dns_norm(c->B, c->cs, c->dinst, c->d_dns);
     launch_dns_capture(c->dns_ctas, c->B, c->cs, c->dinst, c->d_dns);
   }));
   PCF_TRY(launch_prodM(c));
   if (c->mixed) {
     PCF_TRY(launch_tc_analysis(c));
-    PCF_TRY(launch_mode(c, MODE_PHI, 0, 0));
+    PCF_TRY(launch_mode(c, MODE_PHI, 0));
   } else if (c->split && c->fused) {
     PCF_TRY(launch_fused_step(c, MODE_PHI));
   } else if (c->split) {
     PCF_TRY(launch_split_analysis(c, MODE_PHI));
     PCF_TRY(launch_split_solve(c, MODE_PHI));
   } else {
-    PCF_TRY(launch_mode(c, MODE_PHI, 0, 0));
+    PCF_TRY(launch_mode(c, MODE_PHI, 0));
   }
   PCF_TRY(timed(c, 11, [&] { launch_dns_update(c->dns_ctas, c->B, c->cs, c->dinst, c->d_dns); }));
   if (c->any_sym) PCF_TRY(launch_sym(c, -1));
@@ -702,8 +713,7 @@ static bool params_ok(const pcf_params* prm) {
 struct GridTables {
   double *cheb, *rco, *ccw, *kx, *kz, *y, *ub, *tab0, *tab1, *dense0, *dense1;
   float2* cheb_ff = nullptr;
-  double2 *twx, *twz, *tanx, *tanz;
-  unsigned char *rotx, *rotz;
+  fxtw *twfx_x = nullptr, *twfx_z = nullptr;
   float2 *twxf = nullptr, *twzf = nullptr;
   uint16_t* tcA = nullptr;
   uint16_t* tcA5 = nullptr;
@@ -740,20 +750,17 @@ static pcf_status build_tables(pcf_ctx* c, const pcf_params* prm, GridTables* g)
   g->sig[0] = 1.0 / (nu * prm->dt);
   g->sig[1] = 1.0 / (nu * prm->dtau_hat);
   const std::vector<double> tab0 = make_mode_tables(N, kx, kz, g->sig[0], rco);
-  const std::vector<double2> twx = make_twiddles(nx), twz = make_twiddles(nz);
-  std::vector<double2> tanx, tanz;
-  std::vector<unsigned char> rotx, rotz;
-  make_tangent_twiddles(nx, &tanx, &rotx);
-  make_tangent_twiddles(nz, &tanz, &rotz);
   if (upload(cheb, &g->cheb) || upload(rco, &g->rco) || upload(ccw, &g->ccw) || upload(kx, &g->kx) ||
-      upload(kz, &g->kz) || upload(yg, &g->y) || upload(ub, &g->ub) || upload(twx, &g->twx) ||
-      upload(twz, &g->twz) || upload(tab0, &g->tab0) || upload(tanx, &g->tanx) || upload(tanz, &g->tanz) ||
-      upload(rotx, &g->rotx) || upload(rotz, &g->rotz))
+      upload(kz, &g->kz) || upload(yg, &g->y) || upload(ub, &g->ub) || upload(tab0, &g->tab0))
     return PCF_ECUDA;
   for (void* p : {(void*)g->cheb, (void*)g->rco, (void*)g->ccw, (void*)g->kx, (void*)g->kz, (void*)g->y,
-                  (void*)g->ub, (void*)g->twx, (void*)g->twz, (void*)g->tab0, (void*)g->tanx, (void*)g->tanz,
-                  (void*)g->rotx, (void*)g->rotz})
+                  (void*)g->ub, (void*)g->tab0})
     c->allocs.push_back(p);
+  if (prm->precision != PCF_MIXED) {
+    if (upload(make_fx_twiddles(nx), &g->twfx_x) || upload(make_fx_twiddles(nz), &g->twfx_z)) return PCF_ECUDA;
+    c->allocs.push_back(g->twfx_x);
+    c->allocs.push_back(g->twfx_z);
+  }
   std::vector<double> tab1;
   if (prm->dtau_hat == prm->dt) {
     g->tab1 = g->tab0;
@@ -774,7 +781,7 @@ static pcf_status build_tables(pcf_ctx* c, const pcf_params* prm, GridTables* g)
   }
   if (prm->precision == PCF_MIXED) {
     const std::vector<uint16_t> tcm = make_tc_matrices(N);
-    if (upload(to_float2(twx), &g->twxf) || upload(to_float2(twz), &g->twzf) || upload(tcm, &g->tcA))
+    if (upload(to_float2(make_twiddles(nx)), &g->twxf) || upload(to_float2(make_twiddles(nz)), &g->twzf) || upload(tcm, &g->tcA))
       return PCF_ECUDA;
     c->allocs.push_back(g->twxf);
     c->allocs.push_back(g->twzf);
@@ -1148,10 +1155,10 @@ static pcf_status time_mode_tiles(pcf_ctx* c, cudaEvent_t a, cudaEvent_t b, int*
   for (int mpc : cand) {
     if (set_mode_tiles(c, mpc) != PCF_OK) continue;
     PCF_TRY(push_descriptors(c));
-    k_mode<<<c->cta_mode, c->mode_thr, c->sm_mode, c->cs>>>(li_of(c, c->pre_mode), MODE_PHI, 0, mpc, 0);
+    k_mode<<<c->cta_mode, c->mode_thr, c->sm_mode, c->cs>>>(li_of(c, c->pre_mode), MODE_PHI, 0, mpc);
     PCF_CUDA(cudaEventRecord(a, c->cs));
     for (int r = 0; r < 3; ++r)
-      k_mode<<<c->cta_mode, c->mode_thr, c->sm_mode, c->cs>>>(li_of(c, c->pre_mode), MODE_PHI, 0, mpc, 0);
+      k_mode<<<c->cta_mode, c->mode_thr, c->sm_mode, c->cs>>>(li_of(c, c->pre_mode), MODE_PHI, 0, mpc);
     PCF_CUDA(cudaEventRecord(b, c->cs));
     PCF_CUDA(cudaEventSynchronize(b));
     float ms = 0.f;
@@ -1274,7 +1281,7 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
   }
 
   // per-instance workspace, one allocation per buffer kind
-  size_t n_yv = 0, n_ph = 0, n_xz = 0, n_np = 0, n_fr = 0;
+  size_t n_yv = 0, n_ph = 0, n_xz = 0, n_np = 0, n_fr = 0, n_pi = 0;
   c->state_off.assign(B + 1, 0);
   {
     int b = 0;
@@ -1286,6 +1293,7 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
         n_ph += 2ULL * kFieldsSynth * p.ny * p.nx * p.nz;
         n_xz += 3ULL * p.ny * nm;
         n_np += 3ULL * p.ny;
+        n_pi += 2ULL * kFieldsSynth * p.ny;
         n_fr += 6ULL * (p.ny + 1) * nm;
         c->state_off[b + 1] = c->state_off[b] + 3LL * nm * p.ny;
       }
@@ -1296,6 +1304,7 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
   float2 *yvf = nullptr, *xzf = nullptr, *xzc = nullptr;
   float* phf = nullptr;
   int* jc = nullptr;
+  int2* pin = nullptr;
   if (ctx_alloc(c, &np, n_np) || ctx_alloc(c, &c->r_int, (size_t)c->total_state) ||
       ctx_alloc(c, &c->active, (size_t)B) || ctx_alloc(c, &jc, (size_t)B))
     return fail(PCF_ENOMEM);
@@ -1304,12 +1313,13 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
     if (ctx_alloc(c, &yvf, n_yv) || ctx_alloc(c, &phf, n_ph) || ctx_alloc(c, &xzf, n_xz) || ctx_alloc(c, &xzc, n_xz))
       return fail(PCF_ENOMEM);
   } else {
-    if (ctx_alloc(c, &yv, n_yv) || ctx_alloc(c, &ph, n_ph) || ctx_alloc(c, &xz, n_xz) || ctx_alloc(c, &fr, n_fr))
+    if (ctx_alloc(c, &yv, n_yv) || ctx_alloc(c, &ph, n_ph) || ctx_alloc(c, &xz, n_xz) || ctx_alloc(c, &fr, n_fr) ||
+        ctx_alloc(c, &pin, n_pi))
       return fail(PCF_ENOMEM);
   }
   c->hinst.resize(B);
   std::vector<int> per11(B), per3(B), per1(B, 1), per_tcs(B), per_tca(B);
-  size_t o_yv = 0, o_ph = 0, o_xz = 0, o_np = 0, o_fr = 0;
+  size_t o_yv = 0, o_ph = 0, o_xz = 0, o_np = 0, o_fr = 0, o_pi = 0;
   c->split = !c->mixed;
   // the FP32 form's plane kernels keep their transforms in warp registers wherever every
   // instance's nx and nz allow it (unless the caller asks for the shared-memory kernels)
@@ -1340,8 +1350,21 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
       I.inv_nxnz = 1.0 / ((double)p.nx * p.nz);
       I.cheb = g.cheb; I.cheb_ff = g.cheb_ff; I.rco = g.rco; I.ygrid = g.y; I.ubase = g.ub; I.ccw = g.ccw;
       I.kx = g.kx; I.kz = g.kz;
-      I.twx = g.twx; I.twz = g.twz;
-      I.tanx = g.tanx; I.tanz = g.tanz; I.rotx = g.rotx; I.rotz = g.rotz;
+      I.twfx_x = g.twfx_x; I.twfx_z = g.twfx_z;
+      I.mz_mul = div_mul(I.Mz); I.nz_mul = div_mul(p.nz); I.rx_mul = div_mul(p.nx / 8);
+      I.rz_mul = div_mul(p.nz / 8);
+      {
+        // 1/(nx nz) = m 2^e, 1/2 < m <= 1
+        const int n = p.nx * p.nz;
+        int e = 0;
+        while ((2 << e) <= n) ++e;
+        I.nfx_e = -e;
+        if (n != (1 << e)) {
+          const long long z = std::llrint(std::ldexp((long double)(1 << e) / n, 62));
+          I.nfx_l = (int)(uint32_t)(uint64_t)z;
+          I.nfx_h = (int)((z - I.nfx_l) >> 32);
+        }
+      }
       I.tab[0] = g.tab0; I.tab[1] = g.tab1;
       I.dense[0] = g.dense0; I.dense[1] = g.dense1;
       I.sigma[0] = g.sig[0]; I.sigma[1] = g.sig[1];
@@ -1351,13 +1374,14 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
         I.yvf = yvf + o_yv; I.physf = phf + o_ph; I.xzf = xzf + o_xz; I.xzc = xzc + o_xz;
         I.twxf = g.twxf; I.twzf = g.twzf; I.tcA = g.tcA; I.tcA5 = g.tcA5; I.mixed = 1;
       } else {
-        I.yv = yv + o_yv; I.phys = ph + o_ph; I.xz = xz + o_xz; I.frg = fr + o_fr;
+        I.yv = yv + o_yv; I.phys = ph + o_ph; I.xz = xz + o_xz; I.frg = fr + o_fr; I.pinfo = pin + o_pi;
       }
       if (!I.dense[0] || !I.dense[1] || p.solve_kind == 2 || smem_ysolve(I.N, 1) > 227 * 1024) c->split = false;
       o_yv += 2ULL * kFieldsY * p.ny * I.nmodes;
       o_ph += 2ULL * kFieldsSynth * p.ny * p.nx * p.nz;
       o_xz += 3ULL * p.ny * I.nmodes;
       o_np += 3ULL * p.ny;
+      o_pi += 2ULL * kFieldsSynth * p.ny;
       o_fr += 6ULL * (p.ny + 1) * I.nmodes;
       I.hist_stride = B;
       I.sym = p.symmetry;
@@ -1368,12 +1392,18 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
       per3[b] = 3 * p.ny;
       per_tcs[b] = kFieldsY * cheb_tc_tiles(I.nmodes);
       per_tca[b] = 3 * cheb_tc_tiles(I.nmodes);
-      const int elem = c->mixed ? (int)sizeof(float2) : (int)sizeof(double2);
       if (!plane_warp_ok(I)) c->plane_warp = false;
-      c->sm_synth = std::max(c->sm_synth, smem_plane(I, elem));
-      c->sm_prod = std::max(c->sm_prod, smem_plane(I, elem));
-      c->sm_warp = std::max(c->sm_warp, smem_plane_warp(I, elem));
+      c->plane_big = c->plane_big || planes_fx_big(I);
+      c->thr_synth = std::max(c->thr_synth, planes_fx_threads(I, false));
+      c->thr_prod = std::max(c->thr_prod, planes_fx_threads(I, true));
+      if (c->mixed) c->sm_synth = c->sm_prod = std::max(c->sm_synth, smem_plane(I, (int)sizeof(float2)));
+      c->sm_warp = std::max(c->sm_warp, smem_plane_warp(I, (int)sizeof(float2)));
       if (c->mixed) c->sm_tc = std::max(c->sm_tc, c->tc05 ? smem_cheb_tc05(p.ny) : smem_cheb_tc(p.ny));
+    }
+  if (!c->mixed)
+    for (const Inst& I : c->hinst) {
+      c->sm_synth = std::max(c->sm_synth, smem_planes_fx(I, c->thr_synth));
+      c->sm_prod = std::max(c->sm_prod, smem_planes_fx(I, c->thr_prod));
     }
   if (ctx_alloc(c, &c->dinst, (size_t)B)) return fail(PCF_ENOMEM);
   int dummy;
@@ -1389,7 +1419,7 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
   if (c->plane_warp) {
     c->sm_synth = c->sm_prod = c->sm_warp;
     if (set_plane_warp_smem(c->sm_synth, c->sm_prod)) return fail(PCF_ECUDA);
-  } else if (set_plane_smem(c->plane_kind, c->sm_synth, c->sm_prod)) {
+  } else if (c->mixed ? set_plane_smem(c->sm_synth, c->sm_prod) : set_planes_fx_smem(c->sm_synth, c->sm_prod)) {
     return fail(PCF_ECUDA);
   }
   const int want = list[0].modes_per_block;
@@ -1462,12 +1492,12 @@ pcf_status pcf_residual(pcf_ctx* c, const double* u, double* r, double* rnorm) {
   PCF_TRY(launch_synth(c, 0, kFieldsSynth));
   PCF_TRY(launch_prodM(c));
   if (c->mixed) PCF_TRY(launch_tc_analysis(c));
-  PCF_TRY(launch_mode(c, MODE_PHI, 0, 0));
+  PCF_TRY(launch_mode(c, MODE_PHI, 0));
   if (rnorm) {
     if (c->mixed) PCF_TRY(launch_tc_synth(c, 1));
     PCF_TRY(launch_synth(c, 1, 3));
-    launch_norm_planes(c->plane_kind, c->cta_synth3, c->cs, li_of(c, c->pre_synth3), 1);
-    k_norm_final<<<1, 32, 0, c->cs>>>(li_of(c, c->pre_inst), rnorm);
+    launch_plane_sums(c, 1);
+    k_norm_final<<<c->B, 32, 0, c->cs>>>(li_of(c, c->pre_inst), rnorm);
   }
   PCF_TRY(check_launch());
   return leave(c);
@@ -1484,7 +1514,7 @@ pcf_status pcf_adjoint_gradient(pcf_ctx* c, const double* u, const double* r, do
   PCF_TRY(launch_synth(c, 1, kFieldsSynth));
   PCF_TRY(launch_prodN(c));
   if (c->mixed) PCF_TRY(launch_tc_analysis(c));
-  PCF_TRY(launch_mode(c, MODE_PSI_GRAD, 1, 0));
+  PCF_TRY(launch_mode(c, MODE_PSI_GRAD, 1));
   PCF_TRY(check_launch());
   return leave(c);
 }
@@ -1498,7 +1528,7 @@ pcf_status pcf_influence_matrix_solve(pcf_ctx* c, const double* rhs, double* out
   set_pointers(c, nullptr, rhs, out);
   PCF_TRY(enter(c));
   PCF_TRY(push_descriptors(c));
-  PCF_TRY(launch_mode(c, MODE_SOLVE, sig, 0));
+  PCF_TRY(launch_mode(c, MODE_SOLVE, sig));
   PCF_TRY(check_launch());
   return leave(c);
 }
@@ -1730,8 +1760,8 @@ pcf_status pcf_norm(pcf_ctx* c, const double* u, double* out) {
   PCF_TRY(push_descriptors(c));
   PCF_TRY(launch_ysynth(c, 0));
   PCF_TRY(launch_synth(c, 0, 3));
-  launch_norm_planes(c->plane_kind, c->cta_synth3, c->cs, li_of(c, c->pre_synth3), 0);
-  k_norm_final<<<1, 32, 0, c->cs>>>(li_of(c, c->pre_inst), out);
+  launch_plane_sums(c, 0);
+  k_norm_final<<<c->B, 32, 0, c->cs>>>(li_of(c, c->pre_inst), out);
   PCF_TRY(check_launch());
   return leave(c);
 }

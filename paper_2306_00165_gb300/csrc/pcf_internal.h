@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "../../include/pcfadj.h"
+#include "pcf_fx.cuh"
 
 #define PCF_HD __host__ __device__ __forceinline__
 
@@ -96,13 +97,11 @@ struct Inst {
   const double* ccw;
   const double* kx;   // [Mx]
   const double* kz;   // [Mz]
-  const double2* twx; // e^{-2 pi i k/nx}, k < nx
-  const double2* twz; // e^{-2 pi i k/nz}, k < nz
-  const double2* tanx;        // [2][nx] tangent-form twiddles (t, m) of the FP64 plane FFTs:
-  const double2* tanz;        //   forward, then inverse; see TwTan
-  const unsigned char* rotx;  // [nx] their rotation flags (|sin| > |cos|)
-  const unsigned char* rotz;  // [nz]
-  const float2* twxf; // FP32 copies for the mixed-precision form
+  const fxtw* twfx_x; // [2][nx] fixed-point twiddles of the FP64 forms' plane kernels:
+  const fxtw* twfx_z; //   forward (e^{-2 pi i q/n}), then inverse
+  unsigned mz_mul, nz_mul, rx_mul, rz_mul;  // floor(2^32/d) + 1 for d = Mz, nz, nx/8, nz/8 (exact quotients by __umulhi)
+  int nfx_h, nfx_l, nfx_e;  // 1/(nx nz) = (nfx_h, nfx_l) 2^-62 2^nfx_e; nfx_h = 0 for a power of two
+  const float2* twxf; // e^{-2 pi i k/nx}, k < nx, of the mixed form
   const float2* twzf;
   const double* tab[2];  // per-mode solver tables: [0] sigma = 1/(nu dt), [1] sigma = 1/(nu dtau_hat)
   const double* dense[2];  // per-mode dense solve operators (DenseLayout) or null
@@ -112,7 +111,8 @@ struct Inst {
   double2* rhat;
   double2* fhat;
   double2* yv;        // [2][5][ny][Mx][Mz]: slot 0 for u, slot 1 for q
-  double* phys;       // [2][11][ny][nx][nz]: slot 0 for u, slot 1 for q
+  double* phys;       // [2][11][ny][nx][nz] 64-bit integers: slot 0 for u, slot 1 for q
+  int2* pinfo;        // [2][11][ny]: exponent of each plane of phys and the bits of its largest magnitude
   double2* xz;        // [3][ny][Mx][Mz]
   double* normpart;   // [3][ny]
   double* frg;        // [nmodes][3][2][N + 2]: class-split Stokes right-hand sides (FP64 split mode kernels)

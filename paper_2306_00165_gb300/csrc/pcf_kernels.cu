@@ -154,39 +154,12 @@ __device__ C* fft_run_io(C* a, C* b, int L, int LS, int nb, const int* radix, in
   return OUT_ST ? nullptr : cur;
 }
 
-// Twiddles of the plane kernels in shared memory: the standard tables (FP32, float-float), or
-// for FP64 the tangent-form entries of the transform's direction (inv: the inverse
-// transform) and their rotation flags.  PlaneTw<T>::type is the pass functions' view.
+// The x and z twiddle tables, copied to shared memory.
 template <class T>
-struct PlaneTw {
-  using C = typename Cx<T>::c;
-  using type = TwStd<C>;
-  static __device__ __forceinline__ type view(C* tw, unsigned char*) { return type{tw}; }
-  static __device__ __forceinline__ void load(const Inst& I, C* twx, C* twz, unsigned char*, unsigned char*, bool) {
-    const typename Sto<T>::c* sx = twx_of<T>(I);
-    const typename Sto<T>::c* sz = twz_of<T>(I);
-    for (int t = threadIdx.x; t < I.nx; t += blockDim.x) twx[t] = load_c<T>(sx[t]);
-    for (int t = threadIdx.x; t < I.nz; t += blockDim.x) twz[t] = load_c<T>(sz[t]);
-  }
-};
-template <>
-struct PlaneTw<double> {
-  using type = TwTan;
-  static __device__ __forceinline__ type view(double2* tw, unsigned char* rot) { return type{tw, rot}; }
-  static __device__ __forceinline__ void load(const Inst& I, double2* twx, double2* twz, unsigned char* rx,
-                                              unsigned char* rz, bool inv) {
-    const double2* sx = I.tanx + (inv ? I.nx : 0);
-    const double2* sz = I.tanz + (inv ? I.nz : 0);
-    for (int t = threadIdx.x; t < I.nx; t += blockDim.x) {
-      twx[t] = sx[t];
-      rx[t] = I.rotx[t];
-    }
-    for (int t = threadIdx.x; t < I.nz; t += blockDim.x) {
-      twz[t] = sz[t];
-      rz[t] = I.rotz[t];
-    }
-  }
-};
+__device__ __forceinline__ void load_twiddles(const Inst& I, typename Cx<T>::c* twx, typename Cx<T>::c* twz) {
+  for (int t = threadIdx.x; t < I.nx; t += blockDim.x) twx[t] = twx_of<T>(I)[t];
+  for (int t = threadIdx.x; t < I.nz; t += blockDim.x) twz[t] = twz_of<T>(I)[t];
+}
 
 // Shared-memory plan of a plane transform: two buffers of PB complex values; x-stage
 // batches (one per retained z mode) have stride LX = nx + 1, z-stage batches (one per row
@@ -211,13 +184,11 @@ __host__ __device__ inline PlanePlan plane_plan(const Inst& I, int elem) {
   }
   return pp;
 }
-// [B0 | B1 | twx (nx) | twz (nz) | 32 doubles of reduction | rotation flags of twx, twz]
+// [B0 | B1 | twx (nx) | twz (nz) | 32 doubles of reduction]
 size_t smem_plane(const Inst& I, int elem) {
   const PlanePlan pp = plane_plan(I, elem);
-  return (size_t)elem * (2 * (size_t)pp.PB + I.nx + I.nz) + 8 * 32 + (size_t)((I.nx + I.nz + 15) & ~15);
+  return (size_t)elem * (2 * (size_t)pp.PB + I.nx + I.nz) + 8 * 32;
 }
-size_t smem_xzsynth(const Inst& I) { return smem_plane(I, sizeof(double2)); }
-size_t smem_prod(const Inst& I) { return smem_plane(I, sizeof(double2)); }
 
 
 // ------------------------------------------------------------------ plane synthesis
@@ -247,12 +218,10 @@ __global__ void __launch_bounds__(128, PCF_XZ_MINB) k_xzsynth_t(LaunchInfo li, i
   C* B1 = sm + pp.PB;
   C* twx = sm + 2 * pp.PB;
   C* twz = twx + nx;
-  unsigned char* rtx = reinterpret_cast<unsigned char*>(twz + nz) + 8 * 32;
-  unsigned char* rtz = rtx + nx;
-  PlaneTw<T>::load(I, twx, twz, rtx, rtz, true);  // first used after the first pass's barrier
-  const typename PlaneTw<T>::type tx = PlaneTw<T>::view(twx, rtx), tz = PlaneTw<T>::view(twz, rtz);
+  load_twiddles<T>(I, twx, twz);  // first used after the first pass's barrier
+  const TwStd<C> tx{twx}, tz{twz};
   const int LX = pp.LX, LZ = pp.LZ;
-  const typename Sto<T>::c* src = yv_of<T>(I) + (((size_t)slot * kFieldsY + c_src[f]) * I.ny + j) * (size_t)I.nmodes;
+  const C* src = yv_of<T>(I) + (((size_t)slot * kFieldsY + c_src[f]) * I.ny + j) * (size_t)I.nmodes;
   const int fac = c_fac[f];
   // x stage: batch p (retained z mode), element = x bin; the input is the y-values (times
   // i kx or i kz for the x and z derivatives); bins outside |m| <= Kx are zero
@@ -265,7 +234,7 @@ __global__ void __launch_bounds__(128, PCF_XZ_MINB) k_xzsynth_t(LaunchInfo li, i
   // (the other bins are never read: the first pass returns zero for them)
   for (int t = threadIdx.x; t < I.nmodes; t += blockDim.x) {
     const int i = t / Mz, p = t - i * Mz;
-    B0[p * LX + xbin(i, Kx, Mx, nx)] = scaled(load_c<T>(src[t]), i, p);
+    B0[p * LX + xbin(i, Kx, Mx, nx)] = scaled(src[t], i, p);
   }
   __syncthreads();
   const auto ldx = [&](int p, int bin) -> C {
@@ -340,7 +309,7 @@ __device__ __forceinline__ T grad_at(const PlaneSet<T>& F, int c, int d, int e) 
 // (so that the flows without suction keep their instruction count).
 template <class T, bool ADJ, bool VB>
 __device__ __forceinline__ void product_pair(const Inst& I, const PlaneSet<T>& U, const PlaneSet<T>& Q, int c, T Ub,
-                                             T dUb, T Vb, int e0, int e1, T* m, typename Acc<T>::type* sq) {
+                                             T dUb, T Vb, int e0, int e1, T* m, double* sq) {
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int e = h == 0 ? e0 : e1;
@@ -369,7 +338,7 @@ __device__ __forceinline__ void product_pair(const Inst& I, const PlaneSet<T>& U
 template <class T, bool ADJ, int CC, bool VB>
 __device__ __forceinline__ void product_rows(const Inst& I, const PlaneSet<T>& U, const PlaneSet<T>& Q, T Ub, T dUb,
                                              T Vb, int r0, int nrc, int nz, int LZ, typename Cx<T>::c* Z0,
-                                             typename Acc<T>::type* sq) {
+                                             double* sq) {
   for (int t = threadIdx.x; t < nrc * nz; t += blockDim.x) {
     const int r = t / nz, z = t - r * nz;
     const int e0 = (2 * (r0 + r)) * nz + z, e1 = e0 + nz;
@@ -383,7 +352,7 @@ __device__ __forceinline__ void product_rows(const Inst& I, const PlaneSet<T>& U
 template <class T, bool ADJ, bool VB>
 __device__ __forceinline__ void product_rows_c(int c, const Inst& I, const PlaneSet<T>& U, const PlaneSet<T>& Q,
                                                T Ub, T dUb, T Vb, int r0, int nrc, int nz, int LZ,
-                                               typename Cx<T>::c* Z0, typename Acc<T>::type* sq) {
+                                               typename Cx<T>::c* Z0, double* sq) {
   if (c == 0) product_rows<T, ADJ, 0, VB>(I, U, Q, Ub, dUb, Vb, r0, nrc, nz, LZ, Z0, sq);
   else if (c == 1) product_rows<T, ADJ, 1, VB>(I, U, Q, Ub, dUb, Vb, r0, nrc, nz, LZ, Z0, sq);
   else product_rows<T, ADJ, 2, VB>(I, U, Q, Ub, dUb, Vb, r0, nrc, nz, LZ, Z0, sq);
@@ -413,10 +382,8 @@ __global__ void __launch_bounds__(128, ADJ ? 6 : 8) k_prod_t(LaunchInfo li, int 
   C* twx = sm + 2 * pp.PB;
   C* twz = twx + nx;
   double* red = reinterpret_cast<double*>(twz + nz);
-  unsigned char* rtx = reinterpret_cast<unsigned char*>(red + 32);
-  unsigned char* rtz = rtx + nx;
-  PlaneTw<T>::load(I, twx, twz, rtx, rtz, false);
-  const typename PlaneTw<T>::type tx = PlaneTw<T>::view(twx, rtx), tz = PlaneTw<T>::view(twz, rtz);
+  load_twiddles<T>(I, twx, twz);
+  const TwStd<C> tx{twx}, tz{twz};
   const int fs = I.ny * nx * nz;  // between the fields of a slot
   const PlaneSet<T> U{fplane<T>(I, 0, 0, j), fs};
   const PlaneSet<T> Q{ADJ ? fplane<T>(I, 1, 0, j) : nullptr, fs};
@@ -426,7 +393,7 @@ __global__ void __launch_bounds__(128, ADJ ? 6 : 8) k_prod_t(LaunchInfo li, int 
   const bool whole = pp.chunk == nr;
   // the x-stage input X[p][x] lives in B0 when chunked (z chunks use B1), else decided below
   C* X = B0;
-  typename Acc<T>::type sq = 0.0;
+  double sq = 0.0;
   __syncthreads();
   for (int r0 = 0; r0 < nr; r0 += pp.chunk) {
     const int nrc = min(pp.chunk, nr - r0);
@@ -447,7 +414,7 @@ __global__ void __launch_bounds__(128, ADJ ? 6 : 8) k_prod_t(LaunchInfo li, int 
     __syncthreads();
   }
   if (ADJ) {
-    double sqd = acc_value(sq);
+    double sqd = sq;
     for (int o = 16; o > 0; o >>= 1) sqd += __shfl_down_sync(0xffffffffu, sqd, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sqd;
     __syncthreads();
@@ -459,43 +426,13 @@ __global__ void __launch_bounds__(128, ADJ ? 6 : 8) k_prod_t(LaunchInfo li, int 
   }
   C* Y = fft_run<C>(X, X == B0 ? B1 : B0, nx, LX, Mz, I.rx, I.nrx, tx, false);
   const T sc = (T)I.inv_nxnz;
-  typename Sto<T>::c* dst = xz_of<T>(I) + ((size_t)c * I.ny + j) * I.nmodes;
+  C* dst = xz_of<T>(I) + ((size_t)c * I.ny + j) * I.nmodes;
   for (int t = threadIdx.x; t < I.nmodes; t += blockDim.x) {
     const int i = t / Mz, p = t - i * Mz;
     const C v = Y[p * LX + xbin(i, Kx, Mx, nx)];
-    dst[t] = store_c<T>(Cx<T>::mk(v.x * sc, v.y * sc));
+    dst[t] = Cx<T>::mk(v.x * sc, v.y * sc);
   }
-  if (ADJ && step_index >= 0) {
-    // J = ||r1|| once all 3 ny plane sums of the instance are written: the CTA that counts
-    // last computes it (the chain of norm_from_parts, so the bits match the other paths),
-    // writes the history entry, clears the mask when J < tol (the instance stops before this
-    // step's update) and resets the counter for the next launch.
-    __shared__ int last;
-    if (threadIdx.x == 0) {
-      __threadfence();
-      last = atomicAdd(I.jcount, 1) == 3 * I.ny - 1;
-    }
-    __syncthreads();
-    if (last) {  // uniform in the CTA
-      // the plane buffers are free now: stage the per-plane sums and the weights
-      const int ny = I.ny;
-      const double* P = I.normpart;
-      double* ps = reinterpret_cast<double*>(smraw);
-      for (int q = threadIdx.x; q < ny; q += blockDim.x) {
-        ps[q] = __ldcg(P + q) + __ldcg(P + ny + q) + __ldcg(P + 2 * ny + q);
-        ps[ny + q] = I.ccw[q];
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int q = 0; q < ny; ++q) s = fma(ps[ny + q], ps[q], s);
-        const double J = sqrt(0.5 * I.inv_nxnz * s);
-        if (I.hist) I.hist[(size_t)step_index * I.hist_stride] = J;
-        if (I.tol > 0.0 && J < I.tol && I.active) *I.active = 0;
-        *I.jcount = 0;
-      }
-    }
-  }
+  if (ADJ && step_index >= 0) finish_norm(I, step_index);
 }
 
 // CTA = (instance, plane j, component c): sum over the plane of the squared velocity
@@ -508,9 +445,8 @@ __global__ void __launch_bounds__(128) k_norm_planes_t(LaunchInfo li, int slot) 
   const Inst& I = li.insts[b];
   const int c = local % 3, j = local / 3;
   const T* q = fplane<T>(I, slot, c, j);
-  typename Acc<T>::type sa = 0.0;
-  for (int t = threadIdx.x; t < I.nx * I.nz; t += blockDim.x) acc_sq(&sa, q[t]);
-  double sq = acc_value(sa);
+  double sq = 0.0;
+  for (int t = threadIdx.x; t < I.nx * I.nz; t += blockDim.x) acc_sq(&sq, q[t]);
   for (int o = 16; o > 0; o >>= 1) sq += __shfl_down_sync(0xffffffffu, sq, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
   __syncthreads();
@@ -521,53 +457,35 @@ __global__ void __launch_bounds__(128) k_norm_planes_t(LaunchInfo li, int slot) 
   }
 }
 
-// host launchers (the kernel templates are instantiated in this translation unit only)
-// plane arithmetic: 0 FP64, 1 FP32 (mixed form), 2 float-float
-void launch_xzsynth(int kind, int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf) {
-  if (kind == 1) k_xzsynth_t<float><<<ctas, 128, smem, s>>>(li, slot, nf);
-  else if (kind == 2) k_xzsynth_t<ff><<<ctas, 128, smem, s>>>(li, slot, nf);
-  else k_xzsynth_t<double><<<ctas, 128, smem, s>>>(li, slot, nf);
+// host launchers (the kernel templates are instantiated in this translation unit only): FP32
+void launch_xzsynth(int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf) {
+  k_xzsynth_t<float><<<ctas, 128, smem, s>>>(li, slot, nf);
 }
-template <class T, bool VB>
+template <bool VB>
 static void launch_prod_t(bool adj, int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int step_index) {
-  if (adj) k_prod_t<T, true, VB><<<ctas, 128, smem, s>>>(li, step_index);
-  else k_prod_t<T, false, VB><<<ctas, 128, smem, s>>>(li, -1);
+  if (adj) k_prod_t<float, true, VB><<<ctas, 128, smem, s>>>(li, step_index);
+  else k_prod_t<float, false, VB><<<ctas, 128, smem, s>>>(li, -1);
 }
-void launch_prod(int kind, bool adj, bool suction, int ctas, size_t smem, cudaStream_t s, LaunchInfo li,
-                 int step_index) {
-  if (kind == 1) {
-    if (suction) launch_prod_t<float, true>(adj, ctas, smem, s, li, step_index);
-    else launch_prod_t<float, false>(adj, ctas, smem, s, li, step_index);
-  } else if (kind == 2) {
-    if (suction) launch_prod_t<ff, true>(adj, ctas, smem, s, li, step_index);
-    else launch_prod_t<ff, false>(adj, ctas, smem, s, li, step_index);
-  } else {
-    if (suction) launch_prod_t<double, true>(adj, ctas, smem, s, li, step_index);
-    else launch_prod_t<double, false>(adj, ctas, smem, s, li, step_index);
-  }
+void launch_prod(bool adj, bool suction, int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int step_index) {
+  if (suction) launch_prod_t<true>(adj, ctas, smem, s, li, step_index);
+  else launch_prod_t<false>(adj, ctas, smem, s, li, step_index);
 }
-void launch_norm_planes(int kind, int ctas, cudaStream_t s, LaunchInfo li, int slot) {
-  if (kind == 1) k_norm_planes_t<float><<<ctas, 128, 0, s>>>(li, slot);
-  else if (kind == 2) k_norm_planes_t<ff><<<ctas, 128, 0, s>>>(li, slot);
-  else k_norm_planes_t<double><<<ctas, 128, 0, s>>>(li, slot);
+void launch_norm_planes(int ctas, cudaStream_t s, LaunchInfo li, int slot) {
+  k_norm_planes_t<float><<<ctas, 128, 0, s>>>(li, slot);
 }
-template <class T>
-static cudaError_t set_plane_smem_t(size_t synth, size_t prod) {
+cudaError_t set_plane_smem(size_t synth, size_t prod) {
   cudaError_t e;
-  if ((e = raise_smem_limit((const void*)k_xzsynth_t<T>, synth))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_t<T, false, false>, prod))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_t<T, false, true>, prod))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_t<T, true, true>, prod))) return e;
-  return raise_smem_limit((const void*)k_prod_t<T, true, false>, prod);
-}
-cudaError_t set_plane_smem(int kind, size_t synth, size_t prod) {
-  if (kind == 1) return set_plane_smem_t<float>(synth, prod);
-  if (kind == 2) return set_plane_smem_t<ff>(synth, prod);
-  return set_plane_smem_t<double>(synth, prod);
+  if ((e = raise_smem_limit((const void*)k_xzsynth_t<float>, synth))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_t<float, false, false>, prod))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_t<float, false, true>, prod))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_t<float, true, true>, prod))) return e;
+  return raise_smem_limit((const void*)k_prod_t<float, true, false>, prod);
 }
 
+// one warp per instance
 __global__ void k_norm_final(LaunchInfo li, double* out) {
-  for (int b = threadIdx.x; b < li.ninst; b += blockDim.x) out[b] = norm_from_parts(li.insts[b]);
+  const double J = norm_from_parts(li.insts[blockIdx.x]);
+  if (threadIdx.x == 0) out[blockIdx.x] = J;
 }
 
 // ------------------------------------------------------------------ per-mode kernel
@@ -605,7 +523,7 @@ __device__ __forceinline__ void dot2_ldg(const double* col, int stride, const do
   }
 }
 
-__global__ void __launch_bounds__(320) k_mode(LaunchInfo li, int op, int sig, int mpc_arg, int step_index) {
+__global__ void __launch_bounds__(320) k_mode(LaunchInfo li, int op, int sig, int mpc_arg) {
   extern __shared__ double smd[];
   int local;
   const int b = find_inst(li, blockIdx.x, &local);
@@ -620,22 +538,8 @@ __global__ void __launch_bounds__(320) k_mode(LaunchInfo li, int op, int sig, in
   const ChebLayout CL(N);
   const bool solve = (op != MODE_SYNTH_ONLY);
 
-  // descent: J = ||r1|| from the plane sums of k_prod<N>, its history entry and the
-  // convergence decision; step_index < 0: the product kernel has taken them already (the
-  // instance's mask then holds this step's J < tol)
-  if (op == MODE_PSI_UPDATE) {
-    if (!inst_active(I)) return;
-    if (step_index >= 0) {
-      const double J = norm_from_parts(I);
-      if (local == 0 && threadIdx.x == 0 && I.hist) I.hist[(size_t)step_index * I.hist_stride] = J;
-      if (I.tol > 0.0 && J < I.tol) {
-        if (local == 0 && threadIdx.x == 0 && I.active) *I.active = 0;
-        return;
-      }
-    }
-  } else if (op != MODE_SOLVE && op != MODE_SYNTH_ONLY && !inst_active(I)) {
-    return;
-  }
+  // descent: the adjoint product kernel has taken J; the mask holds this step's J < tol
+  if (op != MODE_SOLVE && op != MODE_SYNTH_ONLY && !inst_active(I)) return;
 
   const bool need_cheb = !I.mixed, need_tabs = !I.dense[0];
   double* cheb = smd;

@@ -17,6 +17,7 @@ struct LaunchInfo {
   const Inst* insts;
   const int* prefix;   // CTA prefix over instances (length ninst + 1)
   int ninst;
+  int per = 0;         // CTAs per instance when every instance has the same number, else 0
 };
 
 // Launch over groups of consecutive instances that share one grid.
@@ -37,6 +38,11 @@ __device__ __forceinline__ int run_modes(const GroupLaunch& gl, const Inst& I) {
 }
 
 __device__ __forceinline__ int find_inst(const LaunchInfo& li, int cta, int* local) {
+  if (li.per) {  // no dependent loads on the way to the instance's descriptor
+    const int b = cta / li.per;
+    *local = cta - b * li.per;
+    return b;
+  }
   int lo = 0, hi = li.ninst - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -61,14 +67,39 @@ struct DnsInst {
   double h1, h2;       // ||u|| of the previous two steps
 };
 
-// J = sqrt(0.5 * sum_j w_j * mean_{x,z} |q|^2) from the plane sums (fixed order).
+// J = sqrt(0.5 * sum_j w_j * mean_{x,z} |q|^2) from the plane sums, by one full warp (every
+// lane returns it): strided partial sums, then a shuffle tree, so that the chain is ny/32 + 5
+// additions and not ny.  Every path that computes a norm uses this order.
 __device__ __forceinline__ double norm_from_parts(const Inst& I) {
   double s = 0.0;
-  for (int j = 0; j < I.ny; ++j) {
-    const double pj = I.normpart[j] + I.normpart[I.ny + j] + I.normpart[2 * I.ny + j];
-    s = fma(I.ccw[j], pj, s);
+  for (int q = threadIdx.x & 31; q < I.ny; q += 32) {
+    const double pj = __ldcg(I.normpart + q) + __ldcg(I.normpart + I.ny + q) + __ldcg(I.normpart + 2 * I.ny + q);
+    s = fma(I.ccw[q], pj, s);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return sqrt(0.5 * I.inv_nxnz * s);
+}
+
+// End of an adjoint product CTA, after thread 0 has written its plane sum: the CTA that counts
+// last of the instance's 3 ny computes J (its first warp), writes the history entry, clears
+// the mask when J < tol (the instance stops before this step's update) and resets the counter
+// for the next launch.
+__device__ __forceinline__ void finish_norm(const Inst& I, int step_index) {
+  if (threadIdx.x >= 32) return;
+  int last = 0;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(I.jcount, 1) == 3 * I.ny - 1;
+  }
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  __threadfence();
+  const double J = norm_from_parts(I);
+  if (threadIdx.x == 0) {
+    if (I.hist) I.hist[(size_t)step_index * I.hist_stride] = J;
+    if (I.tol > 0.0 && J < I.tol && I.active) *I.active = 0;
+    *I.jcount = 0;
+  }
 }
 
 // Raise the maximum dynamic shared memory of kernel func on the current device to at least
@@ -84,15 +115,24 @@ int sweep_ctas(int nmodes_run, int threads);
 void launch_sweep(int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int op, int red);
 cudaError_t set_sweep_smem(size_t smem);
 
-// kind: plane arithmetic, 0 FP64, 1 FP32 (mixed form), 2 float-float
-void launch_xzsynth(int kind, int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf);
+// FP32 plane kernels of the mixed form (shared-memory Stockham passes).
 // step_index >= 0 (adjoint product only): the last CTA of each instance also computes J from
 // the plane sums, its history entry and the convergence mask (in place of launch_jnorm)
 // suction: some instance of the launch has a base flow with a wall-normal velocity (ASBL)
-void launch_prod(int kind, bool adj, bool suction, int ctas, size_t smem, cudaStream_t s, LaunchInfo li,
-                 int step_index = -1);
-void launch_norm_planes(int kind, int ctas, cudaStream_t s, LaunchInfo li, int slot);
-cudaError_t set_plane_smem(int kind, size_t synth, size_t prod);
+void launch_xzsynth(int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf);
+void launch_prod(bool adj, bool suction, int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int step_index = -1);
+void launch_norm_planes(int ctas, cudaStream_t s, LaunchInfo li, int slot);
+cudaError_t set_plane_smem(size_t synth, size_t prod);
+// The FP64 forms' plane kernels in 64-bit fixed point (pcf_planes_fx.cu); threads per CTA from
+// the largest plane of the launch.
+bool planes_fx_big(const Inst& I);
+size_t smem_planes_fx(const Inst& I, int threads);
+int planes_fx_threads(const Inst& I, bool prod);
+void launch_xzsynth_fx(bool big, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf);
+void launch_prod_fx(bool big, bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li,
+                    int step_index);
+void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot);
+cudaError_t set_planes_fx_smem(size_t synth, size_t prod);
 // Plane kernels of the FP32 form with the x, z transforms in warp registers
 // (pcf_planes_warp.cu): nx, nz in {32, 64, 96, 128}.
 bool plane_warp_ok(const Inst& I);
@@ -100,13 +140,11 @@ size_t smem_plane_warp(const Inst& I, int elem_bytes);
 void launch_xzsynth_warp(int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf);
 void launch_prod_warp(bool adj, int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int step_index);
 cudaError_t set_plane_warp_smem(size_t synth, size_t prod);
-__global__ void k_mode(LaunchInfo li, int op, int sig, int mpc, int step_index);
+__global__ void k_mode(LaunchInfo li, int op, int sig, int mpc);
 __global__ void k_norm_final(LaunchInfo li, double* out);
 __global__ void k_fp64_probe(double* out, int iters);
 
 size_t smem_plane(const Inst& I, int elem_bytes);
-size_t smem_xzsynth(const Inst& I);
-size_t smem_prod(const Inst& I);
 size_t smem_mode(const Inst& I, int mpc);
 size_t smem_cheb_tc(int ny);
 void launch_cheb_synth_tc(int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int slot);

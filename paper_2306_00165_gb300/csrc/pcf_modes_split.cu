@@ -233,23 +233,14 @@ __global__ void __launch_bounds__(kAnalysisMaxThreads, 4) k_yanalysis(GroupLaunc
 }
 
 // ---------------------------------------------------------------- norm of r1
-// J = ||r1|| of every active instance from the plane sums of the adjoint product kernel
-// (same order of operations as norm_from_parts), its history entry, and the convergence
-// mask (J < tol: the instance stops before this step's update).  One CTA per instance;
-// ny <= 257 (the split kernels serve grids with dense operators, ny <= 129).
-__global__ void __launch_bounds__(128) k_jnorm(const Inst* insts, int step_index) {
-  __shared__ double part[3 * 257];
-  __shared__ double w[257];
+// J = ||r1|| of every active instance from the plane sums of the adjoint product kernel, its
+// history entry, and the convergence mask (J < tol: the instance stops before this step's
+// update).  One warp per instance.
+__global__ void __launch_bounds__(32) k_jnorm(const Inst* insts, int step_index) {
   const Inst& I = insts[blockIdx.x];
   if (!inst_active(I)) return;
-  const int ny = I.ny;
-  for (int t = threadIdx.x; t < 3 * ny; t += blockDim.x) part[t] = I.normpart[t];
-  for (int t = threadIdx.x; t < ny; t += blockDim.x) w[t] = I.ccw[t];
-  __syncthreads();
+  const double J = norm_from_parts(I);
   if (threadIdx.x != 0) return;
-  double s = 0.0;
-  for (int j = 0; j < ny; ++j) s = fma(w[j], part[j] + part[ny + j] + part[2 * ny + j], s);
-  const double J = sqrt(0.5 * I.inv_nxnz * s);
   if (I.hist) I.hist[(size_t)step_index * I.hist_stride] = J;
   if (I.tol > 0.0 && J < I.tol && I.active) *I.active = 0;
 }
@@ -1010,7 +1001,7 @@ void launch_ysolve(int ctas, int nitems, int bufsz, int scr_rows, size_t smem, c
   k_ysolve<<<ctas, kSolveThreads, smem, s>>>(gl, op, nitems, bufsz, scr_rows);
 }
 void launch_jnorm(int ninst, cudaStream_t s, const Inst* insts, int step_index) {
-  k_jnorm<<<ninst, 128, 0, s>>>(insts, step_index);
+  k_jnorm<<<ninst, 32, 0, s>>>(insts, step_index);
 }
 int ysolve_ctas_per_sm(size_t smem) {
   int n = 0;

@@ -253,7 +253,7 @@ extern "C" pcf_status pcf_influence_matrix_solve_noalloc(const pcf_params* prm, 
   const int ctas = (nm + mpc - 1) / mpc;
   // the prefix over the one instance is {0}; LaunchInfo reads prefix[0] only
   LaunchInfo li{reinterpret_cast<const Inst*>(base + L.inst), reinterpret_cast<const int*>(base + L.prefix), 1};
-  k_mode<<<ctas, 128, smem, s>>>(li, MODE_SOLVE, 0, mpc, 0);
+  k_mode<<<ctas, 128, smem, s>>>(li, MODE_SOLVE, 0, mpc);
   if (cudaGetLastError() != cudaSuccess) return PCF_ECUDA;
   return PCF_OK;
 }

@@ -1,0 +1,629 @@
+// x-z plane kernels of the FP64 forms in 64-bit fixed point (pcf_fx.cuh).
+//
+//   k_synth_fx  CTA (instance, y-plane, field): inverse x and z transforms of the y-values;
+//               writes the plane as integers with one exponent
+//   k_prod_fx   CTA (instance, y-plane, component): M(u) or N(q) on the plane, forward z and x
+//               transforms, 2/3 truncation, back to FP64; plane sums of q^2 and J
+//   k_norm_planes_fx  plane sums of squares
+//
+// What bounds them: integer issue.  The same transforms in FP64 were bound by the FP64 pipe
+// (a 32 x 32 plane needs 11 k FP64 instructions, 6.7 k clocks of an SM); the integer
+// butterflies of a plane take under 1 k clocks.
+//
+// A transform of length L = 8 R (R = 2, 4, 6, 8, 12, 16 for L = 16 .. 128) is two register
+// passes: DFTs of length R over the elements n, n + 8, .. (thread n of 8), twiddles, and DFTs
+// of length 8 over each block of eight.  Both passes work in place, so one buffer and one
+// barrier per pass suffice.  Slot of element (block b, member e) in a row: 8 b + (e xor (b mod 8)):
+// the eight lanes of a shared-memory phase meet eight different 16-byte bank groups in both
+// passes without padding; rows have an odd stride for the walks across rows.
+#include "pcf_fx.cuh"
+#include "pcf_kernels.cuh"
+
+namespace pcf {
+
+namespace {
+
+// Threads and resident CTAs the kernels are compiled for: 80 registers for sides up to 64
+// (six 128-thread CTAs), 128 registers for the longer transforms.
+template <bool BIG>
+struct FxCfg {
+  static constexpr int threads = BIG ? 256 : 128, ctas = BIG ? 2 : 6;
+};
+
+__device__ __forceinline__ int fx_slot(int b, int e) { return b * 8 + (e ^ (b & 7)); }
+
+// First pass over nrow rows: ld(row, n) -> element n, result in place in buf.
+template <int R, bool INV, class LD>
+__device__ __forceinline__ void fx_first(int nrow, fxc* buf, int LS, const fxtw* __restrict__ tw, const LD& ld) {
+  for (int t = threadIdx.x; t < 8 * nrow; t += blockDim.x) {
+    const int row = t >> 3, n = t & 7;
+    fxc v[R];
+    ld(row, n, v);
+    FxDft<R, INV>::run(v);
+    fxc* o = buf + row * LS;
+    o[fx_slot(0, n)] = v[0];
+#pragma unroll
+    for (int k = 1; k < R; ++k) {
+      const int4 w = __ldg(reinterpret_cast<const int4*>(tw) + n * k);
+      o[fx_slot(k, n)] = fx_cmul(v[k], fxtw{w.x, w.y, w.z, w.w});
+    }
+  }
+}
+// Second pass: st(row, b, v): v[k] is output b + R k of the row.
+template <int R, bool INV, class ST>
+__device__ __forceinline__ void fx_second(int nrow, const fxc* buf, int LS, const ST& st) {
+  for (int t = threadIdx.x; t < R * nrow; t += blockDim.x) {
+    const int row = t / R, b = t - row * R;
+    const fxc* a = buf + row * LS;
+    fxc v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = a[fx_slot(b, e)];
+    FxDft<8, INV>::run(v);
+    st(row, b, v);
+  }
+}
+
+// f(integral_constant R) for the transform length n = 8 R (uniform in the CTA)
+template <int R_>
+struct FxR {
+  static constexpr int R = R_;
+};
+// BIG: kernels for planes with a side above 64 (R = 12, 16 hold more registers)
+template <bool BIG, class F>
+__device__ __forceinline__ void fx_length(int n, const F& f) {
+  switch (n >> 3) {
+    case 2: f(FxR<2>()); break;
+    case 4: f(FxR<4>()); break;
+    case 6: f(FxR<6>()); break;
+    case 12: if (BIG) f(FxR<12>()); break;
+    case 16: if (BIG) f(FxR<16>()); break;
+    default: f(FxR<8>()); break;
+  }
+}
+
+// ------------------------------------------------------------------ FP64 -> fixed point
+// Integer view of a nonzero finite factor k: mantissa in [2^61, 2^62) and biased exponent.
+struct FxK {
+  fx m;
+  int e, neg, hi;
+};
+__device__ __forceinline__ FxK fx_factor(double k) {
+  const int hi = __double2hiint(k);
+  const fx m = ((fx)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(k);
+  return FxK{m << 9, (hi >> 20) & 0x7ff, hi >> 31, hi & 0x7fffffff};
+}
+__device__ __forceinline__ fx fx_signed(fx a, int neg) {
+  const fx m = (fx)neg;
+  return (a ^ m) - m;
+}
+// v 2^-e0 toward zero, where |v| 2^-e0 < 2^60
+__device__ __forceinline__ fx fx_from(double v, int e0) {
+  const int hi = __double2hiint(v), ec = (hi >> 20) & 0x7ff;
+  const fx m = ((fx)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
+  const int r = 1083 + e0 - ec;
+  return fx_signed(ec == 0 || r > 63 ? 0 : (m << 8) >> r, hi >> 31);
+}
+// k v 2^-e0, negated when neg
+__device__ __forceinline__ fx fx_from_k(double v, const FxK& k, int e0, int neg) {
+  const int hi = __double2hiint(v), ec = (hi >> 20) & 0x7ff;
+  const fx m = ((fx)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
+  const int r = 2106 + e0 - ec - k.e;
+  return fx_signed(ec == 0 || k.e == 0 || r > 63 ? 0 : (fx_mul64(m << 9, k.m) << 2) >> r, (hi >> 31) ^ k.neg ^ neg);
+}
+// Upper bound of |v| (|k v|) as w 2^(e - 14): e and w for the running maximum of e; v zero: e very low
+__device__ __forceinline__ int fx_bexp(int hi) {
+  const int ec = (hi >> 20) & 0x7ff;
+  return ec == 0 ? kFxNone : ec == 0x7ff ? kFxNan : ec - 1023;
+}
+__device__ __forceinline__ unsigned fx_mant15(int hi) { return (((hi & 0xfffff) | 0x100000) >> 6) + 1; }
+
+// Sum over the block of w (pairs (E, S) per warp, S in units of 2^(E - 14)); returns the bit
+// length nb and the exponent E: sum < 2^(nb + E - 14).  sh: 2 ints per warp.
+__device__ __forceinline__ void fx_block_bound(int E, unsigned S, int* sh, int* Eo, int* nb) {
+  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    sh[2 * warp] = E;
+    sh[2 * warp + 1] = (int)S;
+  }
+  __syncthreads();
+  int Em = sh[0];
+  for (int w = 1; w < nw; ++w) Em = max(Em, sh[2 * w]);
+  unsigned tot = 0;
+  for (int w = 0; w < nw; ++w) {
+    const int d = Em - sh[2 * w];
+    tot += (d > 31 ? 0u : (unsigned)sh[2 * w + 1] >> d) + 4u;
+  }
+  *Eo = Em;
+  *nb = 32 - __clz((int)tot);
+}
+
+__device__ __forceinline__ const int2* fx_info(const Inst& I, int slot, int f, int j) {
+  return I.pinfo + ((size_t)slot * kFieldsSynth + f) * I.ny + j;
+}
+// x-storage index i (m = i for i <= Kx, m = i - Mx otherwise) -> FFT bin
+__device__ __forceinline__ int xbin(int i, int Kx, int Mx, int nx) { return i <= Kx ? i : nx - (Mx - i); }
+__device__ __forceinline__ int fx_div(int t, unsigned mul) { return (int)__umulhi((unsigned)t, mul); }
+
+}  // namespace
+
+// x rows (one per retained z mode) and z rows (row pairs) in shared memory: the x array whole,
+// the z rows `chunk` at a time.
+struct FxPlanes {
+  int LX, LZ, chunk;
+};
+// One pass of `threads` threads covers threads/8 row pairs in the first z pass, so more rows
+// at a time would only cost shared memory.
+__host__ __device__ inline FxPlanes fx_planes(const Inst& I, int threads) {
+  FxPlanes p;
+  p.LX = I.nx + 1;
+  p.LZ = I.nz + 1;
+  p.chunk = I.nx / 2 < threads / 8 ? I.nx / 2 : threads / 8 < 16 ? 16 : threads / 8;
+  return p;
+}
+// [x rows | z rows | 64 ints of reduction | exponents of the row pairs and x rows | alignment]
+size_t smem_planes_fx(const Inst& I, int threads) {
+  const FxPlanes p = fx_planes(I, threads);
+  return sizeof(fxc) * ((size_t)I.Mz * p.LX + (size_t)p.chunk * p.LZ) + 4 * (64 + 64 + 64 + 64);
+}
+// Threads per CTA: the synthesis of small planes keeps two warps busy in every pass; the
+// products, with fewer CTAs and a pointwise part, take twice as many.
+bool planes_fx_big(const Inst& I) { return I.nx > 64 || I.nz > 64; }
+int planes_fx_threads(const Inst& I, bool prod) {
+  if (planes_fx_big(I)) return 256;
+  return !prod && I.nx * I.nz <= 1024 ? 64 : 128;
+}
+
+__constant__ int c_fx_src[kFieldsSynth] = {0, 1, 2, 0, 3, 0, 1, 1, 2, 4, 2};
+__constant__ int c_fx_fac[kFieldsSynth] = {0, 0, 0, 1, 0, 2, 1, 2, 1, 0, 2};
+
+// ------------------------------------------------------------------ plane synthesis
+// CTA = (instance, y-plane j, field f), fields as in k_xzsynth_t.  The plane's exponent e0 comes
+// from the sum B of |Re| + |Im| over the plane's modes (p > 0 twice): every intermediate of the
+// two transforms is below 2 B in modulus, and 2 B 2^-e0 <= 2^61.
+template <bool BIG>
+__global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_synth_fx(LaunchInfo li, int slot, int nfields) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  int local;
+  const int b = find_inst(li, blockIdx.x, &local);
+  const Inst& I = li.insts[b];
+  if (!inst_active(I)) return;
+  const int f = local % nfields, j = local / nfields;
+  const int nx = I.nx, nz = I.nz, Mz = I.Mz, Kx = I.Kx, Kz = I.Kz, nm = I.nmodes;
+  const FxPlanes P = fx_planes(I, blockDim.x);
+  fxc* G = reinterpret_cast<fxc*>(smraw);
+  fxc* Z = G + Mz * P.LX;
+  int* red = reinterpret_cast<int*>(Z + P.chunk * P.LZ);
+  const double2* src = I.yv + (((size_t)slot * kFieldsY + c_fx_src[f]) * I.ny + j) * (size_t)nm;
+  const int fac = c_fx_fac[f];
+  // exponent of the plane
+  int E = kFxNone;
+  const unsigned mzm = I.mz_mul;
+  const auto bexp = [&](int t, int hi) {
+    int e = fx_bexp(hi);
+    if (fac == 1) e += fx_bexp(__double2hiint(I.kx[fx_div(t, mzm)]));
+    else if (fac == 2) e += fx_bexp(__double2hiint(I.kz[t - fx_div(t, mzm) * Mz]));
+    return e;
+  };
+  for (int t = threadIdx.x; t < nm; t += blockDim.x) {
+    const double2 s = src[t];
+    E = max(E, max(bexp(t, __double2hiint(s.x)), bexp(t, __double2hiint(s.y))));
+  }
+  E = __reduce_max_sync(0xffffffffu, E);
+  unsigned S = 0;
+  const bool bad = E > kFxNan / 4;
+  if (E > kFxNone / 2 && !bad)
+    for (int t = threadIdx.x; t < nm; t += blockDim.x) {
+      const double2 s = src[t];
+      const int i = fx_div(t, mzm), p = t - i * Mz;
+      const double k = fac == 1 ? I.kx[i] : fac == 2 ? I.kz[p] : 1.0;
+      const int kh = __double2hiint(k) & 0x7fffffff, ek = fx_bexp(kh);
+      const unsigned km = fx_mant15(kh);
+      unsigned w = 0;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        // terms below 2^-28 of the largest: at most 2 units in all, within the slack of the block sum
+        const int hi = __double2hiint(c ? s.y : s.x), d = E - (fx_bexp(hi) + ek);
+        if (d < 28) w += ((fac ? (fx_mant15(hi) * km) >> 14 : fx_mant15(hi)) >> d) + 1;
+      }
+      S += p ? 2 * w : w;
+    }
+  S = __reduce_add_sync(0xffffffffu, S);
+  int nb;
+  fx_block_bound(E, S, red, &E, &nb);
+  int2* info = const_cast<int2*>(fx_info(I, slot, f, j));
+  fx* out = reinterpret_cast<fx*>(I.phys) + (((size_t)slot * kFieldsSynth + f) * I.ny + j) * (size_t)nx * nz;
+  if (E > kFxNan / 4 || E < kFxNone / 2) {  // a NaN or an infinity in the plane, or a zero plane (uniform)
+    if (E < kFxNone / 2)
+      for (int t = threadIdx.x; t < nx * nz; t += blockDim.x) out[t] = 0;
+    if (threadIdx.x == 0) *info = make_int2(E > kFxNan / 4 ? kFxNan : kFxNone, 0);
+    return;
+  }
+  const int e0 = nb + E - 74;
+  // the modes as integers at their x bins (rows p); i k v for the x and z derivatives
+  for (int t = threadIdx.x; t < nm; t += blockDim.x) {
+    const double2 s = src[t];
+    const int i = fx_div(t, mzm), p = t - i * Mz, bin = xbin(i, Kx, I.Mx, nx);
+    fxc v;
+    if (fac == 0) {
+      v = fxc{fx_from(s.x, e0), fx_from(s.y, e0)};
+    } else {
+      const FxK k = fx_factor(fac == 1 ? I.kx[i] : I.kz[p]);
+      v = fxc{fx_from_k(s.y, k, e0, -1), fx_from_k(s.x, k, e0, 0)};
+    }
+    G[p * P.LX + fx_slot(bin >> 3, bin & 7)] = v;
+  }
+  __syncthreads();
+  // x stage, rows p: element = x bin; bins outside |m| <= Kx are zero
+  fx_length<BIG>(nx, [&](auto rc) {
+    constexpr int R = decltype(rc)::R;
+    fx_first<R, true>(Mz, G, P.LX, I.twfx_x + nx, [&](int p, int n, fxc* v) {
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        const int bin = n + 8 * q;
+        v[q] = bin <= Kx || bin >= nx - Kx ? G[p * P.LX + fx_slot(q, n)] : fxc{0, 0};
+      }
+    });
+    __syncthreads();
+    fx_second<R, true>(Mz, G, P.LX, [&](int p, int bk, const fxc* v) {
+      fxc* o = G + p * P.LX;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[fx_slot(bk, e)] = v[e];
+    });
+  });
+  __syncthreads();
+  const int nr = nx / 2, Rx = nx >> 3;
+  const unsigned rxm = I.rx_mul;
+  unsigned mh = 0;
+  for (int r0 = 0; r0 < nr; r0 += P.chunk) {
+    const int nrc = min(P.chunk, nr - r0);
+    fx_length<BIG>(nz, [&](auto rc) {
+      constexpr int R = decltype(rc)::R;
+      // row pair (x1, x2 = x1 + 1) -> one complex row G[x1] + i G[x2] (see k_xzsynth_t)
+      fx_first<R, true>(nrc, Z, P.LZ, I.twfx_z + nz, [&](int r, int n, fxc* v) {
+        const int x1 = 2 * (r0 + r), k3 = fx_div(x1, rxm), k1 = x1 - k3 * Rx;
+        const int s1 = fx_slot(k1, k3), s2 = fx_slot(k1 + 1, k3);
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const int z = n + 8 * q;
+          const bool lo = z <= Kz, hi = z >= nz - Kz;
+          v[q] = fxc{0, 0};
+          if (lo || hi) {
+            const fxc* g = G + (lo ? z : nz - z) * P.LX;
+            fxc g1 = g[s1], g2 = g[s2];
+            if (z == 0) g1.y = g2.y = 0;
+            v[q] = lo ? fxc{g1.x - g2.y, g1.y + g2.x} : fxc{g1.x + g2.y, g2.x - g1.y};
+          }
+        }
+      });
+      __syncthreads();
+      fx_second<R, true>(nrc, Z, P.LZ, [&](int r, int bk, const fxc* v) {
+        fx* o = out + (size_t)(2 * (r0 + r)) * nz + bk;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          o[R * e] = v[e].x;
+          o[nz + R * e] = v[e].y;
+          mh = max(mh, max(fx_maghi(v[e].x), fx_maghi(v[e].y)));
+        }
+      });
+    });
+    __syncthreads();  // the next chunk rewrites Z
+  }
+  mh = __reduce_max_sync(0xffffffffu, mh);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (int)mh;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mh = max(mh, (unsigned)red[w]);
+    *info = make_int2(e0, fx_bits(mh));
+  }
+}
+
+// ------------------------------------------------------------------ products + analysis
+namespace {
+
+__device__ __forceinline__ fx fx_shift(fx x, int s) { return s >= 0 ? x << s : x >> min(-s, 63); }
+// exponent of a plane scaled to 62 bits (kFxNone: zero, kFxNan: not finite)
+__device__ __forceinline__ int fx_e62(int2 inf) { return inf.x == kFxNan || inf.x == kFxNone ? inf.x : inf.x + inf.y - 62; }
+// field of the gradient component d of velocity component c; v_y = -(u_x + w_z) is field 3 plus
+// field 10 (the sign is the caller's)
+__device__ __forceinline__ int fx_grad(int c, int d) {
+  return c == 0 ? 3 + d : c == 2 ? 8 + d : d == 0 ? 6 : d == 1 ? 3 : 7;
+}
+
+// sum over the block of s 2^e, exact in integers, as a double in thread 0
+__device__ double fx_block_sum(unsigned long long s, int e, int* red) {
+  // 24-bit parts: 32 lanes of each stay below 2^29
+  const unsigned a = (unsigned)s & 0xffffffu, b = (unsigned)(s >> 24) & 0xffffffu, c = (unsigned)(s >> 48);
+  const unsigned ra = __reduce_add_sync(0xffffffffu, a), rb = __reduce_add_sync(0xffffffffu, b),
+                 rc = __reduce_add_sync(0xffffffffu, c);
+  const int warp = threadIdx.x >> 5;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) {
+    red[3 * warp] = (int)ra;
+    red[3 * warp + 1] = (int)rb;
+    red[3 * warp + 2] = (int)rc;
+  }
+  __syncthreads();
+  double v = 0.0;
+  if (threadIdx.x == 0) {
+    unsigned long long A = 0, B = 0, Cc = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      A += (unsigned)red[3 * w];
+      B += (unsigned)red[3 * w + 1];
+      Cc += (unsigned)red[3 * w + 2];
+    }
+    B += A >> 24;
+    Cc += B >> 24;
+    const unsigned long long lo = (A & 0xffffffu) | ((B & 0xffffffu) << 24);
+    v = ldexp((double)Cc, e + 48) + ldexp((double)lo, e);
+  }
+  return v;
+}
+
+}  // namespace
+
+// CTA = (instance, plane j, component c).  Every factor is scaled to 62 bits, the products keep
+// their high 64 bits (2^-60 of the largest product) and are summed at the largest term's
+// exponent.  The transforms rescale every row pair and then every x row from its own largest
+// value, found by shuffles among the eight lanes that hold the row.
+template <bool ADJ, bool BIG>
+__global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_fx(LaunchInfo li, int step_index) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  // factors: 0-2 advecting velocity u_b + u; 3-5 gradient of component c of u (M) or q (N);
+  // N: 6-8 q, 9-11 derivative c of u's components; 12: the factor of U' (v, or q_0).
+  // A factor is plane a 2^sa (+ plane b 2^sb) (+ a constant), below 2^62, with exponent se.
+  __shared__ int se[13], ssa[13], ssb[13], ssd[8];
+  __shared__ fx sadd[2];
+  __shared__ int sh_eP, sh_bad;
+  int local;
+  const int b = find_inst(li, blockIdx.x, &local);
+  const Inst& I = li.insts[b];
+  if (!inst_active(I)) return;
+  const int c = local % 3, j = local / 3;
+  const int nx = I.nx, nz = I.nz, Mx = I.Mx, Mz = I.Mz, Kx = I.Kx;
+  const FxPlanes P = fx_planes(I, blockDim.x);
+  fxc* X = reinterpret_cast<fxc*>(smraw);
+  fxc* Z = X + Mz * P.LX;
+  int* red = reinterpret_cast<int*>(Z + P.chunk * P.LZ);
+  int* er = red + 64;   // exponents of the row pairs
+  int* ep = er + 64;    // exponents of the x rows
+  const double dU = I.ubase[I.ny + j];
+  if (threadIdx.x < 32) {
+    const int k = min((int)threadIdx.x, 12);
+    const int slot = k == 12 ? ADJ : k < 3 ? 0 : k < 9 ? ADJ : 0;
+    const int comp = k < 6 ? c : k - 9, dir = k < 6 ? k - 3 : c;
+    const bool grad = (k >= 3 && k < 6) || (k >= 9 && k < 12);
+    const int f = k < 3 ? k : k == 12 ? (ADJ ? 0 : 1) : grad ? fx_grad(comp, dir) : k - 6;
+    const bool two = grad && comp == 1 && dir == 1;
+    const bool used = k < 6 || (ADJ && k < 12) || (k == 12 && c == (ADJ ? 1 : 0));
+    const double cst = k < 2 ? I.ubase[2 * k * I.ny + j] : 0.0;
+    const int2 ia = used ? *fx_info(I, slot, f, j) : make_int2(kFxNone, 0);
+    const int2 ib = two && used ? *fx_info(I, slot, 10, j) : make_int2(kFxNone, 0);
+    const int ea = fx_e62(ia), eb = fx_e62(ib), ec = cst != 0.0 ? fx_bexp(__double2hiint(cst)) - 59 : kFxNone;
+    int e = max(ea, max(eb, ec));
+    if (e != kFxNan && e != kFxNone && (two || ec != kFxNone)) e += 1;  // room for the sum
+    const int sa = ia.x == kFxNone || e == kFxNan ? 0 : ia.x - e, sb = ib.x == kFxNone || e == kFxNan ? 0 : ib.x - e;
+    // terms: 0-2 advection, 3-5 transposed gradient, 6 the base flow's shear
+    const int t = threadIdx.x;
+    int x = __shfl_sync(0xffffffffu, e, t < 3 ? t : (3 + t) & 31);
+    const int y = __shfl_sync(0xffffffffu, e, t < 3 ? 3 + t : (6 + t) & 31);
+    if (t == 6) x = dU != 0.0 ? fx_bexp(__double2hiint(dU)) - 59 : kFxNone;
+    const bool term = t < 3 || (ADJ && t < 6) || t == 6;
+    const int et = !term || x == kFxNone || y == kFxNone ? kFxNone : x + y + 64;
+    const bool nan = term && (x == kFxNan || y == kFxNan) && !(t == 6 && y == kFxNone);
+    const int em = __reduce_max_sync(0xffffffffu, nan ? kFxNone : et);
+    const bool any = __any_sync(0xffffffffu, nan);
+    if (t < 13) {
+      se[t] = e;
+      ssa[t] = sa;
+      ssb[t] = sb;
+    }
+    if (t < 2) sadd[t] = ec != kFxNone && e != kFxNan ? fx_from(cst, e) : 0;
+    if (t < 7) ssd[t] = min(et == kFxNone ? 63 : em - et, 63);
+    if (t == 0) {
+      sh_eP = em;
+      sh_bad = any;
+    }
+  }
+  __syncthreads();
+  const bool bad = sh_bad != 0;
+  int eP = sh_eP;
+  const bool zero = eP < kFxNone / 2;
+  unsigned long long sq = 0;
+  const int eq = ADJ ? se[6 + c] : kFxNone;
+  const bool sqok = ADJ && eq != kFxNan && eq != kFxNone;
+  const int nr = nx / 2;
+  const unsigned nzm = I.nz_mul;
+  const fx dUx = c == (ADJ ? 1 : 0) ? fx_from(dU, fx_bexp(__double2hiint(dU)) - 59) : 0;
+  const int lgz = 32 - __clz(nz - 1), lgx = 32 - __clz(nx - 1);
+  // the factors' planes (offsets uniform in the CTA) and shifts
+  constexpr int NO = ADJ ? 12 : 6;
+  const int fs = I.ny * nx * nz;
+  const fx* const U = reinterpret_cast<const fx*>(I.phys) + (size_t)j * nx * nz;
+  const fx* const Q = U + (ADJ ? (size_t)kFieldsSynth * fs : 0);
+  int of[NO], sa[NO], sd[7];
+#pragma unroll
+  for (int k = 0; k < NO; ++k) {
+    of[k] = fs * (k < 3 ? k : k < 6 ? fx_grad(c, k - 3) : k < 9 ? k - 6 : fx_grad(k - 9, c));
+    sa[k] = ssa[k];
+  }
+#pragma unroll
+  for (int k = 0; k < 7; ++k) sd[k] = ssd[k];
+  const fx add0 = sadd[0], add1 = sadd[1];
+  // One loop over the transform stages, so that the z stage of every chunk of rows and the x
+  // stage run the same instructions (the kernel's straight-line code otherwise exceeds the
+  // instruction cache): job g < nch is chunk g's products and z stage, job nch the x stage.
+  const int nch = bad || (zero && !ADJ) ? 0 : (nr + P.chunk - 1) / P.chunk;
+  const bool live = !bad && !zero;
+  int* align = ep + 64;  // right shift of each row pair's values in the x stage (z stage: none)
+  if (threadIdx.x < 64) align[threadIdx.x] = 0;
+  for (int g = 0; g <= nch; ++g) {
+    const bool xs = g == nch;
+    const int r0 = g * P.chunk, nrc = xs ? 0 : min(P.chunk, nr - r0), base = 2 * r0 * nz;
+    // products of the chunk's rows, two neighbouring points per thread: row 2r in the real
+    // part, 2r + 1 in the imaginary part
+    for (int t = 2 * threadIdx.x; t < 2 * nrc * nz; t += 2 * blockDim.x) {
+      const int row = fx_div(t, nzm), z = t - row * nz, e = base + t;
+      longlong2 x[NO];
+#pragma unroll
+      for (int k = 0; k < NO; ++k)
+        x[k] = __ldg(reinterpret_cast<const longlong2*>((k >= 3 && k < 9 ? Q : U) + of[k] + e));
+      longlong2 b4 = make_longlong2(0, 0), b10 = b4, pv = b4;
+      if (c == 1) {  // v_y = -(u_x + w_z)
+        b4 = __ldg(reinterpret_cast<const longlong2*>(Q + 10 * fs + e));
+        if (ADJ) b10 = __ldg(reinterpret_cast<const longlong2*>(U + 10 * fs + e));
+      }
+      if (!ADJ && c == 0) pv = __ldg(reinterpret_cast<const longlong2*>(U + fs + e));
+      fx val[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        fx v[NO];
+#pragma unroll
+        for (int k = 0; k < NO; ++k) {
+          v[k] = h ? x[k].y : x[k].x;
+          v[k] = k < 2 || k == 4 || k == 10 ? fx_shift(v[k], sa[k]) : v[k] << sa[k];
+        }
+        v[0] += add0;
+        v[1] += add1;
+        if (c == 1) {
+          v[4] = -(v[4] + fx_shift(h ? b4.y : b4.x, ssb[4]));
+          if (ADJ) v[10 % NO] = -(v[10 % NO] + fx_shift(h ? b10.y : b10.x, ssb[10]));
+        }
+        fx a = (fx_mul64(v[0], v[3]) >> sd[0]) + (fx_mul64(v[1], v[4]) >> sd[1]) + (fx_mul64(v[2], v[5]) >> sd[2]);
+        if (!ADJ) {
+          if (c == 0) a += fx_mul64(dUx, (h ? pv.y : pv.x) << ssa[12]) >> sd[6];
+          a = -a;
+        } else {
+          a -= (fx_mul64(v[6 % NO], v[9 % NO]) >> sd[3]) + (fx_mul64(v[7 % NO], v[10 % NO]) >> sd[4]) +
+               (fx_mul64(v[8 % NO], v[11 % NO]) >> sd[5]);
+          if (c == 1) a -= fx_mul64(dUx, v[6 % NO]) >> sd[6];
+          const fx qc = (c == 0 ? v[6 % NO] : c == 1 ? v[7 % NO] : v[8 % NO]) >> 2;  // at most 64 squares below 2^56
+          sq += (unsigned long long)fx_mul64(qc, qc);
+        }
+        val[h] = a;
+      }
+      fxc* o = Z + (row >> 1) * P.LZ;
+      reinterpret_cast<fx*>(o + fx_slot(z >> 3, z & 7))[row & 1] = val[0];
+      reinterpret_cast<fx*>(o + fx_slot(z >> 3, (z & 7) + 1))[row & 1] = val[1];
+    }
+    if (!live) continue;
+    if (xs) {
+      int emax = kFxNone;
+      for (int r = threadIdx.x & 31; r < nr; r += 32) emax = max(emax, er[r]);
+      emax = __reduce_max_sync(0xffffffffu, emax);
+      if (threadIdx.x < nr) align[threadIdx.x] = emax - er[threadIdx.x];
+      eP = emax;
+    }
+    __syncthreads();
+    fxc* const buf = xs ? X : Z;
+    const int LS = xs ? P.LX : P.LZ, rows = xs ? Mz : nrc, lg = xs ? lgx : lgz + 1;
+    int* const eo = xs ? ep : er + r0;
+    fx_length<BIG>(xs ? nx : nz, [&](auto rc) {
+      constexpr int R = decltype(rc)::R;
+      fx_first<R, false>(rows, buf, LS, xs ? I.twfx_x : I.twfx_z, [&](int r, int n, fxc* v) {
+        unsigned mh = 0;
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const fxc a = buf[r * LS + fx_slot(q, n)];
+          const int d = min(align[(n + 8 * q) >> 1], 63);
+          v[q] = fxc{a.x >> d, a.y >> d};
+          mh = max(mh, max(fx_maghi(v[q].x), fx_maghi(v[q].y)));
+        }
+        const unsigned m = 0xffu << (threadIdx.x & 24);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) mh = max(mh, __shfl_xor_sync(m, mh, o));
+        // sqrt(2) n max <= 2^61 (z stage: the unpacking adds two values), 2^62 (x stage)
+        const int s = fx_bits(mh) + 1 + lg - 62;
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = fxc{fx_shift(v[q].x, -s), fx_shift(v[q].y, -s)};
+        if (n == 0) eo[r] = eP + s - (xs ? 0 : 1);
+      });
+      __syncthreads();
+      fx_second<R, false>(rows, buf, LS, [&](int r, int bk, const fxc* v) {
+        fxc* o = buf + r * LS;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) o[fx_slot(bk, e)] = v[e];
+      });
+    });
+    __syncthreads();
+    // rows x1 and x2 of each pair, twice their value: F1 = H_p + conj(H_-p), F2 = -i (H_p - conj(H_-p))
+    for (int t = threadIdx.x; t < nrc * Mz; t += blockDim.x) {
+      const int r = fx_div(t, I.mz_mul), p = t - r * Mz, pm = p == 0 ? 0 : nz - p;
+      const int kp = fx_div(p, I.rz_mul), km = fx_div(pm, I.rz_mul), Rz = nz >> 3;
+      const fxc hp = Z[r * P.LZ + fx_slot(p - kp * Rz, kp)], hm = Z[r * P.LZ + fx_slot(pm - km * Rz, km)];
+      const int x = 2 * (r0 + r);
+      X[p * P.LX + fx_slot(x >> 3, x & 7)] = fxc{hp.x + hm.x, hp.y - hm.y};
+      X[p * P.LX + fx_slot(x >> 3, (x & 7) + 1)] = fxc{hp.y + hm.y, hm.x - hp.x};
+    }
+    if (!xs) __syncthreads();
+  }
+  double2* dst = I.xz + ((size_t)c * I.ny + j) * I.nmodes;
+  const int Rx = nx >> 3;
+  for (int t = threadIdx.x; t < I.nmodes; t += blockDim.x) {
+    const int i = fx_div(t, I.mz_mul), p = t - i * Mz, bin = xbin(i, Kx, Mx, nx), k3 = fx_div(bin, I.rx_mul);
+    double2 o = make_double2(0.0, 0.0);
+    if (bad) o.x = o.y = __longlong_as_double(0x7ff8000000000000LL);
+    if (live) {
+      fxc a = X[p * P.LX + fx_slot(bin - k3 * Rx, k3)];
+      if (I.nfx_h) a = fxc{fx_mulc(a.x, I.nfx_h, I.nfx_l), fx_mulc(a.y, I.nfx_h, I.nfx_l)};
+      const int e0 = ep[p] + I.nfx_e;
+      o = make_double2(__longlong_as_double((long long)fx_double_bits(a.x, e0)),
+                       __longlong_as_double((long long)fx_double_bits(a.y, e0)));
+    }
+    dst[t] = o;
+  }
+  if (ADJ) {
+    const double s = fx_block_sum(sq, sqok ? 2 * eq + 68 : 0, red);
+    if (threadIdx.x == 0)
+      I.normpart[(size_t)c * I.ny + j] = eq == kFxNan || bad ? __longlong_as_double(0x7ff8000000000000LL) : sqok ? s : 0.0;
+  }
+  if (ADJ && step_index >= 0) finish_norm(I, step_index);
+}
+
+// CTA = (instance, plane j, component c): sum over the plane of the squared velocity component
+// c of a slot (0: u, 1: q).
+__global__ void __launch_bounds__(128) k_norm_planes_fx(LaunchInfo li, int slot) {
+  __shared__ int red[64];
+  int local;
+  const int b = find_inst(li, blockIdx.x, &local);
+  const Inst& I = li.insts[b];
+  const int c = local % 3, j = local / 3, n = I.nx * I.nz;
+  const int2 inf = *fx_info(I, slot, c, j);
+  const int e = fx_e62(inf), sa = 62 - inf.y;
+  const bool ok = e != kFxNan && e != kFxNone;
+  const fx* a = reinterpret_cast<const fx*>(I.phys) + (((size_t)slot * kFieldsSynth + c) * I.ny + j) * (size_t)n;
+  unsigned long long sq = 0;
+  if (ok)
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+      const fx q = (a[t] << sa) >> 2;  // at most 128 squares below 2^56 per thread
+      sq += (unsigned long long)fx_mul64(q, q);
+    }
+  const double s = fx_block_sum(sq, ok ? 2 * e + 68 : 0, red);
+  if (threadIdx.x == 0)
+    I.normpart[(size_t)c * I.ny + j] = e == kFxNan ? __longlong_as_double(0x7ff8000000000000LL) : s;
+}
+
+void launch_xzsynth_fx(bool big, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf) {
+  if (big) k_synth_fx<true><<<ctas, threads, smem, s>>>(li, slot, nf);
+  else k_synth_fx<false><<<ctas, threads, smem, s>>>(li, slot, nf);
+}
+void launch_prod_fx(bool big, bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li,
+                    int step_index) {
+  if (big && adj) k_prod_fx<true, true><<<ctas, threads, smem, s>>>(li, step_index);
+  else if (big) k_prod_fx<false, true><<<ctas, threads, smem, s>>>(li, -1);
+  else if (adj) k_prod_fx<true, false><<<ctas, threads, smem, s>>>(li, step_index);
+  else k_prod_fx<false, false><<<ctas, threads, smem, s>>>(li, -1);
+}
+void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot) {
+  k_norm_planes_fx<<<ctas, 128, 0, s>>>(li, slot);
+}
+cudaError_t set_planes_fx_smem(size_t synth, size_t prod) {
+  cudaError_t e;
+  if ((e = raise_smem_limit((const void*)k_synth_fx<false>, synth))) return e;
+  if ((e = raise_smem_limit((const void*)k_synth_fx<true>, synth))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_fx<true, false>, prod))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_fx<true, true>, prod))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_fx<false, true>, prod))) return e;
+  return raise_smem_limit((const void*)k_prod_fx<false, false>, prod);
+}
+
+}  // namespace pcf

@@ -195,10 +195,10 @@ __host__ __device__ inline WarpPlan warp_plan(const Inst& I, int elem) {
 
 template <class T>
 __device__ __forceinline__ void load_twiddles_w(const Inst& I, typename Cx<T>::c* twx, typename Cx<T>::c* twz) {
-  const typename Sto<T>::c* sx = twx_of<T>(I);
-  const typename Sto<T>::c* sz = twz_of<T>(I);
-  for (int t = threadIdx.x; t < I.nx; t += blockDim.x) twx[t] = load_c<T>(sx[t]);
-  for (int t = threadIdx.x; t < I.nz; t += blockDim.x) twz[t] = load_c<T>(sz[t]);
+  const typename Cx<T>::c* sx = twx_of<T>(I);
+  const typename Cx<T>::c* sz = twz_of<T>(I);
+  for (int t = threadIdx.x; t < I.nx; t += blockDim.x) twx[t] = sx[t];
+  for (int t = threadIdx.x; t < I.nz; t += blockDim.x) twz[t] = sz[t];
 }
 
 __constant__ int c_src_w[kFieldsSynth] = {0, 1, 2, 0, 3, 0, 1, 1, 2, 4, 2};
@@ -233,12 +233,12 @@ __global__ void __launch_bounds__(kWarpPlaneThreads, 3) k_xzsynth_w(LaunchInfo l
   C* twx = sm + wp.twx;
   C* twz = sm + wp.twz;
   load_twiddles_w<T>(I, twx, twz);
-  const typename Sto<T>::c* src =
+  const typename Cx<T>::c* src =
       yv_of<T>(I) + (((size_t)slot * kFieldsY + c_src_w[f]) * I.ny + j) * (size_t)I.nmodes;
   const int fac = c_fac_w[f];
   for (int t = threadIdx.x; t < I.nmodes; t += blockDim.x) {
     const int i = t / Mz, p = t - i * Mz;
-    C s = load_c<T>(src[t]);
+    C s = src[t];
     if (fac == 1) { const T k = (T)I.kx[i]; s = Cx<T>::mk(-k * s.y, k * s.x); }
     else if (fac == 2) { const T k = (T)I.kz[p]; s = Cx<T>::mk(-k * s.y, k * s.x); }
     S[i * SP + p] = s;
@@ -505,39 +505,12 @@ __global__ void __launch_bounds__(kWarpPlaneThreads, 2) k_prod_w(LaunchInfo li, 
       }
   }
   __syncthreads();
-  typename Sto<T>::c* dst = xz_of<T>(I) + ((size_t)c * I.ny + j) * I.nmodes;
+  typename Cx<T>::c* dst = xz_of<T>(I) + ((size_t)c * I.ny + j) * I.nmodes;
   for (int t = threadIdx.x; t < I.nmodes; t += blockDim.x) {
     const int i = t / Mz, p = t - i * Mz;
-    dst[t] = store_c<T>(O[i * SP + p]);
+    dst[t] = O[i * SP + p];
   }
-  if (ADJ && step_index >= 0) {
-    // J = ||r1|| once all 3 ny plane sums of the instance are written (the chain of
-    // norm_from_parts, as in the Stockham kernel)
-    __shared__ int last;
-    if (threadIdx.x == 0) {
-      __threadfence();
-      last = atomicAdd(I.jcount, 1) == 3 * I.ny - 1;
-    }
-    __syncthreads();
-    if (last) {
-      const int ny = I.ny;
-      const double* P = I.normpart;
-      double* ps = reinterpret_cast<double*>(smraw);
-      for (int q = threadIdx.x; q < ny; q += blockDim.x) {
-        ps[q] = __ldcg(P + q) + __ldcg(P + ny + q) + __ldcg(P + 2 * ny + q);
-        ps[ny + q] = I.ccw[q];
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int q = 0; q < ny; ++q) s = fma(ps[ny + q], ps[q], s);
-        const double J = sqrt(0.5 * I.inv_nxnz * s);
-        if (I.hist) I.hist[(size_t)step_index * I.hist_stride] = J;
-        if (I.tol > 0.0 && J < I.tol && I.active) *I.active = 0;
-        *I.jcount = 0;
-      }
-    }
-  }
+  if (ADJ && step_index >= 0) finish_norm(I, step_index);
 }
 
 void launch_xzsynth_warp(int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf) {

@@ -78,20 +78,12 @@ void launch_symmetrize(int ctas_x, int ninst, cudaStream_t s, const Inst* insts,
 // h_s = ||u_s|| from the plane sums of u^2 (same arithmetic as the norm of r1), its history
 // entry, and the discrete-extremum test of the previous step:
 //   (h_{s-1} - h_{s-2}) (h_s - h_{s-1}) < 0  ->  u_{s-1} (held in uprev) is a guess.
-// One CTA per instance; D.step counts the steps of the current call.
-__global__ void __launch_bounds__(128) k_dns_norm(const Inst* insts, DnsInst* dns) {
-  __shared__ double part[3 * 257];
-  __shared__ double w[257];
+// One warp per instance; D.step counts the steps of the current call.
+__global__ void __launch_bounds__(32) k_dns_norm(const Inst* insts, DnsInst* dns) {
   const Inst& I = insts[blockIdx.x];
   DnsInst& D = dns[blockIdx.x];
-  const int ny = I.ny;
-  for (int t = threadIdx.x; t < 3 * ny; t += blockDim.x) part[t] = I.normpart[t];
-  for (int t = threadIdx.x; t < ny; t += blockDim.x) w[t] = I.ccw[t];
-  __syncthreads();
+  const double h = norm_from_parts(I);
   if (threadIdx.x != 0) return;
-  double s = 0.0;
-  for (int j = 0; j < ny; ++j) s = fma(w[j], part[j] + part[ny + j] + part[2 * ny + j], s);
-  const double h = sqrt(0.5 * I.inv_nxnz * s);
   const int step = D.step;
   if (D.hist) D.hist[(size_t)step * D.hist_stride] = h;
   int slot = -1;
@@ -135,7 +127,7 @@ int dns_ctas(const Inst& I) {
 }
 
 void launch_dns_norm(int ninst, cudaStream_t s, const Inst* insts, DnsInst* dns) {
-  k_dns_norm<<<ninst, 128, 0, s>>>(insts, dns);
+  k_dns_norm<<<ninst, 32, 0, s>>>(insts, dns);
 }
 void launch_dns_capture(int ctas_x, int ninst, cudaStream_t s, const Inst* insts, const DnsInst* dns) {
   k_dns_capture<<<dim3(ctas_x, ninst), 256, 0, s>>>(insts, dns);
