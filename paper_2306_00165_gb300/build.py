@@ -13,7 +13,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libpcfadj.so")
-SOURCES = ["pcf_kernels.cu", "pcf_host.cu", "pcf_noalloc.cu", "pcf_dmd.cu", "pcf_cheb_tc.cu", "pcf_modes_split.cu",
+SOURCES = ["pcf_kernels.cu", "pcf_host.cu", "pcf_noalloc.cu", "pcf_dmd.cu", "pcf_cheb_tc.cu", "pcf_modes_fx.cu",
            "pcf_fno.cu", "pcf_sym_dns.cu", "pcf_planes_warp.cu", "pcf_cheb_tc05.cu",
            "pcf_sweep.cu", "pcf_planes_fx.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -14,7 +14,6 @@ struct pcf_ctx {
   bool uniform = true;   // every instance on the same problem
   bool suction = false;  // some instance has a base flow with suction (PCF_ASBL)
   int mode_thr = 128;    // threads per CTA of the single per-mode kernel
-  int thr_ya = 256, thr_yy = 128;  // threads per CTA of the split analysis and synthesis
   bool mixed = false;    // mixed-precision form (FP32 planes, split-BF16 Chebyshev, FP64 solves)
   int plane_kind = 0;    // 0 FP64 form, 1 mixed form, 2 float-float form
   // fixed-point plane kernels: threads per CTA; some side above 64
@@ -28,8 +27,7 @@ struct pcf_ctx {
   int* pre_ya_r = nullptr;
   int* pre_yy_r = nullptr;
   int* pre_ys_r = nullptr;
-  int cta_ya_r = 0, cta_yy_r = 0, cta_ys_r = 0, grid_ys_r = 0;
-  double tuned_ms = 0.0; // autotuner: time of the chosen mode-kernel launch
+  int cta_ya_r = 0, cta_yy_r = 0, cta_ys_r = 0;
   cudaStream_t user = nullptr, cs = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   std::vector<void*> allocs;
@@ -45,21 +43,21 @@ struct pcf_ctx {
   int* pre_tca = nullptr;   // tensor-core analysis (mixed form)
   int cta_synth11 = 0, cta_synth3 = 0, cta_prod = 0, cta_mode = 0, cta_tcs = 0, cta_tca = 0;
   size_t sm_synth = 0, sm_prod = 0, sm_mode = 0, sm_tc = 0, sm_warp = 0;
-  // split mode kernels (FP64 form with dense operators): instance groups and geometry
+  // the FP64 forms' fixed-point per-mode kernels (every solve_kind but 1)
   bool split = false;
-  int sgrp = 0;                 // largest instances per group
-  int smt = 1;                  // consecutive modes per CTA of the split analysis
-  int smt_y = 1;                // ... and of the split synthesis (tuned separately)
+  int sgrp = 0;                 // largest instances per group of the solve
+  int np = 8;                   // modes per tile of the analysis and synthesis
   int ngroups = 0;
   int2* d_groups = nullptr;     // [B] (first, count)
-  int* pre_ya = nullptr;        // CTA prefixes over groups [B + 1]
-  int* pre_ys = nullptr;
+  int* pre_ya = nullptr;        // CTA prefixes over instances: analysis, synthesis
   int* pre_yy = nullptr;
+  int* pre_ys = nullptr;        // ... over groups: one CTA per (group, mode)
   int cta_ya = 0, cta_ys = 0, cta_yy = 0;
-  int grid_ys = 0, buf_ys = 0, rows_ys = 0;  // persistent solve: CTAs, stage buffer, scratch rows
-  // the solve's own instance groups (its right-hand sides are per instance, so its grouping
-  // is independent of the analysis and synthesis kernels'); tuned separately
-  int sgrp_s = 0, ngroups_s = 0;
+  int thr_ya = 64, thr_yy = 64, thr_ys = 64, thr_yf = 64;
+  bool fine_y = false, fine_s = false;  // one row and one part per thread (few row pairs)
+  size_t sm_ya = 0, sm_ys = 0, sm_yy = 0, sm_yf = 0;
+  // the step runs the fused half-step kernel (k_ystep_fx), with a separate norm kernel (jn)
+  bool fused = false, jn = false;
   // the split step's Stokes solve by banded sweeps, one thread per chain (k_sweep), in place
   // of the dense solve: CTA prefixes per instance (full and reduced launches) and geometry
   bool sweep = false;
@@ -67,13 +65,6 @@ struct pcf_ctx {
   int* pre_sw_r = nullptr;
   int cta_sw = 0, cta_sw_r = 0, thr_sw = 32;
   size_t sm_sw = 0;
-  int2* d_groups_s = nullptr;
-  bool fused = false;           // the step runs the fused per-mode kernel (k_ystep)
-  int* pre_yf = nullptr;        // its CTA prefix over groups [B + 1]
-  int cta_yf = 0;
-  size_t sm_yf = 0;
-  size_t sm_ya = 0, sm_ys = 0, sm_yy = 0;
-  double tuned_split_ms = 0.0;
   double2* r_int = nullptr;    // internal r1 buffer for descent
   double2* u_dev = nullptr;    // device state for the *_host entry point
   double* hist_dev = nullptr;

@@ -89,6 +89,43 @@ std::vector<double> make_cheb(int N) {
   return t;
 }
 
+// Fixed-point Chebyshev tables (FxTab): columns k of row pairs (2 rp, 2 rp + 1), entries in
+// units of 2^-57 split into 29-bit words.  Analysis (Ae, Ao): coefficient 2k or 2k + 1 from the
+// folded sums, scaled by a power of two so that the largest entry stays at or below 1 (*exp:
+// exponent of a product's unit, 2^55 of theirs, relative to the column's); synthesis
+// (Ce, Co): T_{2k}(y_j), T_{2k+1}(y_j).
+std::vector<int4> make_fxcheb(int N, int* exp) {
+  const int H = N / 2 + 1, half = N / 2, hE = (H + 1) / 2, hO = (half + 1) / 2;
+  int ka = 0;  // 2^ka * 2/N <= 1
+  while ((4 << ka) <= N) ++ka;
+  *exp = -2 - ka;
+  auto cosl_frac = [&](long long a) {
+    return std::cos(3.14159265358979323846264338327950288L * (long double)(a % (2LL * N)) / (long double)N);
+  };
+  auto words = [](long double v) {
+    const long long z = std::llrint(std::ldexp(v, 57));
+    const int h = (int)((z + (1 << 28)) >> 29);
+    return make_int2(h, (int)(z - ((long long)h << 29)));
+  };
+  std::vector<int4> t;
+  auto block = [&](int K, int rows, int hp, auto&& entry) {
+    for (int k = 0; k < K; ++k)
+      for (int rp = 0; rp < hp; ++rp) {
+        const int2 a = words(entry(2 * rp, k)), b = 2 * rp + 1 < rows ? words(entry(2 * rp + 1, k)) : make_int2(0, 0);
+        t.push_back(make_int4(a.x, a.y, b.x, b.y));
+      }
+  };
+  auto inv = [&](int n, int j) {
+    const long double cn = n == 0 || n == N ? 2.0L : 1.0L, cj = j == 0 || j == N ? 2.0L : 1.0L;
+    return std::ldexp(2.0L / (N * cn * cj) * cosl_frac((long long)n * j), ka);
+  };
+  block(H, H, hE, [&](int r, int j) { return inv(2 * r, j); });
+  block(half, half, hO, [&](int r, int j) { return inv(2 * r + 1, j); });
+  block(H, H, hE, [&](int j, int k) { return cosl_frac((long long)j * (2 * k)); });
+  block(half, H, hE, [&](int j, int k) { return cosl_frac((long long)j * (2 * k + 1)); });
+  return t;
+}
+
 std::vector<double> make_rco(int N) {
   const RcoLayout RL(N);
   const int Mh = N / 2 + 1;
@@ -490,50 +527,51 @@ pcf_status launch_tc_analysis(pcf_ctx* c) {
     else launch_cheb_analysis_tc(c->cta_tca, c->sm_tc, c->cs, li_of(c, c->pre_tca));
   });
 }
-// split mode kernels of the FP64 descent step
-GroupLaunch gl_of(pcf_ctx* c, const int* pre, int red = 0) {
-  return GroupLaunch{c->dinst, pre, c->d_groups, c->ngroups, red};
+// per-mode kernels over groups of instances; red: the modes m >= 0 only
+GroupLaunch gl_of(pcf_ctx* c, bool red = false) {
+  return GroupLaunch{c->dinst, red ? c->pre_ys_r : c->pre_ys, c->d_groups, c->ngroups};
 }
-// red: the reduced launch of a symmetric descent step (modes m >= 0 only)
-pcf_status launch_split_analysis(pcf_ctx* c, int op, bool red = false) {
+// Chebyshev coefficients of the products (both forms)
+pcf_status launch_analysis(pcf_ctx* c, bool red = false) {
+  if (c->mixed) return launch_tc_analysis(c);
   return timed(c, 7, [&] {
-    launch_yanalysis(red ? c->cta_ya_r : c->cta_ya, c->thr_ya, c->sm_ya, c->cs,
-                     gl_of(c, red ? c->pre_ya_r : c->pre_ya, red), op, c->plane_kind == 2, c->smt);
+    const int ctas = red ? c->cta_ya_r : c->cta_ya;
+    launch_yana_fx(ctas, c->thr_ya, c->sm_ya, c->cs, li_of(c, red ? c->pre_ya_r : c->pre_ya, ctas), c->np, red ? 1 : 0, c->fine_y);
   });
 }
-GroupLaunch gl_solve(pcf_ctx* c, bool red = false) {
-  return GroupLaunch{c->dinst, red ? c->pre_ys_r : c->pre_ys, c->d_groups_s, c->ngroups_s, red ? 1 : 0};
-}
-pcf_status launch_split_solve(pcf_ctx* c, int op, bool red = false) {
-  if (c->sweep)
-    return timed(c, op == MODE_PHI ? 3 : 6, [&] {
+// Stokes solve and what follows it (op); sig selects the step size's operators
+pcf_status launch_solve(pcf_ctx* c, int op, int sig, bool red = false) {
+  const int cls = op == MODE_PHI ? 3 : 6;
+  if (!c->split) return launch_mode(c, op, sig);
+  if (c->sweep && (op == MODE_PHI || op == MODE_PSI_UPDATE))
+    return timed(c, cls, [&] {
       launch_sweep(red ? c->cta_sw_r : c->cta_sw, c->thr_sw, c->sm_sw, c->cs,
                    LaunchInfo{c->dinst, red ? c->pre_sw_r : c->pre_sw, c->B}, op, red ? 1 : 0);
     });
-  return timed(c, op == MODE_PHI ? 3 : 6, [&] {
-    launch_ysolve(red ? c->grid_ys_r : c->grid_ys, red ? c->cta_ys_r : c->cta_ys, c->buf_ys, c->rows_ys, c->sm_ys,
-                  c->cs, gl_solve(c, red), op);
+  return timed(c, cls, [&] {
+    launch_ysolve_fx(red ? c->cta_ys_r : c->cta_ys, c->thr_ys, c->sm_ys, c->cs, gl_of(c, red), op, sig, c->fine_s);
   });
 }
-pcf_status launch_fused_step(pcf_ctx* c, int op) {
-  return timed(c, op == MODE_PHI ? 3 : 6,
-               [&] { launch_ystep(c->cta_yf, c->sm_yf, c->cs, gl_of(c, c->pre_yf), op); });
+// synth: the half-step ends with the y-synthesis of its result
+pcf_status launch_fused_step(pcf_ctx* c, int op, int synth) {
+  return timed(c, op == MODE_PHI ? 3 : 6, [&] {
+    launch_ystep_fx(c->cta_ys, c->thr_yf, c->sm_yf, c->cs, gl_of(c), op, synth, c->fine_s);
+  });
 }
 pcf_status launch_split_jnorm(pcf_ctx* c, int step_index) {
   return timed(c, 9, [&] { launch_jnorm(c->B, c->cs, c->dinst, step_index); });
 }
-pcf_status launch_split_synth(pcf_ctx* c, int slot, int in_step, bool red = false) {
-  return timed(c, in_step ? 8 : 0, [&] {
-    launch_ysynth_split(red ? c->cta_yy_r : c->cta_yy, c->thr_yy, c->sm_yy, c->cs,
-                        gl_of(c, red ? c->pre_yy_r : c->pre_yy, red), slot, in_step, c->plane_kind == 2, c->smt_y);
-  });
-}
-
-// y-synthesis of the state (slot 0) or of r1 (slot 1) in either form
-pcf_status launch_ysynth(pcf_ctx* c, int slot) {
+// y-synthesis of the state (slot 0) or of r1 (slot 1) in either form; in_step: masked instances
+// are left out; nf: five fields, or three (the values, without y-derivatives)
+pcf_status launch_ysynth(pcf_ctx* c, int slot, int in_step = 0, bool red = false, int nf = kFieldsY) {
   if (c->mixed) return launch_tc_synth(c, slot);
-  if (c->split) return launch_split_synth(c, slot, 0);
-  return launch_mode(c, MODE_SYNTH_ONLY, slot);
+  if (!c->split) return launch_mode(c, MODE_SYNTH_ONLY, slot);
+  return timed(c, in_step ? 8 : 0, [&] {
+    const int* pre = nf == 3 ? c->pre_ya : red ? c->pre_yy_r : c->pre_yy;
+    const int ctas = nf == 3 ? c->cta_ya : red ? c->cta_yy_r : c->cta_yy;
+    launch_ysynth_fx(ctas, c->thr_yy, c->sm_yy, c->cs, li_of(c, pre, ctas), slot, nf, in_step, c->np, red ? 1 : 0,
+                     c->fine_y);
+  });
 }
 
 // projection onto the symmetric subspace: each instance's own mask (mask_override < 0) or mask
@@ -575,60 +613,47 @@ void set_pointers(pcf_ctx* c, const double* u, const double* r, double* f) {
   }
 }
 
-pcf_status step_body(pcf_ctx* c, int s) {
-  if (c->mixed) {
-    if (s > 0) PCF_TRY(launch_tc_synth(c, 0));
-    PCF_TRY(launch_synth(c, 0, kFieldsSynth));
-    PCF_TRY(launch_prodM(c));
-    PCF_TRY(launch_tc_analysis(c));
-    PCF_TRY(launch_mode(c, MODE_PHI, 0));
-    PCF_TRY(launch_tc_synth(c, 1));
-    PCF_TRY(launch_synth(c, 1, kFieldsSynth));
-    PCF_TRY(launch_prodN(c, s));  // with J, its history entry and the convergence mask
-    PCF_TRY(launch_tc_analysis(c));
-    PCF_TRY(launch_mode(c, MODE_PSI_UPDATE, 1));
-    if (c->any_sym) PCF_TRY(launch_sym(c, -1));  // the next step's synthesis reads the projected state
-    return PCF_OK;
-  }
+// Step s of a call; last: the call's last step (its update needs no synthesis).
+pcf_status step_body(pcf_ctx* c, int s, bool last) {
   if (c->split && c->fused) {
     PCF_TRY(launch_synth(c, 0, kFieldsSynth));
     PCF_TRY(launch_prodM(c));
-    PCF_TRY(launch_fused_step(c, MODE_PHI));
+    PCF_TRY(launch_fused_step(c, MODE_PHI, 1));
     PCF_TRY(launch_synth(c, 1, kFieldsSynth));
-    PCF_TRY(launch_prodN(c));
-    PCF_TRY(launch_split_jnorm(c, s));
-    PCF_TRY(launch_fused_step(c, MODE_PSI_UPDATE));
+    PCF_TRY(launch_prodN(c, c->jn ? -1 : s));
+    if (c->jn) PCF_TRY(launch_split_jnorm(c, s));
+    PCF_TRY(launch_fused_step(c, MODE_PSI_UPDATE, !last && !c->any_sym));
     if (c->any_sym) {
       PCF_TRY(launch_sym(c, -1));
       PCF_TRY(launch_ysynth(c, 0));
     }
     return PCF_OK;
   }
-  if (c->split) {
+  if (c->split || c->mixed) {
     // in the symmetric subspace of s2 the per-mode work covers the modes m >= 0; the
     // synthesis mirrors their y-values to -m, and the projection after the update rebuilds
     // the state's modes -m
-    const bool red = c->reduced;
+    const bool red = c->split && c->reduced;
     // the y-values of the state the previous step updated (the call's first step reads the
     // synthesis done at the call's start)
-    if (s > 0) PCF_TRY(launch_split_synth(c, 0, 1, red));
+    if (s > 0) PCF_TRY(launch_ysynth(c, 0, 1, red));
     PCF_TRY(launch_synth(c, 0, kFieldsSynth));
     PCF_TRY(launch_prodM(c));
-    PCF_TRY(launch_split_analysis(c, MODE_PHI, red));
-    PCF_TRY(launch_split_solve(c, MODE_PHI, red));
-    PCF_TRY(launch_split_synth(c, 1, 1, red));
+    PCF_TRY(launch_analysis(c, red));
+    PCF_TRY(launch_solve(c, MODE_PHI, 0, red));
+    PCF_TRY(launch_ysynth(c, 1, 1, red));
     PCF_TRY(launch_synth(c, 1, kFieldsSynth));
     PCF_TRY(launch_prodN(c, s));  // with J, its history entry and the convergence mask
-    PCF_TRY(launch_split_analysis(c, MODE_PSI_UPDATE, red));
-    PCF_TRY(launch_split_solve(c, MODE_PSI_UPDATE, red));
-    if (c->any_sym) PCF_TRY(launch_sym(c, -1, red));
+    PCF_TRY(launch_analysis(c, red));
+    PCF_TRY(launch_solve(c, MODE_PSI_UPDATE, 1, red));
+    if (c->any_sym) PCF_TRY(launch_sym(c, -1, red));  // the next step's synthesis reads the projected state
     return PCF_OK;
   }
   PCF_TRY(launch_synth(c, 0, kFieldsSynth));
   PCF_TRY(launch_prodM(c));
   PCF_TRY(launch_mode(c, MODE_PHI, 0));
   PCF_TRY(launch_synth(c, 1, kFieldsSynth));
-  PCF_TRY(launch_prodN(c, s));  // with J, its history entry and the convergence mask
+  PCF_TRY(launch_prodN(c, s));
   PCF_TRY(launch_mode(c, MODE_PSI_UPDATE, 1));
   if (c->any_sym) {
     PCF_TRY(launch_sym(c, -1));
@@ -648,14 +673,9 @@ pcf_status dns_body(pcf_ctx* c) {
     launch_dns_capture(c->dns_ctas, c->B, c->cs, c->dinst, c->d_dns);
   }));
   PCF_TRY(launch_prodM(c));
-  if (c->mixed) {
-    PCF_TRY(launch_tc_analysis(c));
-    PCF_TRY(launch_mode(c, MODE_PHI, 0));
-  } else if (c->split && c->fused) {
-    PCF_TRY(launch_fused_step(c, MODE_PHI));
-  } else if (c->split) {
-    PCF_TRY(launch_split_analysis(c, MODE_PHI));
-    PCF_TRY(launch_split_solve(c, MODE_PHI));
+  if (c->split || c->mixed) {
+    PCF_TRY(launch_analysis(c));
+    PCF_TRY(launch_solve(c, MODE_PHI, 0));
   } else {
     PCF_TRY(launch_mode(c, MODE_PHI, 0));
   }
@@ -711,8 +731,11 @@ static bool params_ok(const pcf_params* prm) {
 
 // Device tables of one grid (shared by every instance on that grid).
 struct GridTables {
-  double *cheb, *rco, *ccw, *kx, *kz, *y, *ub, *tab0, *tab1, *dense0, *dense1;
-  float2* cheb_ff = nullptr;
+  double *cheb, *rco, *ccw, *kx, *kz, *y, *ub, *tab0, *tab1, *ik2nu = nullptr;
+  double* dense[2] = {nullptr, nullptr};
+  int4 *fxcheb = nullptr, *fxD[2] = {nullptr, nullptr};
+  int* fxDe[2] = {nullptr, nullptr};
+  int fxcheb_e = 0;
   fxtw *twfx_x = nullptr, *twfx_z = nullptr;
   float2 *twxf = nullptr, *twzf = nullptr;
   uint16_t* tcA = nullptr;
@@ -769,16 +792,6 @@ static pcf_status build_tables(pcf_ctx* c, const pcf_params* prm, GridTables* g)
     if (upload(tab1, &g->tab1)) return PCF_ECUDA;
     c->allocs.push_back(g->tab1);
   }
-  if (prm->precision == PCF_FLOAT_FLOAT) {
-    // nearest float-float pairs: hi = fl(x), lo = fl(x - hi)
-    std::vector<float2> cf(cheb.size());
-    for (size_t i = 0; i < cheb.size(); ++i) {
-      const float hi = static_cast<float>(cheb[i]);
-      cf[i] = make_float2(hi, static_cast<float>(cheb[i] - (double)hi));
-    }
-    if (upload(cf, &g->cheb_ff)) return PCF_ECUDA;
-    c->allocs.push_back(g->cheb_ff);
-  }
   if (prm->precision == PCF_MIXED) {
     const std::vector<uint16_t> tcm = make_tc_matrices(N);
     if (upload(to_float2(make_twiddles(nx)), &g->twxf) || upload(to_float2(make_twiddles(nz)), &g->twzf) || upload(tcm, &g->tcA))
@@ -792,17 +805,40 @@ static pcf_status build_tables(pcf_ctx* c, const pcf_params* prm, GridTables* g)
       c->allocs.push_back(g->tcA5);
     }
   }
-  g->dense0 = g->dense1 = nullptr;
-  const bool dense = N <= kDenseMaxN && prm->solve_kind != 1;
-  if (dense) {
-    if (upload(make_dense_tables(N, kx, kz, g->sig[0], rco, tab0), &g->dense0)) return PCF_ECUDA;
-    c->allocs.push_back(g->dense0);
-    if (prm->dtau_hat == prm->dt) {
-      g->dense1 = g->dense0;
-    } else {
-      if (upload(make_dense_tables(N, kx, kz, g->sig[1], rco, tab1), &g->dense1)) return PCF_ECUDA;
-      c->allocs.push_back(g->dense1);
+  if (prm->solve_kind == 1) return PCF_OK;
+  // dense operators: in FP64 for the mixed form, as fixed-point words for the FP64 forms
+  const bool fx = prm->precision != PCF_MIXED;
+  if (fx) {
+    std::vector<double> ik(Mx * Mz, 0.0);
+    for (int m = 1; m < Mx * Mz; ++m) {
+      const double x = kx[m / Mz], z = kz[m % Mz];
+      ik[m] = 1.0 / nu / (x * x + z * z);
     }
+    if (upload(ik, &g->ik2nu) || upload(make_fxcheb(N, &g->fxcheb_e), &g->fxcheb)) return PCF_ECUDA;
+    c->allocs.push_back(g->ik2nu);
+    c->allocs.push_back(g->fxcheb);
+  }
+  for (int q = 0; q < 2; ++q) {
+    if (q == 1 && prm->dtau_hat == prm->dt) {
+      g->dense[1] = g->dense[0];
+      g->fxD[1] = g->fxD[0];
+      g->fxDe[1] = g->fxDe[0];
+      break;
+    }
+    double* d = nullptr;
+    if (upload(make_dense_tables(N, kx, kz, g->sig[q], rco, q ? tab1 : tab0), &d)) return PCF_ECUDA;
+    if (!fx) {
+      g->dense[q] = d;
+      c->allocs.push_back(d);
+      continue;
+    }
+    const bool ok = !ctx_alloc(c, &g->fxD[q], dense_limbs_len(N, Mx * Mz)) &&
+                    !ctx_alloc(c, &g->fxDe[q], dense_exps_len(N, Mx * Mz));
+    if (ok) launch_dense_limbs(d, N, Mx * Mz, g->fxD[q], g->fxDe[q]);
+    const cudaError_t e = cudaDeviceSynchronize();
+    cudaFree(d);
+    if (!ok) return PCF_ENOMEM;
+    PCF_CUDA(e);
   }
   return PCF_OK;
 }
@@ -852,8 +888,6 @@ static pcf_status set_mode_tiles(pcf_ctx* c, int want) {
   return PCF_OK;
 }
 
-// Instance groups of the split mode kernels: runs of consecutive instances on the same grid,
-// at most G per group, and the derived launch geometry.
 // Consecutive instances that share grid and tables, at most G per group.
 static std::vector<int2> make_groups(const pcf_ctx* c, int G) {
   std::vector<int2> groups;
@@ -862,7 +896,7 @@ static std::vector<int2> make_groups(const pcf_ctx* c, int G) {
     bool fresh = groups.empty() || groups.back().y == G;
     if (!fresh) {
       const Inst& P = c->hinst[b - 1];
-      fresh = I.dense[0] != P.dense[0] || I.dense[1] != P.dense[1] || I.cheb != P.cheb || I.nmodes != P.nmodes;
+      fresh = I.fxD[0] != P.fxD[0] || I.fxD[1] != P.fxD[1] || I.kx != P.kx || I.nmodes != P.nmodes;
     }
     if (fresh) groups.push_back(make_int2(b, 1)); else groups.back().y += 1;
   }
@@ -890,261 +924,69 @@ static pcf_status set_sweep(pcf_ctx* c, int threads) {
   return PCF_OK;
 }
 
-// Instance groups of the persistent Stokes solve (at most G instances each): items, prefix,
-// shared-memory layout and grid.
-static pcf_status set_solve_groups(pcf_ctx* c, int G) {
+// Geometry of the fixed-point per-mode kernels: instance groups of the dense solve (at most G
+// instances), mode tiles of the analysis and the synthesis.
+static pcf_status set_modes(pcf_ctx* c, int G) {
   int Nmax = 0;
-  for (const Inst& I : c->hinst) Nmax = std::max(Nmax, I.N);
-  G = std::max(1, std::min(G, split_max_group(Nmax)));
-  while (G > 1 && smem_ysolve(Nmax, G) > 227 * 1024) --G;
+  long long modes = 0;
+  for (const Inst& I : c->hinst) {
+    Nmax = std::max(Nmax, I.N);
+    modes += I.nmodes;
+  }
+  G = std::max(1, std::min(G, kMaxGroup));
+  while (G > 1 && smem_ystep_fx(Nmax, G) > 227 * 1024) --G;
   const std::vector<int2> groups = make_groups(c, G);
   const int ng = (int)groups.size();
   int gmax = 1;
-  for (const int2& gq : groups) gmax = std::max(gmax, gq.y);
+  for (const int2& q : groups) gmax = std::max(gmax, q.y);
   std::vector<int> ps(ng + 1, 0), psr(ng + 1, 0);
   for (int q = 0; q < ng; ++q) {
     const Inst& I = c->hinst[groups[q].x];
-    ps[q + 1] = ps[q] + split_ctas_per_group(1, I.nmodes, 1);
-    psr[q + 1] = psr[q] + split_ctas_per_group(1, (I.Kx + 1) * I.Mz, 1);  // modes m >= 0
+    ps[q + 1] = ps[q] + I.nmodes;
+    psr[q + 1] = psr[q] + (I.Kx + 1) * I.Mz;  // modes m >= 0
   }
-  // the persistent solve lays out every item in buffers sized for the largest grid and group
-  const size_t ss = smem_ysolve(Nmax, gmax);
-  if (ss > 227 * 1024) return PCF_ENOTSUP;
-  if (!c->d_groups_s) {
-    if (ctx_alloc(c, &c->d_groups_s, (size_t)c->B) || ctx_alloc(c, &c->pre_ys, (size_t)c->B + 1) ||
+  if (!c->d_groups) {
+    if (ctx_alloc(c, &c->d_groups, (size_t)c->B) || ctx_alloc(c, &c->pre_ys, (size_t)c->B + 1) ||
         ctx_alloc(c, &c->pre_ys_r, (size_t)c->B + 1))
       return PCF_ENOMEM;
   }
-  PCF_CUDA(cudaMemcpy(c->d_groups_s, groups.data(), sizeof(int2) * ng, cudaMemcpyHostToDevice));
+  PCF_CUDA(cudaMemcpy(c->d_groups, groups.data(), sizeof(int2) * ng, cudaMemcpyHostToDevice));
   PCF_CUDA(cudaMemcpy(c->pre_ys, ps.data(), sizeof(int) * (ng + 1), cudaMemcpyHostToDevice));
   PCF_CUDA(cudaMemcpy(c->pre_ys_r, psr.data(), sizeof(int) * (ng + 1), cudaMemcpyHostToDevice));
-  c->cta_ys_r = psr[ng];
-  c->sgrp_s = G;
-  c->ngroups_s = ng;
-  c->cta_ys = ps[ng];
-  c->sm_ys = ss;
-  c->buf_ys = (int)ysolve_buffer(Nmax, gmax);
-  c->rows_ys = Nmax / 2 + 1;
-  PCF_CUDA(set_split_smem(c->sm_ya, ss, c->sm_yy));
-  int dev = 0, nsm = 0;
-  PCF_CUDA(cudaGetDevice(&dev));
-  PCF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const int per_sm = std::max(1, ysolve_ctas_per_sm(ss));
-  c->grid_ys = std::min(c->cta_ys, nsm * per_sm);
-  c->grid_ys_r = std::min(c->cta_ys_r, nsm * per_sm);
-  return PCF_OK;
-}
-
-// Instance groups of the split analysis and synthesis (at most G instances each) with mt_a and
-// mt_y consecutive modes per CTA (mt_y < 1: the same as mt_a); also resets the solve's groups.
-static pcf_status set_split_groups(pcf_ctx* c, int G, int mt = 1, int mt_y = 0) {
-  int Nmax = 0;
-  for (const Inst& I : c->hinst) Nmax = std::max(Nmax, I.N);
-  G = std::max(1, std::min(G, split_max_group(Nmax)));
-  while (G > 1 && smem_ysolve(Nmax, G) > 227 * 1024) --G;
-  std::vector<int2> groups = make_groups(c, G);
-  const int ng = (int)groups.size();
-  int gmax = 1;
-  for (const int2& gq : groups) gmax = std::max(gmax, gq.y);
-  mt = std::max(1, mt);
-  while (mt > 1 && split_col_pad(gmax) * mt > 32) mt >>= 1;
-  mt_y = mt_y < 1 ? mt : mt_y;
-  while (mt_y > 1 && split_col_pad(gmax) * mt_y > 32) mt_y >>= 1;
-  std::vector<int> pa(ng + 1, 0), py(ng + 1, 0), pf(ng + 1, 0), par(ng + 1, 0), pyr(ng + 1, 0);
-  size_t sa = 0, sy = 0;
-  int thr_a = 64, thr_y = 64;  // threads per CTA: one pass over the row tasks of any group
-  for (int q = 0; q < ng; ++q) {
-    const Inst& I = c->hinst[groups[q].x];
-    const int nrun = (I.Kx + 1) * I.Mz;  // the reduced launches: modes m >= 0
-    pf[q + 1] = pf[q] + I.nmodes;
-    pa[q + 1] = pa[q] + split_ctas_per_group(0, I.nmodes, mt);
-    py[q + 1] = py[q] + split_ctas_per_group(2, I.nmodes, mt_y);
-    par[q + 1] = par[q] + split_ctas_per_group(0, nrun, mt);
-    pyr[q + 1] = pyr[q] + split_ctas_per_group(2, nrun, mt_y);
-    sa = std::max(sa, smem_yanalysis(I.N, groups[q].y, mt));
-    sy = std::max(sy, smem_ysynth(I.N, groups[q].y, mt_y));
-    const bool fp64 = c->plane_kind != 2;
-    thr_a = std::max(thr_a, split_yanalysis_threads(I.N, groups[q].y, mt, fp64));
-    thr_y = std::max(thr_y, split_ysynth_threads(I.N, groups[q].y, mt_y, fp64));
-  }
-  if (std::max(sa, sy) > 227 * 1024) return PCF_ENOTSUP;
-  if (!c->d_groups) {
-    if (ctx_alloc(c, &c->d_groups, (size_t)c->B) || ctx_alloc(c, &c->pre_ya, (size_t)c->B + 1) ||
-        ctx_alloc(c, &c->pre_yy, (size_t)c->B + 1) || ctx_alloc(c, &c->pre_yf, (size_t)c->B + 1) ||
-        ctx_alloc(c, &c->pre_ya_r, (size_t)c->B + 1) || ctx_alloc(c, &c->pre_yy_r, (size_t)c->B + 1))
-      return PCF_ENOMEM;
-  }
-  PCF_CUDA(cudaMemcpy(c->pre_ya_r, par.data(), sizeof(int) * (ng + 1), cudaMemcpyHostToDevice));
-  PCF_CUDA(cudaMemcpy(c->pre_yy_r, pyr.data(), sizeof(int) * (ng + 1), cudaMemcpyHostToDevice));
-  c->cta_ya_r = par[ng];
-  c->cta_yy_r = pyr[ng];
-  PCF_CUDA(cudaMemcpy(c->pre_yf, pf.data(), sizeof(int) * (ng + 1), cudaMemcpyHostToDevice));
-  c->cta_yf = pf[ng];
-  c->sm_yf = smem_ystep(Nmax, gmax);
-  PCF_CUDA(cudaMemcpy(c->d_groups, groups.data(), sizeof(int2) * ng, cudaMemcpyHostToDevice));
-  PCF_CUDA(cudaMemcpy(c->pre_ya, pa.data(), sizeof(int) * (ng + 1), cudaMemcpyHostToDevice));
-  PCF_CUDA(cudaMemcpy(c->pre_yy, py.data(), sizeof(int) * (ng + 1), cudaMemcpyHostToDevice));
   c->sgrp = G;
-  c->smt = mt;
-  c->smt_y = mt_y;
   c->ngroups = ng;
-  c->cta_ya = pa[ng];
-  c->cta_yy = py[ng];
-  c->sm_ya = sa;
-  c->sm_yy = sy;
-  c->thr_ya = thr_a;
-  c->thr_yy = thr_y;
-  if (c->sm_yf <= 227 * 1024) PCF_CUDA(set_ystep_smem(c->sm_yf));
-  // the solve follows the same group size unless tuned on its own (autotune_split)
-  return set_solve_groups(c, G);
-}
-
-// Autotuner of the split mode kernels: time the per-mode work of a whole step (analysis,
-// solve and synthesis of both half-steps, or the fused kernel twice and the norm kernel) on
-// the batch for each candidate group size, mode tile and organisation, and keep the fastest.
-static pcf_status autotune_split(pcf_ctx* c) {
-  const int cand[] = {1, 2, 4, 6, 8};
-  cudaEvent_t a, b;
-  PCF_CUDA(cudaEventCreate(&a));
-  PCF_CUDA(cudaEventCreate(&b));
-  int best = 2, best_mt = 1;
-  bool best_fused = false;
-  float best_ms = 1e30f;
-  int last = 0;
-  for (int G0 : cand) {
-    const int G = std::min(G0, c->B);
-    if (G == last) continue;
-    last = G;
-    for (int mt = 1; mt <= 16 && split_col_pad(G) * mt <= 32; mt *= 2) {
-      if (set_split_groups(c, G, mt) != PCF_OK || c->sgrp != G || c->smt != mt) continue;
-      for (int fuse = 0; fuse < 2; ++fuse) {
-        if (fuse && (mt > 1 || c->sm_yf > 227 * 1024)) continue;  // the fused kernel has no mode tile
-        if (((c->prm.solve_kind == 3 || c->prm.solve_kind == 5) && fuse) || (c->prm.solve_kind == 4 && !fuse))
-          continue;
-        // the per-mode work of a whole step in each organisation (both half-steps; the fused
-        // path also launches the separate norm kernel)
-        auto seq = [&] {
-          if (fuse) {
-            launch_ystep(c->cta_yf, c->sm_yf, c->cs, gl_of(c, c->pre_yf), MODE_PHI);
-            launch_jnorm(c->B, c->cs, c->dinst, 0);
-            launch_ystep(c->cta_yf, c->sm_yf, c->cs, gl_of(c, c->pre_yf), MODE_PSI_UPDATE);
-            return;
-          }
-          for (int op : {(int)MODE_PHI, (int)MODE_PSI_UPDATE}) {
-            launch_yanalysis(c->cta_ya, c->thr_ya, c->sm_ya, c->cs, gl_of(c, c->pre_ya), op, c->plane_kind == 2,
-                             c->smt);
-            launch_ysolve(c->grid_ys, c->cta_ys, c->buf_ys, c->rows_ys, c->sm_ys, c->cs, gl_solve(c), op);
-            launch_ysynth_split(c->cta_yy, c->thr_yy, c->sm_yy, c->cs, gl_of(c, c->pre_yy), op == MODE_PHI ? 1 : 0, 1,
-                                c->plane_kind == 2, c->smt_y);
-          }
-        };
-        seq();
-        PCF_CUDA(cudaEventRecord(a, c->cs));
-        for (int r = 0; r < 3; ++r) seq();
-        PCF_CUDA(cudaEventRecord(b, c->cs));
-        PCF_CUDA(cudaEventSynchronize(b));
-        float ms = 0.f;
-        PCF_CUDA(cudaEventElapsedTime(&ms, a, b));
-        if (ms < best_ms) {
-          best_ms = ms;
-          best = G;
-          best_mt = mt;
-          best_fused = fuse != 0;
-        }
-      }
-    }
+  c->cta_ys = ps[ng];
+  c->cta_ys_r = psr[ng];
+  c->sm_ys = smem_ysolve_fx(Nmax, gmax);
+  c->sm_yf = smem_ystep_fx(Nmax, gmax);
+  // one row and one part per thread while the launch would otherwise leave SMs with less than
+  // eight warps
+  const int hp = (Nmax / 2 + 2) / 2;
+  c->fine_s = (long long)c->cta_ys * 6 * hp * gmax < 152LL * 256;
+  c->thr_ys = ysolve_fx_threads(Nmax, gmax, c->fine_s);
+  c->thr_yf = std::max(c->thr_ys, 256);
+  // tiles of 16 modes while they give every SM four CTAs of the analysis
+  c->np = 3 * (modes / 16) >= 4 * 152 ? 16 : 8;
+  std::vector<int> pa(c->B), py(c->B), par(c->B), pyr(c->B);
+  for (int b = 0; b < c->B; ++b) {
+    const Inst& I = c->hinst[b];
+    const int t = yfx_tiles(I.nmodes, c->np), r = yfx_tiles((I.Kx + 1) * I.Mz, c->np);
+    pa[b] = 3 * t;
+    py[b] = kFieldsY * t;
+    par[b] = 3 * r;
+    pyr[b] = kFieldsY * r;
   }
-  c->tuned_split_ms = best_ms / 3.0;
-  pcf_status st = set_split_groups(c, best, best_mt);
-  c->fused = st == PCF_OK && best_fused;
-  if (st == PCF_OK && !c->fused) {
-    // analysis and synthesis mode tiles, each timed alone
-    auto time5 = [&](auto&& launch, float* ms) -> pcf_status {
-      launch();
-      PCF_CUDA(cudaEventRecord(a, c->cs));
-      for (int r = 0; r < 5; ++r) launch();
-      PCF_CUDA(cudaEventRecord(b, c->cs));
-      PCF_CUDA(cudaEventSynchronize(b));
-      PCF_CUDA(cudaEventElapsedTime(ms, a, b));
-      return PCF_OK;
-    };
-    int mt_a = best_mt, mt_y = best_mt;
-    float ba = 1e30f, by = 1e30f;
-    for (int mt = 1; mt <= 16 && split_col_pad(best) * mt <= 32; mt *= 2) {
-      if (set_split_groups(c, best, mt, mt) != PCF_OK || c->smt != mt || c->smt_y != mt) continue;
-      float ms = 0.f;
-      PCF_TRY(time5([&] {
-        launch_yanalysis(c->cta_ya, c->thr_ya, c->sm_ya, c->cs, gl_of(c, c->pre_ya), MODE_PHI, c->plane_kind == 2,
-                         c->smt);
-      }, &ms));
-      if (ms < ba) { ba = ms; mt_a = mt; }
-      PCF_TRY(time5([&] {
-        launch_ysynth_split(c->cta_yy, c->thr_yy, c->sm_yy, c->cs, gl_of(c, c->pre_yy), 1, 1, c->plane_kind == 2,
-                            c->smt_y);
-      }, &ms));
-      if (ms < by) { by = ms; mt_y = mt; }
-    }
-    st = set_split_groups(c, best, mt_a, mt_y);
-  }
-  float solve_ms = 1e30f;  // five dense solves in the chosen groups
-  if (st == PCF_OK && !c->fused) {
-    // the solve alone over its own group sizes
-    int best_s = c->sgrp_s;
-    float best_s_ms = 1e30f;
-    last = 0;
-    for (int G0 : {1, 2, 4, 8}) {
-      const int G = std::min(G0, c->B);
-      if (G == last) continue;
-      last = G;
-      if (set_solve_groups(c, G) != PCF_OK || c->sgrp_s != G) continue;
-      auto seq = [&] {
-        launch_ysolve(c->grid_ys, c->cta_ys, c->buf_ys, c->rows_ys, c->sm_ys, c->cs, gl_solve(c), MODE_PHI);
-      };
-      seq();
-      PCF_CUDA(cudaEventRecord(a, c->cs));
-      for (int r = 0; r < 5; ++r) seq();
-      PCF_CUDA(cudaEventRecord(b, c->cs));
-      PCF_CUDA(cudaEventSynchronize(b));
-      float ms = 0.f;
-      PCF_CUDA(cudaEventElapsedTime(&ms, a, b));
-      if (ms < best_s_ms) {
-        best_s_ms = ms;
-        best_s = G;
-      }
-    }
-    st = set_solve_groups(c, best_s);
-    solve_ms = best_s_ms;
-  }
-  c->sweep = false;
-  if (st == PCF_OK && !c->fused && c->prm.solve_kind != 3) {
-    // the banded sweeps, one thread per chain, against the dense solve (solve_kind 5: always)
-    int best_t = 0;
-    float best_t_ms = c->prm.solve_kind == 5 ? 1e30f : solve_ms;
-    for (int thr : {32, 64}) {
-      if (set_sweep(c, thr) != PCF_OK) continue;
-      auto seq = [&] {
-        launch_sweep(c->cta_sw, c->thr_sw, c->sm_sw, c->cs, LaunchInfo{c->dinst, c->pre_sw, c->B}, MODE_PHI, 0);
-      };
-      seq();
-      PCF_CUDA(cudaEventRecord(a, c->cs));
-      for (int r = 0; r < 5; ++r) seq();
-      PCF_CUDA(cudaEventRecord(b, c->cs));
-      PCF_CUDA(cudaEventSynchronize(b));
-      float ms = 0.f;
-      PCF_CUDA(cudaEventElapsedTime(&ms, a, b));
-      if (ms < best_t_ms) {
-        best_t_ms = ms;
-        best_t = thr;
-      }
-    }
-    if (best_t > 0) {
-      st = set_sweep(c, best_t);
-      c->sweep = st == PCF_OK;
-    }
-  }
-  cudaEventDestroy(a);
-  cudaEventDestroy(b);
-  return st;
+  PCF_TRY(upload_prefix(c, pa, &c->pre_ya, &c->cta_ya));
+  PCF_TRY(upload_prefix(c, py, &c->pre_yy, &c->cta_yy));
+  PCF_TRY(upload_prefix(c, par, &c->pre_ya_r, &c->cta_ya_r));
+  PCF_TRY(upload_prefix(c, pyr, &c->pre_yy_r, &c->cta_yy_r));
+  c->sm_ya = smem_yana_fx(Nmax, c->np);
+  c->sm_yy = smem_ysynth_fx(Nmax, c->np);
+  c->fine_y = (long long)c->cta_ya * c->np * 2 * hp < 152LL * 256;
+  c->thr_ya = yana_fx_threads(Nmax, c->np, c->fine_y);
+  c->thr_yy = ysynth_fx_threads(Nmax, c->np, c->fine_y);
+  PCF_CUDA(set_modes_fx_smem(c->sm_ya, c->sm_yy, c->sm_ys, c->sm_yf));
+  return PCF_OK;
 }
 
 // Time the Stokes-step mode kernel on the batch for each candidate tile; keep the fastest.
@@ -1171,7 +1013,7 @@ static pcf_status time_mode_tiles(pcf_ctx* c, cudaEvent_t a, cudaEvent_t b, int*
   return PCF_OK;
 }
 
-// Autotuner (laminar input): the mode tile and, for the mixed-precision form, the Stokes
+// Autotuner of the single per-mode kernel (laminar input): its mode tile and, for the mixed-precision form, the Stokes
 // solve variant.  The dense per-mode operators keep the FP64 pipe full; the banded sweeps
 // need ~20x fewer FP64 operations but run as sequential chains and no operator tables stream
 // from memory; which one is faster depends on the grid and the batch, so both are timed.
@@ -1209,15 +1051,33 @@ static pcf_status autotune_tiles(pcf_ctx* c) {
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
-  c->tuned_ms = best_ms / 3.0;
   pcf_status st = set_mode_tiles(c, best);
-  if (st == PCF_OK && c->split) {
-    st = push_descriptors(c);
-    if (st == PCF_OK) st = autotune_split(c);
-  }
   if (cudaStreamSynchronize(c->cs) != cudaSuccess && st == PCF_OK) st = PCF_ECUDA;
   cudaFree(z);
   return st;
+}
+
+// Instances per group of the dense solve: a group shares every operator load, but a CTA is one
+// (group, mode), so the group is as large as leaves every SM two CTAs.
+static int solve_group(const pcf_ctx* c) {
+  int G = kMaxGroup;
+  while (G > 1) {
+    long long ctas = 0;
+    for (const int2& q : make_groups(c, G)) ctas += c->hinst[q.x].nmodes;
+    if (ctas >= 2 * 152) break;
+    G /= 2;
+  }
+  return G;
+}
+
+// The fused half-step (two launches fewer per half-step) wins where the launches dominate.
+static bool fused_step_pays(const pcf_ctx* c) { return c->cta_ys <= 228; }
+
+// Grids whose Chebyshev tables and one mode's scratch exceed a CTA's shared memory in the FP64
+// per-mode kernel (ny above 125) are refused in the FP64 forms.
+static bool fp64_grid_refused(const Inst& I) {
+  const size_t H = I.N / 2 + 1;
+  return 8 * (6 * H * H + 10 * H + 60 * H + 1) > 227 * 1024;
 }
 
 static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, pcf_ctx** out) {
@@ -1299,7 +1159,7 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
       }
   }
   c->total_state = c->state_off[B];
-  double2 *yv = nullptr, *xz = nullptr;
+  double2 *yv = nullptr, *xz = nullptr, *xc = nullptr;
   double *ph = nullptr, *np = nullptr, *fr = nullptr;
   float2 *yvf = nullptr, *xzf = nullptr, *xzc = nullptr;
   float* phf = nullptr;
@@ -1313,14 +1173,14 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
     if (ctx_alloc(c, &yvf, n_yv) || ctx_alloc(c, &phf, n_ph) || ctx_alloc(c, &xzf, n_xz) || ctx_alloc(c, &xzc, n_xz))
       return fail(PCF_ENOMEM);
   } else {
-    if (ctx_alloc(c, &yv, n_yv) || ctx_alloc(c, &ph, n_ph) || ctx_alloc(c, &xz, n_xz) || ctx_alloc(c, &fr, n_fr) ||
-        ctx_alloc(c, &pin, n_pi))
+    if (ctx_alloc(c, &yv, n_yv) || ctx_alloc(c, &ph, n_ph) || ctx_alloc(c, &xz, n_xz) || ctx_alloc(c, &xc, n_xz) ||
+        ctx_alloc(c, &pin, n_pi) || (list[0].solve_kind == 5 && ctx_alloc(c, &fr, n_fr)))
       return fail(PCF_ENOMEM);
   }
   c->hinst.resize(B);
   std::vector<int> per11(B), per3(B), per1(B, 1), per_tcs(B), per_tca(B);
   size_t o_yv = 0, o_ph = 0, o_xz = 0, o_np = 0, o_fr = 0, o_pi = 0;
-  c->split = !c->mixed;
+  c->split = !c->mixed && list[0].solve_kind != 1;
   // the FP32 form's plane kernels keep their transforms in warp registers wherever every
   // instance's nx and nz allow it (unless the caller asks for the shared-memory kernels)
   c->plane_warp = c->mixed && list[0].plane_kernel != 1;
@@ -1348,7 +1208,7 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
       I.nu = 1.0 / p.Re; I.dt = p.dt; I.dtau_hat = p.dtau_hat; I.dtau = 0.0;
       I.inv_nu = 1.0 / I.nu; I.inv_dt = 1.0 / I.dt; I.inv_dtau_hat = 1.0 / I.dtau_hat;
       I.inv_nxnz = 1.0 / ((double)p.nx * p.nz);
-      I.cheb = g.cheb; I.cheb_ff = g.cheb_ff; I.rco = g.rco; I.ygrid = g.y; I.ubase = g.ub; I.ccw = g.ccw;
+      I.cheb = g.cheb; I.rco = g.rco; I.ygrid = g.y; I.ubase = g.ub; I.ccw = g.ccw;
       I.kx = g.kx; I.kz = g.kz;
       I.twfx_x = g.twfx_x; I.twfx_z = g.twfx_z;
       I.mz_mul = div_mul(I.Mz); I.nz_mul = div_mul(p.nz); I.rx_mul = div_mul(p.nx / 8);
@@ -1366,7 +1226,10 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
         }
       }
       I.tab[0] = g.tab0; I.tab[1] = g.tab1;
-      I.dense[0] = g.dense0; I.dense[1] = g.dense1;
+      I.fxcheb = g.fxcheb; I.fxcheb_e = g.fxcheb_e;
+      I.fxD[0] = g.fxD[0]; I.fxD[1] = g.fxD[1]; I.fxDe[0] = g.fxDe[0]; I.fxDe[1] = g.fxDe[1];
+      I.ik2nu = g.ik2nu;
+      I.dense[0] = g.dense[0]; I.dense[1] = g.dense[1];
       I.sigma[0] = g.sig[0]; I.sigma[1] = g.sig[1];
       I.normpart = np + o_np;
       I.jcount = jc + b;
@@ -1374,9 +1237,10 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
         I.yvf = yvf + o_yv; I.physf = phf + o_ph; I.xzf = xzf + o_xz; I.xzc = xzc + o_xz;
         I.twxf = g.twxf; I.twzf = g.twzf; I.tcA = g.tcA; I.tcA5 = g.tcA5; I.mixed = 1;
       } else {
-        I.yv = yv + o_yv; I.phys = ph + o_ph; I.xz = xz + o_xz; I.frg = fr + o_fr; I.pinfo = pin + o_pi;
+        I.yv = yv + o_yv; I.phys = ph + o_ph; I.xz = xz + o_xz; I.xc = xc + o_xz; I.frg = fr ? fr + o_fr : nullptr;
+        I.pinfo = pin + o_pi;
       }
-      if (!I.dense[0] || !I.dense[1] || p.solve_kind == 2 || smem_ysolve(I.N, 1) > 227 * 1024) c->split = false;
+      if (!c->mixed && fp64_grid_refused(I)) return fail(PCF_ENOTSUP);
       o_yv += 2ULL * kFieldsY * p.ny * I.nmodes;
       o_ph += 2ULL * kFieldsSynth * p.ny * p.nx * p.nz;
       o_xz += 3ULL * p.ny * I.nmodes;
@@ -1423,11 +1287,14 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
     return fail(PCF_ECUDA);
   }
   const int want = list[0].modes_per_block;
-  st = want > 0 ? set_mode_tiles(c, want) : autotune_tiles(c);
-  if (st == PCF_OK && want > 0 && c->split) {
-    st = set_split_groups(c, want);
-    c->fused = st == PCF_OK && c->prm.solve_kind == 4 && c->sm_yf <= 227 * 1024;
-    if (st == PCF_OK && c->prm.solve_kind == 5) {
+  if (!c->split) {
+    st = want > 0 ? set_mode_tiles(c, want) : autotune_tiles(c);
+  } else {
+    st = set_modes(c, want > 0 ? want : solve_group(c));
+    const int kind = list[0].solve_kind;
+    c->jn = kind == 4;
+    c->fused = kind == 2 || kind == 4 || (kind == 0 && !c->reduced && want == 0 && fused_step_pays(c));
+    if (st == PCF_OK && kind == 5) {
       st = set_sweep(c, 32);
       c->sweep = st == PCF_OK;
     }
@@ -1465,7 +1332,7 @@ int pcf_symmetric_modes(const pcf_ctx* c) {
 
 int pcf_solve_variant(const pcf_ctx* c) {
   if (!c) return -1;
-  if (c->split) return c->fused ? 3 : (c->sweep ? 4 : 2);
+  if (c->split) return c->fused ? (c->jn ? 3 : 1) : (c->sweep ? 4 : 2);
   return c->hinst[0].dense[0] ? 1 : 0;
 }
 
@@ -1491,10 +1358,10 @@ pcf_status pcf_residual(pcf_ctx* c, const double* u, double* r, double* rnorm) {
   PCF_TRY(launch_ysynth(c, 0));
   PCF_TRY(launch_synth(c, 0, kFieldsSynth));
   PCF_TRY(launch_prodM(c));
-  if (c->mixed) PCF_TRY(launch_tc_analysis(c));
-  PCF_TRY(launch_mode(c, MODE_PHI, 0));
+  if (c->split || c->mixed) PCF_TRY(launch_analysis(c));
+  PCF_TRY(launch_solve(c, MODE_PHI, 0));
   if (rnorm) {
-    if (c->mixed) PCF_TRY(launch_tc_synth(c, 1));
+    if (c->split || c->mixed) PCF_TRY(launch_ysynth(c, 1, 0, false, 3));  // the banded kernel has done it
     PCF_TRY(launch_synth(c, 1, 3));
     launch_plane_sums(c, 1);
     k_norm_final<<<c->B, 32, 0, c->cs>>>(li_of(c, c->pre_inst), rnorm);
@@ -1513,8 +1380,8 @@ pcf_status pcf_adjoint_gradient(pcf_ctx* c, const double* u, const double* r, do
   PCF_TRY(launch_synth(c, 0, kFieldsSynth));
   PCF_TRY(launch_synth(c, 1, kFieldsSynth));
   PCF_TRY(launch_prodN(c));
-  if (c->mixed) PCF_TRY(launch_tc_analysis(c));
-  PCF_TRY(launch_mode(c, MODE_PSI_GRAD, 1));
+  if (c->split || c->mixed) PCF_TRY(launch_analysis(c));
+  PCF_TRY(launch_solve(c, MODE_PSI_GRAD, 1));
   PCF_TRY(check_launch());
   return leave(c);
 }
@@ -1528,7 +1395,7 @@ pcf_status pcf_influence_matrix_solve(pcf_ctx* c, const double* rhs, double* out
   set_pointers(c, nullptr, rhs, out);
   PCF_TRY(enter(c));
   PCF_TRY(push_descriptors(c));
-  PCF_TRY(launch_mode(c, MODE_SOLVE, sig));
+  PCF_TRY(launch_solve(c, MODE_SOLVE, sig));
   PCF_TRY(check_launch());
   return leave(c);
 }
@@ -1550,7 +1417,7 @@ static pcf_status descent_internal(pcf_ctx* c, double* u, double dtau, int nstep
   if (c->any_sym) PCF_TRY(launch_sym(c, -1));  // the run starts in the symmetric subspace
   if (c->timing) {
     PCF_TRY(launch_ysynth(c, 0));
-    for (int s = 0; s < nsteps; ++s) PCF_TRY(step_body(c, s));
+    for (int s = 0; s < nsteps; ++s) PCF_TRY(step_body(c, s, s + 1 == nsteps));
     PCF_TRY(check_launch());
     return leave(c);
   }
@@ -1559,7 +1426,7 @@ static pcf_status descent_internal(pcf_ctx* c, double* u, double dtau, int nstep
     cudaGraph_t g;
     PCF_CUDA(cudaStreamBeginCapture(c->cs, cudaStreamCaptureModeThreadLocal));
     pcf_status st = launch_ysynth(c, 0);
-    for (int s = 0; s < nsteps && st == PCF_OK; ++s) st = step_body(c, s);
+    for (int s = 0; s < nsteps && st == PCF_OK; ++s) st = step_body(c, s, s + 1 == nsteps);
     cudaError_t e = cudaStreamEndCapture(c->cs, &g);
     if (st != PCF_OK) return st;
     PCF_CUDA(e);
@@ -1747,7 +1614,7 @@ pcf_status pcf_kernel_times(pcf_ctx* c, double* ms, long long* launches, int n) 
 
 int pcf_launches_per_step(pcf_ctx* c) {
   if (!c) return 0;
-  const int base = c->split ? (c->fused ? 7 : 10) : c->mixed ? 10 : 6;
+  const int base = c->split ? (c->fused ? (c->jn ? 7 : 6) : 10) : c->mixed ? 10 : 6;
   // symmetric subspace: the projection, plus a separate synthesis where the update kernel
   // synthesises the state itself (fused and single per-mode kernels)
   return base + (c->any_sym ? ((c->split && !c->fused) || c->mixed ? 1 : 2) : 0);
@@ -1758,7 +1625,7 @@ pcf_status pcf_norm(pcf_ctx* c, const double* u, double* out) {
   set_pointers(c, u, nullptr, nullptr);
   PCF_TRY(enter(c));
   PCF_TRY(push_descriptors(c));
-  PCF_TRY(launch_ysynth(c, 0));
+  PCF_TRY(launch_ysynth(c, 0, 0, false, 3));
   PCF_TRY(launch_synth(c, 0, 3));
   launch_plane_sums(c, 0);
   k_norm_final<<<c->B, 32, 0, c->cs>>>(li_of(c, c->pre_inst), out);
@@ -1768,10 +1635,10 @@ pcf_status pcf_norm(pcf_ctx* c, const double* u, double* out) {
 
 pcf_status pcf_split_config(const pcf_ctx* c, int* cfg) {
   if (!c || !cfg) return PCF_EINVAL;
+  const bool tiles = c->split && !c->fused;
   cfg[0] = c->split ? c->sgrp : 0;
-  cfg[1] = c->split ? c->smt : 0;
-  cfg[2] = c->split ? c->smt_y : 0;
-  cfg[3] = c->split && !c->fused ? c->sgrp_s : 0;
+  cfg[1] = cfg[2] = tiles ? c->np : 0;
+  cfg[3] = tiles && !c->sweep ? c->sgrp : 0;
   return PCF_OK;
 }
 

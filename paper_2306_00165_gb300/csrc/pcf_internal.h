@@ -90,7 +90,12 @@ struct Inst {
   double inv_nu, inv_dt, inv_dtau_hat;  // 1/nu, 1/dt, 1/dtau_hat (IEEE quotients, set on the host)
   // tables (device)
   const double* cheb;
-  const float2* cheb_ff;  // the same table as float-float pairs (hi, lo), for the float-float form
+  const int4* fxcheb;  // fixed-point Chebyshev tables of the FP64 forms (FxTab of pcf_modes_fx.cu)
+  int fxcheb_e;        // exponent of the analysis table: its entries are scaled by 2^-fxcheb_e
+  const int4* fxD[2];  // [nmodes][6][Mh][(Mh + 1)/2] dense operators as fixed-point words
+  const int* fxDe[2];  // [nmodes][6][2 ((Mh + 1)/2)] exponents of their rows
+  const double* dense[2];  // mixed form: per-mode dense solve operators in FP64 (DenseLayout) or null
+  const double* ik2nu; // [nmodes] 1/(nu k^2), 0 for the mean mode
   const double* rco;
   const double* ygrid;
   const double* ubase;  // [3][ny]: base-flow profile U(y_j), U'(y_j) and the constant V
@@ -104,7 +109,6 @@ struct Inst {
   const float2* twxf; // e^{-2 pi i k/nx}, k < nx, of the mixed form
   const float2* twzf;
   const double* tab[2];  // per-mode solver tables: [0] sigma = 1/(nu dt), [1] sigma = 1/(nu dtau_hat)
-  const double* dense[2];  // per-mode dense solve operators (DenseLayout) or null
   double sigma[2];
   // buffers (device), uhat layout unless noted
   double2* uhat;
@@ -115,7 +119,8 @@ struct Inst {
   int2* pinfo;        // [2][11][ny]: exponent of each plane of phys and the bits of its largest magnitude
   double2* xz;        // [3][ny][Mx][Mz]
   double* normpart;   // [3][ny]
-  double* frg;        // [nmodes][3][2][N + 2]: class-split Stokes right-hand sides (FP64 split mode kernels)
+  double2* xc;        // [3][nmodes][ny]: Chebyshev coefficients of xz
+  double* frg;        // [nmodes][3][2][N + 2]: class-split Stokes right-hand sides (k_sweep)
   // mixed-precision form: FP32 plane data and Chebyshev coefficients of the products
   float* physf;       // [2][11][ny][nx][nz]
   float2* yvf;        // [2][5][ny][Mx][Mz]

@@ -17,7 +17,6 @@
 #include <mutex>
 #include <utility>
 
-#include "pcf_ff.cuh"
 #include "pcf_kernels.cuh"
 #include "pcf_plane_common.cuh"
 

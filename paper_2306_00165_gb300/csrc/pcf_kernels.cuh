@@ -26,16 +26,7 @@ struct GroupLaunch {
   const int* prefix;   // CTA prefix over groups (length ngroups + 1)
   const int2* groups;  // (first instance, instance count) per group
   int ngroups;
-  // 1: the modes m >= 0 only (storage indices i <= Kx, the first (Kx + 1) Mz modes); the
-  // synthesis also writes the y-values of mode -m from those of m by the s2 relation
-  // a_{-m} = e2_c (-1)^m conj(a_m), which every state in an s2-invariant subspace satisfies
-  int reduced;
 };
-
-// Number of (Fourier) modes a launch over instance I processes.
-__device__ __forceinline__ int run_modes(const GroupLaunch& gl, const Inst& I) {
-  return gl.reduced ? (I.Kx + 1) * I.Mz : I.nmodes;
-}
 
 __device__ __forceinline__ int find_inst(const LaunchInfo& li, int cta, int* local) {
   if (li.per) {  // no dependent loads on the way to the instance's descriptor
@@ -158,37 +149,31 @@ void launch_cheb_analysis_tc05(int ctas, size_t smem, cudaStream_t s, LaunchInfo
 cudaError_t set_cheb_tc05_smem(size_t smem);
 int cheb_tc_tiles(int nmodes);
 
-// Split mode kernels of the FP64 descent step (Chebyshev analysis, dense Stokes solve,
-// Chebyshev synthesis) over groups of instances on the same grid (at most
-// split_max_group() instances; G below is the largest group of a launch).
-// kind: 0 analysis, 1 solve, 2 synthesis.
-// The solve kernel is persistent (ctas <= nitems CTAs loop over the (group, mode, parity)
-// items, double-buffering each item's operands in shared memory).
-int split_ctas_per_group(int kind, int nmodes, int mt);
-int split_col_pad(int G);  // columns of a group of G instances (2 G rounded up to a power of two)
-int split_max_group(int N);
-size_t smem_yanalysis(int N, int G, int mt);
-size_t ysolve_buffer(int N, int G);
-size_t smem_ysolve(int N, int G);
-size_t smem_ysynth(int N, int G, int mt);
-// ff_arith: the Chebyshev dot products in float-float arithmetic (float-float form)
-// mt: consecutive modes per CTA of the analysis and synthesis kernels (col_pad(G) mt <= 32)
-void launch_yanalysis(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int op, bool ff_arith,
-                      int mt);
-void launch_ysolve(int ctas, int nitems, int bufsz, int scr_rows, size_t smem, cudaStream_t s, GroupLaunch gl,
-                   int op);
+// Per-mode kernels of the FP64 forms in 64-bit fixed point (pcf_modes_fx.cu): Chebyshev analysis
+// and synthesis over tiles of np modes of an instance, dense Stokes solve and the fused half-step
+// over groups of instances on one grid (at most kMaxGroup), one CTA per (group, mode).
+constexpr int kMaxGroup = 8;
+int yfx_tiles(int nmodes, int np);
+int yana_fx_threads(int N, int np, bool fine);
+int ysynth_fx_threads(int N, int np, bool fine);
+int ysolve_fx_threads(int N, int G, bool fine);
+size_t smem_yana_fx(int N, int np);
+size_t smem_ysynth_fx(int N, int np);
+size_t smem_ysolve_fx(int N, int G);
+size_t smem_ystep_fx(int N, int G);
+// fine: one matrix row and one part per thread, for launches with few row pairs.
+// red: the modes m >= 0 only (a state invariant under s2); the synthesis mirrors their y-values
+void launch_yana_fx(int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int np, int red, int fine);
+void launch_ysynth_fx(int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf,
+                      int check_active, int np, int red, int fine);
+void launch_ysolve_fx(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int op, int sig, int fine);
+void launch_ystep_fx(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int op, int synth, int fine);
 void launch_jnorm(int ninst, cudaStream_t s, const Inst* insts, int step_index);
-int ysolve_ctas_per_sm(size_t smem);
-void launch_ysynth_split(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int slot,
-                         int check_active, bool ff_arith, int mt);
-// threads per CTA of the split analysis / synthesis: one pass over a CTA's row tasks
-int split_yanalysis_threads(int N, int G, int mt, bool fp64);
-int split_ysynth_threads(int N, int G, int mt, bool fp64);
-cudaError_t set_split_smem(size_t analysis, size_t solve, size_t synth);
-// The fused per-mode half-step (analysis + solve + synthesis), one CTA per (group, mode).
-size_t smem_ystep(int N, int G);
-void launch_ystep(int ctas, size_t smem, cudaStream_t s, GroupLaunch gl, int op);
-cudaError_t set_ystep_smem(size_t smem);
+cudaError_t set_modes_fx_smem(size_t ana, size_t synth, size_t solve, size_t step);
+// dense operators -> fixed-point words (default stream): lengths of the two arrays, conversion
+size_t dense_limbs_len(int N, int nmodes);
+size_t dense_exps_len(int N, int nmodes);
+void launch_dense_limbs(const double* src, int N, int nmodes, int4* dst, int* dexp);
 
 // Symmetric-subspace projection and the DNS helpers (pcf_sym_dns.cu).
 int symmetrize_ctas(const Inst& I);

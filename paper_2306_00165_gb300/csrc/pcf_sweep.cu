@@ -110,7 +110,22 @@ __global__ void __launch_bounds__(T) k_sweep(LaunchInfo li, int red) {
   const bool mean = m == 0;
   const double* tab = I.tab[sig] + (size_t)m * TL.per_mode();
   const double* rco = I.rco;
-  const double* Fr = I.frg + (size_t)m * 6 * L2;
+  double* Fr = I.frg + (size_t)m * 6 * L2;
+  // this chain's right-hand sides F = (state/step + product)/nu: f_v of class pv, part rho, and
+  // f_u, f_w of class 1 - g, the other part (the mean mode: of class g, this part)
+  const double inv_step = OP == MODE_PHI ? I.inv_dt : I.inv_dtau_hat;
+  if (valid) {
+    for (int c = 0; c < 3; ++c) {
+      const int cls = c == 1 || mean ? g : 1 - g, part = c == 1 || mean ? rho : 1 - rho;
+      const double* st = reinterpret_cast<const double*>((OP == MODE_PHI ? I.uhat : I.rhat) + ((size_t)c * nm + m) * ny);
+      const double* xc = reinterpret_cast<const double*>(I.xc + ((size_t)c * nm + m) * ny);
+      double* f = Fr + (c * 2 + part) * L2 + cls * Mh;
+      for (int i = 0; i < (N - cls) / 2 + 1; ++i) {
+        const int k = 2 * (cls + 2 * i) + part;
+        f[i] = fma(st[k], inv_step, xc[k]) * I.inv_nu;
+      }
+    }
+  }
   if (valid) {
     if (mean) {
       // mean mode: v = 0; Dirichlet Helmholtz problems for u (into P) and w (into V), class g
@@ -157,7 +172,6 @@ __global__ void __launch_bounds__(T) k_sweep(LaunchInfo li, int red) {
   }
   __syncwarp();  // the partner lane's xi and eta
   if (!valid) return;
-  const double inv_step = OP == MODE_PHI ? I.inv_dt : I.inv_dtau_hat;
   const auto put = [&](int comp, int n, double val) {
     const size_t gidx = ((size_t)comp * nm + m) * ny + n;
     double* rh = reinterpret_cast<double*>(I.rhat + gidx) + rho;
