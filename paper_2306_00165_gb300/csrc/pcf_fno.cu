@@ -10,6 +10,7 @@
 // weights.  Proposals are judged by the residual norm of the descent (pcf_fno_propose).
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -215,6 +216,276 @@ __global__ void k_sum_parts(const float* part, int G, int E, float* out, int acc
     out[e] = accumulate ? out[e] + s : s;
   }
 }
+// ------------------------------------------------------------------ one mode per CTA
+// The whole network of one Fourier mode, forward and backward, in one CTA: the weights of a mode
+// (W x F encoder and decoder, L matrices W x W) and the activations of 32 samples fit shared
+// memory as BF16 operands, so that a training gradient is one launch plus a reduction over the
+// modes (54 launches of products, element-wise passes and sums before, each bound by its launch
+// and load latency: 584 us at 190 modes, W = 32, F = 132, 32 samples).  What bounds it now: the
+// chain of about 20 small products with a barrier each; weights and gradients cross HBM once.
+// Samples go 32 at a time; the weight gradients of later chunks continue the accumulators of
+// the earlier ones.  Every product rounds the same FP32 values to BF16 and accumulates K in the
+// same 16-wide steps as k_gemm_bf16, so the two paths give the same bits in every per-mode
+// output.
+constexpr int kFnoThreads = 256, kFnoS = 32;
+
+struct FnoFused {
+  const float *X, *T, *w;  // T null: forward only
+  float *Y, *g;            // Y null: not written
+  float* bpart;            // [MP][L + 1][W] sums over samples of dZ_l, then dH_0
+  double* lpart;           // [MP] sums of (Y - T)^2
+  long long oE, obE, oD, obD, oR[8], oL[8], ob[8];
+  int MP, S, W, F, L;
+  float sc;                // 2 / number of outputs
+};
+// shared memory: BF16 arrays with a pitch of 8 more than their (padded) width, whose rows then fall
+// into different 16-byte bank groups, and FP32 arrays
+struct FnoLayout {
+  int FP, PF, PW;  // F rounded up to 16, pitches
+  int Xb, Eb, Db, Hb, Wb, dYb, dZb, dHb, h_end;       // halves
+  int H, Z, dH, dZ, dY, total;                         // floats from byte offset 2 h_end
+  PCF_HD FnoLayout(int W, int F, int L, bool back) {
+    FP = (F + 15) & ~15;
+    PF = FP + 8;
+    PW = W + 8;
+    int o = 0;
+    const auto take = [&](int n) { const int at = o; o += n; return at; };
+    Xb = take(kFnoS * PF);
+    Eb = take(W * PF);
+    Db = take(FP * PW);
+    Hb = take((L + 1) * kFnoS * PW);
+    Wb = take(L * W * PW);
+    dYb = take(back ? kFnoS * PF : 0);
+    dZb = take(back ? kFnoS * PW : 0);
+    dHb = take(back ? kFnoS * PW : 0);
+    h_end = (o + 7) & ~7;
+    o = 0;
+    H = take(kFnoS * W);
+    Z = take(L * kFnoS * W);
+    dH = take(back ? kFnoS * W : 0);
+    dZ = take(back ? kFnoS * W : 0);
+    dY = take(back ? kFnoS * F : 0);
+    total = 2 * h_end + 4 * o;  // bytes
+  }
+};
+
+__device__ __forceinline__ void ldsm4(uint32_t* r, const __nv_bfloat16* p, bool trans) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  if (trans)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+// C(i, j) = init(i, j) + sum_k A(i, k) B(k, j) for i < M, j < N (M, N, K multiples of 16); A is stored
+// [i][k], or [k][i] when AT; B is stored [j][k], or [k][j] when BT.  Warps take 16 x 16 tiles.
+template <bool AT, bool BT, class INIT, class EPI>
+__device__ __forceinline__ void tile_gemm(const __nv_bfloat16* A, int pa, const __nv_bfloat16* B, int pb, int M, int N,
+                                          int K, const INIT& init, const EPI& epi) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nt = N >> 4;
+  const int gq = lane >> 2, tq = lane & 3, r8 = lane & 7, q = lane >> 3;
+  for (int t = warp; t < (M >> 4) * nt; t += kFnoThreads / 32) {
+    const int i0 = (t / nt) << 4, j0 = (t % nt) << 4;
+    float acc[2][4];
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int h = 0; h < 4; ++h) acc[b][h] = init(i0 + gq + (h >= 2 ? 8 : 0), j0 + 8 * b + 2 * tq + (h & 1));
+    for (int k0 = 0; k0 < K; k0 += 16) {
+      uint32_t a[4], b[4];
+      // 8 x 8 blocks in the order (i 0-7, k 0-7), (i 8-15, k 0-7), (i 0-7, k 8-15), (i 8-15, k 8-15)
+      if (AT) ldsm4(a, A + (k0 + r8 + (q & 2 ? 8 : 0)) * pa + i0 + (q & 1 ? 8 : 0), true);
+      else ldsm4(a, A + (i0 + r8 + (q & 1 ? 8 : 0)) * pa + k0 + (q & 2 ? 8 : 0), false);
+      // (k 0-7, j 0-7), (k 8-15, j 0-7), (k 0-7, j 8-15), (k 8-15, j 8-15)
+      if (BT) ldsm4(b, B + (k0 + r8 + (q & 1 ? 8 : 0)) * pb + j0 + (q & 2 ? 8 : 0), true);
+      else ldsm4(b, B + (j0 + r8 + (q & 2 ? 8 : 0)) * pb + k0 + (q & 1 ? 8 : 0), false);
+      mma16816(acc[0], a, b);
+      mma16816(acc[1], a, b + 2);
+    }
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int h = 0; h < 4; ++h) epi(i0 + gq + (h >= 2 ? 8 : 0), j0 + 8 * b + 2 * tq + (h & 1), acc[b][h]);
+  }
+}
+
+__global__ void __launch_bounds__(kFnoThreads, 2) k_fno_mode(FnoFused f) {
+  extern __shared__ __align__(16) unsigned char fsm[];
+  __shared__ double red[kFnoThreads / 32];
+  const int mp = blockIdx.x, W = f.W, F = f.F, L = f.L, S = f.S;
+  const bool back = f.T != nullptr;
+  const FnoLayout Y(W, F, L, back);
+  const int FP = Y.FP, PF = Y.PF, PW = Y.PW;
+  __nv_bfloat16* hb = reinterpret_cast<__nv_bfloat16*>(fsm);
+  float* fb = reinterpret_cast<float*>(fsm + 2 * Y.h_end);
+  __nv_bfloat16 *Xb = hb + Y.Xb, *Eb = hb + Y.Eb, *Db = hb + Y.Db, *Hb = hb + Y.Hb, *Wb = hb + Y.Wb, *dYb = hb + Y.dYb,
+                *dZb = hb + Y.dZb, *dHb = hb + Y.dHb;
+  float *H = fb + Y.H, *Z = fb + Y.Z, *dH = fb + Y.dH, *dZ = fb + Y.dZ, *dY = fb + Y.dY;
+  const auto zero = [](int, int) { return 0.f; };
+  // the mode's weights as BF16 operands (columns past F are zero)
+  const float* E = f.w + f.oE + (size_t)mp * W * F;
+  const float* D = f.w + f.oD + (size_t)mp * F * W;
+  for (int t = threadIdx.x; t < W * FP; t += kFnoThreads) {
+    const int r = t / FP, c = t - r * FP;
+    Eb[r * PF + c] = __float2bfloat16_rn(c < F ? E[r * F + c] : 0.f);
+  }
+  for (int t = threadIdx.x; t < FP * W; t += kFnoThreads) {
+    const int r = t / W, c = t - r * W;
+    Db[r * PW + c] = __float2bfloat16_rn(r < F ? D[t] : 0.f);
+  }
+  for (int t = threadIdx.x; t < L * W * W; t += kFnoThreads) {
+    const int l = t / (W * W), e = t - l * W * W, r = e / W, c = e - r * W;
+    Wb[(l * W + r) * PW + c] = __float2bfloat16_rn(f.w[f.oR[l] + (size_t)mp * W * W + e] + f.w[f.oL[l] + e]);
+  }
+  double loss = 0.0;
+  for (int s0 = 0; s0 < S; s0 += kFnoS) {
+    const int ns = min(kFnoS, S - s0);
+    const bool first = s0 == 0;
+    const float* Xg = f.X + ((size_t)mp * S + s0) * F;
+    __syncthreads();
+    for (int t = threadIdx.x; t < kFnoS * FP; t += kFnoThreads) {
+      const int r = t / FP, c = t - r * FP;
+      Xb[r * PF + c] = __float2bfloat16_rn(r < ns && c < F ? Xg[r * F + c] : 0.f);
+    }
+    __syncthreads();
+    // H_0 = X E^T + bE
+    tile_gemm<false, false>(Xb, PF, Eb, PF, kFnoS, W, FP, zero, [&](int s, int j, float v) {
+      v = s < ns ? v + f.w[f.obE + j] : 0.f;
+      H[s * W + j] = v;
+      Hb[s * PW + j] = __float2bfloat16_rn(v);
+    });
+    __syncthreads();
+    // Z_l = H_l (R_l + L_l)^T + b_l, H_{l+1} = H_l + GELU(Z_l)
+    for (int l = 0; l < L; ++l) {
+      tile_gemm<false, false>(Hb + l * kFnoS * PW, PW, Wb + l * W * PW, PW, kFnoS, W, W, zero, [&](int s, int j, float v) {
+        const float z = v + f.w[f.ob[l] + j];
+        Z[(l * kFnoS + s) * W + j] = z;
+        const float hn = s < ns ? H[s * W + j] + gelu_f(z) : 0.f;
+        H[s * W + j] = hn;
+        Hb[((l + 1) * kFnoS + s) * PW + j] = __float2bfloat16_rn(hn);
+      });
+      __syncthreads();
+    }
+    // Y = H_L D^T + bD; dY = 2 (Y - T)/n
+    const __nv_bfloat16* HL = Hb + L * kFnoS * PW;
+    tile_gemm<false, false>(HL, PW, Db, PW, kFnoS, FP, W, zero, [&](int s, int j, float v) {
+      if (s < ns && j < F) {
+        const size_t at = ((size_t)mp * S + s0 + s) * F + j;
+        v += f.w[f.obD + (size_t)mp * F + j];
+        if (f.Y) f.Y[at] = v;
+        if (back) {
+          const float d = v - f.T[at];
+          loss += (double)d * d;
+          v = f.sc * d;
+        }
+      } else {
+        v = 0.f;
+      }
+      if (back) {
+        if (j < F) dY[s * F + j] = v;
+        dYb[s * PF + j] = __float2bfloat16_rn(v);
+      }
+    });
+    if (!back) continue;
+    __syncthreads();
+    float* gD = f.g + f.oD + (size_t)mp * F * W;
+    float* gbD = f.g + f.obD + (size_t)mp * F;
+    // dD = dY^T H_L, dbD, dH = dY D
+    tile_gemm<true, true>(dYb, PF, HL, PW, FP, W, kFnoS,
+                          [&](int i, int j) { return first || i >= F ? 0.f : gD[i * W + j]; },
+                          [&](int i, int j, float v) { if (i < F) gD[i * W + j] = v; });
+    for (int c = threadIdx.x; c < F; c += kFnoThreads) {
+      float a = first ? 0.f : gbD[c];
+      for (int s = 0; s < ns; ++s) a += dY[s * F + c];
+      gbD[c] = a;
+    }
+    tile_gemm<false, true>(dYb, PF, Db, PW, kFnoS, W, FP, zero, [&](int s, int j, float v) {
+      dH[s * W + j] = v;
+      const float z = v * gelu_df(Z[((L - 1) * kFnoS + s) * W + j]);  // rows past ns: v = 0
+      dZ[s * W + j] = z;
+      dZb[s * PW + j] = __float2bfloat16_rn(z);
+    });
+    __syncthreads();
+    for (int l = L - 1; l >= 0; --l) {
+      float* gR = f.g + f.oR[l] + (size_t)mp * W * W;
+      float* bp = f.bpart + ((size_t)mp * (L + 1) + l) * W;
+      for (int j = threadIdx.x; j < W; j += kFnoThreads) {
+        float a = first ? 0.f : bp[j];
+        for (int s = 0; s < ns; ++s) a += dZ[s * W + j];
+        bp[j] = a;
+      }
+      // dR = dZ^T H_l; dH_l = dH_{l+1} + dZ (R_l + L_l)
+      tile_gemm<true, true>(dZb, PW, Hb + l * kFnoS * PW, PW, W, W, kFnoS,
+                            [&](int i, int j) { return first ? 0.f : gR[i * W + j]; },
+                            [&](int i, int j, float v) { gR[i * W + j] = v; });
+      tile_gemm<false, true>(dZb, PW, Wb + l * W * PW, PW, kFnoS, W, W, zero, [&](int s, int j, float v) {
+        dH[s * W + j] += v;
+      });
+      __syncthreads();
+      for (int t = threadIdx.x; t < kFnoS * W; t += kFnoThreads) {
+        const int s = t / W, j = t - s * W;
+        if (l > 0) {
+          const float z = dH[t] * gelu_df(Z[(l - 1) * kFnoS * W + t]);
+          dZ[t] = z;
+          dZb[s * PW + j] = __float2bfloat16_rn(z);
+        } else {
+          dHb[s * PW + j] = __float2bfloat16_rn(dH[t]);
+        }
+      }
+      __syncthreads();
+    }
+    // dE = dH_0^T X, dbE
+    float* gE = f.g + f.oE + (size_t)mp * W * F;
+    tile_gemm<true, true>(dHb, PW, Xb, PF, W, FP, kFnoS,
+                          [&](int i, int j) { return first || j >= F ? 0.f : gE[i * F + j]; },
+                          [&](int i, int j, float v) { if (j < F) gE[i * F + j] = v; });
+    float* bp = f.bpart + ((size_t)mp * (L + 1) + L) * W;
+    for (int j = threadIdx.x; j < W; j += kFnoThreads) {
+      float a = first ? 0.f : bp[j];
+      for (int s = 0; s < ns; ++s) a += dH[s * W + j];
+      bp[j] = a;
+    }
+  }
+  if (!back) return;
+  for (int o = 16; o > 0; o >>= 1) loss += __shfl_down_sync(0xffffffffu, loss, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = loss;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = 0.0;
+    for (int w = 0; w < kFnoThreads / 32; ++w) a += red[w];
+    f.lpart[mp] = a;
+  }
+}
+
+// Gradients of the shared parameters: dL_l = sum over modes of dR_l, and the bias sums.  A CTA
+// takes 32 outputs, its 8 warps every eighth mode.
+__global__ void __launch_bounds__(256) k_fno_shared(FnoFused f) {
+  __shared__ float part[8][32];
+  const int W = f.W, WW = W * W, nL = f.L * WW, n = nL + (f.L + 1) * W;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+  float a = 0.f;
+  if (e < n) {
+    const bool isL = e < nL;
+    const int l = isL ? e / WW : 0;
+    const float* src = isL ? f.g + f.oR[l] + (e - l * WW) : f.bpart + (e - nL);
+    const size_t st = isL ? WW : (size_t)(f.L + 1) * W;
+#pragma unroll 4
+    for (int mp = warp; mp < f.MP; mp += 8) a += src[mp * st];
+  }
+  part[warp][lane] = a;
+  __syncthreads();
+  if (warp || e >= n) return;
+  for (int k = 1; k < 8; ++k) a += part[k][lane];
+  if (e < nL) {
+    const int l = e / WW;
+    f.g[f.oL[l] + (e - l * WW)] = a;
+  } else {
+    const int b = (e - nL) / W, j = (e - nL) - b * W;
+    f.g[(b < f.L ? f.ob[b] : f.obE) + j] = a;
+  }
+}
+
 // Adam on FP32 master weights
 __global__ void k_adam(float* w, const float* gr, float* m, float* v, long long n, float lr, float b1, float b2,
                        float eps, float c1, float c2) {
@@ -369,6 +640,32 @@ GemmArgs ga(const float* A, long long sAb, long long sAi, long long sAk, const f
   return g;
 }
 
+// The fused per-mode kernel serves widths that are multiples of 16 whose mode fits half an SM's
+// shared memory (two CTAs per SM; larger F leaves the products to k_gemm_bf16).
+size_t fused_smem(const pcf_fno* f, bool back) {
+  if (f->W % 16) return 0;
+  const size_t b = FnoLayout(f->W, f->NY * f->CI, f->L, back).total;
+  return b <= 113 * 1024 ? b : 0;
+}
+// Forward pass (T null), or loss partials and gradients into g.
+pcf_status fused(pcf_fno* f, const float* X, const float* T, int S, float* Y, float* g) {
+  FnoFused a;
+  memset(&a, 0, sizeof(a));
+  a.X = X; a.T = T; a.w = f->w; a.Y = Y; a.g = g; a.bpart = f->part; a.lpart = f->dpart;
+  a.oE = f->off[OE]; a.obE = f->off[ObE]; a.oD = f->off[OD]; a.obD = f->off[ObD];
+  for (int l = 0; l < f->L; ++l) { a.oR[l] = OR(f, l); a.oL[l] = OL(f, l); a.ob[l] = Ob(f, l); }
+  a.MP = f->MP; a.S = S; a.W = f->W; a.F = f->NY * f->CI; a.L = f->L;
+  a.sc = 2.f / (float)((long long)f->MP * S * a.F);
+  const size_t sm = fused_smem(f, T != nullptr);
+  if (raise_smem_limit((const void*)k_fno_mode, sm) != cudaSuccess) return PCF_ECUDA;
+  k_fno_mode<<<f->MP, kFnoThreads, sm, f->s>>>(a);
+  if (T) {
+    const int n = f->L * f->W * f->W + (f->L + 1) * f->W;
+    k_fno_shared<<<(n + 31) / 32, 256, 0, f->s>>>(a);
+  }
+  return cudaGetLastError() == cudaSuccess ? PCF_OK : PCF_ECUDA;
+}
+
 int grid_for(long long n) { return (int)std::min<long long>((n + 255) / 256, 4096); }
 
 // Y = network(X); keeps activations for the backward pass
@@ -398,14 +695,24 @@ void colsum(pcf_fno* f, const float* X, long long rows, int C, float* out) {
   k_sum_parts<<<(C + 255) / 256, 256, 0, f->s>>>(f->part, kPartBlocks, C, out, 0);
 }
 
-// gradients of mean((Y - T)^2) into f->g; the loss via per-block partial sums
-pcf_status backward(pcf_fno* f, const float* X, const float* T, int S, double* loss) {
+// loss = sum of n partial sums / number of outputs (synchronises)
+pcf_status read_loss(pcf_fno* f, int n, long long io, double* loss) {
+  std::vector<double> hp(n);
+  if (cudaMemcpyAsync(hp.data(), f->dpart, sizeof(double) * n, cudaMemcpyDeviceToHost, f->s) ||
+      cudaStreamSynchronize(f->s))
+    return PCF_ECUDA;
+  double sum = 0.0;
+  for (double x : hp) sum += x;
+  *loss = sum / (double)io;
+  return cudaGetLastError() == cudaSuccess ? PCF_OK : PCF_ECUDA;
+}
+
+// gradients of mean((Y - T)^2) into g; the loss via per-block partial sums
+pcf_status backward(pcf_fno* f, const float* X, const float* T, int S, float* g, double* loss) {
   const int MP = f->MP, W = f->W, F = f->NY * f->CI;
   const long long act = (long long)MP * S * W, io = (long long)MP * S * F;
-  float* g = f->g;
   const float* w = f->w;
   k_mse<<<kPartBlocks, 256, 0, f->s>>>(f->Y, T, f->dY, io, f->dpart);
-  std::vector<double> hp(kPartBlocks);
   // decoder: dD[mp] = dY[mp]^T H_L[mp], dbD, dH = dY[mp] D[mp]
   gemm(f->s, ga(f->dY, (long long)S * F, 1, F, f->H[f->L], (long long)S * W, W, 1, g + f->off[OD], (long long)F * W,
                 W, 1, F, W, S, 0.f), MP);
@@ -429,13 +736,18 @@ pcf_status backward(pcf_fno* f, const float* X, const float* T, int S, double* l
   gemm(f->s, ga(f->dH, (long long)S * W, 1, W, X, (long long)S * F, F, 1, g + f->off[OE], (long long)W * F, F, 1, W, F,
                 S, 0.f), MP);
   colsum(f, f->dH, (long long)MP * S, W, g + f->off[ObE]);
-  if (cudaMemcpyAsync(hp.data(), f->dpart, sizeof(double) * kPartBlocks, cudaMemcpyDeviceToHost, f->s) ||
-      cudaStreamSynchronize(f->s))
-    return PCF_ECUDA;
-  double sum = 0.0;
-  for (double x : hp) sum += x;
-  *loss = sum / (double)io;
-  return cudaGetLastError() == cudaSuccess ? PCF_OK : PCF_ECUDA;
+  return read_loss(f, kPartBlocks, io, loss);
+}
+
+// loss and gradients into g by either path
+pcf_status loss_and_grads(pcf_fno* f, const float* X, const float* T, int S, float* g, double* loss) {
+  if (fused_smem(f, true)) {
+    const pcf_status st = fused(f, X, T, S, nullptr, g);
+    return st != PCF_OK ? st : read_loss(f, f->MP, (long long)f->MP * S * f->NY * f->CI, loss);
+  }
+  if (ensure_cap(f, S) != PCF_OK) return PCF_ENOMEM;
+  forward(f, X, S, f->Y);
+  return backward(f, X, T, S, g, loss);
 }
 
 }  // namespace
@@ -466,8 +778,8 @@ pcf_status pcf_fno_create(int MP, int NY, int width, int layers, unsigned long l
   if (cudaMalloc(&f->w, o * sizeof(float)) || cudaMalloc(&f->g, o * sizeof(float)) ||
       cudaMalloc(&f->m, o * sizeof(float)) || cudaMalloc(&f->v, o * sizeof(float)) ||
       cudaMalloc(&f->wsum, (size_t)MP * W * W * sizeof(float)) ||
-      cudaMalloc(&f->part, (size_t)kPartBlocks * 64 * 64 * sizeof(float)) ||
-      cudaMalloc(&f->dpart, kPartBlocks * sizeof(double))) {
+      cudaMalloc(&f->part, std::max<size_t>((size_t)kPartBlocks * 64, (size_t)MP * (layers + 1) * W) * sizeof(float)) ||
+      cudaMalloc(&f->dpart, std::max(kPartBlocks, MP) * sizeof(double))) {
     pcf_fno_destroy(f);
     return PCF_ENOMEM;
   }
@@ -508,6 +820,7 @@ pcf_status pcf_fno_get_params(pcf_fno* f, float* host) {
 
 pcf_status pcf_fno_forward(pcf_fno* f, const float* X, int S, float* Y) {
   if (!f || !X || !Y || S < 1) return PCF_EINVAL;
+  if (fused_smem(f, false)) return fused(f, X, nullptr, S, Y, nullptr);
   if (ensure_cap(f, S) != PCF_OK) return PCF_ENOMEM;
   forward(f, X, S, Y);
   return cudaGetLastError() == cudaSuccess ? PCF_OK : PCF_ECUDA;
@@ -515,22 +828,17 @@ pcf_status pcf_fno_forward(pcf_fno* f, const float* X, int S, float* Y) {
 
 pcf_status pcf_fno_loss_grad(pcf_fno* f, const float* X, const float* T, int S, double* loss, float* grad) {
   if (!f || !X || !T || S < 1) return PCF_EINVAL;
-  if (ensure_cap(f, S) != PCF_OK) return PCF_ENOMEM;
-  forward(f, X, S, f->Y);
   double l = 0.0;
-  const pcf_status st = backward(f, X, T, S, &l);
+  const pcf_status st = loss_and_grads(f, X, T, S, grad ? grad : f->g, &l);
   if (st != PCF_OK) return st;
   if (loss) *loss = l;
-  if (grad && cudaMemcpy(grad, f->g, f->np * sizeof(float), cudaMemcpyDeviceToDevice)) return PCF_ECUDA;
   return PCF_OK;
 }
 
 pcf_status pcf_fno_train_step(pcf_fno* f, const float* X, const float* T, int S, float lr, double* loss) {
   if (!f || !X || !T || S < 1 || !(lr > 0)) return PCF_EINVAL;
-  if (ensure_cap(f, S) != PCF_OK) return PCF_ENOMEM;
-  forward(f, X, S, f->Y);
   double l = 0.0;
-  const pcf_status st = backward(f, X, T, S, &l);
+  const pcf_status st = loss_and_grads(f, X, T, S, f->g, &l);
   if (st != PCF_OK) return st;
   f->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
