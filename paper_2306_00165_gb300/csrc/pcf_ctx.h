@@ -5,8 +5,23 @@
 
 #include "pcf_kernels.cuh"
 
+// Device tables of one grid (shared by every instance on that grid).
+struct GridTables {
+  double *cheb, *rco, *ccw, *kx, *kz, *y, *ub, *tab0, *tab1, *ik2nu = nullptr;
+  double* dense[2] = {nullptr, nullptr};
+  int4 *fxcheb = nullptr, *fxD[2] = {nullptr, nullptr};
+  int* fxDe[2] = {nullptr, nullptr};
+  int fxcheb_e = 0;
+  pcf::fxtw *twfx_x = nullptr, *twfx_z = nullptr;
+  float2 *twxf = nullptr, *twzf = nullptr;
+  uint16_t* tcA = nullptr;
+  uint16_t* tcA5 = nullptr;
+  double sig[2];
+};
+
 struct pcf_ctx {
   pcf_params prm;
+  GridTables gt;  // of the first problem
   int N, Kx, Kz, Mx, Mz, nm, B, mpc;
   long long state_len;  // complex values per instance (instance 0; all instances when uniform)
   std::vector<long long> state_off;  // complex offset of each instance's state, [B+1]
@@ -94,7 +109,10 @@ struct pcf_ctx {
   double2* dmd_cu = nullptr;    // candidate states
   double* dmd_J = nullptr;      // candidate norms (batch)
   double* dmd_c = nullptr;      // candidate coefficient vectors (device)
+  pcf_ctx* dmd_eval = nullptr;  // context over a batch of candidates on this problem's tables
   int dmd_cap = 0;              // columns the DMD workspace holds
   int dmd_ncand_cap = 0;
 };
 
+// A context over `batch` instances of c's (first) problem that shares c's tables: workspace only.
+pcf_status pcf_make_child(pcf_ctx* c, int batch, pcf_ctx** out);

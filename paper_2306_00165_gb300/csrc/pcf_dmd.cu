@@ -13,8 +13,10 @@
 // least-squares amplitudes are all computed from the small R on the host; the steady
 // state b_1 phi_1 = Psi' (Re(b_1 V Sigma^-1 w_1)) is a combination of the snapshots.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
+#include <thread>
 #include <vector>
 
 #include "pcf_ctx.h"
@@ -60,97 +62,105 @@ __global__ void k_psi_extract(const double2* __restrict__ uhat, long long state_
   }
 }
 
-// One thread per (instance, independent mode or mean): rebuild the mode's u, v, w.
-__global__ void k_psi_rebuild(const double* __restrict__ psi, long long psi_len, double2* __restrict__ uhat,
-                              long long state_len, const int* __restrict__ indep, int nindep,
-                              const double* __restrict__ kx, const double* __restrict__ kz, int Mx, int Mz, int ny,
-                              int nm, int B) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per (instance, independent mode or mean): rebuild the mode's u, v, w.  Coefficients
+// sit in shared memory; the lanes share the wall sums and the assembly, four lanes run the
+// derivative recurrence (parts x parity classes).  One thread per mode with its four
+// coefficient columns in local memory took 112 us for 20 states at 32x33x32.
+constexpr int kRebuildWarps = 4, kRebuildLen = 132;
+__device__ __forceinline__ double warp_sum(double s) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+__global__ void __launch_bounds__(32 * kRebuildWarps)
+    k_psi_rebuild(const double* __restrict__ psi, long long psi_len, double2* __restrict__ uhat, long long state_len,
+                  const int* __restrict__ indep, int nindep, const double* __restrict__ kx,
+                  const double* __restrict__ kz, int Mx, int Mz, int ny, int nm, int B) {
+  __shared__ double sh[kRebuildWarps][6][kRebuildLen];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t = blockIdx.x * kRebuildWarps + warp;
   if (t >= B * (nindep + 1)) return;
   const int b = t / (nindep + 1), q = t - b * (nindep + 1);
   const int N = ny - 1;
   const int segv = N - 3, sege = N - 1, seg = 2 * segv + 2 * sege;
   const double* in = psi + (size_t)b * psi_len;
   double2* u = uhat + (size_t)b * state_len;
-  double vr[130], vi[130], er[130], ei[130];
+  double *vr = sh[warp][0], *vi = sh[warp][1], *er = sh[warp][2], *ei = sh[warp][3], *xr = sh[warp][4], *xi = sh[warp][5];
+  // the top coefficient of each parity class from sum a_n = 0
+  const auto dirichlet = [&](double* a) {
+    for (int par = 0; par < 2; ++par) {
+      const int top = (N % 2 == par) ? N : N - 1;
+      double s = 0.0;
+      for (int n = par + 2 * lane; n < top; n += 64) s += a[n];
+      s = warp_sum(s);
+      if (lane == 0) a[top] = -s;
+    }
+    __syncwarp();
+  };
   if (q == nindep) {
     // mean u, w: Dirichlet completion, imaginary part zero; v = 0
     const double* o = in + (size_t)nindep * seg;
     for (int c = 0; c < 2; ++c) {
-      for (int n = 0; n <= N; ++n) vr[n] = n < sege ? o[c * sege + n] : 0.0;
-      for (int par = 0; par < 2; ++par) {
-        const int top = (N % 2 == par) ? N : N - 1;
-        double s = 0.0;
-        for (int n = par; n < top; n += 2) s += vr[n];
-        vr[top] = -s;
-      }
+      for (int n = lane; n <= N; n += 32) vr[n] = n < sege ? o[c * sege + n] : 0.0;
+      __syncwarp();
+      dirichlet(vr);
       const int comp = c == 0 ? 0 : 2;
-      for (int n = 0; n <= N; ++n) u[((size_t)comp * nm + 0) * ny + n] = make_double2(vr[n], 0.0);
+      for (int n = lane; n <= N; n += 32) u[((size_t)comp * nm + 0) * ny + n] = make_double2(vr[n], 0.0);
+      __syncwarp();
     }
-    for (int n = 0; n <= N; ++n) u[((size_t)1 * nm + 0) * ny + n] = make_double2(0.0, 0.0);
+    for (int n = lane; n <= N; n += 32) u[((size_t)1 * nm + 0) * ny + n] = make_double2(0.0, 0.0);
     return;
   }
   const int i = indep[2 * q], j = indep[2 * q + 1], m = i * Mz + j;
   const double* o = in + (size_t)q * seg;
-  for (int n = 0; n <= N; ++n) {
+  for (int n = lane; n <= N; n += 32) {
     vr[n] = n < segv ? o[n] : 0.0;
     vi[n] = n < segv ? o[segv + n] : 0.0;
     er[n] = n < sege ? o[2 * segv + n] : 0.0;
     ei[n] = n < sege ? o[2 * segv + sege + n] : 0.0;
   }
+  __syncwarp();
   // v: for each parity class the two top coefficients from sum a_n = 0, sum n^2 a_n = 0
   for (int par = 0; par < 2; ++par) {
     const int hi = (N % 2 == par) ? N : N - 1, lo = hi - 2;
-    double s0r = 0, s1r = 0, s0i = 0, s1i = 0;
-    for (int n = par; n < lo; n += 2) {
-      const double n2 = (double)n * n;
-      s0r += vr[n];
-      s1r += n2 * vr[n];
-      s0i += vi[n];
-      s1i += n2 * vi[n];
+    for (int part = 0; part < 2; ++part) {
+      double* v = part ? vi : vr;
+      double s0 = 0, s1 = 0;
+      for (int n = par + 2 * lane; n < lo; n += 64) {
+        s0 += v[n];
+        s1 = fma((double)(n * n), v[n], s1);
+      }
+      s0 = warp_sum(s0);
+      s1 = warp_sum(s1);
+      const double h2 = (double)hi * hi, l2 = (double)lo * lo, det = l2 - h2;
+      if (lane == 0) {
+        v[hi] = (s1 - s0 * l2) / det;
+        v[lo] = (s0 * h2 - s1) / det;
+      }
     }
-    const double h2 = (double)hi * hi, l2 = (double)lo * lo, det = l2 - h2;
-    vr[hi] = (s1r - s0r * l2) / det;
-    vr[lo] = (s0r * h2 - s1r) / det;
-    vi[hi] = (s1i - s0i * l2) / det;
-    vi[lo] = (s0i * h2 - s1i) / det;
   }
-  // eta: top coefficient of each class from sum a_n = 0
-  for (int par = 0; par < 2; ++par) {
-    const int top = (N % 2 == par) ? N : N - 1;
-    double sr = 0, si = 0;
-    for (int n = par; n < top; n += 2) {
-      sr += er[n];
-      si += ei[n];
+  __syncwarp();
+  dirichlet(er);
+  dirichlet(ei);
+  // dv/dy by the coefficient recurrence
+  if (lane < 4) {
+    const double* v = lane & 1 ? vi : vr;
+    double* x = lane & 1 ? xi : xr;
+    double acc = 0.0;
+    const int n0 = (N - (lane >> 1));  // class of N, or of N - 1
+    for (int n = n0; n >= 0; n -= 2) {
+      if (n + 1 <= N) acc = fma(2.0 * (n + 1), v[n + 1], acc);
+      x[n] = n == 0 ? 0.5 * acc : acc;
     }
-    er[top] = -sr;
-    ei[top] = -si;
   }
-  const double a = kx[i], c = kz[j], k2 = a * a + c * c;
-  // xi = -dv/dy by the coefficient recurrence, then u, w
-  double br2 = 0, br1 = 0, bi2 = 0, bi1 = 0;  // b_{n+2}, b_{n+1}
-  double xr[130], xi[130];
-  for (int n = N; n >= 0; --n) {
-    double br = 0.0, bi = 0.0;
-    if (n + 1 <= N) {
-      br = br2 + 2.0 * (n + 1) * vr[n + 1];
-      bi = bi2 + 2.0 * (n + 1) * vi[n + 1];
-    }
-    br2 = br1;
-    bi2 = bi1;
-    br1 = br;
-    bi1 = bi;
-    xr[n] = br;
-    xi[n] = bi;
-  }
-  xr[0] *= 0.5;
-  xi[0] *= 0.5;
+  __syncwarp();
+  const double a = kx[i], c = kz[j], ik2 = 1.0 / (a * a + c * c);
   const int mconj = (Mx - i) * Mz;  // storage index of (-m, 0)
-  for (int n = 0; n <= N; ++n) {
+  for (int n = lane; n <= N; n += 32) {
     const double xre = -xr[n], xim = -xi[n];
-    const double2 uu = make_double2((a * xim + c * ei[n]) / k2, -(a * xre + c * er[n]) / k2);
+    const double2 uu = make_double2((a * xim + c * ei[n]) * ik2, -(a * xre + c * er[n]) * ik2);
     const double2 vv = make_double2(vr[n], vi[n]);
-    const double2 ww = make_double2((c * xim - a * ei[n]) / k2, (-c * xre + a * er[n]) / k2);
+    const double2 ww = make_double2((c * xim - a * ei[n]) * ik2, (-c * xre + a * er[n]) * ik2);
     u[((size_t)0 * nm + m) * ny + n] = uu;
     u[((size_t)1 * nm + m) * ny + n] = vv;
     u[((size_t)2 * nm + m) * ny + n] = ww;
@@ -223,16 +233,82 @@ __global__ void k_qr_update(double* __restrict__ A, long long rows, long long ld
   }
 }
 
-// cand[c][i] = sum_k C[c][k] S[i][k+1]  (k < M): steady states as combinations of snapshots
-__global__ void k_combine(const double* __restrict__ S, long long rows, long long ld, int M,
-                          const double* __restrict__ C, int ncand, double* __restrict__ out, long long out_ld) {
+// Tall-skinny QR, R only: CTA b factors the rows [b RB, (b + 1) RB) of A (n columns, leading
+// dimension ld) by Householder reflections in shared memory and writes its R as rows b n ..
+// b n + n - 1 of out (leading dimension ldo, zeros below the diagonal); the stacked R's are
+// factored again until one CTA is left.  A warp takes a column's projection and update; the
+// warp that updates the next pivot column also takes its norm, so that a step has one barrier.
+// The column-by-column QR over the whole matrix (three launches per column, each waiting for
+// sums over all rows) took 940 us for 20218 x 21; this takes four launches.
+constexpr int kTsqrThreads = 512;
+__global__ void __launch_bounds__(kTsqrThreads) k_tsqr(const double* __restrict__ A, long long ld, long long rows, int n,
+                                                       int RB, double* __restrict__ out, long long ldo) {
+  extern __shared__ double q[];  // [n][RB + 1]
+  __shared__ double s_alpha, s_f;  // R_jj and 2 / v^T v of the pivot column (0: no reflection)
+  const int P = RB + 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kTsqrThreads / 32;
+  const long long r0 = (long long)blockIdx.x * RB;
+  const int m = (int)min((long long)RB, rows - r0);
+  for (int t = threadIdx.x; t < n * RB; t += kTsqrThreads) {
+    const int k = t / RB, i = t - k * RB;
+    q[k * P + i] = i < m ? A[(size_t)k * ld + r0 + i] : 0.0;
+  }
+  __syncthreads();
+  // pivot j: x = a_j[j:], alpha = -sign(x_j) |x|, v = x - alpha e_j in place
+  const auto pivot = [&](int j) {
+    double* x = q + j * P;
+    double s = 0.0;
+    for (int i = j + lane; i < RB; i += 32) s = fma(x[i], x[i], s);
+    s = warp_sum(s);
+    if (lane == 0) {
+      const double xj = x[j], nrm = sqrt(s), al = xj >= 0.0 ? -nrm : nrm, vtv = 2.0 * (s - al * xj);
+      s_alpha = al;
+      s_f = vtv > 0.0 ? 2.0 / vtv : 0.0;
+      x[j] = xj - al;
+    }
+    __syncwarp();
+  };
+  if (warp == 0) pivot(0);
+  __syncthreads();
+  for (int j = 0; j < n; ++j) {
+    const double f = s_f, al = s_alpha;
+    __syncthreads();  // the next pivot overwrites them
+    const double* v = q + j * P;
+    for (int k = j + 1 + warp; k < n; k += nw) {
+      double* a = q + k * P;
+      double s = 0.0;
+      for (int i = j + lane; i < RB; i += 32) s = fma(v[i], a[i], s);
+      s = warp_sum(s) * f;
+      for (int i = j + lane; i < RB; i += 32) a[i] = fma(-s, v[i], a[i]);
+      __syncwarp();
+      if (k == j + 1) pivot(k);
+    }
+    __syncthreads();
+    // row j of R: the diagonal, and the updated columns
+    for (int k = threadIdx.x; k < n; k += kTsqrThreads) {
+      const double d = k < j ? 0.0 : k == j ? al : q[k * P + j];
+      out[(size_t)k * ldo + (size_t)blockIdx.x * n + j] = d;
+    }
+  }
+}
+
+// cand[c][i] = sum_k C[c][k] S[i][k+1]  (k < M): steady states as combinations of snapshots, four
+// candidates per thread on each load
+__global__ void __launch_bounds__(256) k_combine(const double* __restrict__ S, long long rows, long long ld, int M,
+                                                 const double* __restrict__ C, int ncand, double* __restrict__ out,
+                                                 long long out_ld) {
+  const int c0 = 4 * blockIdx.y;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < rows;
        i += (long long)gridDim.x * blockDim.x) {
-    for (int c = 0; c < ncand; ++c) {
-      double s = 0.0;
-      for (int k = 0; k < M; ++k) s = fma(C[(size_t)c * M + k], S[(size_t)(k + 1) * ld + i], s);
-      out[(size_t)c * out_ld + i] = s;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k = 0; k < M; ++k) {
+      const double x = S[(size_t)(k + 1) * ld + i];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c0 + c < ncand) s[c] = fma(C[(size_t)(c0 + c) * M + k], x, s[c]);
     }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (c0 + c < ncand) out[(size_t)(c0 + c) * out_ld + i] = s[c];
   }
 }
 
@@ -275,7 +351,7 @@ pcf_status ensure_indep(pcf_ctx* c) {
 pcf_status ensure_dmd(pcf_ctx* c, int ncol) {
   if (c->dmd_cap >= ncol) return PCF_OK;
   const int cap = std::max(ncol, 32);
-  const int ncand = ((cap + c->B - 1) / c->B) * c->B;
+  const int ncand = cap + std::max(c->B, 32);  // whole batches of either evaluation context
   double *A, *part, *coef, *cpsi, *J, *cc;
   double2* cu;
   DMD_CUDA(cudaMalloc(&A, sizeof(double) * (size_t)c->psi_len * cap));
@@ -283,7 +359,7 @@ pcf_status ensure_dmd(pcf_ctx* c, int ncol) {
   DMD_CUDA(cudaMalloc(&coef, sizeof(double) * 2 * (size_t)cap));
   DMD_CUDA(cudaMalloc(&cpsi, sizeof(double) * (size_t)c->psi_len * ncand));
   DMD_CUDA(cudaMalloc(&cu, sizeof(double2) * (size_t)c->state_len * ncand));
-  DMD_CUDA(cudaMalloc(&J, sizeof(double) * (size_t)c->B));
+  DMD_CUDA(cudaMalloc(&J, sizeof(double) * (size_t)ncand));
   DMD_CUDA(cudaMalloc(&cc, sizeof(double) * (size_t)cap * ncand));
   for (void* p : {(void*)A, (void*)part, (void*)coef, (void*)cpsi, (void*)cu, (void*)J, (void*)cc})
     c->allocs.push_back(p);
@@ -316,6 +392,73 @@ pcf_status sync_out(pcf_ctx* c) {
     if (s_ != PCF_OK) return s_; \
   } while (0)
 
+// R of the QR of the ncol snapshots (columns of S, leading dimension ld), row-major, on the host.
+pcf_status snapshot_r(pcf_ctx* c, const double* S, long long ld, int ncol, std::vector<double>* R) {
+  const long long rows = c->psi_len;
+  R->assign((size_t)ncol * ncol, 0.0);
+  std::vector<double> h((size_t)ncol * ncol);
+  const int RB = std::max(256, 2 * ncol);
+  const size_t sm = sizeof(double) * (size_t)ncol * (RB + 1);
+  const auto blocks = [&](long long r) { return (r + RB - 1) / RB; };
+  const long long n1 = blocks(rows) * ncol, n2 = blocks(n1) * ncol;  // rows of the first two levels' outputs
+  if (sm <= 227 * 1024 - 64 && n1 + n2 <= rows) {
+    // two levels at a time in the workspace (rows x cap): level 1, 3, .. at its start, 2, 4, .. behind it
+    DMD_CUDA(raise_smem_limit((const void*)k_tsqr, sm));
+    const double* src = S;
+    long long r = rows, l = ld;
+    for (int level = 0;; ++level) {
+      const long long nb = blocks(r), ro = nb * ncol;
+      double* dst = level & 1 ? c->dmd_A + n1 * ncol : c->dmd_A;
+      k_tsqr<<<(int)nb, kTsqrThreads, sm, c->cs>>>(src, l, r, ncol, RB, dst, ro);
+      src = dst;
+      r = l = ro;
+      if (nb == 1) break;
+    }
+    DMD_CUDA(cudaGetLastError());
+    DMD_CUDA(cudaMemcpyAsync(h.data(), src, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, c->cs));
+    DMD_CUDA(cudaStreamSynchronize(c->cs));
+    for (int j = 0; j < ncol; ++j)
+      for (int k = j; k < ncol; ++k) (*R)[(size_t)j * ncol + k] = h[(size_t)k * ncol + j];
+    return PCF_OK;
+  }
+  // more columns than a CTA's shared memory holds, or few rows: column by column over the whole
+  // matrix, copied into the workspace (column-major, ld = rows)
+  DMD_CUDA(cudaMemcpy2DAsync(c->dmd_A, sizeof(double) * rows, S, sizeof(double) * ld, sizeof(double) * rows, ncol,
+                             cudaMemcpyDeviceToDevice, c->cs));
+  double* alpha = c->dmd_coef + c->dmd_cap;
+  for (int j = 0; j < ncol; ++j) {
+    k_qr_dots<<<kQrBlocks, 256, 0, c->cs>>>(c->dmd_A, rows, rows, j, ncol, c->dmd_part);
+    k_qr_reflect<<<1, 128, 0, c->cs>>>(c->dmd_A, rows, j, ncol, c->dmd_part, kQrBlocks, c->dmd_coef, alpha);
+    if (j + 1 < ncol) k_qr_update<<<kQrBlocks, 256, 0, c->cs>>>(c->dmd_A, rows, rows, j, ncol, c->dmd_coef);
+  }
+  DMD_CUDA(cudaGetLastError());
+  std::vector<double> al(ncol);
+  DMD_CUDA(cudaMemcpy2DAsync(h.data(), sizeof(double) * ncol, c->dmd_A, sizeof(double) * rows,
+                             sizeof(double) * ncol, ncol, cudaMemcpyDeviceToHost, c->cs));
+  DMD_CUDA(cudaMemcpyAsync(al.data(), alpha, sizeof(double) * ncol, cudaMemcpyDeviceToHost, c->cs));
+  DMD_CUDA(cudaStreamSynchronize(c->cs));
+  for (int j = 0; j < ncol; ++j) {
+    (*R)[(size_t)j * ncol + j] = al[j];
+    for (int k = j + 1; k < ncol; ++k) (*R)[(size_t)j * ncol + k] = h[(size_t)k * ncol + j];
+  }
+  return PCF_OK;
+}
+
+// Context that evaluates the candidates' residuals, up to `want` at a time: c itself, or one over
+// more instances of the same problem (at most 32, within 1 GiB of plane buffers), made on first use
+// and kept with c.  One candidate per pass left the GPU mostly idle: 19 passes of 90 us.
+pcf_ctx* eval_ctx(pcf_ctx* c, int want) {
+  const long long per = 2LL * kFieldsSynth * c->prm.nx * c->prm.ny * c->prm.nz * 8;
+  const int nb = (int)std::min<long long>(std::min(want, 32), (1LL << 30) / per);
+  if (nb <= c->B) return c;
+  if (c->dmd_eval && c->dmd_eval->B < nb) {
+    pcf_destroy(c->dmd_eval);
+    c->dmd_eval = nullptr;
+  }
+  if (!c->dmd_eval && pcf_make_child(c, nb, &c->dmd_eval) != PCF_OK) c->dmd_eval = nullptr;
+  return c->dmd_eval ? c->dmd_eval : c;
+}
+
 }  // namespace
 
 extern "C" {
@@ -340,7 +483,7 @@ pcf_status pcf_from_snapshot(pcf_ctx* c, const double* psi, double* u_hat) {
   DMD_TRY(ensure_indep(c));
   DMD_TRY(sync_in(c));
   const int n = c->B * (c->nindep + 1);
-  k_psi_rebuild<<<(n + 127) / 128, 128, 0, c->cs>>>(psi, c->psi_len, (double2*)u_hat, c->state_len, c->d_indep,
+  k_psi_rebuild<<<(n + kRebuildWarps - 1) / kRebuildWarps, 32 * kRebuildWarps, 0, c->cs>>>(psi, c->psi_len, (double2*)u_hat, c->state_len, c->d_indep,
                                                     c->nindep, c->hinst[0].kx, c->hinst[0].kz, c->Mx, c->Mz,
                                                     c->prm.ny, c->nm, c->B);
   DMD_CUDA(cudaGetLastError());
@@ -357,27 +500,9 @@ pcf_status pcf_dmd_extrapolate(pcf_ctx* c, const double* S, long long ld, int M,
   DMD_TRY(ensure_dmd(c, ncol));
   DMD_TRY(sync_in(c));
   const long long rows = c->psi_len;
-  // copy the snapshots into the QR workspace (column-major, ld = rows)
-  DMD_CUDA(cudaMemcpy2DAsync(c->dmd_A, sizeof(double) * rows, S, sizeof(double) * ld, sizeof(double) * rows, ncol,
-                             cudaMemcpyDeviceToDevice, c->cs));
-  double* alpha = c->dmd_coef + c->dmd_cap;
-  for (int j = 0; j < ncol; ++j) {
-    k_qr_dots<<<kQrBlocks, 256, 0, c->cs>>>(c->dmd_A, rows, rows, j, ncol, c->dmd_part);
-    k_qr_reflect<<<1, 128, 0, c->cs>>>(c->dmd_A, rows, j, ncol, c->dmd_part, kQrBlocks, c->dmd_coef, alpha);
-    if (j + 1 < ncol) k_qr_update<<<kQrBlocks, 256, 0, c->cs>>>(c->dmd_A, rows, rows, j, ncol, c->dmd_coef);
-  }
-  DMD_CUDA(cudaGetLastError());
-  std::vector<double> Rcm((size_t)ncol * ncol), al(ncol);
-  DMD_CUDA(cudaMemcpy2DAsync(Rcm.data(), sizeof(double) * ncol, c->dmd_A, sizeof(double) * rows,
-                             sizeof(double) * ncol, ncol, cudaMemcpyDeviceToHost, c->cs));
-  DMD_CUDA(cudaMemcpyAsync(al.data(), alpha, sizeof(double) * ncol, cudaMemcpyDeviceToHost, c->cs));
-  DMD_CUDA(cudaStreamSynchronize(c->cs));
   // R (row-major, ncol x ncol, upper triangular)
-  std::vector<double> R((size_t)ncol * ncol, 0.0);
-  for (int j = 0; j < ncol; ++j) {
-    R[(size_t)j * ncol + j] = al[j];
-    for (int k = j + 1; k < ncol; ++k) R[(size_t)j * ncol + k] = Rcm[(size_t)k * ncol + j];
-  }
+  std::vector<double> R;
+  DMD_TRY(snapshot_r(c, S, ld, ncol, &R));
   // Psi ~ R0 = R[:, 0:M], Psi' ~ R1 = R[:, 1:M+1], last snapshot t = R[:, M]
   std::vector<double> R0((size_t)ncol * M), R1((size_t)ncol * M), t(ncol);
   for (int i = 0; i < ncol; ++i) {
@@ -396,8 +521,9 @@ pcf_status pcf_dmd_extrapolate(pcf_ctx* c, const double* S, long long ld, int M,
   // candidates r = rstar .. 1: coefficient vectors over the snapshots s_1..s_M
   std::vector<double> Cc((size_t)rstar * M, 0.0);
   std::vector<int> rank_of(rstar);
-  int ncand = 0;
-  for (int r = rstar; r >= 1; --r) {
+  // the ranks are independent small dense problems: one host thread each, at most eight (about
+  // 60 us apiece at 20 snapshots)
+  const auto candidate = [&](int r, double* cv) -> bool {
     std::vector<double> VS((size_t)M * r);  // V_r Sigma_r^-1
     for (int i = 0; i < M; ++i)
       for (int k = 0; k < r; ++k) VS[(size_t)i * r + k] = V[(size_t)i * M + k] / s[k];
@@ -416,7 +542,7 @@ pcf_status pcf_dmd_extrapolate(pcf_ctx* c, const double* S, long long ld, int M,
         At[(size_t)a * r + b] = v;
       }
     std::vector<la::cd> lam, W;
-    if (!la::eig_general(r, At, lam, W)) continue;
+    if (!la::eig_general(r, At, lam, W)) return false;
     int q1 = 0;
     double best = 1e300;
     for (int q = 0; q < r; ++q) {
@@ -428,40 +554,66 @@ pcf_status pcf_dmd_extrapolate(pcf_ctx* c, const double* S, long long ld, int M,
     }
     std::vector<double> cp = la::lstsq_svd(ncol, r, X, t);
     std::vector<la::cd> bvec(cp.begin(), cp.end());
-    if (!la::csolve(r, W, bvec)) continue;
+    if (!la::csolve(r, W, bvec)) return false;
     const la::cd b1 = bvec[q1];
-    double* cv = Cc.data() + (size_t)ncand * M;
     for (int l = 0; l < M; ++l) {
       la::cd a = 0;
       for (int k = 0; k < r; ++k) a += VS[(size_t)l * r + k] * W[(size_t)k * r + q1];
       cv[l] = std::real(b1 * a);
     }
-    rank_of[ncand++] = r;
+    return true;
+  };
+  std::vector<char> ok(rstar, 0);
+  std::atomic<int> next(0);
+  std::atomic<bool> failed(false);
+  const auto work = [&]() noexcept {
+    try {
+      for (int k = next++; k < rstar; k = next++) ok[k] = candidate(rstar - k, Cc.data() + (size_t)k * M);
+    } catch (...) {
+      failed = true;
+    }
+  };
+  {
+    std::vector<std::thread> pool;
+    try {
+      pool.reserve(7);
+      for (int t = 1; t < std::min(rstar, 8); ++t) pool.emplace_back(work);
+    } catch (...) {  // no more threads: the others and this one take the rest
+    }
+    work();
+    for (std::thread& t : pool) t.join();
   }
+  if (failed) return PCF_ENOMEM;
+  int ncand = 0;
+  for (int k = 0; k < rstar; ++k)
+    if (ok[k]) {
+      if (ncand < k) std::copy_n(Cc.data() + (size_t)k * M, M, Cc.data() + (size_t)ncand * M);
+      rank_of[ncand++] = rstar - k;
+    }
   if (ncand == 0) return PCF_ENAN;
-  // candidate states on the device
-  DMD_CUDA(cudaMemcpyAsync(c->dmd_c, Cc.data(), sizeof(double) * (size_t)ncand * M, cudaMemcpyHostToDevice, c->cs));
-  k_combine<<<std::min<long long>((rows + 255) / 256, 2048), 256, 0, c->cs>>>(S, rows, ld, M, c->dmd_c, ncand,
-                                                                             c->dmd_cpsi, rows);
+  // candidate states on the device, padded to whole batches with the last candidate
+  pcf_ctx* ev = eval_ctx(c, M);
+  const int nb = (ncand + ev->B - 1) / ev->B * ev->B;
+  Cc.resize((size_t)nb * M);
+  for (int k = ncand; k < nb; ++k) std::copy_n(Cc.data() + (size_t)(ncand - 1) * M, M, Cc.data() + (size_t)k * M);
+  DMD_CUDA(cudaMemcpyAsync(c->dmd_c, Cc.data(), sizeof(double) * (size_t)nb * M, cudaMemcpyHostToDevice, c->cs));
+  k_combine<<<dim3((unsigned)std::min<long long>((rows + 255) / 256, 2048), (nb + 3) / 4), 256, 0, c->cs>>>(
+      S, rows, ld, M, c->dmd_c, nb, c->dmd_cpsi, rows);
   DMD_CUDA(cudaGetLastError());
-  const int nb = (ncand + c->B - 1) / c->B * c->B;
-  for (int k = ncand; k < nb; ++k)  // pad to whole batches with the last candidate
-    DMD_CUDA(cudaMemcpyAsync(c->dmd_cpsi + (size_t)k * rows, c->dmd_cpsi + (size_t)(ncand - 1) * rows,
-                             sizeof(double) * rows, cudaMemcpyDeviceToDevice, c->cs));
   {
     const int n = nb * (c->nindep + 1);
-    k_psi_rebuild<<<(n + 127) / 128, 128, 0, c->cs>>>(c->dmd_cpsi, rows, c->dmd_cu, c->state_len, c->d_indep,
-                                                      c->nindep, c->hinst[0].kx, c->hinst[0].kz, c->Mx, c->Mz,
-                                                      c->prm.ny, c->nm, nb);
+    k_psi_rebuild<<<(n + kRebuildWarps - 1) / kRebuildWarps, 32 * kRebuildWarps, 0, c->cs>>>(
+        c->dmd_cpsi, rows, c->dmd_cu, c->state_len, c->d_indep, c->nindep, c->hinst[0].kx, c->hinst[0].kz, c->Mx,
+        c->Mz, c->prm.ny, c->nm, nb);
     DMD_CUDA(cudaGetLastError());
   }
   DMD_CUDA(cudaEventRecord(c->ev_out, c->cs));
   DMD_CUDA(cudaStreamWaitEvent(c->user, c->ev_out, 0));
   std::vector<double> Jc(nb);
-  for (int g = 0; g < nb; g += c->B) {
-    DMD_TRY(pcf_residual(c, (const double*)(c->dmd_cu + (size_t)g * c->state_len), (double*)c->r_int, c->dmd_J));
-    DMD_CUDA(cudaMemcpyAsync(Jc.data() + g, c->dmd_J, sizeof(double) * c->B, cudaMemcpyDeviceToHost, c->user));
+  for (int g = 0; g < nb; g += ev->B) {
+    DMD_TRY(pcf_residual(ev, (const double*)(c->dmd_cu + (size_t)g * c->state_len), (double*)ev->r_int, c->dmd_J + g));
   }
+  DMD_CUDA(cudaMemcpyAsync(Jc.data(), c->dmd_J, sizeof(double) * nb, cudaMemcpyDeviceToHost, c->user));
   DMD_CUDA(cudaStreamSynchronize(c->user));
   int bi = -1;
   for (int k = 0; k < ncand; ++k)  // candidates are ordered by decreasing rank: ties keep the larger r

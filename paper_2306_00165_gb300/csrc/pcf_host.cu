@@ -729,20 +729,6 @@ static bool params_ok(const pcf_params* prm) {
          !((prm->symmetry & PCF_SYM_S1) && prm->base_flow != PCF_COUETTE);
 }
 
-// Device tables of one grid (shared by every instance on that grid).
-struct GridTables {
-  double *cheb, *rco, *ccw, *kx, *kz, *y, *ub, *tab0, *tab1, *ik2nu = nullptr;
-  double* dense[2] = {nullptr, nullptr};
-  int4 *fxcheb = nullptr, *fxD[2] = {nullptr, nullptr};
-  int* fxDe[2] = {nullptr, nullptr};
-  int fxcheb_e = 0;
-  fxtw *twfx_x = nullptr, *twfx_z = nullptr;
-  float2 *twxf = nullptr, *twzf = nullptr;
-  uint16_t* tcA = nullptr;
-  uint16_t* tcA5 = nullptr;
-  double sig[2];
-};
-
 static pcf_status build_tables(pcf_ctx* c, const pcf_params* prm, GridTables* g) {
   const int N = prm->ny - 1, nx = prm->nx, ny = prm->ny, nz = prm->nz;
   const int Kx = nx / 3 - 1, Kz = nz / 3 - 1, Mx = 2 * Kx + 1, Mz = Kz + 1;
@@ -1080,7 +1066,9 @@ static bool fp64_grid_refused(const Inst& I) {
   return 8 * (6 * H * H + 10 * H + 60 * H + 1) > 227 * 1024;
 }
 
-static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, pcf_ctx** out) {
+// shared: the tables of list[0]'s problem (nlist 1), owned by another context; else they are built
+static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, pcf_ctx** out,
+                               const GridTables* shared = nullptr) {
   if (!list || nlist < 1 || !out) return PCF_EINVAL;
   int B = 0;
   for (int k = 0; k < nlist; ++k) {
@@ -1131,14 +1119,20 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
     }
     if (found < 0) {
       GridTables g;
-      pcf_status st = build_tables(c, &list[k], &g);
-      if (st != PCF_OK) return fail(st);
+      if (shared) {
+        g = *shared;
+      } else {
+        pcf_status st = build_tables(c, &list[k], &g);
+        if (st != PCF_OK) return fail(st);
+      }
       gts.push_back(g);
       found = (int)gts.size() - 1;
     }
     grid_of[k] = found;
     if (found != 0) c->uniform = false;
   }
+
+  c->gt = gts[0];
 
   // per-instance workspace, one allocation per buffer kind
   size_t n_yv = 0, n_ph = 0, n_xz = 0, n_np = 0, n_fr = 0, n_pi = 0;
@@ -1310,6 +1304,15 @@ pcf_status pcf_create(const pcf_params* prm, void* stream, pcf_ctx** out) {
   return create_batch(prm, 1, stream, out);
 }
 
+}  // extern "C"
+pcf_status pcf_make_child(pcf_ctx* c, int batch, pcf_ctx** out) {
+  pcf_params p = c->prm;
+  p.batch = batch;
+  p.symmetry = PCF_SYM_NONE;
+  return create_batch(&p, 1, c->user, out, &c->gt);
+}
+extern "C" {
+
 pcf_status pcf_batch_create(const pcf_params* list, int n, void* stream, pcf_ctx** out) {
   return create_batch(list, n, stream, out);
 }
@@ -1338,6 +1341,7 @@ int pcf_solve_variant(const pcf_ctx* c) {
 
 void pcf_destroy(pcf_ctx* c) {
   if (!c) return;
+  if (c->dmd_eval) pcf_destroy(c->dmd_eval);
   if (c->cs) cudaStreamSynchronize(c->cs);
   for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
   for (auto& kv : c->dns_graphs) cudaGraphExecDestroy(kv.second);
