@@ -949,10 +949,12 @@ static pcf_status set_modes(pcf_ctx* c, int G) {
   // eight warps
   const int hp = (Nmax / 2 + 2) / 2;
   c->fine_s = (long long)c->cta_ys * 6 * hp * gmax < 152LL * 256;
-  c->thr_ys = ysolve_fx_threads(Nmax, gmax, c->fine_s);
+  c->thr_ys = ysolve_fx_threads(Nmax, gmax, c->fine_s, c->cta_ys >= 5 * 152);
   c->thr_yf = std::max(c->thr_ys, 256);
-  // tiles of 16 modes while they give every SM four CTAs of the analysis
-  c->np = 3 * (modes / 16) >= 4 * 152 ? 16 : 8;
+  // Eight modes per tile, sixteen where eight would leave a CTA of the synthesis less than four
+  // warps of tasks and the tiles still give every SM four CTAs (32 x 33 x 32, batch 32: synthesis
+  // 47 us against 51; 128 x 97 x 128 the other way: 121 against 122, analysis 67 against 77).
+  c->np = 8 * hp < 128 && 3 * (modes / 16) >= 4 * 152 ? 16 : 8;
   std::vector<int> pa(c->B), py(c->B), par(c->B), pyr(c->B);
   for (int b = 0; b < c->B; ++b) {
     const Inst& I = c->hinst[b];

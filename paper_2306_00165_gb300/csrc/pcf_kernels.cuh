@@ -156,7 +156,7 @@ constexpr int kMaxGroup = 8;
 int yfx_tiles(int nmodes, int np);
 int yana_fx_threads(int N, int np, bool fine);
 int ysynth_fx_threads(int N, int np, bool fine);
-int ysolve_fx_threads(int N, int G, bool fine);
+int ysolve_fx_threads(int N, int G, bool fine, bool many);
 size_t smem_yana_fx(int N, int np);
 size_t smem_ysynth_fx(int N, int np);
 size_t smem_ysolve_fx(int N, int G);

@@ -735,10 +735,21 @@ static int one_pass(int tasks, int most) {
 }
 // threads per CTA; fine: one row and one part per thread
 int yana_fx_threads(int N, int np, bool fine) {
-  return one_pass(fine ? 2 * np * (N + 1) : np * ((N / 2 + 2) / 2 + (N / 2 + 1) / 2), 320);
+  return one_pass(fine ? 2 * np * (N + 1) : np * ((N / 2 + 2) / 2 + (N / 2 + 1) / 2), 256);
 }
-int ysynth_fx_threads(int N, int np, bool fine) { return one_pass(np * (fine ? N + 2 : (N / 2 + 2) / 2), 320); }
-int ysolve_fx_threads(int N, int G, bool fine) { return one_pass(6 * ((N / 2 + 2) / 2) * G * (fine ? 4 : 1), 256); }
+int ysynth_fx_threads(int N, int np, bool fine) { return one_pass(np * (fine ? N + 2 : (N / 2 + 2) / 2), fine ? 320 : 256); }
+// many: the launch has at least five CTAs for every SM.  Small CTAs then keep more of their ten
+// dependent phases in flight: 96 or 128 threads, whichever leaves fewer lanes idle, while that
+// takes at most four passes (128 x 97 x 128: 147 us with 96 threads, 166 with 160; 64 x 65 x 64,
+// batch 2: 43 with 128, 48 with 224; 96 x 31 x 48, batch 3: 28 with 96, 35 with 160).  Groups of
+// more columns and launches of few CTAs want one pass (32 x 33 x 32, batch 8: 20.5 us with 256
+// threads, 24.6 with 96; 24 x 32^3 + 24 x 48^3 + 16 x 64^3 in groups of eight: 358 with 224, 492
+// with 96).
+int ysolve_fx_threads(int N, int G, bool fine, bool many) {
+  const int tasks = 6 * ((N / 2 + 2) / 2) * G * (fine ? 4 : 1);
+  if (many && tasks <= 4 * 96) return (tasks + 95) / 96 * 96 <= (tasks + 127) / 128 * 128 ? 96 : 128;
+  return one_pass(tasks, 256);
+}
 size_t smem_yana_fx(int N, int np) { return 16 * ((size_t)(N + 1) * (np + 1) + (size_t)np * (N + 2)) + 16 * (size_t)np; }
 size_t smem_ysynth_fx(int N, int np) { return 16 * (size_t)(N + 1) * (np + 1) + 24 * (size_t)np; }
 size_t smem_ysolve_fx(int N, int G) { return 16 * 6 * (size_t)(N + 1) * G + 64 * (size_t)G; }

@@ -24,10 +24,10 @@ namespace pcf {
 namespace {
 
 // Threads and resident CTAs the kernels are compiled for: 80 registers for sides up to 64
-// (six 128-thread CTAs), 128 registers for the longer transforms.
+// (six 128-thread CTAs), 128 registers (512 threads per SM) for the longer transforms.
 template <bool BIG>
 struct FxCfg {
-  static constexpr int threads = BIG ? 256 : 128, ctas = BIG ? 2 : 6;
+  static constexpr int threads = BIG ? 512 : 128, ctas = BIG ? 1 : 6;
 };
 
 __device__ __forceinline__ int fx_slot(int b, int e) { return b * 8 + (e ^ (b & 7)); }
@@ -165,12 +165,22 @@ size_t smem_planes_fx(const Inst& I, int threads) {
   const FxPlanes p = fx_planes(I, threads);
   return sizeof(fxc) * ((size_t)I.Mz * p.LX + (size_t)p.chunk * p.LZ) + 4 * (64 + 64 + 64 + 64);
 }
-// Threads per CTA: the synthesis of small planes keeps two warps busy in every pass; the
-// products, with fewer CTAs and a pointwise part, take twice as many.
+// Threads per CTA.  Sides up to 64: the synthesis of small planes keeps two warps busy in every
+// pass (32 x 33 x 32, batch 8: 32.1 us, with 128 threads 34.7); the products, with fewer CTAs and
+// a pointwise part, take 128 (21.5 us, with 64 threads 22.9).  Longer sides: the plane's x rows
+// fill much of the shared memory, so the smallest CTA that leaves the SM the most threads (128 x
+// 97 x 128: synthesis 233 us with 512 threads, 280 with 256, 397 with 128; 96 x 31 x 48, batch 3:
+// 64 us with 128 threads, 74 with 256); the products take at least 256 (there 40 and 51 us, with
+// 128 threads 47 and 62).
 bool planes_fx_big(const Inst& I) { return I.nx > 64 || I.nz > 64; }
 int planes_fx_threads(const Inst& I, bool prod) {
-  if (planes_fx_big(I)) return 256;
-  return !prod && I.nx * I.nz <= 1024 ? 64 : 128;
+  if (!planes_fx_big(I)) return !prod && I.nx * I.nz <= 1024 ? 64 : 128;
+  int best = 128, most = 0;
+  for (int t = 128; t <= FxCfg<true>::threads; t *= 2) {
+    const int fit = (int)(228 * 1024 / (smem_planes_fx(I, t) + 1024)), n = t * std::min(fit, 512 / t);
+    if (n > most) best = t, most = n;
+  }
+  return prod ? std::max(best, 256) : best;
 }
 
 __constant__ int c_fx_src[kFieldsSynth] = {0, 1, 2, 0, 3, 0, 1, 1, 2, 4, 2};

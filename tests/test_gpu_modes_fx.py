@@ -71,3 +71,24 @@ def test_a_mode_that_is_not_finite_stays_in_its_instance(pcf):
     assert np.isnan(got[1, 1, 2, 1].real).all()
     got[1, :, 2, 1] = clean[1, :, 2, 1]
     assert np.array_equal(got, clean)
+
+
+@pytest.mark.parametrize("grids", [[(64, 9, 64, 1)], [(64, 13, 64, 4)], [(64, 21, 64, 1), (16, 13, 16, 2)],
+                                   [(128, 9, 64, 1), (96, 11, 96, 1), (16, 9, 16, 1)]])
+def test_launch_shapes_give_the_same_bits(pcf, grids):
+    """The thread counts, tiles and groups a batch chooses move no bit: every sum is an exact
+    integer sum.  Many small CTAs (96 and 128 threads), tiles of 16 modes, planes of unequal
+    sizes in one launch, each against its instances one by one."""
+    us = [gi.random_perturbation(*g[:3], 0.1, 60 + k) for g in grids for k in range(g[3])]
+    s = pcf.Solver.batched(grids, solve_kind=3)
+    u = torch.from_numpy(np.concatenate([x.ravel() for x in us])).cuda()
+    H = s.descent_step(u, 0.01, 1).cpu().numpy()
+    got = u.cpu().numpy()
+    for b, x in enumerate(us):
+        one = pcf.Solver(*s.grids[b][:3], batch=1, solve_kind=3)
+        v = torch.from_numpy(x[None]).cuda()
+        h = one.descent_step(v, 0.01, 1).cpu().numpy()
+        assert np.array_equal(got[s.offsets[b]:s.offsets[b + 1]], v.cpu().numpy().ravel())
+        assert np.array_equal(H[:, b], h[:, 0])
+        one.close()
+    s.close()
