@@ -23,11 +23,11 @@ namespace pcf {
 
 namespace {
 
-// Threads and resident CTAs the kernels are compiled for: 80 registers for sides up to 64
-// (six 128-thread CTAs), 128 registers (512 threads per SM) for the longer transforms.
+// Threads and resident CTAs the kernels are compiled for: 80 registers for sides up to 64 (768
+// threads per SM), 128 registers (512 threads per SM) for the longer transforms.
 template <bool BIG>
 struct FxCfg {
-  static constexpr int threads = BIG ? 512 : 128, ctas = BIG ? 1 : 6;
+  static constexpr int threads = BIG ? 512 : 256, ctas = BIG ? 1 : 3;
 };
 
 __device__ __forceinline__ int fx_slot(int b, int e) { return b * 8 + (e ^ (b & 7)); }
@@ -96,45 +96,79 @@ __device__ __forceinline__ fx fx_signed(fx a, int neg) {
   const fx m = (fx)neg;
   return (a ^ m) - m;
 }
-// v 2^-e0 toward zero, where |v| 2^-e0 < 2^60
+// a 2^-r to the nearest, 0 <= a < 2^62; r > 63 gives 0
+__device__ __forceinline__ fx fx_round(fx a, int r) { return r > 63 ? 0 : (a + (fx)((1ULL << r) >> 1)) >> r; }
+// v 2^-e0 to the nearest, where |v| 2^-e0 < 2^61
 __device__ __forceinline__ fx fx_from(double v, int e0) {
   const int hi = __double2hiint(v), ec = (hi >> 20) & 0x7ff;
   const fx m = ((fx)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
-  const int r = 1083 + e0 - ec;
-  return fx_signed(ec == 0 || r > 63 ? 0 : (m << 8) >> r, hi >> 31);
+  return fx_signed(ec == 0 ? 0 : fx_round(m << 8, 1083 + e0 - ec), hi >> 31);
 }
 // k v 2^-e0, negated when neg
 __device__ __forceinline__ fx fx_from_k(double v, const FxK& k, int e0, int neg) {
   const int hi = __double2hiint(v), ec = (hi >> 20) & 0x7ff;
   const fx m = ((fx)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
-  const int r = 2106 + e0 - ec - k.e;
-  return fx_signed(ec == 0 || k.e == 0 || r > 63 ? 0 : (fx_mul64(m << 9, k.m) << 2) >> r, (hi >> 31) ^ k.neg ^ neg);
+  return fx_signed(ec == 0 || k.e == 0 ? 0 : fx_round(fx_mul64(m << 9, k.m) << 2, 2106 + e0 - ec - k.e),
+                   (hi >> 31) ^ k.neg ^ neg);
 }
-// Upper bound of |v| (|k v|) as w 2^(e - 14): e and w for the running maximum of e; v zero: e very low
+// Exponent of a double: kFxNone (zero, denormal), kFxNan (not finite) or floor(log2 |v|)
 __device__ __forceinline__ int fx_bexp(int hi) {
   const int ec = (hi >> 20) & 0x7ff;
   return ec == 0 ? kFxNone : ec == 0x7ff ? kFxNan : ec - 1023;
 }
-__device__ __forceinline__ unsigned fx_mant15(int hi) { return (((hi & 0xfffff) | 0x100000) >> 6) + 1; }
+__device__ __forceinline__ float fx_pow2f(int e) { return e < -126 ? 0.f : __int_as_float((e + 127) << 23); }
 
-// Sum over the block of w (pairs (E, S) per warp, S in units of 2^(E - 14)); returns the bit
-// length nb and the exponent E: sum < 2^(nb + E - 14).  sh: 2 ints per warp.
-__device__ __forceinline__ void fx_block_bound(int E, unsigned S, int* sh, int* Eo, int* nb) {
+// Running sum of magnitudes w |v| of doubles of any size, in single precision: a double with
+// biased exponent lim counts as 2^33 times its mantissa.  Values up to 2^60 above it are added as
+// they are (2^14 of them with weights below 2^8 stay finite), a larger one becomes the new
+// reference; values below 2^-160 of it vanish.  Truncated mantissas and the sum's rounding stay
+// within the factor 1 + 2^-9 of the bound taken from it.
+struct FxSum {
+  float acc = 0.f;
+  int lim = -4096;
+  unsigned top = 0;  // largest |v| (high word) with a weight other than zero
+  __device__ __forceinline__ static float mag(int habs, int off) { return __int_as_float(max(habs - off, 0) << 3); }
+  __device__ __forceinline__ void add(int hx, int hy, float w) {
+    const int m = max(hx, hy), em = m >> 20;
+    top = max(top, (unsigned)m);
+    if (em > lim + 60) {
+      acc *= fx_pow2f(lim - em);
+      lim = em;
+    }
+    const int off = (lim - 160) << 20;
+    acc = fmaf(w, mag(hx, off) + mag(hy, off), acc);
+  }
+};
+// The block's sum times g: true when some weighted value is not zero; *bits: sum < 2^bits.  any:
+// largest |v| of the thread's values, *all that of the block's.  sh: 4 ints per warp.
+__device__ __forceinline__ bool fx_block_bound(FxSum a, float g, unsigned any, int* sh, unsigned* all, int* bits) {
   const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int L = __reduce_max_sync(0xffffffffu, a.lim);
+  float v = a.acc * fx_pow2f(a.lim - L);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  any = __reduce_max_sync(0xffffffffu, any);
+  const unsigned top = __reduce_max_sync(0xffffffffu, a.top);
   if ((threadIdx.x & 31) == 0) {
-    sh[2 * warp] = E;
-    sh[2 * warp + 1] = (int)S;
+    sh[4 * warp] = L;
+    sh[4 * warp + 1] = __float_as_int(v);
+    sh[4 * warp + 2] = (int)any;
+    sh[4 * warp + 3] = (int)top;
   }
   __syncthreads();
-  int Em = sh[0];
-  for (int w = 1; w < nw; ++w) Em = max(Em, sh[2 * w]);
-  unsigned tot = 0;
+  int Lm = sh[0];
+  unsigned tm = 0, am = 0;
   for (int w = 0; w < nw; ++w) {
-    const int d = Em - sh[2 * w];
-    tot += (d > 31 ? 0u : (unsigned)sh[2 * w + 1] >> d) + 4u;
+    Lm = max(Lm, sh[4 * w]);
+    am = max(am, (unsigned)sh[4 * w + 2]);
+    tm = max(tm, (unsigned)sh[4 * w + 3]);
   }
-  *Eo = Em;
-  *nb = 32 - __clz((int)tot);
+  float tot = 0.f;
+  for (int w = 0; w < nw; ++w) tot += __int_as_float(sh[4 * w + 1]) * fx_pow2f(sh[4 * w] - Lm);
+  tot *= g * (1.f + 0x1p-9f);
+  *all = am;
+  *bits = (__float_as_int(tot) >> 23) - 126 + Lm - 1056;
+  return tm >= 0x00100000u;
 }
 
 __device__ __forceinline__ const int2* fx_info(const Inst& I, int slot, int f, int j) {
@@ -166,15 +200,19 @@ size_t smem_planes_fx(const Inst& I, int threads) {
   return sizeof(fxc) * ((size_t)I.Mz * p.LX + (size_t)p.chunk * p.LZ) + 4 * (64 + 64 + 64 + 64);
 }
 // Threads per CTA.  Sides up to 64: the synthesis of small planes keeps two warps busy in every
-// pass (32 x 33 x 32, batch 8: 32.1 us, with 128 threads 34.7); the products, with fewer CTAs and
-// a pointwise part, take 128 (21.5 us, with 64 threads 22.9).  Longer sides: the plane's x rows
-// fill much of the shared memory, so the smallest CTA that leaves the SM the most threads (128 x
-// 97 x 128: synthesis 233 us with 512 threads, 280 with 256, 397 with 128; 96 x 31 x 48, batch 3:
-// 64 us with 128 threads, 74 with 256); the products take at least 256 (there 40 and 51 us, with
-// 128 threads 47 and 62).
+// pass (32 x 33 x 32, batch 8: 28 us, with 128 threads 32), larger ones four (64 x 65 x 64, batch
+// 2: 55 us, with 96 threads 62, with 256 58).  The products take all row pairs of a plane in one
+// pass: with few CTAs per SM the loads of their factors are what the time goes to (64 x 65 x 64,
+// batch 2: 37 and 51 us with 256 threads, 41 and 67 with 128; 48 x 49 x 48, batch 4: 29 and 41 us
+// with 192, 30 and 45 with 128, 35 and 58 with 256; 32 x 33 x 32, batch 8: 20 and 30 us with
+// 128, 25 and 36 with 256).  Longer sides: the plane's x rows fill much of the shared memory, so
+// the smallest CTA that leaves the SM the most threads (128 x 97 x 128: synthesis 205 us with 512
+// threads; before the single-precision bound 233 with 512, 280 with 256, 397 with 128; 96 x 31 x
+// 48, batch 3: 56 us with 128); the products take at least 256 (there 40 and 51 us, with 128
+// threads 47 and 62).
 bool planes_fx_big(const Inst& I) { return I.nx > 64 || I.nz > 64; }
 int planes_fx_threads(const Inst& I, bool prod) {
-  if (!planes_fx_big(I)) return !prod && I.nx * I.nz <= 1024 ? 64 : 128;
+  if (!planes_fx_big(I)) return prod ? std::max(128, 4 * I.nx) : I.nx * I.nz <= 1024 ? 64 : 128;
   int best = 128, most = 0;
   for (int t = 128; t <= FxCfg<true>::threads; t *= 2) {
     const int fit = (int)(228 * 1024 / (smem_planes_fx(I, t) + 1024)), n = t * std::min(fit, 512 / t);
@@ -189,7 +227,7 @@ __constant__ int c_fx_fac[kFieldsSynth] = {0, 0, 0, 1, 0, 2, 1, 2, 1, 0, 2};
 // ------------------------------------------------------------------ plane synthesis
 // CTA = (instance, y-plane j, field f), fields as in k_xzsynth_t.  The plane's exponent e0 comes
 // from the sum B of |Re| + |Im| over the plane's modes (p > 0 twice): every intermediate of the
-// two transforms is below 2 B in modulus, and 2 B 2^-e0 <= 2^61.
+// two transforms is below 2 B in modulus, and 2 B 2^-e0 < 2^62.
 template <bool BIG>
 __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_synth_fx(LaunchInfo li, int slot, int nfields) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -205,50 +243,38 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_synth
   int* red = reinterpret_cast<int*>(Z + P.chunk * P.LZ);
   const double2* src = I.yv + (((size_t)slot * kFieldsY + c_fx_src[f]) * I.ny + j) * (size_t)nm;
   const int fac = c_fx_fac[f];
-  // exponent of the plane
-  int E = kFxNone;
+  // Bound of the plane: one pass in single precision (a pass for the largest exponent and one
+  // in integers took 90 instructions per mode, this one 25)
   const unsigned mzm = I.mz_mul;
-  const auto bexp = [&](int t, int hi) {
-    int e = fx_bexp(hi);
-    if (fac == 1) e += fx_bexp(__double2hiint(I.kx[fx_div(t, mzm)]));
-    else if (fac == 2) e += fx_bexp(__double2hiint(I.kz[t - fx_div(t, mzm) * Mz]));
-    return e;
-  };
-  for (int t = threadIdx.x; t < nm; t += blockDim.x) {
-    const double2 s = src[t];
-    E = max(E, max(bexp(t, __double2hiint(s.x)), bexp(t, __double2hiint(s.y))));
-  }
-  E = __reduce_max_sync(0xffffffffu, E);
-  unsigned S = 0;
-  const bool bad = E > kFxNan / 4;
-  if (E > kFxNone / 2 && !bad)
-    for (int t = threadIdx.x; t < nm; t += blockDim.x) {
-      const double2 s = src[t];
-      const int i = fx_div(t, mzm), p = t - i * Mz;
-      const double k = fac == 1 ? I.kx[i] : fac == 2 ? I.kz[p] : 1.0;
-      const int kh = __double2hiint(k) & 0x7fffffff, ek = fx_bexp(kh);
-      const unsigned km = fx_mant15(kh);
-      unsigned w = 0;
+  FxSum sum;
+  unsigned any = 0;
+  for (int t0 = threadIdx.x; t0 < nm; t0 += 4 * blockDim.x) {
+    double2 s[4];
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        // terms below 2^-28 of the largest: at most 2 units in all, within the slack of the block sum
-        const int hi = __double2hiint(c ? s.y : s.x), d = E - (fx_bexp(hi) + ek);
-        if (d < 28) w += ((fac ? (fx_mant15(hi) * km) >> 14 : fx_mant15(hi)) >> d) + 1;
-      }
-      S += p ? 2 * w : w;
+    for (int q = 0; q < 4; ++q) s[q] = t0 + q * (int)blockDim.x < nm ? src[t0 + q * blockDim.x] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int t = t0 + q * blockDim.x, i = fx_div(t, mzm), p = t - i * Mz;
+      const int hx = __double2hiint(s[q].x) & 0x7fffffff, hy = __double2hiint(s[q].y) & 0x7fffffff;
+      any = max(any, (unsigned)max(hx, hy));
+      // |k| in units of the smallest wavenumber
+      const int k = fac == 0 ? 1 : fac == 1 ? (i <= Kx ? i : I.Mx - i) : p;
+      if (t < nm && k) sum.add(hx, hy, (float)(p ? 2 * k : k));
     }
-  S = __reduce_add_sync(0xffffffffu, S);
-  int nb;
-  fx_block_bound(E, S, red, &E, &nb);
+  }
+  const int k1 = fac == 0 ? 0x3ff00000 : __double2hiint(fac == 1 ? I.kx[1] : I.kz[1]), ek = fx_bexp(k1);
+  int eb;
+  const bool live = fx_block_bound(sum, __int_as_float(0x3f800000 | (k1 & 0xfffff) << 3), any, red, &any, &eb);
+  const bool bad = any >= 0x7ff00000u || ek == kFxNan;
   int2* info = const_cast<int2*>(fx_info(I, slot, f, j));
   fx* out = reinterpret_cast<fx*>(I.phys) + (((size_t)slot * kFieldsSynth + f) * I.ny + j) * (size_t)nx * nz;
-  if (E > kFxNan / 4 || E < kFxNone / 2) {  // a NaN or an infinity in the plane, or a zero plane (uniform)
-    if (E < kFxNone / 2)
+  if (bad || !live) {  // a NaN or an infinity in the plane, or a zero plane (uniform)
+    if (!bad)
       for (int t = threadIdx.x; t < nx * nz; t += blockDim.x) out[t] = 0;
-    if (threadIdx.x == 0) *info = make_int2(E > kFxNan / 4 ? kFxNan : kFxNone, 0);
+    if (threadIdx.x == 0) *info = make_int2(bad ? kFxNan : kFxNone, 0);
     return;
   }
-  const int e0 = nb + E - 74;
+  const int e0 = eb + ek - 61;
   // the modes as integers at their x bins (rows p); i k v for the x and z derivatives
   for (int t = threadIdx.x; t < nm; t += blockDim.x) {
     const double2 s = src[t];
@@ -397,6 +423,14 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
   int* er = red + 64;   // exponents of the row pairs
   int* ep = er + 64;    // exponents of the x rows
   const double dU = I.ubase[I.ny + j];
+  // the factors' planes (offsets uniform in the CTA)
+  constexpr int NO = ADJ ? 12 : 6;
+  const int fs = I.ny * nx * nz;
+  const fx* const U = reinterpret_cast<const fx*>(I.phys) + (size_t)j * nx * nz;
+  const fx* const Q = U + (ADJ ? (size_t)kFieldsSynth * fs : 0);
+  int of[NO];
+#pragma unroll
+  for (int k = 0; k < NO; ++k) of[k] = fs * (k < 3 ? k : k < 6 ? fx_grad(c, k - 3) : k < 9 ? k - 6 : fx_grad(k - 9, c));
   if (threadIdx.x < 32) {
     const int k = min((int)threadIdx.x, 12);
     const int slot = k == 12 ? ADJ : k < 3 ? 0 : k < 9 ? ADJ : 0;
@@ -445,17 +479,9 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
   const unsigned nzm = I.nz_mul;
   const fx dUx = c == (ADJ ? 1 : 0) ? fx_from(dU, fx_bexp(__double2hiint(dU)) - 59) : 0;
   const int lgz = 32 - __clz(nz - 1), lgx = 32 - __clz(nx - 1);
-  // the factors' planes (offsets uniform in the CTA) and shifts
-  constexpr int NO = ADJ ? 12 : 6;
-  const int fs = I.ny * nx * nz;
-  const fx* const U = reinterpret_cast<const fx*>(I.phys) + (size_t)j * nx * nz;
-  const fx* const Q = U + (ADJ ? (size_t)kFieldsSynth * fs : 0);
-  int of[NO], sa[NO], sd[7];
+  int sa[NO], sd[7];
 #pragma unroll
-  for (int k = 0; k < NO; ++k) {
-    of[k] = fs * (k < 3 ? k : k < 6 ? fx_grad(c, k - 3) : k < 9 ? k - 6 : fx_grad(k - 9, c));
-    sa[k] = ssa[k];
-  }
+  for (int k = 0; k < NO; ++k) sa[k] = ssa[k];
 #pragma unroll
   for (int k = 0; k < 7; ++k) sd[k] = ssd[k];
   const fx add0 = sadd[0], add1 = sadd[1];

@@ -74,3 +74,25 @@ def test_a_value_that_is_not_finite_reaches_the_norm(pcf, bad):
     r_ref, J_ref = o.residual(clean)
     assert abs(float(J[1]) - J_ref) <= TOL * J_ref
     assert _rel(r.cpu().numpy()[1], r_ref) <= TOL
+
+
+@pytest.mark.parametrize("low,high", [(-300, 300), (-70, 0), (0, 150), (-990, -900)])
+def test_bound_of_a_plane_with_a_wide_range(pcf, low, high):
+    """The block exponent comes from a running single-precision sum with a moving reference:
+    modes spread over hundreds of binary orders, in any order, and a mean far above or below the
+    modes that enter a derivative."""
+    grid = (32, 9, 16)
+    rng = np.random.default_rng(5)
+    u0 = gi.random_perturbation(*grid, 0.1, 74)
+    o = PCFOracle(*grid)
+    s = pcf.Solver(*grid, batch=1)
+    e = rng.integers(low, high, size=u0.shape[1:3])
+    for i in range(1, (e.shape[0] + 1) // 2):
+        e[-i, 0] = e[i, 0]  # the modes p = 0 stay Hermitian in m
+    for mean in (low, high):
+        e[0, 0] = mean
+        v = u0 * 2.0 ** (e[None, :, :, None] - max(0.0, high))
+        r, _ = s.residual(torch.from_numpy(v[None]).cuda())
+        assert _rel(r.cpu().numpy()[0], o.residual(v)[0]) <= TOL
+        if low >= -300:  # the norm's square stays in range
+            assert abs(float(s.norm(torch.from_numpy(v[None]).cuda())[0]) - o.norm(v)) <= TOL * o.norm(v)
