@@ -510,9 +510,9 @@ pcf_status launch_prodN(pcf_ctx* c, int step_index = -1) {
 }
 
 // plane sums of the squared velocity of a slot
-void launch_plane_sums(pcf_ctx* c, int slot) {
-  if (c->mixed) launch_norm_planes(c->cta_synth3, c->cs, li_of(c, c->pre_synth3), slot);
-  else launch_norm_planes_fx(c->cta_synth3, c->cs, li_of(c, c->pre_synth3, c->cta_synth3), slot);
+void launch_plane_sums(pcf_ctx* c, int slot, DnsInst* dns = nullptr) {
+  if (c->mixed) launch_norm_planes(c->cta_synth3, c->cs, li_of(c, c->pre_synth3), slot, dns);
+  else launch_norm_planes_fx(c->cta_synth3, c->cs, li_of(c, c->pre_synth3, c->cta_synth3), slot, dns);
 }
 
 pcf_status launch_tc_synth(pcf_ctx* c, int slot) {
@@ -662,16 +662,12 @@ pcf_status step_body(pcf_ctx* c, int s, bool last) {
   return PCF_OK;
 }
 
-// One DNS step u <- u + dt r1 (pcf_dns): ||u|| and the extremum capture of the previous
-// step, M(u), the Stokes step of §4 step 1 (writing r1), the update, and the y-synthesis of
-// the new state for the next step.
+// One DNS step u <- u + dt r1 (pcf_dns): ||u|| and the extremum test of the previous step (its
+// capture comes with the update), M(u), the Stokes step of §4 step 1 (writing r1), the update,
+// and the y-synthesis of the new state for the next step.
 pcf_status dns_body(pcf_ctx* c) {
   PCF_TRY(launch_synth(c, 0, kFieldsSynth));
-  PCF_TRY(timed(c, 11, [&] {
-    launch_plane_sums(c, 0);
-    launch_dns_norm(c->B, c->cs, c->dinst, c->d_dns);
-    launch_dns_capture(c->dns_ctas, c->B, c->cs, c->dinst, c->d_dns);
-  }));
+  PCF_TRY(timed(c, 11, [&] { launch_plane_sums(c, 0, c->d_dns); }));
   PCF_TRY(launch_prodM(c));
   if (c->split || c->mixed) {
     PCF_TRY(launch_analysis(c));

@@ -435,9 +435,9 @@ __global__ void __launch_bounds__(128, ADJ ? 6 : 8) k_prod_t(LaunchInfo li, int 
 }
 
 // CTA = (instance, plane j, component c): sum over the plane of the squared velocity
-// component c of a slot (0: u, 1: q).
+// component c of a slot (0: u, 1: q); dns: the end of a DNS step's norm as well.
 template <class T>
-__global__ void __launch_bounds__(128) k_norm_planes_t(LaunchInfo li, int slot) {
+__global__ void __launch_bounds__(128) k_norm_planes_t(LaunchInfo li, int slot, DnsInst* dns) {
   __shared__ double red[32];
   int local;
   const int b = find_inst(li, blockIdx.x, &local);
@@ -454,6 +454,7 @@ __global__ void __launch_bounds__(128) k_norm_planes_t(LaunchInfo li, int slot) 
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
     I.normpart[(size_t)c * I.ny + j] = s;
   }
+  if (dns) finish_dns(I, dns[b]);
 }
 
 // host launchers (the kernel templates are instantiated in this translation unit only): FP32
@@ -469,8 +470,8 @@ void launch_prod(bool adj, bool suction, int ctas, size_t smem, cudaStream_t s, 
   if (suction) launch_prod_t<true>(adj, ctas, smem, s, li, step_index);
   else launch_prod_t<false>(adj, ctas, smem, s, li, step_index);
 }
-void launch_norm_planes(int ctas, cudaStream_t s, LaunchInfo li, int slot) {
-  k_norm_planes_t<float><<<ctas, 128, 0, s>>>(li, slot);
+void launch_norm_planes(int ctas, cudaStream_t s, LaunchInfo li, int slot, DnsInst* dns) {
+  k_norm_planes_t<float><<<ctas, 128, 0, s>>>(li, slot, dns);
 }
 cudaError_t set_plane_smem(size_t synth, size_t prod) {
   cudaError_t e;

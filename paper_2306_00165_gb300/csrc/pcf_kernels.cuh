@@ -72,25 +72,52 @@ __device__ __forceinline__ double norm_from_parts(const Inst& I) {
   return sqrt(0.5 * I.inv_nxnz * s);
 }
 
-// End of an adjoint product CTA, after thread 0 has written its plane sum: the CTA that counts
-// last of the instance's 3 ny computes J (its first warp), writes the history entry, clears
-// the mask when J < tol (the instance stops before this step's update) and resets the counter
-// for the next launch.
-__device__ __forceinline__ void finish_norm(const Inst& I, int step_index) {
-  if (threadIdx.x >= 32) return;
+// First warp of a CTA whose thread 0 has written its plane sum: true in the CTA that counts last
+// of the instance's 3 ny (thread 0 then resets the counter).
+__device__ __forceinline__ bool last_plane(const Inst& I) {
   int last = 0;
   if (threadIdx.x == 0) {
     __threadfence();
     last = atomicAdd(I.jcount, 1) == 3 * I.ny - 1;
   }
-  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  if (!__shfl_sync(0xffffffffu, last, 0)) return false;
   __threadfence();
+  return true;
+}
+
+// End of an adjoint product CTA: the last one computes J, writes the history entry and clears
+// the mask when J < tol (the instance stops before this step's update).
+__device__ __forceinline__ void finish_norm(const Inst& I, int step_index) {
+  if (threadIdx.x >= 32 || !last_plane(I)) return;
   const double J = norm_from_parts(I);
   if (threadIdx.x == 0) {
     if (I.hist) I.hist[(size_t)step_index * I.hist_stride] = J;
     if (I.tol > 0.0 && J < I.tol && I.active) *I.active = 0;
     *I.jcount = 0;
   }
+}
+
+// End of a plane-sum CTA of a DNS step: the last one has h_s = ||u_s|| (same arithmetic as the norm
+// of r1), writes its history entry and makes the discrete-extremum test of the previous step:
+//   (h_{s-1} - h_{s-2}) (h_s - h_{s-1}) < 0  ->  u_{s-1} (held in uprev until this step's update) is
+// a guess.  D.step counts the steps of the current call.
+__device__ __forceinline__ void finish_dns(const Inst& I, DnsInst& D) {
+  if (threadIdx.x >= 32 || !last_plane(I)) return;
+  const double h = norm_from_parts(I);
+  if (threadIdx.x != 0) return;
+  *I.jcount = 0;
+  const int step = D.step;
+  if (D.hist) D.hist[(size_t)step * D.hist_stride] = h;
+  int slot = -1;
+  if (step >= 2 && (D.h1 - D.h2) * (h - D.h1) < 0.0) {
+    const int k = *D.count;
+    if (k < D.gmax) slot = k;
+    *D.count = k + 1;
+  }
+  D.slot = slot;
+  D.h2 = D.h1;
+  D.h1 = h;
+  D.step = step + 1;
 }
 
 // Raise the maximum dynamic shared memory of kernel func on the current device to at least
@@ -112,7 +139,7 @@ cudaError_t set_sweep_smem(size_t smem);
 // suction: some instance of the launch has a base flow with a wall-normal velocity (ASBL)
 void launch_xzsynth(int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf);
 void launch_prod(bool adj, bool suction, int ctas, size_t smem, cudaStream_t s, LaunchInfo li, int step_index = -1);
-void launch_norm_planes(int ctas, cudaStream_t s, LaunchInfo li, int slot);
+void launch_norm_planes(int ctas, cudaStream_t s, LaunchInfo li, int slot, DnsInst* dns);
 cudaError_t set_plane_smem(size_t synth, size_t prod);
 // The FP64 forms' plane kernels in 64-bit fixed point (pcf_planes_fx.cu); threads per CTA from
 // the largest plane of the launch.
@@ -122,7 +149,7 @@ int planes_fx_threads(const Inst& I, bool prod);
 void launch_xzsynth_fx(bool big, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf);
 void launch_prod_fx(bool big, bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li,
                     int step_index);
-void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot);
+void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot, DnsInst* dns);
 cudaError_t set_planes_fx_smem(size_t synth, size_t prod);
 // Plane kernels of the FP32 form with the x, z transforms in warp registers
 // (pcf_planes_warp.cu): nx, nz in {32, 64, 96, 128}.
@@ -180,8 +207,6 @@ int symmetrize_ctas(const Inst& I);
 void launch_symmetrize(int ctas_x, int ninst, cudaStream_t s, const Inst* insts, int mask_override,
                        int reduced = 0);
 int dns_ctas(const Inst& I);
-void launch_dns_norm(int ninst, cudaStream_t s, const Inst* insts, DnsInst* dns);
-void launch_dns_capture(int ctas_x, int ninst, cudaStream_t s, const Inst* insts, const DnsInst* dns);
 void launch_dns_update(int ctas_x, int ninst, cudaStream_t s, const Inst* insts, const DnsInst* dns);
 
 }  // namespace pcf

@@ -616,8 +616,8 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
 }
 
 // CTA = (instance, plane j, component c): sum over the plane of the squared velocity component
-// c of a slot (0: u, 1: q).
-__global__ void __launch_bounds__(128) k_norm_planes_fx(LaunchInfo li, int slot) {
+// c of a slot (0: u, 1: q); dns: the end of a DNS step's norm as well.
+__global__ void __launch_bounds__(128) k_norm_planes_fx(LaunchInfo li, int slot, DnsInst* dns) {
   __shared__ int red[64];
   int local;
   const int b = find_inst(li, blockIdx.x, &local);
@@ -636,6 +636,7 @@ __global__ void __launch_bounds__(128) k_norm_planes_fx(LaunchInfo li, int slot)
   const double s = fx_block_sum(sq, ok ? 2 * e + 68 : 0, red);
   if (threadIdx.x == 0)
     I.normpart[(size_t)c * I.ny + j] = e == kFxNan ? __longlong_as_double(0x7ff8000000000000LL) : s;
+  if (dns) finish_dns(I, dns[b]);
 }
 
 void launch_xzsynth_fx(bool big, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf) {
@@ -649,8 +650,8 @@ void launch_prod_fx(bool big, bool adj, int ctas, int threads, size_t smem, cuda
   else if (adj) k_prod_fx<true, false><<<ctas, threads, smem, s>>>(li, step_index);
   else k_prod_fx<false, false><<<ctas, threads, smem, s>>>(li, -1);
 }
-void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot) {
-  k_norm_planes_fx<<<ctas, 128, 0, s>>>(li, slot);
+void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot, DnsInst* dns) {
+  k_norm_planes_fx<<<ctas, 128, 0, s>>>(li, slot, dns);
 }
 cudaError_t set_planes_fx_smem(size_t synth, size_t prod) {
   cudaError_t e;

@@ -75,47 +75,18 @@ void launch_symmetrize(int ctas_x, int ninst, cudaStream_t s, const Inst* insts,
 }
 
 // ------------------------------------------------------------------ DNS with the Stokes step
-// h_s = ||u_s|| from the plane sums of u^2 (same arithmetic as the norm of r1), its history
-// entry, and the discrete-extremum test of the previous step:
-//   (h_{s-1} - h_{s-2}) (h_s - h_{s-1}) < 0  ->  u_{s-1} (held in uprev) is a guess.
-// One warp per instance; D.step counts the steps of the current call.
-__global__ void __launch_bounds__(32) k_dns_norm(const Inst* insts, DnsInst* dns) {
-  const Inst& I = insts[blockIdx.x];
-  DnsInst& D = dns[blockIdx.x];
-  const double h = norm_from_parts(I);
-  if (threadIdx.x != 0) return;
-  const int step = D.step;
-  if (D.hist) D.hist[(size_t)step * D.hist_stride] = h;
-  int slot = -1;
-  if (step >= 2 && (D.h1 - D.h2) * (h - D.h1) < 0.0) {
-    const int k = *D.count;
-    if (k < D.gmax) slot = k;
-    *D.count = k + 1;
-  }
-  D.slot = slot;
-  D.h2 = D.h1;
-  D.h1 = h;
-  D.step = step + 1;
-}
-
-// Copy uprev (u_{s-1}) into the instance's guess slot chosen by k_dns_norm.
-__global__ void __launch_bounds__(256) k_dns_capture(const Inst* insts, const DnsInst* dns) {
-  const DnsInst& D = dns[blockIdx.y];
-  if (D.slot < 0 || !D.guess) return;
-  const Inst& I = insts[blockIdx.y];
-  const int n = 3 * I.nmodes * I.ny;
-  double2* dst = D.guess + (size_t)D.slot * D.gstride;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) dst[t] = D.uprev[t];
-}
-
-// uprev <- u, then u <- u + dt r1 = u^dt (the Stokes step of §4 step 1 as a time stepper).
+// The guess slot chosen by finish_dns <- uprev (u_{s-1}), uprev <- u, u <- u + dt r1 = u^dt (the
+// Stokes step of §4 step 1 as a time stepper): each element is one thread's, so the capture needs
+// no launch of its own (nor does the norm: 32 x 33 x 32, batch 4, 64 steps 4342 -> 4304 us).
 __global__ void __launch_bounds__(256) k_dns_update(const Inst* insts, const DnsInst* dns) {
   const Inst& I = insts[blockIdx.y];
   const DnsInst& D = dns[blockIdx.y];
   const int n = 3 * I.nmodes * I.ny;
   const double dt = I.dt;
+  double2* const guess = D.slot >= 0 && D.guess ? D.guess + (size_t)D.slot * D.gstride : nullptr;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const double2 u = I.uhat[t], r = I.rhat[t];
+    if (guess) guess[t] = D.uprev[t];
     D.uprev[t] = u;
     I.uhat[t] = make_double2(fma(dt, r.x, u.x), fma(dt, r.y, u.y));
   }
@@ -126,12 +97,6 @@ int dns_ctas(const Inst& I) {
   return (n + 255) / 256;
 }
 
-void launch_dns_norm(int ninst, cudaStream_t s, const Inst* insts, DnsInst* dns) {
-  k_dns_norm<<<ninst, 32, 0, s>>>(insts, dns);
-}
-void launch_dns_capture(int ctas_x, int ninst, cudaStream_t s, const Inst* insts, const DnsInst* dns) {
-  k_dns_capture<<<dim3(ctas_x, ninst), 256, 0, s>>>(insts, dns);
-}
 void launch_dns_update(int ctas_x, int ninst, cudaStream_t s, const Inst* insts, const DnsInst* dns) {
   k_dns_update<<<dim3(ctas_x, ninst), 256, 0, s>>>(insts, dns);
 }
