@@ -26,6 +26,8 @@
 // shared-memory load).  What bounds the kernels at small grids is latency (a handful of
 // phases between barriers), at large ones the multiply-adds and, in the solve of a single
 // instance, the operators streamed from HBM (16 bytes per two entries).
+// Measured (us per launch, FP64 -> now): 32 x 33 x 32, batch 8: analysis 20 -> 12, solves 29 / 30 ->
+// 20 / 20, synthesis 28 -> 20; 128 x 97 x 128: 199 -> 68, 289 / 327 (sweeps) -> 139 / 139, 310 -> 121.
 #include <algorithm>
 
 #include "pcf_fx.cuh"
@@ -334,6 +336,10 @@ __device__ __forceinline__ void put_part(double2* d, int part, double x, double 
 }
 
 // ---------------------------------------------------------------- Stokes solve
+// -x when neg, on the integer pipe
+__device__ __forceinline__ double flip(double x, bool neg) {
+  return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
+}
 // One mode, nI instances (columns).  coef(i, c, n, part): Chebyshev coefficient of the products (0
 // for MODE_SOLVE).  C3, R3: [3][ny][nI] arrays; sm_i: 16 nI ints.  done(i, c, n, part, new value) receives
 // r1 (PHI), the updated state (PSI_UPDATE) or f.
@@ -369,10 +375,10 @@ __device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI,
       g = S(2, part);
       h = 0.0;
     } else {
-      const double u = S(0, 1 - part), w = S(2, 1 - part), sg = part ? 1.0 : -1.0;
+      const double u = S(0, 1 - part), w = S(2, 1 - part), kxg = flip(kx, !part), kzg = flip(kz, !part);
       a = S(1, part);
-      g = fma(sg * kx, u, sg * kz * w);
-      h = fma(sg * kz, u, -sg * kx * w);
+      g = fma(kxg, u, kzg * w);
+      h = fma(kzg, u, -kxg * w);
     }
     double* o = reinterpret_cast<double*>(C3 + n * nI + i) + part;
     o[0] = a;
@@ -458,45 +464,54 @@ __device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI,
     deriv_chains(reinterpret_cast<fx*>(C3), C, N, nullptr);
     __syncthreads();
   }
-  // u = -i (kx xi + kz eta)/k^2, w = -i (kz xi - kx eta)/k^2, and the finite-difference quotient
-  const double inv_nu = I0.inv_nu, ik = I0.ik2nu[m], kxs = kx * ik, kzs = kz * ik;
+  // u = -i (kx xi + kz eta)/k^2, w = -i (kz xi - kx eta)/k^2, and the finite-difference quotient.
+  // The subtraction goes into the products' chain, d = (w - u) or (r - w) by two fused
+  // multiply-adds from the far end: 15 of the 77-clock FP64 instructions per value of three
+  // components instead of 22 (first half-step) and 25, and one rounding of u+ less before the
+  // cancellation (128 x 97 x 128: 148 and 150 -> 139 us; 32 x 33 x 32, batch 8: 20.5 and 22 -> 20).
+  const bool psi = op == MODE_PSI_UPDATE || op == MODE_PSI_GRAD;
+  const double ik = I0.ik2nu[m], kxs = kx * ik, kzs = kz * ik, inu = flip(I0.inv_nu, psi);
   for (int t = threadIdx.x; t < 2 * nI * ny; t += blockDim.x) {
     const int i = CN.row(t >> 1), part = t & 1, n = (t >> 1) - i * ny;
     if (!live[i]) continue;
     const Inst& I = insts[first + i];
     const double* R = reinterpret_cast<const double*>(R3 + n * nI + i);
-    double w[3];
+    // component c: ac x + bc y
+    double x0, x2, y, a0, a2, b0, b2;
     if (mean) {
-      w[0] = R[part] * inv_nu;
-      w[1] = 0.0;
-      w[2] = R[4 * AS + part] * inv_nu;
+      x0 = R[part];
+      x2 = R[4 * AS + part];
+      a0 = a2 = inu;
+      b0 = b2 = y = 0.0;
     } else {
       // the other part of dv/dy and of eta
       const fx bx = n < N ? reinterpret_cast<const fx*>(C3 + (n + 1) * nI + i)[1 - part] : 0;
-      const double b = fx_out(bx, dot_exp(ct[2 * i + 1 - part], -2)), e = R[4 * AS + 1 - part];
-      const double sg = part ? -1.0 : 1.0;
-      w[0] = fma(sg * kzs, e, -sg * kxs * b);
-      w[1] = R[part] * inv_nu;
-      w[2] = fma(-sg * kxs, e, -sg * kzs * b);
+      y = fx_out(bx, dot_exp(ct[2 * i + 1 - part], -2));
+      x0 = x2 = R[4 * AS + 1 - part];
+      const bool sg = (part != 0) != psi;
+      a0 = flip(kzs, sg);
+      b2 = -a0;
+      b0 = a2 = flip(kxs, !sg);
     }
+    const double x1 = mean ? 0.0 : R[part];
+    const size_t gi = 2 * ((size_t)m * ny + n) + part, gc = 2 * (size_t)nm * ny;
+    const double* u = reinterpret_cast<const double*>(I.uhat) + gi;
+    double* rh = reinterpret_cast<double*>(I.rhat) + gi;
+    double d[3], up[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const size_t gi = 2 * (((size_t)c * nm + m) * ny + n) + part;
-      double o = w[c];
-      if (op == MODE_PHI) {
-        o = (o - reinterpret_cast<const double*>(I.uhat)[gi]) * ist;
-        reinterpret_cast<double*>(I.rhat)[gi] = o;
-      } else if (op == MODE_SOLVE) {
-        reinterpret_cast<double*>(I.fhat)[gi] = o;
-      } else {
-        o = (reinterpret_cast<const double*>(I.rhat)[gi] - o) * ist;
-        if (op == MODE_PSI_UPDATE) {
-          o = fma(I.dtau, o, reinterpret_cast<const double*>(I.uhat)[gi]);
-          reinterpret_cast<double*>(I.uhat)[gi] = o;
-        } else {
-          reinterpret_cast<double*>(I.fhat)[gi] = o;
-        }
-      }
+      up[c] = op == MODE_PHI || op == MODE_PSI_UPDATE ? u[c * gc] : 0.0;
+      d[c] = op == MODE_PHI ? -up[c] : psi ? rh[c * gc] : 0.0;
+    }
+    d[0] = fma(a0, x0, fma(b0, y, d[0]));
+    d[1] = fma(inu, x1, d[1]);
+    d[2] = fma(a2, x2, fma(b2, y, d[2]));
+    const double step = op == MODE_PSI_UPDATE ? I.dtau * ist : ist;
+    double* out = op == MODE_PHI ? rh : reinterpret_cast<double*>(op == MODE_PSI_UPDATE ? I.uhat : I.fhat) + gi;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double o = op == MODE_PSI_UPDATE ? fma(step, d[c], up[c]) : op == MODE_SOLVE ? d[c] : d[c] * step;
+      out[c * gc] = o;
       done(i, c, n, part, o);
     }
   }
