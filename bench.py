@@ -35,8 +35,20 @@ WORKLOAD = "PCF Re=400 box 2pi/1.14 x 2 x 2pi/2.5, 32x33x32, 8 streak/roll guess
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the kernel classes,
 # read from one ncu capture of the current kernels on this workload; reset an entry to None
 # when that kernel changes.
-# Capture of the tangent-twiddle plane kernels (--mode-tile 4, one step's launches).
-TRAFFIC_BYTES = {"xzsynth_u": 4.096768e6, "xzsynth_q": 4.096768e6, "prod_M": 23.83616e6, "prod_N": 47.641088e6}
+# Capture of the fixed-point plane kernels (one step at this grid and batch).
+TRAFFIC_BYTES = {"xzsynth_u": 4.098e6, "xzsynth_q": 4.102e6, "prod_M": 23.89e6, "prod_N": 47.75e6}
+
+# A 64-bit fixed-point multiply-add is three 32 x 32 -> 64 bit integer multiply-adds, which run
+# at 24.4 lanes per clock per SM on GB300 (measured with an instruction loop).
+FIXED_POINT_MAC_PER_CLK_SM = 24.4 / 3.0
+
+
+def fixed_point_peak_tflops(nsm, sm_max_mhz):
+    """Multiply-adds of the FP64 forms' fixed-point arithmetic as TFLOP/s (2 per multiply-add)."""
+    return 2.0 * FIXED_POINT_MAC_PER_CLK_SM * nsm * sm_max_mhz * 1e6 / 1e12
+
+
+FX_PEAK_SOURCE = "64-bit fixed-point multiply-adds: 3 integer multiply-adds each at 24.4 lanes/clk/SM (measured)"
 
 
 def _peaks():
@@ -338,8 +350,8 @@ def _mixed_roofline(s4, u, flush, grid, args, nk=5):
 
 
 def _form_roofline(s, u, flush, grids, args, nk=5):
-    """Per-kernel CUDA-event times of a form's step (eager launches) and the FP64 roofline of
-    its dominant kernel: algorithmic flops of every grid's instances per launch (kernel_flops)
+    """Per-kernel CUDA-event times of a form's step (eager launches) and the fixed-point roofline
+    of its dominant kernel: algorithmic flops of every grid's instances per launch (kernel_flops)
     over the kernel's average launch time."""
     import torch
     s.set_kernel_timing(True)
@@ -356,11 +368,11 @@ def _form_roofline(s, u, flush, grids, args, nk=5):
             flops[k] = flops.get(k, 0.0) + v
     dom = max((k for k in kt if kt[k][1]), key=lambda k: kt[k][0])
     dom_ms = kt[dom][0] / kt[dom][1]
-    peak_tf = args.fp64_peak_gflops / 1e3
+    peak_tf = args.fx_peak_tflops
     achieved = flops.get(dom, 0.0) / (dom_ms * 1e-3) / 1e12
     return {"bound": "alu", "kernel": dom, "achieved": round(achieved, 4), "peak": round(peak_tf, 4),
             "unit": "TFLOP/s", "frac": round(achieved / peak_tf, 4), "traffic": None,
-            "peak_source": "measured FP64 DFMA throughput (k_fp64_probe) on this GPU",
+            "peak_source": FX_PEAK_SOURCE,
             "kernel_ms_per_launch": round(dom_ms, 5),
             "per_kernel_ms_per_step": {k: round(v[0] / nk, 5) for k, v in kt.items() if v[1]}}
 
@@ -570,7 +582,7 @@ def run_forms(pcf, gi, flush, stream, dev, args):
     ss.close()
     if not args.no_robust:
         out["robustness"] = run_robustness(pcf, gi, dev, args)
-    # float-float form (x-z transforms and products in pairs of FP32) vs the FP64 path
+    # float-float form (runs the FP64 form's fixed-point kernels) vs the FP64 path
     u8 = gi.batch(gi.streak_roll, range(BATCH), *GRID)
     res = {}
     for name, prec in (("fp64", pcf.FP64), ("ff", pcf.FLOAT_FLOAT)):
@@ -583,8 +595,8 @@ def run_forms(pcf, gi, flush, stream, dev, args):
         sf.close()
     rf, r64 = res["ff"][1], res["fp64"][1]
     out["float_float"] = {
-        "config": "8 streak/roll guesses, 32x33x32, Re 400; x-z FFTs and products in float-float (pairs of FP32, "
-                  "~48 bits) on the FP32 pipe, Chebyshev transforms / solves / norms / state FP64",
+        "config": "8 streak/roll guesses, 32x33x32, Re 400; the float-float form accepts ~48-bit x-z FFTs "
+                  "and products; it runs the FP64 form's 64-bit fixed-point kernels",
         "gradient_evals_per_s": BATCH * 1e3 / res["ff"][0], "ms_per_step": res["ff"][0],
         "fp64_ms_per_step": res["fp64"][0], "speedup_vs_fp64": res["fp64"][0] / res["ff"][0],
         "r1_rel_error_vs_fp64_path_per_component": {
@@ -832,20 +844,17 @@ def run_ours(args):
     dom_ms = kt[dom][0] / max(1, kt[dom][1])
     fp64 = pcf.probe_fp64_peak()
     achieved = flops[dom] / (dom_ms * 1e-3) / 1e12
-    peak_tf = fp64 / 1e3
+    nsm = torch.cuda.get_device_properties(dev).multi_processor_count
+    peak_tf = fixed_point_peak_tflops(nsm, ck.get("sm_max_mhz") or 2070)
+    args.fx_peak_tflops = peak_tf
+    # the transforms and solves run in fixed point on the integer pipe, so the FP64 pipe's measured
+    # rate is context only
     roof = {"bound": "alu", "achieved": round(achieved, 4), "peak": round(peak_tf, 4), "unit": "TFLOP/s",
             "frac": round(achieved / peak_tf, 4), "traffic": TRAFFIC_BYTES.get(dom), "kernel": dom,
-            "peak_source": "measured FP64 DFMA throughput (k_fp64_probe) on this GPU",
+            "peak_source": FX_PEAK_SOURCE, "measured_fp64_dfma_tflops": round(fp64 / 1e3, 4),
             "kernel_share": round(kt[dom][0] / total_ms, 4), "mode_tile": s.mode_tile(), "split_config": s.split_config(),
             "kernel_ms_per_launch": round(dom_ms, 5),
             "per_kernel_ms_per_step": {k: round(v[0] / nk, 5) for k, v in kt.items()}}
-    # the same against the FP64 pipe's nominal rate (2 DFMA per clock per SM at the maximum SM
-    # clock); a DFMA-only loop (k_fp64_probe) sustains about 0.84 of it on GB300
-    nsm = torch.cuda.get_device_properties(dev).multi_processor_count
-    if ck.get("sm_max_mhz"):
-        nominal = nsm * 4.0 * ck["sm_max_mhz"] * 1e6 / 1e12
-        roof.update(nominal_fp64_peak=round(nominal, 4), frac_vs_nominal=round(achieved / nominal, 4),
-                    probe_vs_nominal=round(peak_tf / nominal, 4))
 
     if rank == 0:
         line = {"metric": "gradient evals/s", "value": value, "unit": "gradient evals/s", "n_gpus": ws,

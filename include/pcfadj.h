@@ -55,12 +55,16 @@ typedef enum {
 } pcf_status;
 
 typedef enum {
-  PCF_FP64 = 0,         /* the plain method: FP64 throughout */
+  PCF_FP64 = 0,         /* the plain method: FP64 state, tables and results.  The transforms,
+                           products and Stokes solves run in 64-bit fixed point with block
+                           exponents (units of 2^-60 of a plane's and 2^-55 of a column's sum of
+                           magnitudes), which is no coarser than FP64 arithmetic there */
   PCF_MIXED = 1,        /* FP32 x-z transforms and products, split-BF16 tensor-core Chebyshev
                            transforms, FP64 Stokes solves, norms and state; ny <= 113
                            (PCF_ENOTSUP above) */
-  PCF_FLOAT_FLOAT = 2   /* x-z transforms and products in float-float arithmetic (pairs of
-                           FP32, ~48 significant bits) on the FP32 pipe; everything else FP64 */
+  PCF_FLOAT_FLOAT = 2   /* accepts x-z transforms and products of ~48 significant bits; since the
+                           fixed-point kernels are both more accurate and faster than pairs of
+                           FP32, it runs the same kernels as PCF_FP64 */
 } pcf_precision;
 
 /* Problem description; all instances of a context share one grid.
@@ -74,20 +78,18 @@ typedef struct pcf_params {
   double Lx, Lz, Re;
   double dt, dtau_hat;
   int precision;        /* pcf_precision; PCF_FP64 for the plain method */
-  int modes_per_block;  /* tile of the per-mode kernels (Fourier modes per CTA of the single
-                           per-mode kernel; instances per group of the split kernels);
-                           0 = autotuned */
-  int solve_kind;       /* 0: dense per-mode operators when ny <= 129, else banded sweeps; the
-                           autotuner picks the kernel organisation (FP64 form, ny <= 97: split
-                           or fused kernels over instance groups; mixed form: dense against
-                           sweeps), see pcf_solve_variant.  1: banded sweeps.  2: dense
-                           operators inside the single per-mode kernel.  3: FP64 split
-                           analysis / solve / synthesis kernels with the dense solve.  4: FP64
-                           fused per-mode half-step kernel.  2, 3 and 4 give bit-identical
-                           results.  5: FP64 split analysis and synthesis kernels with the
-                           Stokes solve by banded sweeps, one thread per chain (group g, mode,
-                           real or imaginary part); with 0 the autotuner times it against the
-                           dense solve. */
+  int modes_per_block;  /* FP64 forms: instances per group of the dense solve; mixed form and
+                           solve_kind 1: Fourier modes per CTA of the per-mode kernel; 0 = chosen
+                           by the library (mixed form: timed at creation) */
+  int solve_kind;       /* 0: chosen by the library, see pcf_solve_variant (FP64 forms: dense
+                           operators in separate kernels, or in the fused half-step kernel where
+                           the launch is small; mixed form: dense operators against sweeps, timed
+                           at creation).  1: banded sweeps in the per-mode kernel.  2: fused
+                           per-mode half-step kernel (analysis, dense solve, synthesis).  3:
+                           separate analysis / solve / synthesis kernels.  4: as 2, with J in a
+                           kernel of its own.  2, 3 and 4 give bit-identical results.  5: the
+                           separate kernels with the Stokes solve by banded sweeps, one thread
+                           per chain (group g, mode, real or imaginary part). */
   int base_flow;        /* pcf_base_flow: the laminar base flow u_b = (U(y), V, 0) */
   int symmetry;         /* pcf_symmetry mask enforced along the descent and the DNS (0: none).
                            s1 requires PCF_COUETTE (it maps the Poiseuille profile to its
@@ -95,7 +97,7 @@ typedef struct pcf_params {
   int plane_kernel;     /* x-z plane kernels of the mixed form (FP32): 0 = transforms in warp
                            registers when every instance has nx, nz in {32, 64, 96, 128}, else
                            the shared-memory Stockham kernels; 1 = always the Stockham kernels.
-                           The FP64 and float-float forms always use the Stockham kernels.
+                           Ignored by the FP64 and float-float forms.
                            pcf_plane_variant reports the choice. */
   int contraction_kernel; /* Chebyshev transforms of the mixed form (split-BF16, FP32
                            accumulation): 0 = tcgen05 MMAs with the accumulator in tensor
@@ -166,7 +168,7 @@ pcf_status pcf_create(const pcf_params* params, void* stream, pcf_ctx** out);
  * step captured in one CUDA graph, with per-instance convergence masks in pcf_run).
  * Instance states are stored back to back in the order given; pcf_state_offset gives
  * each one's offset.  Tables are shared between instances on the same problem.  With
- * list[0].modes_per_block = 0 an autotuner times the mode kernel for several tiles on
+ * list[0].modes_per_block = 0 the mixed form times its mode kernel for several tiles on
  * the batch and keeps the fastest (pcf_mode_tile).  DMD entry points require every
  * instance on one problem (PCF_ENOTSUP otherwise). */
 pcf_status pcf_batch_create(const pcf_params* list, int n, void* stream, pcf_ctx** out);
@@ -175,18 +177,17 @@ pcf_status pcf_batch_create(const pcf_params* list, int n, void* stream, pcf_ctx
  * (instance = batch gives the total); -1 for an invalid instance. */
 long long pcf_state_offset(const pcf_ctx* ctx, int instance);
 
-/* Fourier modes per CTA chosen for the per-mode kernels of the descent step (by the
- * autotuner or the caller). */
+/* Instances per group of the dense solve (FP64 forms), or Fourier modes per CTA of the
+ * per-mode kernel (mixed form, solve_kind 1). */
 int pcf_mode_tile(const pcf_ctx* ctx);
 
-/* Stokes solve the descent step uses: 0 banded tau sweeps inside the per-mode kernel,
- * 1 dense per-mode operators inside the per-mode kernel, 2 dense operators in the split
- * analysis / solve / synthesis kernels over instance groups, 3 dense operators in the fused
- * per-mode half-step kernel over instance groups, 4 banded sweeps with one thread per chain
- * between the split analysis and synthesis kernels (2, 3 and 4: FP64 and float-float forms).
- * With solve_kind 0 the FP64 form times 2 against 3 and then the chosen dense solve against
- * 4, the mixed-precision form 0 against 1, at creation, and each keeps the faster.  -1 for a
- * NULL context. */
+/* Stokes solve the descent step uses: 0 banded tau sweeps inside the per-mode kernel, 1 dense
+ * per-mode operators inside one kernel per half-step (the mixed form's per-mode kernel; the
+ * FP64 forms' fused kernel), 2 dense operators between separate analysis and synthesis kernels,
+ * 3 the fused kernel with J in a kernel of its own, 4 banded sweeps with one thread per chain
+ * between the separate kernels.  With solve_kind 0 the FP64 forms take 1 where the solve has at
+ * most 228 CTAs and no reduced symmetric state, else 2; the mixed form times 0 against 1 at
+ * creation.  -1 for a NULL context. */
 int pcf_solve_variant(const pcf_ctx* ctx);
 
 /* x-z plane kernels the context launches: 0 shared-memory Stockham passes, 1 transforms in
@@ -394,22 +395,21 @@ pcf_status pcf_probe_fp64_peak(void* stream, double* gflops);
  * Kernel classes: 0 ysynth, 1 xzsynth_u, 2 prod_M, 3 mode_phi, 4 xzsynth_q,
  * 5 prod_N, 6 mode_psi, 7 yanalysis, 8 ysynth_step, 9 jnorm, 10 symmetrize, 11 dns_aux,
  * 12 cheb_synth_tc, 13 cheb_analysis_tc.
- * In the FP64 form with dense per-mode operators (ny <= 97) the per-mode work of a step
- * runs as three kernels: 7 (Chebyshev analysis + right-hand side, twice per step), 3/6
- * (Stokes solve and update of the NSE / dummy step), 8 (Chebyshev synthesis of r1 and of
- * the new u).  J, its history and the convergence mask come from the last CTA of each
- * instance in 5, except with the fused half-step kernel, where 9 computes them; without
- * dense operators 3/6 hold the whole per-mode kernel and 7, 8, 9 stay empty.  10 is the
- * projection onto the symmetric subspace, 11 the small kernels around pcf_dns; 12 and 13 are the
+ * In the FP64 forms the per-mode work of a step runs as three kernels: 7 (Chebyshev analysis,
+ * twice per step), 3/6 (Stokes solve and update of the NSE / dummy step), 8 (Chebyshev
+ * synthesis of r1 and of the new u), or as the fused kernel, counted in 3/6.  J, its history and
+ * the convergence mask come from the last CTA of each instance in 5, except with solve_kind 4,
+ * where 9 computes them.  With solve_kind 1 and in the mixed form
+ * 3/6 hold the whole per-mode kernel and 7, 8, 9 stay empty.  10 is the
+ * projection onto the symmetric subspace, 11 the kernels around pcf_dns; 12 and 13 are the
  * mixed form's tensor-core Chebyshev synthesis and analysis (its mode kernel, 3/6, then holds
  * only the Stokes solve). */
 pcf_status pcf_set_kernel_timing(pcf_ctx* ctx, int enable);
 
-/* Organisation the autotuner chose for the split per-mode kernels (FP64 and float-float
- * forms): cfg[0] instances per group of the analysis and synthesis kernels, cfg[1] and cfg[2]
- * consecutive modes per CTA of the analysis and of the synthesis, cfg[3] instances per group
- * of the Stokes solve.  Zeros where the context does not use those kernels (fused solve:
- * cfg[3] = 0).  cfg: host int[4]. */
+/* Organisation of the FP64 forms' per-mode kernels: cfg[0] instances per group of the solve,
+ * cfg[1] and cfg[2] modes per CTA of the separate analysis and synthesis kernels, cfg[3]
+ * instances per group of the separate dense solve.  Zeros where the context does not use those
+ * kernels.  cfg: host int[4]. */
 pcf_status pcf_split_config(const pcf_ctx* ctx, int* cfg);
 
 /* Kernel launches of one pcf_descent_step call of nsteps steps (the entry synthesis, and

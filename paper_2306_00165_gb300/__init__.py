@@ -366,14 +366,15 @@ class Solver:
         return int(self.lib.pcf_symmetric_modes(self._h))
 
     def solve_variant(self):
-        """0 banded sweeps, 1 dense operators (single per-mode kernel), 2 dense split kernels."""
+        """0 banded sweeps and 1 dense operators in one kernel per half-step, 2 dense operators and 4 banded
+        sweeps between separate transforms, 3 as 1 with a separate J kernel."""
         return int(self.lib.pcf_solve_variant(self._h))
 
     def launches_per_step(self):
         return int(self.lib.pcf_launches_per_step(self._h))
 
     def split_config(self):
-        """Autotuned organisation of the split per-mode kernels: dict of group sizes and mode tiles."""
+        """Organisation of the FP64 forms' per-mode kernels: dict of group sizes and mode tiles."""
         cfg = (ctypes.c_int * 4)()
         _check(self.lib.pcf_split_config(self._h, cfg))
         return {"group": cfg[0], "analysis_mode_tile": cfg[1], "synthesis_mode_tile": cfg[2], "solve_group": cfg[3]}

@@ -30,7 +30,6 @@ struct pcf_ctx {
   bool suction = false;  // some instance has a base flow with suction (PCF_ASBL)
   int mode_thr = 128;    // threads per CTA of the single per-mode kernel
   bool mixed = false;    // mixed-precision form (FP32 planes, split-BF16 Chebyshev, FP64 solves)
-  int plane_kind = 0;    // 0 FP64 form, 1 mixed form, 2 float-float form
   // fixed-point plane kernels: threads per CTA; some side above 64
   int thr_synth = 64, thr_prod = 64;
   bool plane_big = false;

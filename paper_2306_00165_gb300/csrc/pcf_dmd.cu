@@ -455,7 +455,10 @@ pcf_ctx* eval_ctx(pcf_ctx* c, int want) {
     pcf_destroy(c->dmd_eval);
     c->dmd_eval = nullptr;
   }
-  if (!c->dmd_eval && pcf_make_child(c, nb, &c->dmd_eval) != PCF_OK) c->dmd_eval = nullptr;
+  if (!c->dmd_eval && pcf_make_child(c, nb, &c->dmd_eval) != PCF_OK) {
+    c->dmd_eval = nullptr;
+    cudaGetLastError();  // a failed allocation is answered by c itself
+  }
   return c->dmd_eval ? c->dmd_eval : c;
 }
 

@@ -1090,7 +1090,6 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
   c->state_len = 3LL * c->nm * list[0].ny;
   c->user = (cudaStream_t)stream;
   c->mixed = list[0].precision == PCF_MIXED;
-  c->plane_kind = c->mixed ? 1 : list[0].precision == PCF_FLOAT_FLOAT ? 2 : 0;
   auto fail = [&](pcf_status s) {
     pcf_destroy(c);
     return s;

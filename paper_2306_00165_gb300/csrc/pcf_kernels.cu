@@ -1,18 +1,16 @@
-// CUDA kernels (sm_103a) of one adjoint-descent step for plane Couette flow.
+// Kernels of the mixed form and of the per-mode Stokes solve (sm_103a): FP32 plane transforms and
+// products as radix-4/2/3 Stockham passes in shared memory (CTA = one y-plane of one field or
+// product component), and k_mode, the FP64 solve of a few Fourier modes per CTA by dense
+// operators or banded sweeps.
 //
 // Data flow of one descent step (paper §4, steps 1-5), per instance:
-//   k_mode(SYNTH)      uhat -> y-values of u and du/dy at the Gauss-Lobatto points
-//   k_xzsynth(slot 0)  -> 11 physical fields u, grad u on each y-plane (inverse FFT in x, z)
-//   k_prod_M           -> M(u) per plane, forward FFT in z, x, 2/3 truncation
-//   k_mode(PHI)        -> Chebyshev analysis, Stokes step (step 1), r1 (step 2), synthesis of r1
-//   k_xzsynth(slot 1)  -> 11 physical fields r1, grad r1
-//   k_prod_N           -> N(r1) per plane (+ plane sums of r1^2 for J), forward FFT
-//   k_mode(PSI_UPDATE) -> analysis, Stokes step of the dummy dynamics (step 3), f (step 4),
-//                         u += dtau f (step 5), synthesis of the new u for the next step
-// The mode kernels work on Chebyshev columns of a few Fourier modes per CTA; the plane
-// kernels on one y-plane of one field (or product component) per CTA.  All arithmetic is
-// FP64; the FP64 pipe is the bound on GB300, so the transforms are radix-4/2/3 Stockham
-// FFTs in shared memory (x, z) and parity-folded dense Chebyshev matrices (y).
+//   y-synthesis        uhat -> y-values of u and du/dy at the Gauss-Lobatto points
+//   plane synthesis    -> 11 physical fields u, grad u on each y-plane (inverse FFT in x, z)
+//   products M         -> M(u) per plane, forward FFT in z, x, 2/3 truncation
+//   k_mode(PHI)        -> Stokes step (step 1), r1 (step 2); y-synthesis and planes of r1
+//   products N         -> N(r1) per plane (+ plane sums of r1^2 for J), forward FFT
+//   k_mode(PSI_UPDATE) -> Stokes step of the dummy dynamics (step 3), f (step 4), u += dtau f (step 5)
+// Dense operators keep the FP64 pipe, which bounds k_mode, full.
 #include <map>
 #include <mutex>
 #include <utility>
