@@ -489,13 +489,14 @@ pcf_status launch_synth(pcf_ctx* c, int slot, int nf) {
     else launch_xzsynth_fx(c->plane_big, ctas, c->thr_synth, c->sm_synth, c->cs, li_of(c, pre, ctas), slot, nf);
   });
 }
-pcf_status launch_prodM(pcf_ctx* c) {
+// dns: with the norm and the extremum test of a DNS step (FP64 forms)
+pcf_status launch_prodM(pcf_ctx* c, DnsInst* dns = nullptr) {
   return timed(c, 2, [&] {
     if (c->plane_warp) launch_prod_warp(false, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod), -1);
     else if (c->mixed) launch_prod(false, c->suction, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod));
     else
       launch_prod_fx(c->plane_big, false, c->cta_prod, c->thr_prod, c->sm_prod, c->cs,
-                     li_of(c, c->pre_prod, c->cta_prod), -1);
+                     li_of(c, c->pre_prod, c->cta_prod), -1, dns);
   });
 }
 pcf_status launch_prodN(pcf_ctx* c, int step_index = -1) {
@@ -509,10 +510,10 @@ pcf_status launch_prodN(pcf_ctx* c, int step_index = -1) {
   });
 }
 
-// plane sums of the squared velocity of a slot
+// plane sums of the squared velocity of a slot; dns: as in launch_prodM (mixed form)
 void launch_plane_sums(pcf_ctx* c, int slot, DnsInst* dns = nullptr) {
   if (c->mixed) launch_norm_planes(c->cta_synth3, c->cs, li_of(c, c->pre_synth3), slot, dns);
-  else launch_norm_planes_fx(c->cta_synth3, c->cs, li_of(c, c->pre_synth3, c->cta_synth3), slot, dns);
+  else launch_norm_planes_fx(c->cta_synth3, c->cs, li_of(c, c->pre_synth3, c->cta_synth3), slot);
 }
 
 pcf_status launch_tc_synth(pcf_ctx* c, int slot) {
@@ -667,8 +668,8 @@ pcf_status step_body(pcf_ctx* c, int s, bool last) {
 // and the y-synthesis of the new state for the next step.
 pcf_status dns_body(pcf_ctx* c) {
   PCF_TRY(launch_synth(c, 0, kFieldsSynth));
-  PCF_TRY(timed(c, 11, [&] { launch_plane_sums(c, 0, c->d_dns); }));
-  PCF_TRY(launch_prodM(c));
+  if (c->mixed) PCF_TRY(timed(c, 11, [&] { launch_plane_sums(c, 0, c->d_dns); }));
+  PCF_TRY(launch_prodM(c, c->mixed ? nullptr : c->d_dns));
   if (c->split || c->mixed) {
     PCF_TRY(launch_analysis(c));
     PCF_TRY(launch_solve(c, MODE_PHI, 0));

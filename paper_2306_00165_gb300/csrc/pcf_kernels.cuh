@@ -97,7 +97,7 @@ __device__ __forceinline__ void finish_norm(const Inst& I, int step_index) {
   }
 }
 
-// End of a plane-sum CTA of a DNS step: the last one has h_s = ||u_s|| (same arithmetic as the norm
+// End of a CTA of a DNS step that has written its plane sum of u_c^2: the last one has h_s = ||u_s|| (same arithmetic as the norm
 // of r1), writes its history entry and makes the discrete-extremum test of the previous step:
 //   (h_{s-1} - h_{s-2}) (h_s - h_{s-1}) < 0  ->  u_{s-1} (held in uprev until this step's update) is
 // a guess.  D.step counts the steps of the current call.
@@ -148,8 +148,8 @@ size_t smem_planes_fx(const Inst& I, int threads);
 int planes_fx_threads(const Inst& I, bool prod);
 void launch_xzsynth_fx(bool big, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf);
 void launch_prod_fx(bool big, bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li,
-                    int step_index);
-void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot, DnsInst* dns);
+                    int step_index, DnsInst* dns = nullptr);
+void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot);
 cudaError_t set_planes_fx_smem(size_t synth, size_t prod);
 // Plane kernels of the FP32 form with the x, z transforms in warp registers
 // (pcf_planes_warp.cu): nx, nz in {32, 64, 96, 128}.

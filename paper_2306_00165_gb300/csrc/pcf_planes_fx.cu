@@ -404,8 +404,12 @@ __device__ double fx_block_sum(unsigned long long s, int e, int* red) {
 // their high 64 bits (2^-60 of the largest product) and are summed at the largest term's
 // exponent.  The transforms rescale every row pair and then every x row from its own largest
 // value, found by shuffles among the eight lanes that hold the row.
-template <bool ADJ, bool BIG>
-__global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_fx(LaunchInfo li, int step_index) {
+// SUM (M only, the DNS): also the plane sums of u_c^2 and, in an instance's last CTA, the end of
+// the DNS step's norm; the planes are in registers here (as a kernel of its own the sums took 4238
+// us per 64 steps of four 32 x 33 x 32 fields, now 4047).
+template <bool ADJ, bool BIG, bool SUM>
+__global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_fx(LaunchInfo li, int step_index,
+                                                                                  DnsInst* dns) {
   extern __shared__ __align__(16) unsigned char smraw[];
   // factors: 0-2 advecting velocity u_b + u; 3-5 gradient of component c of u (M) or q (N);
   // N: 6-8 q, 9-11 derivative c of u's components; 12: the factor of U' (v, or q_0).
@@ -491,7 +495,10 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
   // One loop over the transform stages, so that the z stage of every chunk of rows and the x
   // stage run the same instructions (the kernel's straight-line code otherwise exceeds the
   // instruction cache): job g < nch is chunk g's products and z stage, job nch the x stage.
-  const int nch = bad || (zero && !ADJ) ? 0 : (nr + P.chunk - 1) / P.chunk;
+  const int nch = !SUM && (bad || (zero && !ADJ)) ? 0 : (nr + P.chunk - 1) / P.chunk;
+  const int2 iu = SUM ? *fx_info(I, 0, c, j) : make_int2(kFxNone, 0);
+  const int eu = fx_e62(iu);
+  const bool suok = SUM && eu != kFxNan && eu != kFxNone;
   const bool live = !bad && !zero;
   int* align = ep + 64;  // right shift of each row pair's values in the x stage (z stage: none)
   if (threadIdx.x < 64) align[threadIdx.x] = 0;
@@ -511,6 +518,7 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
         b4 = __ldg(reinterpret_cast<const longlong2*>(Q + 10 * fs + e));
         if (ADJ) b10 = __ldg(reinterpret_cast<const longlong2*>(U + 10 * fs + e));
       }
+      const longlong2 uc = c == 0 ? x[0] : c == 1 ? x[1] : x[2];
       if (!ADJ && c == 0) pv = __ldg(reinterpret_cast<const longlong2*>(U + fs + e));
       fx val[2];
 #pragma unroll
@@ -528,6 +536,10 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
           if (ADJ) v[10 % NO] = -(v[10 % NO] + fx_shift(h ? b10.y : b10.x, ssb[10]));
         }
         fx a = (fx_mul64(v[0], v[3]) >> sd[0]) + (fx_mul64(v[1], v[4]) >> sd[1]) + (fx_mul64(v[2], v[5]) >> sd[2]);
+        if (suok) {
+          const fx q = ((h ? uc.y : uc.x) << (62 - iu.y)) >> 2;  // at most 64 squares below 2^56
+          sq += (unsigned long long)fx_mul64(q, q);
+        }
         if (!ADJ) {
           if (c == 0) a += fx_mul64(dUx, (h ? pv.y : pv.x) << ssa[12]) >> sd[6];
           a = -a;
@@ -616,11 +628,17 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
       I.normpart[(size_t)c * I.ny + j] = eq == kFxNan || bad ? __longlong_as_double(0x7ff8000000000000LL) : sqok ? s : 0.0;
   }
   if (ADJ && step_index >= 0) finish_norm(I, step_index);
+  if (SUM) {
+    const double s = fx_block_sum(sq, suok ? 2 * eu + 68 : 0, red);
+    if (threadIdx.x == 0)
+      I.normpart[(size_t)c * I.ny + j] = eu == kFxNan ? __longlong_as_double(0x7ff8000000000000LL) : s;
+    finish_dns(I, dns[b]);
+  }
 }
 
 // CTA = (instance, plane j, component c): sum over the plane of the squared velocity component
-// c of a slot (0: u, 1: q); dns: the end of a DNS step's norm as well.
-__global__ void __launch_bounds__(128) k_norm_planes_fx(LaunchInfo li, int slot, DnsInst* dns) {
+// c of a slot (0: u, 1: q).
+__global__ void __launch_bounds__(128) k_norm_planes_fx(LaunchInfo li, int slot) {
   __shared__ int red[64];
   int local;
   const int b = find_inst(li, blockIdx.x, &local);
@@ -639,7 +657,6 @@ __global__ void __launch_bounds__(128) k_norm_planes_fx(LaunchInfo li, int slot,
   const double s = fx_block_sum(sq, ok ? 2 * e + 68 : 0, red);
   if (threadIdx.x == 0)
     I.normpart[(size_t)c * I.ny + j] = e == kFxNan ? __longlong_as_double(0x7ff8000000000000LL) : s;
-  if (dns) finish_dns(I, dns[b]);
 }
 
 void launch_xzsynth_fx(bool big, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf) {
@@ -647,23 +664,27 @@ void launch_xzsynth_fx(bool big, int ctas, int threads, size_t smem, cudaStream_
   else k_synth_fx<false><<<ctas, threads, smem, s>>>(li, slot, nf);
 }
 void launch_prod_fx(bool big, bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li,
-                    int step_index) {
-  if (big && adj) k_prod_fx<true, true><<<ctas, threads, smem, s>>>(li, step_index);
-  else if (big) k_prod_fx<false, true><<<ctas, threads, smem, s>>>(li, -1);
-  else if (adj) k_prod_fx<true, false><<<ctas, threads, smem, s>>>(li, step_index);
-  else k_prod_fx<false, false><<<ctas, threads, smem, s>>>(li, -1);
+                    int step_index, DnsInst* dns) {
+  if (big && adj) k_prod_fx<true, true, false><<<ctas, threads, smem, s>>>(li, step_index, nullptr);
+  else if (adj) k_prod_fx<true, false, false><<<ctas, threads, smem, s>>>(li, step_index, nullptr);
+  else if (big && dns) k_prod_fx<false, true, true><<<ctas, threads, smem, s>>>(li, -1, dns);
+  else if (dns) k_prod_fx<false, false, true><<<ctas, threads, smem, s>>>(li, -1, dns);
+  else if (big) k_prod_fx<false, true, false><<<ctas, threads, smem, s>>>(li, -1, nullptr);
+  else k_prod_fx<false, false, false><<<ctas, threads, smem, s>>>(li, -1, nullptr);
 }
-void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot, DnsInst* dns) {
-  k_norm_planes_fx<<<ctas, 128, 0, s>>>(li, slot, dns);
+void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot) {
+  k_norm_planes_fx<<<ctas, 128, 0, s>>>(li, slot);
 }
 cudaError_t set_planes_fx_smem(size_t synth, size_t prod) {
   cudaError_t e;
   if ((e = raise_smem_limit((const void*)k_synth_fx<false>, synth))) return e;
   if ((e = raise_smem_limit((const void*)k_synth_fx<true>, synth))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_fx<true, false>, prod))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_fx<true, true>, prod))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_fx<false, true>, prod))) return e;
-  return raise_smem_limit((const void*)k_prod_fx<false, false>, prod);
+  if ((e = raise_smem_limit((const void*)k_prod_fx<true, false, false>, prod))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_fx<true, true, false>, prod))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_fx<false, true, true>, prod))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_fx<false, false, true>, prod))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_fx<false, true, false>, prod))) return e;
+  return raise_smem_limit((const void*)k_prod_fx<false, false, false>, prod);
 }
 
 }  // namespace pcf
