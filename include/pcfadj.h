@@ -31,8 +31,8 @@
  * that returns anything but PCF_OK has enqueued no partial update of its outputs
  * unless noted; nothing aborts the process.
  *
- * Grids: nx, nz in {16, 32, 48, 64, 96, 128} (products of 2, 3, 4), ny odd with
- * 9 <= ny <= 129; batch >= 1.
+ * Grids: nx, nz even products of 2 and 3 from 16 to 128 (16, 18, 24, 32, 36, 48, 54, 64, 72, 96,
+ * 108, 128), ny odd with 9 <= ny <= 129; batch >= 1.
  */
 #ifndef PCFADJ_H
 #define PCFADJ_H

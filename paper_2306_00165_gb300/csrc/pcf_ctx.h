@@ -30,9 +30,8 @@ struct pcf_ctx {
   bool suction = false;  // some instance has a base flow with suction (PCF_ASBL)
   int mode_thr = 128;    // threads per CTA of the single per-mode kernel
   bool mixed = false;    // mixed-precision form (FP32 planes, split-BF16 Chebyshev, FP64 solves)
-  // fixed-point plane kernels: threads per CTA; some side above 64
-  int thr_synth = 64, thr_prod = 64;
-  bool plane_big = false;
+  // fixed-point plane kernels: threads per CTA, variant (planes_fx_kind)
+  int thr_synth = 64, thr_prod = 64, plane_kind = 0;
   bool plane_warp = false;  // FP32 plane kernels with the transforms in warp registers
   bool tc05 = false;        // Chebyshev contractions of the mixed form on tcgen05 (else mma.sync)
   // descent steps in the symmetric subspace run the per-mode kernels on the modes m >= 0 only

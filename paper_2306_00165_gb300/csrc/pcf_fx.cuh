@@ -121,6 +121,12 @@ constexpr int kS8h = 759250125, kS8l = -25716447;        // sqrt(1/2)
 constexpr int kS3h = 929887697, kS3l = -1332128537;      // sin(pi/3)
 constexpr int kC16h = 992008094, kC16l = 1696238673;     // cos(pi/8)
 constexpr int kS16h = 410903207, kS16l = -1364630830;    // sin(pi/8)
+constexpr int kC91h = 822533958, kC91l = -1633652124;    // cos(2 pi/9)
+constexpr int kS91h = 690187940, kS91l = 2016164183;     // sin(2 pi/9)
+constexpr int kC92h = 186453311, kC92l = 96060625;       // cos(4 pi/9)
+constexpr int kS92h = 1057429273, kS92l = 37236404;      // sin(4 pi/9)
+constexpr int kC94h = -1008987269, kC94l = 1537591498;   // cos(8 pi/9)
+constexpr int kS94h = 367241333, kS94l = -1978927779;    // sin(8 pi/9)
 
 // v exp(+-i pi/4) and v exp(+-3 i pi/4) (+ for the inverse transform)
 template <bool INV>
@@ -134,7 +140,7 @@ PCF_HD fxc fx_w83(fxc v) {
   return fxc{fx_mulc(a, kS8h, kS8l), fx_mulc(b, kS8h, kS8l)};
 }
 
-// dft<R, INV>(v): v[k] <- sum_n v[n] exp(+-2 pi i n k/R), natural order, for R = 2, 3, 4, 6, 8,
+// dft<R, INV>(v): v[k] <- sum_n v[n] exp(+-2 pi i n k/R), natural order, for R = 2, 3, 4, 6, 8, 9,
 // 12, 16.  6 and 12 use the prime-factor index maps (no inner twiddles).
 template <int R, bool INV>
 struct FxDft;
@@ -205,6 +211,33 @@ struct FxDft<8, INV> {
   }
 };
 template <bool INV>
+struct FxDft<9, INV> {
+  static PCF_HD void run(fxc* v) {
+    // 3 x 3: n = 3 n1 + n2, twiddles exp(+-2 pi i n2 k1/9), k = k1 + 3 k2
+    const int sg = INV ? 1 : -1;
+    const fxtw w1{kC91h, kC91l, sg * kS91h, sg * kS91l}, w2{kC92h, kC92l, sg * kS92h, sg * kS92l};
+    const fxtw w4{kC94h, kC94l, sg * kS94h, sg * kS94l};
+    fxc q[3][3];  // [n2][k1]
+#pragma unroll
+    for (int n2 = 0; n2 < 3; ++n2) {
+#pragma unroll
+      for (int n1 = 0; n1 < 3; ++n1) q[n2][n1] = v[3 * n1 + n2];
+      FxDft<3, INV>::run(q[n2]);
+    }
+    q[1][1] = fx_cmul(q[1][1], w1);
+    q[1][2] = fx_cmul(q[1][2], w2);
+    q[2][1] = fx_cmul(q[2][1], w2);
+    q[2][2] = fx_cmul(q[2][2], w4);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+      fxc c[3] = {q[0][k1], q[1][k1], q[2][k1]};
+      FxDft<3, INV>::run(c);
+#pragma unroll
+      for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = c[k2];
+    }
+  }
+};
+template <bool INV>
 struct FxDft<12, INV> {
   static PCF_HD void run(fxc* v) {
     // n = 4 n1 + 3 n2, k = 4 k1 + 9 k2 (mod 12)
@@ -256,5 +289,31 @@ struct FxDft<16, INV> {
     }
   }
 };
+
+// ------------------------------------------------------------------ transforms of a row
+// A transform of length L = R S is two passes, in place: DFTs of length R over the elements n,
+// n + S, .. (n < S), twiddles, and DFTs of length S over each block of S.  S = 8 wherever R = L/8 is
+// one of 2, 4, 6, 8, 12, 16; the other even products of 2 and 3 up to 128 have S = 3, 6 or 9.  R is
+// even: neighbouring outputs b = 2 r, 2 r + 1 of the second pass lie in the same S-strided set.
+struct FxPlan {
+  int R, S;
+};
+PCF_HD FxPlan fx_plan(int L) {
+  switch (L) {
+    case 18: return FxPlan{6, 3};
+    case 24: return FxPlan{4, 6};
+    case 36: return FxPlan{6, 6};
+    case 54: return FxPlan{6, 9};
+    case 72: return FxPlan{12, 6};
+    case 108: return FxPlan{12, 9};
+    default: return FxPlan{L >> 3, 8};
+  }
+}
+// Slot of element (block b, member e) in a row.  S = 8: the eight lanes of a shared-memory phase
+// meet eight different 16-byte bank groups in both passes without padding.
+template <int S>
+PCF_HD int fx_slot(int b, int e) {
+  return S == 8 ? b * 8 + (e ^ (b & 7)) : b * S + e;
+}
 
 }  // namespace pcf

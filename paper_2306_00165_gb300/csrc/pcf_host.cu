@@ -486,7 +486,7 @@ pcf_status launch_synth(pcf_ctx* c, int slot, int nf) {
   return timed(c, slot == 0 ? 1 : 4, [&] {
     if (c->plane_warp) launch_xzsynth_warp(ctas, c->sm_synth, c->cs, li_of(c, pre), slot, nf);
     else if (c->mixed) launch_xzsynth(ctas, c->sm_synth, c->cs, li_of(c, pre), slot, nf);
-    else launch_xzsynth_fx(c->plane_big, ctas, c->thr_synth, c->sm_synth, c->cs, li_of(c, pre, ctas), slot, nf);
+    else launch_xzsynth_fx(c->plane_kind, ctas, c->thr_synth, c->sm_synth, c->cs, li_of(c, pre, ctas), slot, nf);
   });
 }
 // dns: with the norm and the extremum test of a DNS step (FP64 forms)
@@ -495,7 +495,7 @@ pcf_status launch_prodM(pcf_ctx* c, DnsInst* dns = nullptr) {
     if (c->plane_warp) launch_prod_warp(false, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod), -1);
     else if (c->mixed) launch_prod(false, c->suction, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod));
     else
-      launch_prod_fx(c->plane_big, false, c->cta_prod, c->thr_prod, c->sm_prod, c->cs,
+      launch_prod_fx(c->plane_kind, false, c->cta_prod, c->thr_prod, c->sm_prod, c->cs,
                      li_of(c, c->pre_prod, c->cta_prod), -1, dns);
   });
 }
@@ -505,7 +505,7 @@ pcf_status launch_prodN(pcf_ctx* c, int step_index = -1) {
     else if (c->mixed)
       launch_prod(true, c->suction, c->cta_prod, c->sm_prod, c->cs, li_of(c, c->pre_prod), step_index);
     else
-      launch_prod_fx(c->plane_big, true, c->cta_prod, c->thr_prod, c->sm_prod, c->cs,
+      launch_prod_fx(c->plane_kind, true, c->cta_prod, c->thr_prod, c->sm_prod, c->cs,
                      li_of(c, c->pre_prod, c->cta_prod), step_index);
   });
 }
@@ -1203,8 +1203,8 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
       I.cheb = g.cheb; I.rco = g.rco; I.ygrid = g.y; I.ubase = g.ub; I.ccw = g.ccw;
       I.kx = g.kx; I.kz = g.kz;
       I.twfx_x = g.twfx_x; I.twfx_z = g.twfx_z;
-      I.mz_mul = div_mul(I.Mz); I.nz_mul = div_mul(p.nz); I.rx_mul = div_mul(p.nx / 8);
-      I.rz_mul = div_mul(p.nz / 8);
+      I.mz_mul = div_mul(I.Mz); I.nz_mul = div_mul(p.nz); I.rx_mul = div_mul(fx_plan(p.nx).R);
+      I.rz_mul = div_mul(fx_plan(p.nz).R);
       {
         // 1/(nx nz) = m 2^e, 1/2 < m <= 1
         const int n = p.nx * p.nz;
@@ -1249,7 +1249,7 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
       per_tcs[b] = kFieldsY * cheb_tc_tiles(I.nmodes);
       per_tca[b] = 3 * cheb_tc_tiles(I.nmodes);
       if (!plane_warp_ok(I)) c->plane_warp = false;
-      c->plane_big = c->plane_big || planes_fx_big(I);
+      c->plane_kind = std::max(c->plane_kind, planes_fx_kind(I));
       c->thr_synth = std::max(c->thr_synth, planes_fx_threads(I, false));
       c->thr_prod = std::max(c->thr_prod, planes_fx_threads(I, true));
       if (c->mixed) c->sm_synth = c->sm_prod = std::max(c->sm_synth, smem_plane(I, (int)sizeof(float2)));
@@ -1275,7 +1275,7 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
   if (c->plane_warp) {
     c->sm_synth = c->sm_prod = c->sm_warp;
     if (set_plane_warp_smem(c->sm_synth, c->sm_prod)) return fail(PCF_ECUDA);
-  } else if (c->mixed ? set_plane_smem(c->sm_synth, c->sm_prod) : set_planes_fx_smem(c->sm_synth, c->sm_prod)) {
+  } else if (c->mixed ? set_plane_smem(c->sm_synth, c->sm_prod) : set_planes_fx_smem(c->plane_kind, c->sm_synth, c->sm_prod)) {
     return fail(PCF_ECUDA);
   }
   const int want = list[0].modes_per_block;

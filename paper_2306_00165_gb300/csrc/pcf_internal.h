@@ -104,7 +104,7 @@ struct Inst {
   const double* kz;   // [Mz]
   const fxtw* twfx_x; // [2][nx] fixed-point twiddles of the FP64 forms' plane kernels:
   const fxtw* twfx_z; //   forward (e^{-2 pi i q/n}), then inverse
-  unsigned mz_mul, nz_mul, rx_mul, rz_mul;  // floor(2^32/d) + 1 for d = Mz, nz, nx/8, nz/8 (exact quotients by __umulhi)
+  unsigned mz_mul, nz_mul, rx_mul, rz_mul;  // floor(2^32/d) + 1 for d = Mz, nz and the R of nx, nz (exact quotients by __umulhi)
   int nfx_h, nfx_l, nfx_e;  // 1/(nx nz) = (nfx_h, nfx_l) 2^-62 2^nfx_e; nfx_h = 0 for a power of two
   const float2* twxf; // e^{-2 pi i k/nx}, k < nx, of the mixed form
   const float2* twzf;

@@ -143,14 +143,14 @@ void launch_norm_planes(int ctas, cudaStream_t s, LaunchInfo li, int slot, DnsIn
 cudaError_t set_plane_smem(size_t synth, size_t prod);
 // The FP64 forms' plane kernels in 64-bit fixed point (pcf_planes_fx.cu); threads per CTA from
 // the largest plane of the launch.
-bool planes_fx_big(const Inst& I);
+int planes_fx_kind(const Inst& I);  // a launch takes the largest of its instances'
 size_t smem_planes_fx(const Inst& I, int threads);
 int planes_fx_threads(const Inst& I, bool prod);
-void launch_xzsynth_fx(bool big, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf);
-void launch_prod_fx(bool big, bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li,
+void launch_xzsynth_fx(int kind, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf);
+void launch_prod_fx(int kind, bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li,
                     int step_index, DnsInst* dns = nullptr);
 void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot);
-cudaError_t set_planes_fx_smem(size_t synth, size_t prod);
+cudaError_t set_planes_fx_smem(int kind, size_t synth, size_t prod);
 // Plane kernels of the FP32 form with the x, z transforms in warp registers
 // (pcf_planes_warp.cu): nx, nz in {32, 64, 96, 128}.
 bool plane_warp_ok(const Inst& I);

@@ -13,12 +13,9 @@
 // Measured (us per launch, FP64 Stockham passes -> now): 32 x 33 x 32, batch 8: synthesis 75 -> 28,
 // products M 41 -> 20, N 55 -> 30; 128 x 97 x 128: 1025 -> 205, 381 -> 105, 529 -> 157.
 //
-// A transform of length L = 8 R (R = 2, 4, 6, 8, 12, 16 for L = 16 .. 128) is two register
-// passes: DFTs of length R over the elements n, n + 8, .. (thread n of 8), twiddles, and DFTs
-// of length 8 over each block of eight.  Both passes work in place, so one buffer and one
-// barrier per pass suffice.  Slot of element (block b, member e) in a row: 8 b + (e xor (b mod 8)):
-// the eight lanes of a shared-memory phase meet eight different 16-byte bank groups in both
-// passes without padding; rows have an odd stride for the walks across rows.
+// A transform of length L = R S (fx_plan) is two register passes, thread n of S in the first,
+// thread b of R in the second.  Both work in place, so one buffer and one barrier per pass
+// suffice; rows have an odd stride for the walks across rows.
 #include "pcf_fx.cuh"
 #include "pcf_kernels.cuh"
 
@@ -26,61 +23,93 @@ namespace pcf {
 
 namespace {
 
+// Kernels for planes whose sides are 8 R: up to 64, or longer (R = 12, 16 hold more registers); and
+// for planes with a side of 18, 24, 36, 54, 72 or 108, which also do the others.
+enum FxKind : int { FX_SMALL = 0, FX_BIG = 1, FX_ANY = 2 };
 // Threads and resident CTAs the kernels are compiled for: 80 registers for sides up to 64 (768
 // threads per SM), 128 registers (512 threads per SM) for the longer transforms.
-template <bool BIG>
+template <int KIND>
 struct FxCfg {
-  static constexpr int threads = BIG ? 512 : 256, ctas = BIG ? 1 : 3;
+  static constexpr int threads = KIND ? 512 : 256, ctas = KIND ? 1 : 3;
 };
 
-__device__ __forceinline__ int fx_slot(int b, int e) { return b * 8 + (e ^ (b & 7)); }
+// R and S of length n
+template <int KIND>
+__device__ __forceinline__ FxPlan fx_plan_of(int n) {
+  return KIND == FX_ANY ? fx_plan(n) : FxPlan{n >> 3, 8};
+}
+__device__ __forceinline__ int fx_div(int t, unsigned mul) { return (int)__umulhi((unsigned)t, mul); }
+// slot of element i + odd of a row on its way into a transform (i even when odd is 1), and of output
+// b + R k
+template <int KIND>
+__device__ __forceinline__ int fx_in(FxPlan P, int i, int odd = 0) {
+  if (KIND == FX_ANY && P.S != 8) return i + odd;  // (i / S) S + i mod S
+  return fx_slot<8>(i >> 3, (i & 7) + odd);
+}
+template <int KIND>
+__device__ __forceinline__ int fx_out(FxPlan P, int b, int k) {
+  return KIND == FX_ANY && P.S != 8 ? b * P.S + k : fx_slot<8>(b, k);
+}
 
-// First pass over nrow rows: ld(row, n) -> element n, result in place in buf.
-template <int R, bool INV, class LD>
+// First pass over nrow rows: ld(row, n) -> element n, result in place in buf.  A row's S threads
+// lie in a group of G lanes; the spare lanes (S < G) repeat the last one's loads and store nothing.
+template <int R, int S, bool INV, class LD>
 __device__ __forceinline__ void fx_first(int nrow, fxc* buf, int LS, const fxtw* __restrict__ tw, const LD& ld) {
-  for (int t = threadIdx.x; t < 8 * nrow; t += blockDim.x) {
-    const int row = t >> 3, n = t & 7;
+  constexpr int LG = S <= 8 ? 3 : 4, G = 1 << LG;
+  for (int t = threadIdx.x; t < G * nrow; t += blockDim.x) {
+    const int row = t >> LG, lane = t & (G - 1), n = S < G ? min(lane, S - 1) : lane;
     fxc v[R];
     ld(row, n, v);
+    if (S < G && lane >= S) continue;
     FxDft<R, INV>::run(v);
     fxc* o = buf + row * LS;
-    o[fx_slot(0, n)] = v[0];
+    o[fx_slot<S>(0, n)] = v[0];
 #pragma unroll
     for (int k = 1; k < R; ++k) {
       const int4 w = __ldg(reinterpret_cast<const int4*>(tw) + n * k);
-      o[fx_slot(k, n)] = fx_cmul(v[k], fxtw{w.x, w.y, w.z, w.w});
+      o[fx_slot<S>(k, n)] = fx_cmul(v[k], fxtw{w.x, w.y, w.z, w.w});
     }
   }
 }
 // Second pass: st(row, b, v): v[k] is output b + R k of the row.
-template <int R, bool INV, class ST>
+template <int R, int S, bool INV, class ST>
 __device__ __forceinline__ void fx_second(int nrow, const fxc* buf, int LS, const ST& st) {
   for (int t = threadIdx.x; t < R * nrow; t += blockDim.x) {
     const int row = t / R, b = t - row * R;
     const fxc* a = buf + row * LS;
-    fxc v[8];
+    fxc v[S];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = a[fx_slot(b, e)];
-    FxDft<8, INV>::run(v);
+    for (int e = 0; e < S; ++e) v[e] = a[fx_slot<S>(b, e)];
+    FxDft<S, INV>::run(v);
     st(row, b, v);
   }
 }
 
-// f(integral_constant R) for the transform length n = 8 R (uniform in the CTA)
-template <int R_>
-struct FxR {
-  static constexpr int R = R_;
+// f(FxRS<R, S>) for the transform length n (uniform in the CTA); the host chooses a KIND that has it
+// (planes_fx_kind)
+template <int R_, int S_>
+struct FxRS {
+  static constexpr int R = R_, S = S_;
 };
-// BIG: kernels for planes with a side above 64 (R = 12, 16 hold more registers)
-template <bool BIG, class F>
+template <int KIND, class F>
 __device__ __forceinline__ void fx_length(int n, const F& f) {
+  if (KIND == FX_ANY) {
+    switch (n) {
+      case 18: f(FxRS<6, 3>()); return;
+      case 24: f(FxRS<4, 6>()); return;
+      case 36: f(FxRS<6, 6>()); return;
+      case 54: f(FxRS<6, 9>()); return;
+      case 72: f(FxRS<12, 6>()); return;
+      case 108: f(FxRS<12, 9>()); return;
+    }
+  }
   switch (n >> 3) {
-    case 2: f(FxR<2>()); break;
-    case 4: f(FxR<4>()); break;
-    case 6: f(FxR<6>()); break;
-    case 12: if (BIG) f(FxR<12>()); break;
-    case 16: if (BIG) f(FxR<16>()); break;
-    default: f(FxR<8>()); break;
+    case 2: f(FxRS<2, 8>()); break;
+    case 4: f(FxRS<4, 8>()); break;
+    case 6: f(FxRS<6, 8>()); break;
+    case 12: if (KIND) f(FxRS<12, 8>()); break;
+    case 16: if (KIND) f(FxRS<16, 8>()); break;
+    default: f(FxRS<8, 8>()); break;  // 64
   }
 }
 
@@ -179,7 +208,6 @@ __device__ __forceinline__ const int2* fx_info(const Inst& I, int slot, int f, i
 }
 // x-storage index i (m = i for i <= Kx, m = i - Mx otherwise) -> FFT bin
 __device__ __forceinline__ int xbin(int i, int Kx, int Mx, int nx) { return i <= Kx ? i : nx - (Mx - i); }
-__device__ __forceinline__ int fx_div(int t, unsigned mul) { return (int)__umulhi((unsigned)t, mul); }
 
 }  // namespace
 
@@ -213,11 +241,15 @@ size_t smem_planes_fx(const Inst& I, int threads) {
 // threads; before the single-precision bound 233 with 512, 280 with 256, 397 with 128; 96 x 31 x
 // 48, batch 3: 56 us with 128); the products take at least 256 (there 40 and 51 us, with 128
 // threads 47 and 62).
-bool planes_fx_big(const Inst& I) { return I.nx > 64 || I.nz > 64; }
+// Planes with a side that is not 8 R are rare; they take the longer sides' rule.
+int planes_fx_kind(const Inst& I) {
+  if (fx_plan(I.nx).S != 8 || fx_plan(I.nz).S != 8) return FX_ANY;
+  return I.nx > 64 || I.nz > 64 ? FX_BIG : FX_SMALL;
+}
 int planes_fx_threads(const Inst& I, bool prod) {
-  if (!planes_fx_big(I)) return prod ? std::max(128, 4 * I.nx) : I.nx * I.nz <= 1024 ? 64 : 128;
+  if (planes_fx_kind(I) == FX_SMALL) return prod ? std::max(128, 4 * I.nx) : I.nx * I.nz <= 1024 ? 64 : 128;
   int best = 128, most = 0;
-  for (int t = 128; t <= FxCfg<true>::threads; t *= 2) {
+  for (int t = 128; t <= FxCfg<FX_BIG>::threads; t *= 2) {
     const int fit = (int)(228 * 1024 / (smem_planes_fx(I, t) + 1024)), n = t * std::min(fit, 512 / t);
     if (n > most) best = t, most = n;
   }
@@ -231,8 +263,8 @@ __constant__ int c_fx_fac[kFieldsSynth] = {0, 0, 0, 1, 0, 2, 1, 2, 1, 0, 2};
 // CTA = (instance, y-plane j, field f): u, v, w, u_x, u_y, u_z, v_x, v_z, w_x, w_y, w_z.  The
 // plane's exponent e0 comes from the sum B of |Re| + |Im| over the plane's modes (p > 0 twice):
 // every intermediate of the two transforms is below 2 B in modulus, and 2 B 2^-e0 < 2^62.
-template <bool BIG>
-__global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_synth_fx(LaunchInfo li, int slot, int nfields) {
+template <int KIND>
+__global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_synth_fx(LaunchInfo li, int slot, int nfields) {
   extern __shared__ __align__(16) unsigned char smraw[];
   int local;
   const int b = find_inst(li, blockIdx.x, &local);
@@ -278,6 +310,7 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_synth
     return;
   }
   const int e0 = eb + ek - 61;
+  const FxPlan px = fx_plan_of<KIND>(nx);
   // the modes as integers at their x bins (rows p); i k v for the x and z derivatives
   for (int t = threadIdx.x; t < nm; t += blockDim.x) {
     const double2 s = src[t];
@@ -289,41 +322,41 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_synth
       const FxK k = fx_factor(fac == 1 ? I.kx[i] : I.kz[p]);
       v = fxc{fx_from_k(s.y, k, e0, -1), fx_from_k(s.x, k, e0, 0)};
     }
-    G[p * P.LX + fx_slot(bin >> 3, bin & 7)] = v;
+    G[p * P.LX + fx_in<KIND>(px, bin)] = v;
   }
   __syncthreads();
   // x stage, rows p: element = x bin; bins outside |m| <= Kx are zero
-  fx_length<BIG>(nx, [&](auto rc) {
-    constexpr int R = decltype(rc)::R;
-    fx_first<R, true>(Mz, G, P.LX, I.twfx_x + nx, [&](int p, int n, fxc* v) {
+  fx_length<KIND>(nx, [&](auto rc) {
+    constexpr int R = decltype(rc)::R, S = decltype(rc)::S;
+    fx_first<R, S, true>(Mz, G, P.LX, I.twfx_x + nx, [&](int p, int n, fxc* v) {
 #pragma unroll
       for (int q = 0; q < R; ++q) {
-        const int bin = n + 8 * q;
-        v[q] = bin <= Kx || bin >= nx - Kx ? G[p * P.LX + fx_slot(q, n)] : fxc{0, 0};
+        const int bin = n + S * q;
+        v[q] = bin <= Kx || bin >= nx - Kx ? G[p * P.LX + fx_slot<S>(q, n)] : fxc{0, 0};
       }
     });
     __syncthreads();
-    fx_second<R, true>(Mz, G, P.LX, [&](int p, int bk, const fxc* v) {
+    fx_second<R, S, true>(Mz, G, P.LX, [&](int p, int bk, const fxc* v) {
       fxc* o = G + p * P.LX;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) o[fx_slot(bk, e)] = v[e];
+      for (int e = 0; e < S; ++e) o[fx_slot<S>(bk, e)] = v[e];
     });
   });
   __syncthreads();
-  const int nr = nx / 2, Rx = nx >> 3;
+  const int nr = nx / 2, Rx = px.R;
   const unsigned rxm = I.rx_mul;
   unsigned mh = 0;
   for (int r0 = 0; r0 < nr; r0 += P.chunk) {
     const int nrc = min(P.chunk, nr - r0);
-    fx_length<BIG>(nz, [&](auto rc) {
-      constexpr int R = decltype(rc)::R;
+    fx_length<KIND>(nz, [&](auto rc) {
+      constexpr int R = decltype(rc)::R, S = decltype(rc)::S;
       // row pair (x1, x2 = x1 + 1) -> one complex row G[x1] + i G[x2]
-      fx_first<R, true>(nrc, Z, P.LZ, I.twfx_z + nz, [&](int r, int n, fxc* v) {
+      fx_first<R, S, true>(nrc, Z, P.LZ, I.twfx_z + nz, [&](int r, int n, fxc* v) {
         const int x1 = 2 * (r0 + r), k3 = fx_div(x1, rxm), k1 = x1 - k3 * Rx;
-        const int s1 = fx_slot(k1, k3), s2 = fx_slot(k1 + 1, k3);
+        const int s1 = fx_out<KIND>(px, k1, k3), s2 = fx_out<KIND>(px, k1 + 1, k3);
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-          const int z = n + 8 * q;
+          const int z = n + S * q;
           const bool lo = z <= Kz, hi = z >= nz - Kz;
           v[q] = fxc{0, 0};
           if (lo || hi) {
@@ -335,10 +368,10 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_synth
         }
       });
       __syncthreads();
-      fx_second<R, true>(nrc, Z, P.LZ, [&](int r, int bk, const fxc* v) {
+      fx_second<R, S, true>(nrc, Z, P.LZ, [&](int r, int bk, const fxc* v) {
         fx* o = out + (size_t)(2 * (r0 + r)) * nz + bk;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
+        for (int e = 0; e < S; ++e) {
           o[R * e] = v[e].x;
           o[nz + R * e] = v[e].y;
           mh = max(mh, max(fx_maghi(v[e].x), fx_maghi(v[e].y)));
@@ -403,13 +436,13 @@ __device__ double fx_block_sum(unsigned long long s, int e, int* red) {
 // CTA = (instance, plane j, component c).  Every factor is scaled to 62 bits, the products keep
 // their high 64 bits (2^-60 of the largest product) and are summed at the largest term's
 // exponent.  The transforms rescale every row pair and then every x row from its own largest
-// value, found by shuffles among the eight lanes that hold the row.
+// value, found by shuffles among the lanes that hold the row.
 // SUM (M only, the DNS): also the plane sums of u_c^2 and, in an instance's last CTA, the end of
 // the DNS step's norm; the planes are in registers here (as a kernel of its own the sums took 4238
 // us per 64 steps of four 32 x 33 x 32 fields, now 4047).
-template <bool ADJ, bool BIG, bool SUM>
-__global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_fx(LaunchInfo li, int step_index,
-                                                                                  DnsInst* dns) {
+template <bool ADJ, int KIND, bool SUM>
+__global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_prod_fx(LaunchInfo li, int step_index,
+                                                                                    DnsInst* dns) {
   extern __shared__ __align__(16) unsigned char smraw[];
   // factors: 0-2 advecting velocity u_b + u; 3-5 gradient of component c of u (M) or q (N);
   // N: 6-8 q, 9-11 derivative c of u's components; 12: the factor of U' (v, or q_0).
@@ -553,8 +586,8 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
         val[h] = a;
       }
       fxc* o = Z + (row >> 1) * P.LZ;
-      reinterpret_cast<fx*>(o + fx_slot(z >> 3, z & 7))[row & 1] = val[0];
-      reinterpret_cast<fx*>(o + fx_slot(z >> 3, (z & 7) + 1))[row & 1] = val[1];
+      reinterpret_cast<fx*>(o + fx_in<KIND>(fx_plan_of<KIND>(nz), z))[row & 1] = val[0];
+      reinterpret_cast<fx*>(o + fx_in<KIND>(fx_plan_of<KIND>(nz), z, 1))[row & 1] = val[1];
     }
     if (!live) continue;
     if (xs) {
@@ -568,20 +601,20 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
     fxc* const buf = xs ? X : Z;
     const int LS = xs ? P.LX : P.LZ, rows = xs ? Mz : nrc, lg = xs ? lgx : lgz + 1;
     int* const eo = xs ? ep : er + r0;
-    fx_length<BIG>(xs ? nx : nz, [&](auto rc) {
-      constexpr int R = decltype(rc)::R;
-      fx_first<R, false>(rows, buf, LS, xs ? I.twfx_x : I.twfx_z, [&](int r, int n, fxc* v) {
+    fx_length<KIND>(xs ? nx : nz, [&](auto rc) {
+      constexpr int R = decltype(rc)::R, S = decltype(rc)::S, G = S <= 8 ? 8 : 16;
+      fx_first<R, S, false>(rows, buf, LS, xs ? I.twfx_x : I.twfx_z, [&](int r, int n, fxc* v) {
         unsigned mh = 0;
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-          const fxc a = buf[r * LS + fx_slot(q, n)];
-          const int d = min(align[(n + 8 * q) >> 1], 63);
+          const fxc a = buf[r * LS + fx_slot<S>(q, n)];
+          const int d = min(align[(n + S * q) >> 1], 63);
           v[q] = fxc{a.x >> d, a.y >> d};
           mh = max(mh, max(fx_maghi(v[q].x), fx_maghi(v[q].y)));
         }
-        const unsigned m = 0xffu << (threadIdx.x & 24);
+        const unsigned m = ((1u << G) - 1) << (threadIdx.x & 31 & ~(G - 1));
 #pragma unroll
-        for (int o = 1; o < 8; o <<= 1) mh = max(mh, __shfl_xor_sync(m, mh, o));
+        for (int o = 1; o < G; o <<= 1) mh = max(mh, __shfl_xor_sync(m, mh, o));
         // sqrt(2) n max <= 2^61 (z stage: the unpacking adds two values), 2^62 (x stage)
         const int s = fx_bits(mh) + 1 + lg - 62;
 #pragma unroll
@@ -589,32 +622,32 @@ __global__ void __launch_bounds__(FxCfg<BIG>::threads, FxCfg<BIG>::ctas) k_prod_
         if (n == 0) eo[r] = eP + s - (xs ? 0 : 1);
       });
       __syncthreads();
-      fx_second<R, false>(rows, buf, LS, [&](int r, int bk, const fxc* v) {
+      fx_second<R, S, false>(rows, buf, LS, [&](int r, int bk, const fxc* v) {
         fxc* o = buf + r * LS;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) o[fx_slot(bk, e)] = v[e];
+        for (int e = 0; e < S; ++e) o[fx_slot<S>(bk, e)] = v[e];
       });
     });
     __syncthreads();
     // rows x1 and x2 of each pair, twice their value: F1 = H_p + conj(H_-p), F2 = -i (H_p - conj(H_-p))
     for (int t = threadIdx.x; t < nrc * Mz; t += blockDim.x) {
       const int r = fx_div(t, I.mz_mul), p = t - r * Mz, pm = p == 0 ? 0 : nz - p;
-      const int kp = fx_div(p, I.rz_mul), km = fx_div(pm, I.rz_mul), Rz = nz >> 3;
-      const fxc hp = Z[r * P.LZ + fx_slot(p - kp * Rz, kp)], hm = Z[r * P.LZ + fx_slot(pm - km * Rz, km)];
+      const int kp = fx_div(p, I.rz_mul), km = fx_div(pm, I.rz_mul), Rz = fx_plan_of<KIND>(nz).R;
+      const fxc hp = Z[r * P.LZ + fx_out<KIND>(fx_plan_of<KIND>(nz), p - kp * Rz, kp)], hm = Z[r * P.LZ + fx_out<KIND>(fx_plan_of<KIND>(nz), pm - km * Rz, km)];
       const int x = 2 * (r0 + r);
-      X[p * P.LX + fx_slot(x >> 3, x & 7)] = fxc{hp.x + hm.x, hp.y - hm.y};
-      X[p * P.LX + fx_slot(x >> 3, (x & 7) + 1)] = fxc{hp.y + hm.y, hm.x - hp.x};
+      X[p * P.LX + fx_in<KIND>(fx_plan_of<KIND>(nx), x)] = fxc{hp.x + hm.x, hp.y - hm.y};
+      X[p * P.LX + fx_in<KIND>(fx_plan_of<KIND>(nx), x, 1)] = fxc{hp.y + hm.y, hm.x - hp.x};
     }
     if (!xs) __syncthreads();
   }
   double2* dst = I.xz + ((size_t)c * I.ny + j) * I.nmodes;
-  const int Rx = nx >> 3;
+  const int Rx = fx_plan_of<KIND>(nx).R;
   for (int t = threadIdx.x; t < I.nmodes; t += blockDim.x) {
     const int i = fx_div(t, I.mz_mul), p = t - i * Mz, bin = xbin(i, Kx, Mx, nx), k3 = fx_div(bin, I.rx_mul);
     double2 o = make_double2(0.0, 0.0);
     if (bad) o.x = o.y = __longlong_as_double(0x7ff8000000000000LL);
     if (live) {
-      fxc a = X[p * P.LX + fx_slot(bin - k3 * Rx, k3)];
+      fxc a = X[p * P.LX + fx_out<KIND>(fx_plan_of<KIND>(nx), bin - k3 * Rx, k3)];
       if (I.nfx_h) a = fxc{fx_mulc(a.x, I.nfx_h, I.nfx_l), fx_mulc(a.y, I.nfx_h, I.nfx_l)};
       const int e0 = ep[p] + I.nfx_e;
       o = make_double2(__longlong_as_double((long long)fx_double_bits(a.x, e0)),
@@ -659,32 +692,39 @@ __global__ void __launch_bounds__(128) k_norm_planes_fx(LaunchInfo li, int slot)
     I.normpart[(size_t)c * I.ny + j] = e == kFxNan ? __longlong_as_double(0x7ff8000000000000LL) : s;
 }
 
-void launch_xzsynth_fx(bool big, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf) {
-  if (big) k_synth_fx<true><<<ctas, threads, smem, s>>>(li, slot, nf);
-  else k_synth_fx<false><<<ctas, threads, smem, s>>>(li, slot, nf);
+void launch_xzsynth_fx(int kind, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf) {
+  if (kind == FX_ANY) k_synth_fx<FX_ANY><<<ctas, threads, smem, s>>>(li, slot, nf);
+  else if (kind == FX_BIG) k_synth_fx<FX_BIG><<<ctas, threads, smem, s>>>(li, slot, nf);
+  else k_synth_fx<FX_SMALL><<<ctas, threads, smem, s>>>(li, slot, nf);
 }
-void launch_prod_fx(bool big, bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li,
+template <int KIND>
+static void launch_prod_kind(bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int step_index,
+                             DnsInst* dns) {
+  if (adj) k_prod_fx<true, KIND, false><<<ctas, threads, smem, s>>>(li, step_index, nullptr);
+  else if (dns) k_prod_fx<false, KIND, true><<<ctas, threads, smem, s>>>(li, -1, dns);
+  else k_prod_fx<false, KIND, false><<<ctas, threads, smem, s>>>(li, -1, nullptr);
+}
+void launch_prod_fx(int kind, bool adj, int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li,
                     int step_index, DnsInst* dns) {
-  if (big && adj) k_prod_fx<true, true, false><<<ctas, threads, smem, s>>>(li, step_index, nullptr);
-  else if (adj) k_prod_fx<true, false, false><<<ctas, threads, smem, s>>>(li, step_index, nullptr);
-  else if (big && dns) k_prod_fx<false, true, true><<<ctas, threads, smem, s>>>(li, -1, dns);
-  else if (dns) k_prod_fx<false, false, true><<<ctas, threads, smem, s>>>(li, -1, dns);
-  else if (big) k_prod_fx<false, true, false><<<ctas, threads, smem, s>>>(li, -1, nullptr);
-  else k_prod_fx<false, false, false><<<ctas, threads, smem, s>>>(li, -1, nullptr);
+  (kind == FX_ANY   ? launch_prod_kind<FX_ANY>
+   : kind == FX_BIG ? launch_prod_kind<FX_BIG>
+                    : launch_prod_kind<FX_SMALL>)(adj, ctas, threads, smem, s, li, step_index, dns);
 }
 void launch_norm_planes_fx(int ctas, cudaStream_t s, LaunchInfo li, int slot) {
   k_norm_planes_fx<<<ctas, 128, 0, s>>>(li, slot);
 }
-cudaError_t set_planes_fx_smem(size_t synth, size_t prod) {
+template <int KIND>
+static cudaError_t set_kind_smem(size_t synth, size_t prod) {
   cudaError_t e;
-  if ((e = raise_smem_limit((const void*)k_synth_fx<false>, synth))) return e;
-  if ((e = raise_smem_limit((const void*)k_synth_fx<true>, synth))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_fx<true, false, false>, prod))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_fx<true, true, false>, prod))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_fx<false, true, true>, prod))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_fx<false, false, true>, prod))) return e;
-  if ((e = raise_smem_limit((const void*)k_prod_fx<false, true, false>, prod))) return e;
-  return raise_smem_limit((const void*)k_prod_fx<false, false, false>, prod);
+  if ((e = raise_smem_limit((const void*)k_synth_fx<KIND>, synth))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_fx<true, KIND, false>, prod))) return e;
+  if ((e = raise_smem_limit((const void*)k_prod_fx<false, KIND, true>, prod))) return e;
+  return raise_smem_limit((const void*)k_prod_fx<false, KIND, false>, prod);
+}
+cudaError_t set_planes_fx_smem(int kind, size_t synth, size_t prod) {
+  return kind == FX_ANY   ? set_kind_smem<FX_ANY>(synth, prod)
+         : kind == FX_BIG ? set_kind_smem<FX_BIG>(synth, prod)
+                          : set_kind_smem<FX_SMALL>(synth, prod);
 }
 
 }  // namespace pcf
