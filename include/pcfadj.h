@@ -89,7 +89,9 @@ typedef struct pcf_params {
                            separate analysis / solve / synthesis kernels.  4: as 2, with J in a
                            kernel of its own.  2, 3 and 4 give bit-identical results.  5: the
                            separate kernels with the Stokes solve by banded sweeps, one thread
-                           per chain (group g, mode, real or imaginary part). */
+                           per chain (group g, mode, real or imaginary part).  A batch with a problem of
+                           kind 1 runs the per-mode kernel for all of its problems; otherwise the
+                           first problem's kind counts. */
   int base_flow;        /* pcf_base_flow: the laminar base flow u_b = (U(y), V, 0) */
   int symmetry;         /* pcf_symmetry mask enforced along the descent and the DNS (0: none).
                            s1 requires PCF_COUETTE (it maps the Poiseuille profile to its

@@ -56,7 +56,7 @@ struct pcf_ctx {
   int* pre_tca = nullptr;   // tensor-core analysis (mixed form)
   int cta_synth11 = 0, cta_synth3 = 0, cta_prod = 0, cta_mode = 0, cta_tcs = 0, cta_tca = 0;
   size_t sm_synth = 0, sm_prod = 0, sm_mode = 0, sm_tc = 0, sm_warp = 0;
-  // the FP64 forms' fixed-point per-mode kernels (every solve_kind but 1)
+  // the FP64 forms' fixed-point per-mode kernels (no problem of solve_kind 1)
   bool split = false;
   int sgrp = 0;                 // largest instances per group of the solve
   int np = 8;                   // modes per tile of the analysis and synthesis

@@ -1172,7 +1172,11 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
   c->hinst.resize(B);
   std::vector<int> per11(B), per3(B), per1(B, 1), per_tcs(B), per_tca(B);
   size_t o_yv = 0, o_ph = 0, o_xz = 0, o_np = 0, o_fr = 0, o_pi = 0;
-  c->split = !c->mixed && list[0].solve_kind != 1;
+  // a problem of solve_kind 1 has no dense operators: a batch with one runs the per-mode kernel,
+  // which solves each instance with what its problem has
+  c->split = !c->mixed;
+  for (int k = 0; k < nlist; ++k)
+    if (list[k].solve_kind == 1) c->split = false;
   // the FP32 form's plane kernels keep their transforms in warp registers wherever every
   // instance's nx and nz allow it (unless the caller asks for the shared-memory kernels)
   c->plane_warp = c->mixed && list[0].plane_kernel != 1;
