@@ -66,9 +66,9 @@ struct pcf_ctx {
   int* pre_yy = nullptr;
   int* pre_ys = nullptr;        // ... over groups: one CTA per (group, mode)
   int cta_ya = 0, cta_ys = 0, cta_yy = 0;
-  int thr_ya = 64, thr_yy = 64, thr_ys = 64, thr_yf = 64;
+  int thr_ya = 64, thr_yy = 64, thr_ys = 64, thr_yf = 64, thr_y64 = 64;
   bool fine_y = false, fine_s = false;  // one row and one part per thread (few row pairs)
-  size_t sm_ya = 0, sm_ys = 0, sm_yy = 0, sm_yf = 0;
+  size_t sm_ya = 0, sm_ys = 0, sm_yy = 0, sm_yf = 0, sm_y64 = 0;
   // the step runs the fused half-step kernel (k_ystep_fx), with a separate norm kernel (jn)
   bool fused = false, jn = false;
   // the split step's Stokes solve by banded sweeps, one thread per chain (k_sweep), in place

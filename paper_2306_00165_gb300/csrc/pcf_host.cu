@@ -544,6 +544,8 @@ pcf_status launch_analysis(pcf_ctx* c, bool red = false) {
 pcf_status launch_solve(pcf_ctx* c, int op, int sig, bool red = false) {
   const int cls = op == MODE_PHI ? 3 : 6;
   if (!c->split) return launch_mode(c, op, sig);
+  if (op == MODE_SOLVE)
+    return timed(c, cls, [&] { launch_ysolve_f64(c->cta_ys, c->thr_y64, c->sm_y64, c->cs, gl_of(c), sig); });
   if (c->sweep && (op == MODE_PHI || op == MODE_PSI_UPDATE))
     return timed(c, cls, [&] {
       launch_sweep(red ? c->cta_sw_r : c->cta_sw, c->thr_sw, c->sm_sw, c->cs,
@@ -789,7 +791,7 @@ static pcf_status build_tables(pcf_ctx* c, const pcf_params* prm, GridTables* g)
     }
   }
   if (prm->solve_kind == 1) return PCF_OK;
-  // dense operators: in FP64 for the mixed form, as fixed-point words for the FP64 forms
+  // dense operators: in FP64, and for the FP64 forms as fixed-point words too
   const bool fx = prm->precision != PCF_MIXED;
   if (fx) {
     std::vector<double> ik(Mx * Mz, 0.0);
@@ -810,16 +812,13 @@ static pcf_status build_tables(pcf_ctx* c, const pcf_params* prm, GridTables* g)
     }
     double* d = nullptr;
     if (upload(make_dense_tables(N, kx, kz, g->sig[q], rco, q ? tab1 : tab0), &d)) return PCF_ECUDA;
-    if (!fx) {
-      g->dense[q] = d;
-      c->allocs.push_back(d);
-      continue;
-    }
+    g->dense[q] = d;
+    c->allocs.push_back(d);
+    if (!fx) continue;
     const bool ok = !ctx_alloc(c, &g->fxD[q], dense_limbs_len(N, Mx * Mz)) &&
                     !ctx_alloc(c, &g->fxDe[q], dense_exps_len(N, Mx * Mz));
     if (ok) launch_dense_limbs(d, N, Mx * Mz, g->fxD[q], g->fxDe[q]);
     const cudaError_t e = cudaDeviceSynchronize();
-    cudaFree(d);
     if (!ok) return PCF_ENOMEM;
     PCF_CUDA(e);
   }
@@ -942,6 +941,8 @@ static pcf_status set_modes(pcf_ctx* c, int G) {
   c->cta_ys_r = psr[ng];
   c->sm_ys = smem_ysolve_fx(Nmax, gmax);
   c->sm_yf = smem_ystep_fx(Nmax, gmax);
+  c->sm_y64 = smem_ysolve_f64(Nmax, gmax);
+  c->thr_y64 = ysolve_f64_threads(Nmax, gmax);
   // one row and one part per thread while the launch would otherwise leave SMs with less than
   // eight warps
   const int hp = (Nmax / 2 + 2) / 2;
@@ -970,7 +971,7 @@ static pcf_status set_modes(pcf_ctx* c, int G) {
   c->fine_y = (long long)c->cta_ya * c->np * 2 * hp < 152LL * 256;
   c->thr_ya = yana_fx_threads(Nmax, c->np, c->fine_y);
   c->thr_yy = ysynth_fx_threads(Nmax, c->np, c->fine_y);
-  PCF_CUDA(set_modes_fx_smem(c->sm_ya, c->sm_yy, c->sm_ys, c->sm_yf));
+  PCF_CUDA(set_modes_fx_smem(c->sm_ya, c->sm_yy, c->sm_ys, c->sm_yf, c->sm_y64));
   return PCF_OK;
 }
 

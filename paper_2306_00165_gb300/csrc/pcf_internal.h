@@ -94,7 +94,7 @@ struct Inst {
   int fxcheb_e;        // exponent of the analysis table: its entries are scaled by 2^-fxcheb_e
   const int4* fxD[2];  // [nmodes][6][Mh][(Mh + 1)/2] dense operators as fixed-point words
   const int* fxDe[2];  // [nmodes][6][2 ((Mh + 1)/2)] exponents of their rows
-  const double* dense[2];  // mixed form: per-mode dense solve operators in FP64 (DenseLayout) or null
+  const double* dense[2];  // per-mode dense solve operators in FP64 (DenseLayout) or null
   const double* ik2nu; // [nmodes] 1/(nu k^2), 0 for the mean mode
   const double* rco;
   const double* ygrid;

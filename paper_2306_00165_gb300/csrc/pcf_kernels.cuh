@@ -194,9 +194,13 @@ void launch_yana_fx(int ctas, int threads, size_t smem, cudaStream_t s, LaunchIn
 void launch_ysynth_fx(int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf,
                       int check_active, int np, int red, int fine);
 void launch_ysolve_fx(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int op, int sig, int fine);
+// the solve of a given right-hand side (MODE_SOLVE), in FP64
+int ysolve_f64_threads(int N, int G);
+size_t smem_ysolve_f64(int N, int G);
+void launch_ysolve_f64(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int sig);
 void launch_ystep_fx(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int op, int synth, int fine);
 void launch_jnorm(int ninst, cudaStream_t s, const Inst* insts, int step_index);
-cudaError_t set_modes_fx_smem(size_t ana, size_t synth, size_t solve, size_t step);
+cudaError_t set_modes_fx_smem(size_t ana, size_t synth, size_t solve, size_t step, size_t solve64);
 // dense operators -> fixed-point words (default stream): lengths of the two arrays, conversion
 size_t dense_limbs_len(int N, int nmodes);
 size_t dense_exps_len(int N, int nmodes);

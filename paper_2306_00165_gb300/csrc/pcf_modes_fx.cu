@@ -7,6 +7,7 @@
 //   k_ysolve_fx  CTA (group of instances, mode): right-hand side, dense Stokes operators of both
 //                parity groups, xi = -dv/dy, assembly, finite-difference quotient and update
 //   k_ystep_fx   CTA (group of instances, mode): the three in one, intermediates in shared memory
+//   k_ysolve_f64 CTA (group of instances, mode): the solve of a given right-hand side, in FP64
 //
 // Every product is a matrix (the same for all columns of a CTA) times columns.  A column's
 // values are integers of one exponent, scaled so that the sum of their magnitudes is just below
@@ -340,8 +341,7 @@ __device__ __forceinline__ void put_part(double2* d, int part, double x, double 
 __device__ __forceinline__ double flip(double x, bool neg) {
   return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
 }
-// One mode, nI instances (columns).  coef(i, c, n, part): Chebyshev coefficient of the products (0
-// for MODE_SOLVE).  C3, R3: [3][ny][nI] arrays; sm_i: 16 nI ints.  done(i, c, n, part, new value) receives
+// One mode, nI instances (columns).  coef(i, c, n, part): Chebyshev coefficient of the products.  C3, R3: [3][ny][nI] arrays; sm_i: 16 nI ints.  done(i, c, n, part, new value) receives
 // r1 (PHI), the updated state (PSI_UPDATE) or f.
 template <class COEF, class DONE>
 __device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI, int m, int op, int sig, const int* live,
@@ -357,7 +357,7 @@ __device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI,
   const int ix = m / Mz, pz = m - ix * Mz;
   const double kx = I0.kx[ix], kz = I0.kz[pz];
   const bool mean = m == 0;
-  const double ist = op == MODE_SOLVE ? 1.0 : sig == 0 ? I0.inv_dt : I0.inv_dtau_hat;
+  const double ist = sig == 0 ? I0.inv_dt : I0.inv_dtau_hat;
   const bool in_u = op == MODE_PHI;
   __syncthreads();
   // S = state/step + product; f_v = S_v, g = i (kx S_u + kz S_w), h = i (kz S_u - kx S_w); mean
@@ -501,7 +501,7 @@ __device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI,
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       up[c] = op == MODE_PHI || op == MODE_PSI_UPDATE ? u[c * gc] : 0.0;
-      d[c] = op == MODE_PHI ? -up[c] : psi ? rh[c * gc] : 0.0;
+      d[c] = op == MODE_PHI ? -up[c] : rh[c * gc];
     }
     d[0] = fma(a0, x0, fma(b0, y, d[0]));
     d[1] = fma(inu, x1, d[1]);
@@ -510,7 +510,7 @@ __device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI,
     double* out = op == MODE_PHI ? rh : reinterpret_cast<double*>(op == MODE_PSI_UPDATE ? I.uhat : I.fhat) + gi;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const double o = op == MODE_PSI_UPDATE ? fma(step, d[c], up[c]) : op == MODE_SOLVE ? d[c] : d[c] * step;
+      const double o = op == MODE_PSI_UPDATE ? fma(step, d[c], up[c]) : d[c] * step;
       out[c * gc] = o;
       done(i, c, n, part, o);
     }
@@ -622,15 +622,127 @@ __global__ void __launch_bounds__(256, 3) k_ysolve_fx(GroupLaunch gl, int op, in
   const int2 grp = gl.groups[find_group(gl, blockIdx.x, &m)];
   const int first = grp.x, nI = grp.y;
   const Inst& I0 = gl.insts[first];
-  if (threadIdx.x < nI) live[threadIdx.x] = op == MODE_SOLVE || inst_active(gl.insts[first + threadIdx.x]);
+  if (threadIdx.x < nI) live[threadIdx.x] = inst_active(gl.insts[first + threadIdx.x]);
   const int AS = I0.ny * nI, ny = I0.ny, nm = I0.nmodes;
   int* smi = reinterpret_cast<int*>(smx + 6 * AS);
   solve_mode(gl.insts, first, nI, m, op, sig, live, smx, smx + 3 * AS, smi, fine != 0,
              [&](int i, int c, int n, int part) {
-               if (op == MODE_SOLVE) return 0.0;
                return reinterpret_cast<const double*>(gl.insts[first + i].xc)[2 * (((size_t)c * nm + m) * ny + n) + part];
              },
              [](int, int, int, int, double) {});
+}
+
+// The Stokes solve of a caller's right-hand side (rhat -> fhat).  Its result is the operators' alone:
+// no transform's rounding hides the tail of a decaying Chebyshev spectrum, and units of a whole
+// column's sum would take its digits (spectrum exp(-n/2), ny = 49: coefficient 46 of v off by
+// 1.5e-10 of itself in fixed point, by 6e-14 here).  So the operators are applied in FP64, as stored.
+// Bound by the FP64 pipe, which takes a warp's instruction in the same 77 clocks whatever its
+// active lanes: one output (row, instance, part) per thread, v rows and eta rows in passes of their
+// own, so that a warp's lanes carry chains of about one length.  us, several modes per CTA in FP64
+// / fixed point / here: 32 x 33 x 32, batch 8: 30 / 19 / 25; 96 x 31 x 48, batch 3: 56 / 24 / 33;
+// 128 x 97 x 128: 980 / 126 / 260.
+// X: [3][ny][2 nI] doubles f_v, g, h; V, Q: [ny][2 nI] v and eta (mean mode: u, w); Y: dv/dy.
+__global__ void __launch_bounds__(256) k_ysolve_f64(GroupLaunch gl, int sig) {
+  extern __shared__ __align__(16) double2 smx[];
+  __shared__ int bad[2][2 * kMaxGroup];  // an input of v (u), of eta (w) that is not finite, per column
+  int m;
+  const int2 grp = gl.groups[find_group(gl, blockIdx.x, &m)];
+  const int first = grp.x, nI = grp.y, W = 2 * nI;
+  const Inst& I0 = gl.insts[first];
+  const int N = I0.N, ny = I0.ny, nm = I0.nmodes, Mz = I0.Mz, H = N / 2 + 1, half = N / 2, AS = ny * W;
+  double* X = reinterpret_cast<double*>(smx);
+  double *V = X + 3 * AS, *Q = V + AS, *Y = X;  // Y over f_v, once v is done
+  const int ix = m / Mz, pz = m - ix * Mz;
+  const double kx = I0.kx[ix], kz = I0.kz[pz];
+  const bool mean = m == 0;
+  const Cols C(W, W), CN(ny, ny);
+  for (int t = threadIdx.x; t < 4 * kMaxGroup; t += blockDim.x) (&bad[0][0])[t] = 0;
+  __syncthreads();
+  for (int t = threadIdx.x; t < 2 * nI * ny; t += blockDim.x) {
+    const int i = CN.row(t >> 1), part = t & 1, n = (t >> 1) - i * ny;
+    const double* F = reinterpret_cast<const double*>(gl.insts[first + i].rhat + (size_t)m * ny + n);
+    const size_t gc = 2 * (size_t)nm * ny;
+    double a, g, h;
+    if (mean) {
+      a = F[part];
+      g = 0.0;
+      h = F[2 * gc + part];
+    } else {
+      // g = i (kx F_u + kz F_w), h = i (kz F_u - kx F_w)
+      const double u = F[1 - part], w = F[2 * gc + 1 - part], kxg = flip(kx, !part), kzg = flip(kz, !part);
+      a = F[gc + part];
+      g = fma(kxg, u, kzg * w);
+      h = fma(kzg, u, -kxg * w);
+    }
+    double* o = X + n * W + 2 * i + part;
+    o[0] = a;
+    o[AS] = g;
+    o[2 * AS] = h;
+    if (ec_of(a) == 0x7ff || ec_of(g) == 0x7ff) bad[0][2 * i + part] = 1;
+    if (ec_of(h) == 0x7ff) bad[1][2 * i + part] = 1;
+  }
+  __syncthreads();
+  const DenseLayout DL(N);
+  const double* D = I0.dense[sig] + (size_t)m * DL.per_mode();
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  // sum of an operator row (entries Mh apart) over one parity class of a column
+  const auto dot = [&](const double* A, const double* x, int K, double s) {
+    int k = 0;
+    for (; k + 4 <= K; k += 4) {
+      double a[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) a[q] = __ldg(A + (k + q) * H);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) s = fma(a[q], x[2 * (k + q) * W], s);
+    }
+    for (; k < K; ++k) s = fma(__ldg(A + k * H), x[2 * k * W], s);
+    return s;
+  };
+  // rows of class 0, then of class 1; neighbouring threads take the columns of one row
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int t = threadIdx.x; t < AS; t += blockDim.x) {
+      const int rn = C.row(t), col = t - rn * W, cls = rn >= H, r = cls ? rn - H : rn, n = 2 * r + cls;
+      const int own = cls ? half : H, other = cls ? H : half;
+      double s;
+      if (mean) s = dot(D + DL.at(cls, DL.kEh, r, 0), X + pass * 2 * AS + cls * W + col, own, 0.0);
+      else if (pass == 0)
+        s = dot(D + DL.at(cls, DL.kAg, r, 0), X + AS + (1 - cls) * W + col, other,
+                dot(D + DL.at(cls, DL.kAv, r, 0), X + cls * W + col, own, 0.0));
+      else s = dot(D + DL.at(1 - cls, DL.kEh, r, 0), X + 2 * AS + cls * W + col, own, 0.0);
+      (pass ? Q : V)[n * W + col] = bad[pass][col] ? nan : s;
+    }
+  }
+  __syncthreads();
+  if (!mean) {  // dv/dy: b_n = b_{n+2} + 2 (n+1) v_{n+1}, b_0 half
+    for (int t = threadIdx.x; t < 2 * W; t += blockDim.x) {
+      const int odd = t >= W, col = t - odd * W;
+      double b = bad[0][col] ? nan : 0.0;
+      Y[(N - odd) * W + col] = odd ? b = fma(2.0 * N, V[N * W + col], b) : b;
+      for (int n = N - odd - 2; n >= 0; n -= 2) {
+        b = fma(2.0 * (n + 1), V[(n + 1) * W + col], b);
+        Y[n * W + col] = n ? b : 0.5 * b;
+      }
+    }
+    __syncthreads();
+  }
+  // u = -i (kx xi + kz eta)/(nu k^2), w = -i (kz xi - kx eta)/(nu k^2), xi = -dv/dy
+  const double ik = I0.ik2nu[m], kxs = kx * ik, kzs = kz * ik, inu = I0.inv_nu;
+  for (int t = threadIdx.x; t < 2 * nI * ny; t += blockDim.x) {
+    const int i = CN.row(t >> 1), part = t & 1, n = (t >> 1) - i * ny, at = n * W + 2 * i;
+    const size_t gc = 2 * (size_t)nm * ny;
+    double* out = reinterpret_cast<double*>(gl.insts[first + i].fhat + (size_t)m * ny + n) + part;
+    if (mean) {
+      out[0] = inu * V[at + part];
+      out[gc] = 0.0;
+      out[2 * gc] = inu * Q[at + part];
+    } else {
+      const double y = Y[at + 1 - part], e = Q[at + 1 - part], a0 = flip(kzs, part != 0), b0 = flip(kxs, part == 0);
+      out[0] = fma(a0, e, b0 * y);
+      out[gc] = inu * V[at + part];
+      out[2 * gc] = fma(b0, e, -a0 * y);
+    }
+  }
 }
 
 __global__ void __launch_bounds__(256, 2) k_ystep_fx(GroupLaunch gl, int op, int synth, int fine) {
@@ -779,6 +891,12 @@ void launch_ysynth_fx(int ctas, int threads, size_t smem, cudaStream_t s, Launch
 void launch_ysolve_fx(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int op, int sig, int fine) {
   k_ysolve_fx<<<ctas, threads, smem, s>>>(gl, op, sig, fine);
 }
+// one pass over the columns of a row each for v and for eta
+int ysolve_f64_threads(int N, int G) { return one_pass(2 * G * (N + 1), 256); }
+size_t smem_ysolve_f64(int N, int G) { return 8 * 5 * (size_t)(N + 1) * 2 * G; }
+void launch_ysolve_f64(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int sig) {
+  k_ysolve_f64<<<ctas, threads, smem, s>>>(gl, sig);
+}
 void launch_ystep_fx(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int op, int synth, int fine) {
   k_ystep_fx<<<ctas, threads, smem, s>>>(gl, op, synth, fine);
 }
@@ -790,11 +908,12 @@ size_t dense_exps_len(int N, int nmodes) { return (size_t)nmodes * 12 * ((N / 2 
 void launch_dense_limbs(const double* src, int N, int nmodes, int4* dst, int* dexp) {
   k_dense_limbs<<<dim3(6, nmodes), 64>>>(src, N / 2 + 1, dst, dexp);
 }
-cudaError_t set_modes_fx_smem(size_t ana, size_t synth, size_t solve, size_t step) {
+cudaError_t set_modes_fx_smem(size_t ana, size_t synth, size_t solve, size_t step, size_t solve64) {
   cudaError_t e;
   if ((e = raise_smem_limit((const void*)k_yana_fx, ana))) return e;
   if ((e = raise_smem_limit((const void*)k_ysynth_fx, synth))) return e;
   if ((e = raise_smem_limit((const void*)k_ysolve_fx, solve))) return e;
+  if ((e = raise_smem_limit((const void*)k_ysolve_f64, solve64))) return e;
   return raise_smem_limit((const void*)k_ystep_fx, step);
 }
 
