@@ -77,6 +77,15 @@ PCF_HD fxc fx_i(fxc v) {
 
 // Arithmetic shift right by r in 0..: amounts of 64 and more give 0 (the value is below a unit).
 PCF_HD fx fx_sra(fx x, int r) { return r > 63 ? 0 : x >> r; }
+// r in 0..31: two shifts
+PCF_HD fx fx_sra31(fx x, int r) {
+#ifdef __CUDA_ARCH__
+  const int lo = (int)(uint32_t)(uint64_t)x, hi = (int)(x >> 32);
+  return ((fx)(hi >> r) << 32) | __funnelshift_r((unsigned)lo, (unsigned)hi, r);
+#else
+  return x >> r;
+#endif
+}
 // Bits of the magnitude: |x| < 2^bits from the high word of x ^ (x >> 63).
 PCF_HD uint32_t fx_maghi(fx x) {
   const int h = (int)(x >> 32);

@@ -10,8 +10,8 @@
 // (a 32 x 32 plane needs 11 k FP64 instructions, 6.7 k clocks of an SM); the integer
 // butterflies of a plane take under 1 k clocks.
 //
-// Measured (us per launch, FP64 Stockham passes -> now): 32 x 33 x 32, batch 8: synthesis 75 -> 28,
-// products M 41 -> 20, N 55 -> 30; 128 x 97 x 128: 1025 -> 205, 381 -> 105, 529 -> 157.
+// Measured (us per launch, FP64 Stockham passes -> now): 32 x 33 x 32, batch 8: synthesis 75 -> 29,
+// products M 41 -> 20, N 55 -> 30; 128 x 97 x 128: 1025 -> 208, 381 -> 105, 529 -> 157.
 //
 // A transform of length L = R S (fx_plan) is two register passes, thread n of S in the first,
 // thread b of R in the second.  Both work in place, so one buffer and one barrier per pass
@@ -231,13 +231,13 @@ size_t smem_planes_fx(const Inst& I, int threads) {
   return sizeof(fxc) * ((size_t)I.Mz * p.LX + (size_t)p.chunk * p.LZ) + 4 * (64 + 64 + 64 + 64);
 }
 // Threads per CTA.  Sides up to 64: the synthesis of small planes keeps two warps busy in every
-// pass (32 x 33 x 32, batch 8: 28 us, with 128 threads 32), larger ones four (64 x 65 x 64, batch
-// 2: 55 us, with 96 threads 62, with 256 58).  The products take all row pairs of a plane in one
+// pass (32 x 33 x 32, batch 8: 29 us, with 128 threads 32), larger ones four (64 x 65 x 64, batch
+// 2: 58 us, with 96 threads 62, with 256 58).  The products take all row pairs of a plane in one
 // pass: with few CTAs per SM the loads of their factors are what the time goes to (64 x 65 x 64,
 // batch 2: 37 and 51 us with 256 threads, 41 and 67 with 128; 48 x 49 x 48, batch 4: 29 and 41 us
 // with 192, 30 and 45 with 128, 35 and 58 with 256; 32 x 33 x 32, batch 8: 20 and 30 us with
 // 128, 25 and 36 with 256).  Longer sides: the plane's x rows fill much of the shared memory, so
-// the smallest CTA that leaves the SM the most threads (128 x 97 x 128: synthesis 205 us with 512
+// the smallest CTA that leaves the SM the most threads (128 x 97 x 128: synthesis 208 us with 512
 // threads; before the single-precision bound 233 with 512, 280 with 256, 397 with 128; 96 x 31 x
 // 48, batch 3: 56 us with 128); the products take at least 256 (there 40 and 51 us, with 128
 // threads 47 and 62).
@@ -262,7 +262,12 @@ __constant__ int c_fx_fac[kFieldsSynth] = {0, 0, 0, 1, 0, 2, 1, 2, 1, 0, 2};
 // ------------------------------------------------------------------ plane synthesis
 // CTA = (instance, y-plane j, field f): u, v, w, u_x, u_y, u_z, v_x, v_z, w_x, w_y, w_z.  The
 // plane's exponent e0 comes from the sum B of |Re| + |Im| over the plane's modes (p > 0 twice):
-// every intermediate of the two transforms is below 2 B in modulus, and 2 B 2^-e0 < 2^62.
+// every intermediate of the two transforms is below 2 B in modulus, and 2 B 2^-e0 < 2^62.  The x
+// stage runs each row p (a z mode) at an exponent of its own, from the row's largest value, and its
+// results are rounded to e0: at e0 the rounding of the inputs, summed over all the modes, would be
+// ten times the rounding of the rest (a flat spectrum at 128 x 33 x 128: modes of r1 off by 2.9e-15 of
+// themselves in the median; 6.4e-16 with row exponents, 9.2e-16 in FP64 arithmetic; 32 x 33 x 32, batch
+// 8: 28 -> 29 us, 128 x 97 x 128: 205 -> 208).
 template <int KIND>
 __global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_synth_fx(LaunchInfo li, int slot, int nfields) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -276,6 +281,7 @@ __global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_syn
   fxc* G = reinterpret_cast<fxc*>(smraw);
   fxc* Z = G + Mz * P.LX;
   int* red = reinterpret_cast<int*>(Z + P.chunk * P.LZ);
+  int* row = red + 64;  // exponents of the rows p
   const double2* src = I.yv + (((size_t)slot * kFieldsY + c_fx_src[f]) * I.ny + j) * (size_t)nm;
   const int fac = c_fx_fac[f];
   // Bound of the plane: one pass in single precision (a pass for the largest exponent and one
@@ -283,6 +289,8 @@ __global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_syn
   const unsigned mzm = I.mz_mul;
   FxSum sum;
   unsigned any = 0;
+  for (int p = threadIdx.x; p < Mz; p += blockDim.x) row[p] = 0;
+  __syncthreads();
   for (int t0 = threadIdx.x; t0 < nm; t0 += 4 * blockDim.x) {
     double2 s[4];
 #pragma unroll
@@ -294,7 +302,11 @@ __global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_syn
       any = max(any, (unsigned)max(hx, hy));
       // |k| in units of the smallest wavenumber
       const int k = fac == 0 ? 1 : fac == 1 ? (i <= Kx ? i : I.Mx - i) : p;
-      if (t < nm && k) sum.add(hx, hy, (float)(p ? 2 * k : k));
+      if (t < nm && k) {
+        sum.add(hx, hy, (float)(p ? 2 * k : k));
+        const int m = max(hx, hy) >> 20, e = m + (fac ? 32 - __clz(k) : 0);
+        if (m && e > row[p]) atomicMax(row + p, e);
+      }
     }
   }
   const int k1 = fac == 0 ? 0x3ff00000 : __double2hiint(fac == 1 ? I.kx[1] : I.kz[1]), ek = fx_bexp(k1);
@@ -311,16 +323,22 @@ __global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_syn
   }
   const int e0 = eb + ek - 61;
   const FxPlan px = fx_plan_of<KIND>(nx);
+  // a row's values are below 2^(row - 1022) (times 2^(ek + 1) for a derivative) in each part, and a
+  // transform of its Mx modes below 2^cr times that
+  const int cr = 32 - __clz((3 * I.Mx) >> 1) - 1022 - 62 + (fac ? ek + 1 : 0);
+  for (int p = threadIdx.x; p < Mz; p += blockDim.x) row[p] = max(min(row[p] + cr, e0), e0 - 31);
+  __syncthreads();
   // the modes as integers at their x bins (rows p); i k v for the x and z derivatives
   for (int t = threadIdx.x; t < nm; t += blockDim.x) {
     const double2 s = src[t];
     const int i = fx_div(t, mzm), p = t - i * Mz, bin = xbin(i, Kx, I.Mx, nx);
+    const int e = row[p];
     fxc v;
     if (fac == 0) {
-      v = fxc{fx_from(s.x, e0), fx_from(s.y, e0)};
+      v = fxc{fx_from(s.x, e), fx_from(s.y, e)};
     } else {
       const FxK k = fx_factor(fac == 1 ? I.kx[i] : I.kz[p]);
-      v = fxc{fx_from_k(s.y, k, e0, -1), fx_from_k(s.x, k, e0, 0)};
+      v = fxc{fx_from_k(s.y, k, e, -1), fx_from_k(s.x, k, e, 0)};
     }
     G[p * P.LX + fx_in<KIND>(px, bin)] = v;
   }
@@ -338,8 +356,10 @@ __global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_syn
     __syncthreads();
     fx_second<R, S, true>(Mz, G, P.LX, [&](int p, int bk, const fxc* v) {
       fxc* o = G + p * P.LX;
+      const int d = e0 - row[p];
+      const unsigned h = (1u << d) >> 1;
 #pragma unroll
-      for (int e = 0; e < S; ++e) o[fx_slot<S>(bk, e)] = v[e];
+      for (int e = 0; e < S; ++e) o[fx_slot<S>(bk, e)] = fxc{fx_sra31(v[e].x + h, d), fx_sra31(v[e].y + h, d)};
     });
   });
   __syncthreads();
