@@ -77,6 +77,8 @@ PCF_HD fxc fx_i(fxc v) {
 
 // Arithmetic shift right by r in 0..: amounts of 64 and more give 0 (the value is below a unit).
 PCF_HD fx fx_sra(fx x, int r) { return r > 63 ? 0 : x >> r; }
+// a 2^-r to the nearest, 0 <= a < 2^62, r >= 0; r > 63 gives 0
+PCF_HD fx fx_round(fx a, int r) { return r > 63 ? 0 : (a + (fx)((1ULL << r) >> 1)) >> r; }
 // r in 0..31: two shifts
 PCF_HD fx fx_sra31(fx x, int r) {
 #ifdef __CUDA_ARCH__
@@ -107,6 +109,18 @@ PCF_HD int fx_clz64(uint64_t v) {
 }
 // |x| < 2^fx_bits(maghi): 64 - clz of the 64-bit magnitude with a low word of ones
 PCF_HD int fx_bits(uint32_t maghi) { return 64 - fx_clz32(maghi); }
+
+// Words of a matrix-vector product, x = h 2^28 + l with |l| <= 2^27: for entries up to 2^57 and columns
+// whose magnitudes sum to less than 2^59 both words are 32-bit, and for up to 65 terms the sums of
+// h h' (below 2^60) and of h l' + l h' (below 2^63) are exact.  l l' is left out: at most 65 2^54 of
+// the 2^116 that the largest entry times the column's sum stand for, 2^-56 of it (random words: 2^-61).
+// Split at 29 bits it was 2^-54.
+PCF_HD void fx_words(fx x, int* h, int* l) {
+  *h = (int)((x + (1 << 27)) >> 28);
+  *l = (int)(x - ((fx)*h << 28));
+}
+// h h' and cross sums -> units of 2^55
+PCF_HD fx fx_fold(fx h, fx c) { return (h << 1) + ((c + (1 << 26)) >> 27); }
 
 // Nearest double to x 2^e, by integer instructions (an FP64 conversion and scaling occupy the
 // FP64 pipe for as long as 60 integer instructions); exponents outside the normal range give

@@ -90,7 +90,7 @@ std::vector<double> make_cheb(int N) {
 }
 
 // Fixed-point Chebyshev tables (FxTab): columns k of row pairs (2 rp, 2 rp + 1), entries in
-// units of 2^-57 split into 29-bit words.  Analysis (Ae, Ao): coefficient 2k or 2k + 1 from the
+// units of 2^-57 split into words at 28 bits.  Analysis (Ae, Ao): coefficient 2k or 2k + 1 from the
 // folded sums, scaled by a power of two so that the largest entry stays at or below 1 (*exp:
 // exponent of a product's unit, 2^55 of theirs, relative to the column's); synthesis
 // (Ce, Co): T_{2k}(y_j), T_{2k+1}(y_j).
@@ -104,8 +104,9 @@ std::vector<int4> make_fxcheb(int N, int* exp) {
   };
   auto words = [](long double v) {
     const long long z = std::llrint(std::ldexp(v, 57));
-    const int h = (int)((z + (1 << 28)) >> 29);
-    return make_int2(h, (int)(z - ((long long)h << 29)));
+    int2 w;
+    fx_words(z, &w.x, &w.y);
+    return w;
   };
   std::vector<int4> t;
   auto block = [&](int K, int rows, int hp, auto&& entry) {

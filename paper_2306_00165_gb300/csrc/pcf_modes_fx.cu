@@ -11,13 +11,15 @@
 //
 // Every product is a matrix (the same for all columns of a CTA) times columns.  A column's
 // values are integers of one exponent, scaled so that the sum of their magnitudes is just below
-// 2^59, and split into two words, x = xh 2^29 + xl; a matrix row's entries are below 2^57, split
-// the same way.  A product element is
-//   2^58 sum(ah xh) + 2^29 sum(ah xl + al xh)
-// with both sums exact in 64 bits for up to 65 terms (sum |xh| <= 2^30, so the first stays below
-// 2^59 and the second below 2^63; the words' low product is below 2^-58 of the whole): three
-// 32 x 32 + 64 multiply-adds per term, 0.12 clocks of an SM where an FP64 multiply-add takes
-// 0.60.  The unit is 2^-61 of (largest entry of the row) x (sum of the column's magnitudes).
+// 2^59, and split into two words, x = xh 2^28 + xl; a matrix row's entries are at most 2^57, split the
+// same way.  A product element is
+//   2^56 sum(ah xh) + 2^28 sum(ah xl + al xh)
+// with both sums exact in 64 bits for up to 65 terms (fx_words): three 32 x 32 + 64 multiply-adds per
+// term, 0.12 clocks of an SM where an FP64 multiply-add takes 0.60.  In units of (largest entry of the
+// row) x (sum of the column's magnitudes) the entries are rounded at 2^-58, the column is cut at
+// 2^-59, the words' low product is at most 2^-56 (typically 2^-61) and the result's unit is 2^-61:
+// finer than FP64's rounding of the largest terms, but the same for every element, so that a
+// coefficient far below its column's sum has fewer digits than FP64 would give it.
 // Scaling from the sum, and not from K times the largest value, is what keeps the solve's error
 // at FP64's: r1 = (u+ - u)/dt cancels the leading digits of u+.  Sums are exact, so every
 // organisation gives the same bits.
@@ -55,7 +57,7 @@ __device__ __forceinline__ int mag(int hi, int n, int eb, int ecm) {
   const int d = ecm - eb;
   return eb <= 0 || d > 27 ? 0 : (int)(m >> d) + 1;
 }
-// v in units of 2^(q - 1096): the sum of the column's magnitudes is below 2^59
+// v in units of 2^(q - 1096), to the nearest: the sum of the column's magnitudes is below 2^59
 __device__ __forceinline__ fx col_fx(double v, int q) {
   const int hi = __double2hiint(v), ec = (hi >> 20) & 0x7ff, r = q - 15 - ec;
   const fx m = ((fx)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
@@ -68,8 +70,10 @@ __device__ __forceinline__ double fx_out(fx s, int e) {
                         : __longlong_as_double((long long)fx_double_bits(s, e));
 }
 __device__ __forceinline__ int4 limbs(fx re, fx im) {
-  const int rh = (int)((re + (1 << 28)) >> 29), ih = (int)((im + (1 << 28)) >> 29);
-  return make_int4(rh, (int)(re - ((fx)rh << 29)), ih, (int)(im - ((fx)ih << 29)));
+  int4 w;
+  fx_words(re, &w.x, &w.y);
+  fx_words(im, &w.z, &w.w);
+  return w;
 }
 // sums of two rows (0, 1) x (re, im): high and cross products
 struct Acc {
@@ -89,8 +93,6 @@ __device__ __forceinline__ void mac(Acc& a, int4 m, int4 x) {
   a.c3 += (fx)m.z * x.w;
   a.c3 += (fx)m.w * x.z;
 }
-// in units of 2^55
-__device__ __forceinline__ fx fold(fx h, fx c) { return (h << 3) + ((c + (1 << 25)) >> 26); }
 // rows 2 rp, 2 rp + 1 of a matrix (column k at A + k hp + rp) times column x (element k at x + k s)
 __device__ __forceinline__ Acc dot(const int4* __restrict__ A, int hp, const int4* x, int s, int K) {
   Acc a;
@@ -128,7 +130,7 @@ __device__ __forceinline__ fx dot_fine(const int2* __restrict__ A, int sa, const
     c += (fx)m.x * v.y;
     c += (fx)m.y * v.x;
   }
-  return fold(h, c);
+  return fx_fold(h, c);
 }
 __device__ __forceinline__ const int2* words(const int4* p, int half) { return reinterpret_cast<const int2*>(p) + half; }
 
@@ -227,9 +229,9 @@ __device__ __forceinline__ void ana_mac(const double2* X, const Cols& C, int N, 
                        : dot(tab + T.Ao() + rp, T.hO, x0 + N * C.pitch + col, -C.pitch, T.half);
     const int er = dot_exp(cm[2 * col], ea), ei = dot_exp(cm[2 * col + 1], ea);
     const int n0 = 4 * rp + (even ? 0 : 1), rows = even ? T.H : T.half;
-    *out(col, n0) = make_double2(fx_out(fold(a.h0, a.c0), er), fx_out(fold(a.h1, a.c1), ei));
+    *out(col, n0) = make_double2(fx_out(fx_fold(a.h0, a.c0), er), fx_out(fx_fold(a.h1, a.c1), ei));
     if (2 * rp + 1 < rows)
-      *out(col, n0 + 2) = make_double2(fx_out(fold(a.h2, a.c2), er), fx_out(fold(a.h3, a.c3), ei));
+      *out(col, n0 + 2) = make_double2(fx_out(fx_fold(a.h2, a.c2), er), fx_out(fx_fold(a.h3, a.c3), ei));
   }
 }
 
@@ -318,9 +320,9 @@ __device__ __forceinline__ void syn_mac(const double2* X, const Cols& C, int N, 
   for (int t = threadIdx.x; t < C.n * T.hE; t += blockDim.x) {
     const int rp = C.row(t), col = t - rp * C.n;
     const Acc e = dot(tab + T.Ce() + rp, T.hE, x0 + col, 2 * C.pitch, KE);
-    const fx e0 = fold(e.h0, e.c0), e1 = fold(e.h1, e.c1), e2 = fold(e.h2, e.c2), e3 = fold(e.h3, e.c3);
+    const fx e0 = fx_fold(e.h0, e.c0), e1 = fx_fold(e.h1, e.c1), e2 = fx_fold(e.h2, e.c2), e3 = fx_fold(e.h3, e.c3);
     const Acc o = dot(tab + T.Co() + rp, T.hE, x0 + C.pitch + col, 2 * C.pitch, T.half);
-    const fx o0 = fold(o.h0, o.c0), o1 = fold(o.h1, o.c1), o2 = fold(o.h2, o.c2), o3 = fold(o.h3, o.c3);
+    const fx o0 = fx_fold(o.h0, o.c0), o1 = fx_fold(o.h1, o.c1), o2 = fx_fold(o.h2, o.c2), o3 = fx_fold(o.h3, o.c3);
     const int er = unit(2 * col), ei = unit(2 * col + 1), j = 2 * rp;
     put(col, j, 2, fx_out(e0 + o0, er), fx_out(e1 + o1, ei));
     if (j < T.half) put(col, N - j, 2, fx_out(e0 - o0, er), fx_out(e1 - o1, ei));
@@ -427,8 +429,8 @@ __device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI,
     }
     if (2 * rp >= rows) continue;
     const Acc a = dot(A, hp, x, 2 * nI, K);
-    o[0] = make_longlong2(fold(a.h0, a.c0), fold(a.h1, a.c1));
-    if (2 * rp + 1 < rows) o[2 * nI] = make_longlong2(fold(a.h2, a.c2), fold(a.h3, a.c3));
+    o[0] = make_longlong2(fx_fold(a.h0, a.c0), fx_fold(a.h1, a.c1));
+    if (2 * rp + 1 < rows) o[2 * nI] = make_longlong2(fx_fold(a.h2, a.c2), fx_fold(a.h3, a.c3));
   }
   __syncthreads();
   // v = Av f_v + Ag g at the larger exponent, eta; as doubles in R3[0], R3[2] (mean: u, w)
@@ -824,11 +826,11 @@ __global__ void __launch_bounds__(32) k_jnorm(const Inst* insts, int step_index)
   if (I.tol > 0.0 && J < I.tol && I.active) *I.active = 0;
 }
 
-// A matrix entry in units where its row's largest (biased exponent e) is just below 2^57
+// A matrix entry in units where its row's largest (biased exponent e) is below 2^57, to the nearest
 __device__ __forceinline__ fx row_fx(double v, int e) {
   const int hi = __double2hiint(v), ec = (hi >> 20) & 0x7ff, r = e - ec;
   const fx m = ((fx)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
-  return neg_if(ec == 0 || r > 63 ? 0 : (m << 4) >> r, hi);
+  return neg_if(ec == 0 ? 0 : fx_round(m << 4, r), hi);
 }
 // Dense operators (DenseLayout) of every mode as limbs: block bl of mode m in CTA (bl, m), with
 // each row's exponent.

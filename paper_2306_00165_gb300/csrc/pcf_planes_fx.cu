@@ -128,8 +128,6 @@ __device__ __forceinline__ fx fx_signed(fx a, int neg) {
   const fx m = (fx)neg;
   return (a ^ m) - m;
 }
-// a 2^-r to the nearest, 0 <= a < 2^62; r > 63 gives 0
-__device__ __forceinline__ fx fx_round(fx a, int r) { return r > 63 ? 0 : (a + (fx)((1ULL << r) >> 1)) >> r; }
 // v 2^-e0 to the nearest, where |v| 2^-e0 < 2^61
 __device__ __forceinline__ fx fx_from(double v, int e0) {
   const int hi = __double2hiint(v), ec = (hi >> 20) & 0x7ff;
