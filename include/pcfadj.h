@@ -23,7 +23,8 @@
  *
  * Memory: unless an argument says "host", every pointer is a DEVICE pointer owned
  * by the caller; the library never frees it.  The context owns its workspace and
- * tables (allocated once in pcf_create).
+ * tables (allocated in pcf_create; what only pcf_dns, the *_host variants, the snapshot and the DMD
+ * calls need is allocated at the first of them and kept).
  *
  * Streams: every call is enqueued on the stream given to pcf_create and returns
  * without synchronising, except where noted (pcf_dmd_extrapolate and the *_host

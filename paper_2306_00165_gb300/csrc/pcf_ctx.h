@@ -82,7 +82,8 @@ struct pcf_ctx {
   double2* u_dev = nullptr;    // device state for the *_host entry point
   double* hist_dev = nullptr;
   int hist_cap = 0;
-  int* active = nullptr;
+  int* active = nullptr;  // convergence masks of a run
+  int* first = nullptr;   // mask of pcf_residual_first (a run's DMD jump keeps the run's masks)
   std::map<int, cudaGraphExec_t> graphs;
   // symmetric subspace and DNS
   bool any_sym = false;         // some instance enforces a symmetry
@@ -114,3 +115,5 @@ struct pcf_ctx {
 
 // A context over `batch` instances of c's (first) problem that shares c's tables: workspace only.
 pcf_status pcf_make_child(pcf_ctx* c, int batch, pcf_ctx** out);
+// pcf_residual of the first n instances; the others' outputs are not defined.
+pcf_status pcf_residual_first(pcf_ctx* c, int n, const double* u, double* r, double* rnorm);

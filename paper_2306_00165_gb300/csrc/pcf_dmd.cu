@@ -351,7 +351,8 @@ pcf_status ensure_indep(pcf_ctx* c) {
 pcf_status ensure_dmd(pcf_ctx* c, int ncol) {
   if (c->dmd_cap >= ncol) return PCF_OK;
   const int cap = std::max(ncol, 32);
-  const int ncand = cap + std::max(c->B, 32);  // whole batches of either evaluation context
+  // whole batches of either evaluation context (norms of the masked instances are written too)
+  const int ncand = cap + std::max(c->B, 32);
   double *A, *part, *coef, *cpsi, *J, *cc;
   double2* cu;
   DMD_CUDA(cudaMalloc(&A, sizeof(double) * (size_t)c->psi_len * cap));
@@ -444,12 +445,13 @@ pcf_status snapshot_r(pcf_ctx* c, const double* S, long long ld, int ncol, std::
   return PCF_OK;
 }
 
-// Context that evaluates the candidates' residuals, up to `want` at a time: c itself, or one over
-// more instances of the same problem (at most 32, within 1 GiB of plane buffers), made on first use
-// and kept with c.  One candidate per pass left the GPU mostly idle: 19 passes of 90 us.
+// Context that evaluates `want` candidates' residuals, all or many at a time: c itself, or one over
+// more instances of the same problem (multiples of four, at most 32, within 1 GiB of plane buffers),
+// made on first use and kept with c until it or a call with more candidates ends it.  One candidate
+// per pass left the GPU mostly idle: 19 passes of 90 us.
 pcf_ctx* eval_ctx(pcf_ctx* c, int want) {
   const long long per = 2LL * kFieldsSynth * c->prm.nx * c->prm.ny * c->prm.nz * 8;
-  const int nb = (int)std::min<long long>(std::min(want, 32), (1LL << 30) / per);
+  const int nb = (int)std::min<long long>(std::min((want + 3) / 4 * 4, 32), (1LL << 30) / per);
   if (nb <= c->B) return c;
   if (c->dmd_eval && c->dmd_eval->B < nb) {
     pcf_destroy(c->dmd_eval);
@@ -594,29 +596,28 @@ pcf_status pcf_dmd_extrapolate(pcf_ctx* c, const double* S, long long ld, int M,
       rank_of[ncand++] = rstar - k;
     }
   if (ncand == 0) return PCF_ENAN;
-  // candidate states on the device, padded to whole batches with the last candidate
-  pcf_ctx* ev = eval_ctx(c, M);
-  const int nb = (ncand + ev->B - 1) / ev->B * ev->B;
-  Cc.resize((size_t)nb * M);
-  for (int k = ncand; k < nb; ++k) std::copy_n(Cc.data() + (size_t)(ncand - 1) * M, M, Cc.data() + (size_t)k * M);
-  DMD_CUDA(cudaMemcpyAsync(c->dmd_c, Cc.data(), sizeof(double) * (size_t)nb * M, cudaMemcpyHostToDevice, c->cs));
-  k_combine<<<dim3((unsigned)std::min<long long>((rows + 255) / 256, 2048), (nb + 3) / 4), 256, 0, c->cs>>>(
-      S, rows, ld, M, c->dmd_c, nb, c->dmd_cpsi, rows);
+  // candidate states on the device; the instances past the last candidate are masked (evaluating
+  // copies of it instead, a call of rank 2 took as long as one of rank 20)
+  pcf_ctx* ev = eval_ctx(c, ncand);
+  DMD_CUDA(cudaMemcpyAsync(c->dmd_c, Cc.data(), sizeof(double) * (size_t)ncand * M, cudaMemcpyHostToDevice, c->cs));
+  k_combine<<<dim3((unsigned)std::min<long long>((rows + 255) / 256, 2048), (ncand + 3) / 4), 256, 0, c->cs>>>(
+      S, rows, ld, M, c->dmd_c, ncand, c->dmd_cpsi, rows);
   DMD_CUDA(cudaGetLastError());
   {
-    const int n = nb * (c->nindep + 1);
+    const int n = ncand * (c->nindep + 1);
     k_psi_rebuild<<<(n + kRebuildWarps - 1) / kRebuildWarps, 32 * kRebuildWarps, 0, c->cs>>>(
         c->dmd_cpsi, rows, c->dmd_cu, c->state_len, c->d_indep, c->nindep, c->hinst[0].kx, c->hinst[0].kz, c->Mx,
-        c->Mz, c->prm.ny, c->nm, nb);
+        c->Mz, c->prm.ny, c->nm, ncand);
     DMD_CUDA(cudaGetLastError());
   }
   DMD_CUDA(cudaEventRecord(c->ev_out, c->cs));
   DMD_CUDA(cudaStreamWaitEvent(c->user, c->ev_out, 0));
-  std::vector<double> Jc(nb);
-  for (int g = 0; g < nb; g += ev->B) {
-    DMD_TRY(pcf_residual(ev, (const double*)(c->dmd_cu + (size_t)g * c->state_len), (double*)ev->r_int, c->dmd_J + g));
+  std::vector<double> Jc(ncand);
+  for (int g = 0; g < ncand; g += ev->B) {
+    DMD_TRY(pcf_residual_first(ev, std::min(ev->B, ncand - g), (const double*)(c->dmd_cu + (size_t)g * c->state_len),
+                               (double*)ev->r_int, c->dmd_J + g));
   }
-  DMD_CUDA(cudaMemcpyAsync(Jc.data(), c->dmd_J, sizeof(double) * nb, cudaMemcpyDeviceToHost, c->user));
+  DMD_CUDA(cudaMemcpyAsync(Jc.data(), c->dmd_J, sizeof(double) * ncand, cudaMemcpyDeviceToHost, c->user));
   DMD_CUDA(cudaStreamSynchronize(c->user));
   int bi = -1;
   for (int k = 0; k < ncand; ++k)  // candidates are ordered by decreasing rank: ties keep the larger r

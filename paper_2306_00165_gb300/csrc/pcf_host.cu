@@ -565,15 +565,15 @@ pcf_status launch_fused_step(pcf_ctx* c, int op, int synth) {
 pcf_status launch_split_jnorm(pcf_ctx* c, int step_index) {
   return timed(c, 9, [&] { launch_jnorm(c->B, c->cs, c->dinst, step_index); });
 }
-// y-synthesis of the state (slot 0) or of r1 (slot 1) in either form; in_step: masked instances
-// are left out; nf: five fields, or three (the values, without y-derivatives)
+// y-synthesis of the state (slot 0) or of r1 (slot 1) in either form; in_step: counted in the
+// step's class; nf: five fields, or three (the values, without y-derivatives)
 pcf_status launch_ysynth(pcf_ctx* c, int slot, int in_step = 0, bool red = false, int nf = kFieldsY) {
   if (c->mixed) return launch_tc_synth(c, slot);
   if (!c->split) return launch_mode(c, MODE_SYNTH_ONLY, slot);
   return timed(c, in_step ? 8 : 0, [&] {
     const int* pre = nf == 3 ? c->pre_ya : red ? c->pre_yy_r : c->pre_yy;
     const int ctas = nf == 3 ? c->cta_ya : red ? c->cta_yy_r : c->cta_yy;
-    launch_ysynth_fx(ctas, c->thr_yy, c->sm_yy, c->cs, li_of(c, pre, ctas), slot, nf, in_step, c->np, red ? 1 : 0,
+    launch_ysynth_fx(ctas, c->thr_yy, c->sm_yy, c->cs, li_of(c, pre, ctas), slot, nf, c->np, red ? 1 : 0,
                      c->fine_y);
   });
 }
@@ -1160,7 +1160,7 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
   int* jc = nullptr;
   int2* pin = nullptr;
   if (ctx_alloc(c, &np, n_np) || ctx_alloc(c, &c->r_int, (size_t)c->total_state) ||
-      ctx_alloc(c, &c->active, (size_t)B) || ctx_alloc(c, &jc, (size_t)B))
+      ctx_alloc(c, &c->active, (size_t)B) || ctx_alloc(c, &c->first, (size_t)B) || ctx_alloc(c, &jc, (size_t)B))
     return fail(PCF_ENOMEM);
   if (cudaMemset(jc, 0, sizeof(int) * B) != cudaSuccess) return fail(PCF_ECUDA);
   if (c->mixed) {
@@ -1360,8 +1360,19 @@ void pcf_destroy(pcf_ctx* c) {
 
 pcf_status pcf_residual(pcf_ctx* c, const double* u, double* r, double* rnorm) {
   if (!c || !u || !r) return PCF_EINVAL;
+  return pcf_residual_first(c, c->B, u, r, rnorm);
+}
+
+}  // extern "C"
+pcf_status pcf_residual_first(pcf_ctx* c, int n, const double* u, double* r, double* rnorm) {
   set_pointers(c, u, r, nullptr);
   PCF_TRY(enter(c));
+  if (n < c->B) {
+    std::vector<int> mask(c->B, 0);
+    std::fill_n(mask.begin(), n, 1);
+    for (int b = 0; b < c->B; ++b) c->hinst[b].active = c->first + b;
+    PCF_CUDA(cudaMemcpyAsync(c->first, mask.data(), sizeof(int) * c->B, cudaMemcpyHostToDevice, c->cs));
+  }
   PCF_TRY(push_descriptors(c));
   PCF_TRY(launch_ysynth(c, 0));
   PCF_TRY(launch_synth(c, 0, kFieldsSynth));
@@ -1377,6 +1388,7 @@ pcf_status pcf_residual(pcf_ctx* c, const double* u, double* r, double* rnorm) {
   PCF_TRY(check_launch());
   return leave(c);
 }
+extern "C" {
 
 pcf_status pcf_adjoint_gradient(pcf_ctx* c, const double* u, const double* r, double* f) {
   if (!c || !u || !r || !f) return PCF_EINVAL;

@@ -192,7 +192,7 @@ size_t smem_ystep_fx(int N, int G);
 // red: the modes m >= 0 only (a state invariant under s2); the synthesis mirrors their y-values
 void launch_yana_fx(int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int np, int red, int fine);
 void launch_ysynth_fx(int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf,
-                      int check_active, int np, int red, int fine);
+                      int np, int red, int fine);
 void launch_ysolve_fx(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int op, int sig, int fine);
 // the solve of a given right-hand side (MODE_SOLVE), in FP64
 int ysolve_f64_threads(int N, int G);

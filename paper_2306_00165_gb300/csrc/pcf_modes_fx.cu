@@ -344,9 +344,9 @@ __device__ __forceinline__ double flip(double x, bool neg) {
   return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
 }
 // One mode, nI instances (columns).  coef(i, c, n, part): Chebyshev coefficient of the products.  C3, R3: [3][ny][nI] arrays; sm_i: 16 nI ints.  done(i, c, n, part, new value) receives
-// r1 (PHI), the updated state (PSI_UPDATE) or f.
+// r1 (PHI), the updated state (PSI_UPDATE) or f.  alive: false in every thread when live is all zero.
 template <class COEF, class DONE>
-__device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI, int m, int op, int sig, const int* live,
+__device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI, int m, int op, int sig, bool alive, const int* live,
                                            double2* C3, double2* R3, int* sm_i, bool fine, const COEF& coef, const DONE& done) {
   const Inst& I0 = insts[first];
   const int N = I0.N, ny = I0.ny, nm = I0.nmodes, Mz = I0.Mz, Mh = N / 2 + 1, hp = (Mh + 1) / 2;
@@ -361,7 +361,7 @@ __device__ __forceinline__ void solve_mode(const Inst* insts, int first, int nI,
   const bool mean = m == 0;
   const double ist = sig == 0 ? I0.inv_dt : I0.inv_dtau_hat;
   const bool in_u = op == MODE_PHI;
-  __syncthreads();
+  if (!__syncthreads_or(alive)) return;
   // S = state/step + product; f_v = S_v, g = i (kx S_u + kz S_w), h = i (kz S_u - kx S_w); mean
   // mode: S_u and S_w (all times nu: the factor 1/nu is in the outputs)
   // One thread per (instance, n, part): an FP64 instruction occupies its quarter of the SM for 77
@@ -574,12 +574,12 @@ __global__ void __launch_bounds__(320, 3) k_yana_fx(LaunchInfo li, int np, int r
 }
 
 // Fields 0 .. nf - 1 (nf = 5, or 3 for the values alone).
-__global__ void __launch_bounds__(320, 3) k_ysynth_fx(LaunchInfo li, int slot, int nf, int check_active, int np, int red, int fine) {
+__global__ void __launch_bounds__(320, 3) k_ysynth_fx(LaunchInfo li, int slot, int nf, int np, int red, int fine) {
   extern __shared__ __align__(16) double2 smx[];
   int local;
   const int b = find_inst(li, blockIdx.x, &local);
   const Inst& I = li.insts[b];
-  if (check_active && !inst_active(I)) return;
+  if (!inst_active(I)) return;
   const int N = I.N, ny = I.ny, nm = I.nmodes, nrun = red ? (I.Kx + 1) * I.Mz : nm;
   const int tile = local / nf, q = local - nf * tile, m0 = tile * np, c = field_comp(q);
   const bool deriv = q >= 3;
@@ -624,10 +624,11 @@ __global__ void __launch_bounds__(256, 3) k_ysolve_fx(GroupLaunch gl, int op, in
   const int2 grp = gl.groups[find_group(gl, blockIdx.x, &m)];
   const int first = grp.x, nI = grp.y;
   const Inst& I0 = gl.insts[first];
-  if (threadIdx.x < nI) live[threadIdx.x] = inst_active(gl.insts[first + threadIdx.x]);
+  bool alive = false;
+  if (threadIdx.x < nI) live[threadIdx.x] = alive = inst_active(gl.insts[first + threadIdx.x]);
   const int AS = I0.ny * nI, ny = I0.ny, nm = I0.nmodes;
   int* smi = reinterpret_cast<int*>(smx + 6 * AS);
-  solve_mode(gl.insts, first, nI, m, op, sig, live, smx, smx + 3 * AS, smi, fine != 0,
+  solve_mode(gl.insts, first, nI, m, op, sig, alive, live, smx, smx + 3 * AS, smi, fine != 0,
              [&](int i, int c, int n, int part) {
                return reinterpret_cast<const double*>(gl.insts[first + i].xc)[2 * (((size_t)c * nm + m) * ny + n) + part];
              },
@@ -778,7 +779,7 @@ __global__ void __launch_bounds__(256, 2) k_ystep_fx(GroupLaunch gl, int op, int
     return Y + c * AS + n * nI + i;
   });
   __syncthreads();
-  solve_mode(gl.insts, first, nI, m, op, op == MODE_PHI ? 0 : 1, live, X, R, smi, fine != 0,
+  solve_mode(gl.insts, first, nI, m, op, op == MODE_PHI ? 0 : 1, true, live, X, R, smi, fine != 0,
              [&](int i, int c, int n, int part) { return reinterpret_cast<const double*>(Y + c * AS + n * nI + i)[part]; },
              [&](int i, int c, int n, int part, double v) {
                reinterpret_cast<double*>(Y + c * AS + n * nI + i)[part] = v;
@@ -887,8 +888,8 @@ void launch_yana_fx(int ctas, int threads, size_t smem, cudaStream_t s, LaunchIn
   k_yana_fx<<<ctas, threads, smem, s>>>(li, np, red, fine);
 }
 void launch_ysynth_fx(int ctas, int threads, size_t smem, cudaStream_t s, LaunchInfo li, int slot, int nf,
-                      int check_active, int np, int red, int fine) {
-  k_ysynth_fx<<<ctas, threads, smem, s>>>(li, slot, nf, check_active, np, red, fine);
+                      int np, int red, int fine) {
+  k_ysynth_fx<<<ctas, threads, smem, s>>>(li, slot, nf, np, red, fine);
 }
 void launch_ysolve_fx(int ctas, int threads, size_t smem, cudaStream_t s, GroupLaunch gl, int op, int sig, int fine) {
   k_ysolve_fx<<<ctas, threads, smem, s>>>(gl, op, sig, fine);

@@ -694,6 +694,7 @@ __global__ void __launch_bounds__(128) k_norm_planes_fx(LaunchInfo li, int slot)
   int local;
   const int b = find_inst(li, blockIdx.x, &local);
   const Inst& I = li.insts[b];
+  if (!inst_active(I)) return;
   const int c = local % 3, j = local / 3, n = I.nx * I.nz;
   const int2 inf = *fx_info(I, slot, c, j);
   const int e = fx_e62(inf), sa = 62 - inf.y;
