@@ -1,6 +1,9 @@
 // Context of the pcfadj library (internal; shared by the host translation units).
 #pragma once
+#include <atomic>
 #include <map>
+#include <memory>
+#include <thread>
 #include <vector>
 
 #include "pcf_kernels.cuh"
@@ -109,6 +112,12 @@ struct pcf_ctx {
   double* dmd_J = nullptr;      // candidate norms (batch)
   double* dmd_c = nullptr;      // candidate coefficient vectors (device)
   pcf_ctx* dmd_eval = nullptr;  // context over a batch of candidates on this problem's tables
+  // host threads of DMD calls, joined by a later call or with the context
+  struct Helper {
+    std::thread thread;
+    std::shared_ptr<std::atomic<bool>> ended;
+  };
+  std::vector<Helper> helpers;
   int dmd_cap = 0;              // columns the DMD workspace holds
   int dmd_ncand_cap = 0;
 };

@@ -15,7 +15,10 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <condition_variable>
 #include <cstdio>
+#include <memory>
+#include <mutex>
 #include <thread>
 #include <vector>
 
@@ -464,6 +467,100 @@ pcf_ctx* eval_ctx(pcf_ctx* c, int want) {
   return c->dmd_eval ? c->dmd_eval : c;
 }
 
+// The candidates of all ranks: independent small dense problems (about 60 us apiece at 20 snapshots),
+// taken one by one by the calling thread and by up to seven helpers.  The call waits for the ranks and
+// not for the helpers, which a later call or pcf_destroy joins: on busy cores a helper may get its
+// first time slice only milliseconds later (joined at once, a jump of rank 6 at 32 x 33 x 32 took 3.5 ms
+// beside threads that spin on every core, and 1.1 ms otherwise).
+struct Ranks {
+  int ncol = 0, M = 0, rstar = 0;
+  std::vector<double> U, s, V, R1, t, C;
+  std::vector<char> ok;  // rank rstar - k has coefficients C + k M
+  std::atomic<int> next{0};
+  std::atomic<bool> failed{false};
+  std::mutex lock;
+  std::condition_variable all;
+  int done = 0;
+
+  bool candidate(int r, double* cv) const {
+    std::vector<double> VS((size_t)M * r);  // V_r Sigma_r^-1
+    for (int i = 0; i < M; ++i)
+      for (int k = 0; k < r; ++k) VS[(size_t)i * r + k] = V[(size_t)i * M + k] / s[k];
+    std::vector<double> X((size_t)ncol * r, 0.0);  // R1 V_r Sigma_r^-1
+    for (int i = 0; i < ncol; ++i)
+      for (int k = 0; k < r; ++k) {
+        double a = 0;
+        for (int l = 0; l < M; ++l) a += R1[(size_t)i * M + l] * VS[(size_t)l * r + k];
+        X[(size_t)i * r + k] = a;
+      }
+    std::vector<double> At((size_t)r * r, 0.0);  // U_r^T X
+    for (int a = 0; a < r; ++a)
+      for (int b = 0; b < r; ++b) {
+        double v = 0;
+        for (int i = 0; i < ncol; ++i) v += U[(size_t)i * M + a] * X[(size_t)i * r + b];
+        At[(size_t)a * r + b] = v;
+      }
+    std::vector<la::cd> lam, W;
+    if (!la::eig_general(r, At, lam, W)) return false;
+    int q1 = 0;
+    double best = 1e300;
+    for (int q = 0; q < r; ++q) {
+      const double w = std::abs(std::log(lam[q]));
+      if (w < best) {
+        best = w;
+        q1 = q;
+      }
+    }
+    std::vector<double> cp = la::lstsq_svd(ncol, r, X, t);
+    std::vector<la::cd> bvec(cp.begin(), cp.end());
+    if (!la::csolve(r, W, bvec)) return false;
+    const la::cd b1 = bvec[q1];
+    for (int l = 0; l < M; ++l) {
+      la::cd a = 0;
+      for (int k = 0; k < r; ++k) a += VS[(size_t)l * r + k] * W[(size_t)k * r + q1];
+      cv[l] = std::real(b1 * a);
+    }
+    return true;
+  }
+  void work() noexcept {
+    for (int k = next++; k < rstar; k = next++) {
+      try {
+        ok[k] = candidate(rstar - k, C.data() + (size_t)k * M);
+      } catch (...) {
+        failed = true;
+      }
+      const std::lock_guard<std::mutex> g(lock);
+      if (++done == rstar) all.notify_all();
+    }
+  }
+  void wait() {
+    std::unique_lock<std::mutex> g(lock);
+    all.wait(g, [&] { return done == rstar; });
+  }
+};
+// Helpers for P while seven at most run or wait for a core.
+void start_helpers(pcf_ctx* c, const std::shared_ptr<Ranks>& P) {
+  const auto ended = [](pcf_ctx::Helper& h) {
+    if (!h.ended->load()) return false;
+    h.thread.join();
+    return true;
+  };
+  c->helpers.erase(std::remove_if(c->helpers.begin(), c->helpers.end(), ended), c->helpers.end());
+  try {
+    c->helpers.reserve(7);
+    const size_t want = std::min(P->rstar, 8) - 1;
+    while (c->helpers.size() < want) {
+      auto end = std::make_shared<std::atomic<bool>>(false);
+      c->helpers.push_back({std::thread([P, end] {
+                              P->work();
+                              *end = true;
+                            }),
+                            end});
+    }
+  } catch (...) {  // no more threads: the others and the caller take the rest
+  }
+}
+
 }  // namespace
 
 extern "C" {
@@ -517,78 +614,27 @@ pcf_status pcf_dmd_extrapolate(pcf_ctx* c, const double* S, long long ld, int M,
     }
     t[i] = R[(size_t)i * ncol + M];
   }
-  std::vector<double> U, s, V;
-  la::svd_jacobi(ncol, M, R0, U, s, V);
+  auto P = std::make_shared<Ranks>();
+  P->ncol = ncol;
+  P->M = M;
+  la::svd_jacobi(ncol, M, R0, P->U, P->s, P->V);
   int rstar = 0;
   for (int k = 0; k < M; ++k)
-    if (s[k] > rank_tol * s[0]) ++rstar;
+    if (P->s[k] > rank_tol * P->s[0]) ++rstar;
   if (rstar == 0) return PCF_ENAN;
   // candidates r = rstar .. 1: coefficient vectors over the snapshots s_1..s_M
-  std::vector<double> Cc((size_t)rstar * M, 0.0);
+  P->rstar = rstar;
+  P->R1 = std::move(R1);
+  P->t = std::move(t);
+  P->C.assign((size_t)rstar * M, 0.0);
+  P->ok.assign(rstar, 0);
   std::vector<int> rank_of(rstar);
-  // the ranks are independent small dense problems: one host thread each, at most eight (about
-  // 60 us apiece at 20 snapshots)
-  const auto candidate = [&](int r, double* cv) -> bool {
-    std::vector<double> VS((size_t)M * r);  // V_r Sigma_r^-1
-    for (int i = 0; i < M; ++i)
-      for (int k = 0; k < r; ++k) VS[(size_t)i * r + k] = V[(size_t)i * M + k] / s[k];
-    std::vector<double> X((size_t)ncol * r, 0.0);  // R1 V_r Sigma_r^-1
-    for (int i = 0; i < ncol; ++i)
-      for (int k = 0; k < r; ++k) {
-        double a = 0;
-        for (int l = 0; l < M; ++l) a += R1[(size_t)i * M + l] * VS[(size_t)l * r + k];
-        X[(size_t)i * r + k] = a;
-      }
-    std::vector<double> At((size_t)r * r, 0.0);  // U_r^T X
-    for (int a = 0; a < r; ++a)
-      for (int b = 0; b < r; ++b) {
-        double v = 0;
-        for (int i = 0; i < ncol; ++i) v += U[(size_t)i * M + a] * X[(size_t)i * r + b];
-        At[(size_t)a * r + b] = v;
-      }
-    std::vector<la::cd> lam, W;
-    if (!la::eig_general(r, At, lam, W)) return false;
-    int q1 = 0;
-    double best = 1e300;
-    for (int q = 0; q < r; ++q) {
-      const double w = std::abs(std::log(lam[q]));
-      if (w < best) {
-        best = w;
-        q1 = q;
-      }
-    }
-    std::vector<double> cp = la::lstsq_svd(ncol, r, X, t);
-    std::vector<la::cd> bvec(cp.begin(), cp.end());
-    if (!la::csolve(r, W, bvec)) return false;
-    const la::cd b1 = bvec[q1];
-    for (int l = 0; l < M; ++l) {
-      la::cd a = 0;
-      for (int k = 0; k < r; ++k) a += VS[(size_t)l * r + k] * W[(size_t)k * r + q1];
-      cv[l] = std::real(b1 * a);
-    }
-    return true;
-  };
-  std::vector<char> ok(rstar, 0);
-  std::atomic<int> next(0);
-  std::atomic<bool> failed(false);
-  const auto work = [&]() noexcept {
-    try {
-      for (int k = next++; k < rstar; k = next++) ok[k] = candidate(rstar - k, Cc.data() + (size_t)k * M);
-    } catch (...) {
-      failed = true;
-    }
-  };
-  {
-    std::vector<std::thread> pool;
-    try {
-      pool.reserve(7);
-      for (int t = 1; t < std::min(rstar, 8); ++t) pool.emplace_back(work);
-    } catch (...) {  // no more threads: the others and this one take the rest
-    }
-    work();
-    for (std::thread& t : pool) t.join();
-  }
-  if (failed) return PCF_ENOMEM;
+  start_helpers(c, P);
+  P->work();
+  P->wait();
+  if (P->failed) return PCF_ENOMEM;
+  std::vector<double>& Cc = P->C;
+  const std::vector<char>& ok = P->ok;
   int ncand = 0;
   for (int k = 0; k < rstar; ++k)
     if (ok[k]) {

@@ -1345,6 +1345,7 @@ int pcf_solve_variant(const pcf_ctx* c) {
 
 void pcf_destroy(pcf_ctx* c) {
   if (!c) return;
+  for (pcf_ctx::Helper& h : c->helpers) h.thread.join();
   if (c->dmd_eval) pcf_destroy(c->dmd_eval);
   if (c->cs) cudaStreamSynchronize(c->cs);
   for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);

@@ -1,0 +1,52 @@
+"""A DMD jump beside threads that keep every core busy: the call's host helpers get a core late, and the
+call does not wait for them.  The bound is an idle machine's time plus 1 ms, less than one time slice of
+a thread that waits for a core."""
+import os
+import subprocess
+import sys
+import time
+
+import numpy as np
+import pytest
+
+import pcf_inputs as gi
+from oracle import PCFOracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def test_time_on_busy_cores():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2306_00165_gb300 as pcf
+    pcf.load_library()
+    grid = (32, 33, 32)
+    o = PCFOracle(*grid)
+    rng = np.random.default_rng(0)
+    star = o.to_psi(gi.random_perturbation(*grid, 0.05, 1))
+    a = 0.01 * rng.standard_normal((5, o.psi_dim()))
+    S = np.stack([star + np.linspace(0.5, 0.95, 5) ** k @ a for k in range(21)])
+    S, s = torch.from_numpy(S).cuda(), pcf.Solver(*grid)
+
+    def best(n):
+        t = []
+        for _ in range(n):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            u, r, J = s.dmd_extrapolate(S, rank_tol=1e-10)
+            t.append(time.perf_counter() - t0)
+        return min(t), (u.clone(), r, J)
+    time.sleep(0.5)  # threads of the array library stop spinning
+    idle, first = best(10)
+    spin = [subprocess.Popen([sys.executable, "-c", "while True: pass"]) for _ in range(os.cpu_count())]
+    try:
+        time.sleep(0.5)
+        busy, again = best(20)
+    finally:
+        for p in spin:
+            p.kill()
+            p.wait()
+    assert torch.equal(first[0], again[0]) and first[1:] == again[1:]
+    assert busy <= idle + 1e-3
+    s.close()
