@@ -224,7 +224,10 @@ __global__ void k_sum_parts(const float* part, int G, int E, float* out, int acc
 // and load latency: 584 us at 190 modes, W = 32, F = 132, 32 samples).  What bounds it now: the
 // chain of about 20 small products with a barrier each; weights and gradients cross HBM once.
 // Samples go 32 at a time; the weight gradients of later chunks continue the accumulators of
-// the earlier ones.  Every product rounds the same FP32 values to BF16 and accumulates K in the
+// the earlier ones.  In the forward pass, which carries nothing from chunk to chunk, blockIdx.y shares
+// them out while the modes alone leave the GPU less than two CTAs per SM: 45 modes of 1024 samples (W =
+// 32, F = 68) took 216 us on 45 CTAs and 58 so; the products by k_gemm_bf16 take 157.  The gradient's
+// chunks stay with their mode (699 us there, by products 1333).  Every product rounds the same FP32 values to BF16 and accumulates K in the
 // same 16-wide steps as k_gemm_bf16, so the two paths give the same bits in every per-mode
 // output.
 constexpr int kFnoThreads = 256, kFnoS = 32;
@@ -339,7 +342,7 @@ __global__ void __launch_bounds__(kFnoThreads, 2) k_fno_mode(FnoFused f) {
     Wb[(l * W + r) * PW + c] = __float2bfloat16_rn(f.w[f.oR[l] + (size_t)mp * W * W + e] + f.w[f.oL[l] + e]);
   }
   double loss = 0.0;
-  for (int s0 = 0; s0 < S; s0 += kFnoS) {
+  for (int s0 = blockIdx.y * kFnoS; s0 < S; s0 += gridDim.y * kFnoS) {
     const int ns = min(kFnoS, S - s0);
     const bool first = s0 == 0;
     const float* Xg = f.X + ((size_t)mp * S + s0) * F;
@@ -578,7 +581,7 @@ using namespace pcf;
 
 // ------------------------------------------------------------------ network object
 struct pcf_fno {
-  int MP, NY, W, L, CI;
+  int MP, NY, W, L, CI, sms = 0;
   cudaStream_t s = nullptr;
   long long np = 0;
   std::vector<long long> off;  // parameter offsets: P bP Q bQ, then per layer R L K b
@@ -658,7 +661,8 @@ pcf_status fused(pcf_fno* f, const float* X, const float* T, int S, float* Y, fl
   a.sc = 2.f / (float)((long long)f->MP * S * a.F);
   const size_t sm = fused_smem(f, T != nullptr);
   if (raise_smem_limit((const void*)k_fno_mode, sm) != cudaSuccess) return PCF_ECUDA;
-  k_fno_mode<<<f->MP, kFnoThreads, sm, f->s>>>(a);
+  const int chunks = (S + kFnoS - 1) / kFnoS, parts = T ? 1 : std::max(1, std::min(chunks, 2 * f->sms / f->MP));
+  k_fno_mode<<<dim3(f->MP, parts), kFnoThreads, sm, f->s>>>(a);
   if (T) {
     const int n = f->L * f->W * f->W + (f->L + 1) * f->W;
     k_fno_shared<<<(n + 31) / 32, 256, 0, f->s>>>(a);
@@ -759,6 +763,11 @@ pcf_status pcf_fno_create(int MP, int NY, int width, int layers, unsigned long l
   pcf_fno* f = new pcf_fno();
   f->MP = MP; f->NY = NY; f->W = width; f->L = layers; f->CI = 4;
   f->s = (cudaStream_t)stream;
+  int dev = 0;
+  if (cudaGetDevice(&dev) || cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev)) {
+    delete f;
+    return PCF_ECUDA;
+  }
   const int W = width, F = NY * 4;
   long long o = 0;
   auto add = [&](long long n) { f->off.push_back(o); o += n; };
