@@ -227,9 +227,8 @@ __global__ void k_sum_parts(const float* part, int G, int E, float* out, int acc
 // the earlier ones.  In the forward pass, which carries nothing from chunk to chunk, blockIdx.y shares
 // them out while the modes alone leave the GPU less than two CTAs per SM: 45 modes of 1024 samples (W =
 // 32, F = 68) took 216 us on 45 CTAs and 58 so; the products by k_gemm_bf16 take 157.  The gradient's
-// chunks stay with their mode (699 us there, by products 1333).  Every product rounds the same FP32 values to BF16 and accumulates K in the
-// same 16-wide steps as k_gemm_bf16, so the two paths give the same bits in every per-mode
-// output.
+// chunks stay with their mode (699 us there, by products 1333).  Every product rounds the same FP32
+// values to BF16 as k_gemm_bf16 does; the tests hold both to one reference that rounds there.
 constexpr int kFnoThreads = 256, kFnoS = 32;
 
 struct FnoFused {
