@@ -185,12 +185,12 @@ long long pcf_state_offset(const pcf_ctx* ctx, int instance);
 int pcf_mode_tile(const pcf_ctx* ctx);
 
 /* Stokes solve the descent step uses: 0 banded tau sweeps inside the per-mode kernel, 1 dense
- * per-mode operators inside one kernel per half-step (the mixed form's per-mode kernel; the
- * FP64 forms' fused kernel), 2 dense operators between separate analysis and synthesis kernels,
- * 3 the fused kernel with J in a kernel of its own, 4 banded sweeps with one thread per chain
- * between the separate kernels.  With solve_kind 0 the FP64 forms take 1 where the solve has at
- * most 228 CTAs and no reduced symmetric state, else 2; the mixed form times 0 against 1 at
- * creation.  -1 for a NULL context. */
+ * per-mode operators inside one kernel per half-step (the mixed form's per-mode kernel; the FP64
+ * forms with solve_kind 2), 2 dense operators between separate analysis and synthesis kernels, 3
+ * dense operators in the fused per-mode half-step kernel over instance groups (FP64 forms with
+ * solve_kind 4, or 0 where the solve has at most 228 CTAs and no reduced symmetric state), 4 banded
+ * sweeps with one thread per chain between the separate kernels.  The mixed form times 0 against 1
+ * at creation.  -1 for a NULL context. */
 int pcf_solve_variant(const pcf_ctx* ctx);
 
 /* x-z plane kernels the context launches: 0 shared-memory Stockham passes, 1 transforms in
@@ -409,10 +409,10 @@ pcf_status pcf_probe_fp64_peak(void* stream, double* gflops);
  * only the Stokes solve). */
 pcf_status pcf_set_kernel_timing(pcf_ctx* ctx, int enable);
 
-/* Organisation of the FP64 forms' per-mode kernels: cfg[0] instances per group of the solve,
- * cfg[1] and cfg[2] modes per CTA of the separate analysis and synthesis kernels, cfg[3]
- * instances per group of the separate dense solve.  Zeros where the context does not use those
- * kernels.  cfg: host int[4]. */
+/* Organisation of the FP64 forms' per-mode kernels: cfg[0] instances per group of the analysis and
+ * synthesis (separate kernels: 1; the fused kernel's groups), cfg[1] and cfg[2] modes per CTA of the
+ * separate analysis and synthesis kernels, cfg[3] instances per group of the separate dense solve.
+ * Zeros where the context does not use those kernels.  cfg: host int[4]. */
 pcf_status pcf_split_config(const pcf_ctx* ctx, int* cfg);
 
 /* Kernel launches of one pcf_descent_step call of nsteps steps (the entry synthesis, and

@@ -367,7 +367,7 @@ class Solver:
 
     def solve_variant(self):
         """0 banded sweeps and 1 dense operators in one kernel per half-step, 2 dense operators and 4 banded
-        sweeps between separate transforms, 3 as 1 with a separate J kernel."""
+        sweeps between separate transforms, 3 the fused half-step kernel (see include/pcfadj.h)."""
         return int(self.lib.pcf_solve_variant(self._h))
 
     def launches_per_step(self):

@@ -1339,7 +1339,7 @@ int pcf_symmetric_modes(const pcf_ctx* c) {
 
 int pcf_solve_variant(const pcf_ctx* c) {
   if (!c) return -1;
-  if (c->split) return c->fused ? (c->jn ? 3 : 1) : (c->sweep ? 4 : 2);
+  if (c->split) return c->fused ? (c->prm.solve_kind == 2 ? 1 : 3) : (c->sweep ? 4 : 2);
   return c->hinst[0].dense[0] ? 1 : 0;
 }
 
@@ -1657,7 +1657,7 @@ pcf_status pcf_norm(pcf_ctx* c, const double* u, double* out) {
 pcf_status pcf_split_config(const pcf_ctx* c, int* cfg) {
   if (!c || !cfg) return PCF_EINVAL;
   const bool tiles = c->split && !c->fused;
-  cfg[0] = c->split ? c->sgrp : 0;
+  cfg[0] = tiles ? 1 : c->split ? c->sgrp : 0;
   cfg[1] = cfg[2] = tiles ? c->np : 0;
   cfg[3] = tiles && !c->sweep ? c->sgrp : 0;
   return PCF_OK;
