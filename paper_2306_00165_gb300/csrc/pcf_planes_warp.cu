@@ -38,12 +38,6 @@ __device__ __forceinline__ float2 cshfl(float2 v, int s) {
 __device__ __forceinline__ float2 cshflx(float2 v, int m) {
   return make_float2(__shfl_xor_sync(kFull, v.x, m), __shfl_xor_sync(kFull, v.y, m));
 }
-__device__ __forceinline__ double2 cshfl(double2 v, int s) {
-  return make_double2(__shfl_sync(kFull, v.x, s), __shfl_sync(kFull, v.y, s));
-}
-__device__ __forceinline__ double2 cshflx(double2 v, int m) {
-  return make_double2(__shfl_xor_sync(kFull, v.x, m), __shfl_xor_sync(kFull, v.y, m));
-}
 
 // Twiddles of the 32-point stage of lane `lane`, forward sign: stage s (pair distance
 // h = 16 >> s) multiplies the upper lane's difference by W_32^{(lane mod h) 16/h}; tw is a
