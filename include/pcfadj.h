@@ -188,9 +188,9 @@ int pcf_mode_tile(const pcf_ctx* ctx);
  * per-mode operators inside one kernel per half-step (the mixed form's per-mode kernel; the FP64
  * forms with solve_kind 2), 2 dense operators between separate analysis and synthesis kernels, 3
  * dense operators in the fused per-mode half-step kernel over instance groups (FP64 forms with
- * solve_kind 4, or 0 where the solve has at most 228 CTAs and no reduced symmetric state), 4 banded
- * sweeps with one thread per chain between the separate kernels.  The mixed form times 0 against 1
- * at creation.  -1 for a NULL context. */
+ * solve_kind 4, or 0 where the solve has at most three CTAs for two SMs and no reduced symmetric
+ * state), 4 banded sweeps with one thread per chain between the separate kernels.  The mixed form
+ * times 0 against 1 at creation.  -1 for a NULL context. */
 int pcf_solve_variant(const pcf_ctx* ctx);
 
 /* x-z plane kernels the context launches: 0 shared-memory Stockham passes, 1 transforms in

@@ -26,6 +26,7 @@ struct pcf_ctx {
   pcf_params prm;
   GridTables gt;  // of the first problem
   int N, Kx, Kz, Mx, Mz, nm, B, mpc;
+  int sms = 0;          // multiprocessors of the device (152 where the launch rules were measured)
   long long state_len;  // complex values per instance (instance 0; all instances when uniform)
   std::vector<long long> state_off;  // complex offset of each instance's state, [B+1]
   long long total_state = 0;

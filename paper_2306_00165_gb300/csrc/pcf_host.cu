@@ -947,13 +947,13 @@ static pcf_status set_modes(pcf_ctx* c, int G) {
   // one row and one part per thread while the launch would otherwise leave SMs with less than
   // eight warps
   const int hp = (Nmax / 2 + 2) / 2;
-  c->fine_s = (long long)c->cta_ys * 6 * hp * gmax < 152LL * 256;
-  c->thr_ys = ysolve_fx_threads(Nmax, gmax, c->fine_s, c->cta_ys >= 5 * 152);
+  c->fine_s = (long long)c->cta_ys * 6 * hp * gmax < 256LL * c->sms;
+  c->thr_ys = ysolve_fx_threads(Nmax, gmax, c->fine_s, c->cta_ys >= 5 * c->sms);
   c->thr_yf = std::max(c->thr_ys, 256);
   // Eight modes per tile, sixteen where eight would leave a CTA of the synthesis less than four
   // warps of tasks and the tiles still give every SM four CTAs (32 x 33 x 32, batch 32: synthesis
   // 47 us against 51; 128 x 97 x 128 the other way: 121 against 122, analysis 67 against 77).
-  c->np = 8 * hp < 128 && 3 * (modes / 16) >= 4 * 152 ? 16 : 8;
+  c->np = 8 * hp < 128 && 3 * (modes / 16) >= 4 * c->sms ? 16 : 8;
   std::vector<int> pa(c->B), py(c->B), par(c->B), pyr(c->B);
   for (int b = 0; b < c->B; ++b) {
     const Inst& I = c->hinst[b];
@@ -969,7 +969,7 @@ static pcf_status set_modes(pcf_ctx* c, int G) {
   PCF_TRY(upload_prefix(c, pyr, &c->pre_yy_r, &c->cta_yy_r));
   c->sm_ya = smem_yana_fx(Nmax, c->np);
   c->sm_yy = smem_ysynth_fx(Nmax, c->np);
-  c->fine_y = (long long)c->cta_ya * c->np * 2 * hp < 152LL * 256;
+  c->fine_y = (long long)c->cta_ya * c->np * 2 * hp < 256LL * c->sms;
   c->thr_ya = yana_fx_threads(Nmax, c->np, c->fine_y);
   c->thr_yy = ysynth_fx_threads(Nmax, c->np, c->fine_y);
   PCF_CUDA(set_modes_fx_smem(c->sm_ya, c->sm_yy, c->sm_ys, c->sm_yf, c->sm_y64));
@@ -1051,14 +1051,15 @@ static int solve_group(const pcf_ctx* c) {
   while (G > 1) {
     long long ctas = 0;
     for (const int2& q : make_groups(c, G)) ctas += c->hinst[q.x].nmodes;
-    if (ctas >= 2 * 152) break;
+    if (ctas >= 2 * c->sms) break;
     G /= 2;
   }
   return G;
 }
 
-// The fused half-step (two launches fewer per half-step) wins where the launches dominate.
-static bool fused_step_pays(const pcf_ctx* c) { return c->cta_ys <= 228; }
+// The fused half-step (two launches fewer per half-step) wins where the launches dominate, up to
+// three CTAs for two SMs.
+static bool fused_step_pays(const pcf_ctx* c) { return 2 * c->cta_ys <= 3 * c->sms; }
 
 // Grids whose Chebyshev tables and one mode's scratch exceed a CTA's shared memory in the FP64
 // per-mode kernel (ny above 125) are refused in the FP64 forms.
@@ -1097,6 +1098,10 @@ static pcf_status create_batch(const pcf_params* list, int nlist, void* stream, 
     pcf_destroy(c);
     return s;
   };
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return fail(PCF_ECUDA);
   if (cudaStreamCreateWithFlags(&c->cs, cudaStreamNonBlocking) != cudaSuccess) return fail(PCF_ECUDA);
   if (cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming) != cudaSuccess) return fail(PCF_ECUDA);
   if (cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming) != cudaSuccess) return fail(PCF_ECUDA);
