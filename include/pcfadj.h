@@ -33,7 +33,8 @@
  * unless noted; nothing aborts the process.
  *
  * Grids: nx, nz even products of 2 and 3 from 16 to 128 (16, 18, 24, 32, 36, 48, 54, 64, 72, 96,
- * 108, 128), ny odd with 9 <= ny <= 129; batch >= 1.
+ * 108, 128), ny odd with 9 <= ny <= 129; batch >= 1.  The FP64 and float-float forms take ny up to
+ * 125 and the mixed form up to 113 (PCF_ENOTSUP above).
  */
 #ifndef PCFADJ_H
 #define PCFADJ_H
@@ -57,9 +58,14 @@ typedef enum {
 
 typedef enum {
   PCF_FP64 = 0,         /* the plain method: FP64 state, tables and results.  The transforms,
-                           products and Stokes solves run in 64-bit fixed point with block
-                           exponents (units of 2^-60 of a plane's and 2^-55 of a column's sum of
-                           magnitudes), which is no coarser than FP64 arithmetic there */
+                           products and the steps' Stokes solves run in 64-bit fixed point with
+                           block exponents: a unit is 2^-61 of the sum of a plane's (x stage: a
+                           row's) magnitudes, and a matrix product is good to 2^-56 of its row's
+                           largest entry times its column's sum.  Fields, norms and Fourier modes
+                           come out as accurate as in FP64 arithmetic; a Chebyshev coefficient far
+                           below its column's sum has fewer digits than FP64 arithmetic alone
+                           would leave it, and magnitudes below the normal range count as zero.
+                           pcf_influence_matrix_solve works in FP64 */
   PCF_MIXED = 1,        /* FP32 x-z transforms and products, split-BF16 tensor-core Chebyshev
                            transforms, FP64 Stokes solves, norms and state; ny <= 113
                            (PCF_ENOTSUP above) */

@@ -3,10 +3,10 @@
 // GB300 issues 1.67 FP64 multiply-adds per clock and SM, but 58 64-bit integer additions, 31
 // high products of 32-bit words and 24 32 x 32 + 64 multiply-adds (measured with independent
 // chains on every SM).  A transform whose data are 64-bit integers with one exponent per block
-// (a plane, a row, a column) therefore runs several times faster than in FP64, and its rounding
-// is finer: blocks are scaled from the sum of the magnitudes that enter them, so that a unit is
-// about 2^-60 of that sum where FP64 rounds at 2^-53 of each intermediate.  Integer sums are
-// exact, so results do not depend on how the work is split.
+// (a plane, a row, a column) therefore runs several times faster than in FP64, and the block as a
+// whole is rounded more finely: blocks are scaled from the sum of the magnitudes that enter them, so
+// that a unit is about 2^-60 of that sum.  A value far below its block's sum has fewer digits than
+// FP64 would give it.  Integer sums are exact, so results do not depend on how the work is split.
 //
 // Conventions: a block value is X 2^e with X a signed 64-bit integer, |X| < 2^62 wherever a
 // complex rotation follows; a block that holds an infinity or a NaN is marked (kFxNan) and
@@ -48,7 +48,7 @@ PCF_HD int fx_hi(fx x) { return (int)((x + 0x80000000LL) >> 32); }
 PCF_HD int fx_lo(fx x) { return (int)(uint32_t)(uint64_t)x; }
 
 // round(x (h 2^32 + l) 2^-62): the cross products are summed in 64 bits and rounded once; the
-// product of the low words is below a quarter of the unit.
+// product of the low words, left out, is at most one unit and zero on average.
 PCF_HD fx fx_mulc(fx x, int h, int l) {
   const int xh = fx_hi(x), xl = fx_lo(x);
   const fx t = (fx)xh * l + (fx)xl * h + (1LL << 29);
