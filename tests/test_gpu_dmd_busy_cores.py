@@ -1,6 +1,6 @@
 """A DMD jump beside threads that keep every core busy: the call's host helpers get a core late, and the
-call does not wait for them.  The bound is an idle machine's time plus 1 ms, less than one time slice of
-a thread that waits for a core."""
+call does not wait for them.  The bound is an idle machine's time plus 2 ms, less than one time slice
+(about 3 ms) of a thread that a new one waits for."""
 import os
 import subprocess
 import sys
@@ -48,5 +48,5 @@ def test_time_on_busy_cores():
             p.kill()
             p.wait()
     assert torch.equal(first[0], again[0]) and first[1:] == again[1:]
-    assert busy <= idle + 1e-3
+    assert busy <= idle + 2e-3
     s.close()

@@ -46,12 +46,13 @@ def test_result_does_not_depend_on_the_evaluation_batch(pcf, batch, precision):
 
 
 def test_low_rank_costs_less_than_full_rank(pcf):
-    """Two candidates of 64 x 65 x 64 take well under the time of eleven; with every spare instance
-    evaluated as well both took that of twenty."""
+    """Two candidates of 64 x 65 x 64 take well under the time of twenty; with every spare instance
+    evaluated as well both took about that."""
     grid = (64, 65, 64)
     s, times = pcf.Solver(*grid), []
-    sets = [_snapshots(grid, 19, 20), _snapshots(grid, 1, 20)]
-    for S in sets:
+    low = _snapshots(grid, 1, 20)
+    noise = torch.randn(low.shape, dtype=low.dtype, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    for S in (low + 1e-3 * low.abs() * noise, low):
         best = np.inf
         for _ in range(6):
             torch.cuda.synchronize()
