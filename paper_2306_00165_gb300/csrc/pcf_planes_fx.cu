@@ -321,6 +321,9 @@ __global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_syn
   }
   const int e0 = eb + ek - 61;
   const FxPlan px = fx_plan_of<KIND>(nx);
+  // kept for the end of the kernel (in a register it made the 80-register variant spill: uneven batch of
+  // 64, 789 us a launch against 768)
+  if (KIND == FX_SMALL && threadIdx.x == 0) row[63] = e0;
   // a row's values are below 2^(row - 1022) (times 2^(ek + 1) for a derivative) in each part, and a
   // transform of its Mx modes below 2^cr times that
   const int cr = 32 - __clz((3 * I.Mx) >> 1) - 1022 - 62 + (fac ? ek + 1 : 0);
@@ -403,7 +406,7 @@ __global__ void __launch_bounds__(FxCfg<KIND>::threads, FxCfg<KIND>::ctas) k_syn
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mh = max(mh, (unsigned)red[w]);
-    *info = make_int2(e0, fx_bits(mh));
+    *info = make_int2(KIND == FX_SMALL ? row[63] : e0, fx_bits(mh));
   }
 }
 
